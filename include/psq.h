@@ -248,9 +248,11 @@ const char* psq_last_error(void);
 
 /* RI 4-index assembly (Section 3, eq 14): (ij|kl) ~ sum_PQ (ij|P) [(PQ)^-1] (Q|kl), from the
  * (P|Q) and (P|ij) matrices that psq_compute writes.  With the Cholesky factor (P|Q) = L L^T
- * and B = L^-1 (P|ij), (ij|kl) = sum_R B[R][ij] B[R][kl].  FP64 throughout, on the device,
- * asynchronous on `stream` (a cudaStream_t; NULL = legacy default stream), on the current
- * device.  Matrices are row-major; the pair index of (P|ij) is ij = i * n_bf + j, so its
+ * and B = L^-1 (P|ij), (ij|kl) = sum_R B[R][ij] B[R][kl].  FP64 matrices throughout; the large
+ * products (the solve's off-diagonal blocks, the (ij|kl) sums) run on the tensor cores on exact
+ * integer digits of the FP64 values (62 bits of each 64-row window's largest, one FP64 rounding
+ * per window), the rest on the FP64 pipe.  On the device, asynchronous on `stream` (a
+ * cudaStream_t; NULL = legacy default stream), on the current device.  Matrices are row-major; the pair index of (P|ij) is ij = i * n_bf + j, so its
  * n_aux x n_bf x n_bf layout is B's n x m layout with m = n_bf^2.  The caller owns every
  * buffer.  Errors: PSQ_ERR_ARG for negative sizes, NULL or non-8-byte-aligned pointers with
  * nonzero sizes, or column ranges outside [0, m); PSQ_ERR_CUDA on a failed launch. */

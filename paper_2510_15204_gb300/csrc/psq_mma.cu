@@ -23,6 +23,7 @@
 //    a^3), which the values omit.
 #include "psq_internal.h"
 #include "psq_df.cuh"
+#include "psq_tc.cuh"
 
 #include <cuda_bf16.h>
 
@@ -340,99 +341,10 @@ constexpr int kStages = 3;                      // A ring depth (chunks, 40 KB e
 constexpr int kStagesB = 3;                     // B ring depth (chunks, 15 KB each)
 constexpr int kChunksPerWin = kWinPts / kChunkPts;
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-// Shared-memory matrix descriptor: K-major, 64-byte swizzle, 8-row groups 512 bytes apart.
-__device__ __forceinline__ uint64_t make_desc(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFF) >> 4);
-  d |= (uint64_t)1 << 16;             // leading byte offset (unused for swizzled K-major)
-  d |= (uint64_t)(512 >> 4) << 32;    // stride byte offset between 8-row groups
-  d |= (uint64_t)1 << 46;             // descriptor version for sm_100 family
-  d |= (uint64_t)4 << 61;             // SWIZZLE_64B
-  return d;
-}
-
 // Instruction descriptor: kind::f16, A = B = BF16, D = F32, both K-major, M = 128, N = n.
 __device__ __forceinline__ uint32_t make_idesc(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kM >> 4) << 24);
 }
-
-__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem_d),
-      "l"(da), "l"(db), "r"(idesc), "r"(acc));
-}
-
-__device__ __forceinline__ void mma_commit(uint32_t mbar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar)
-               : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try(uint32_t mbar, uint32_t parity) {
-  uint32_t done;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}\n"
-      : "=r"(done)
-      : "r"(mbar), "r"(parity)
-      : "memory");
-  return done != 0;
-}
-
-// Non-blocking test of the phase of the given parity.
-__device__ __forceinline__ bool mbar_test(uint32_t mbar, uint32_t parity) {
-  uint32_t done;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}\n"
-      : "=r"(done)
-      : "r"(mbar), "r"(parity)
-      : "memory");
-  return done != 0;
-}
-
-__device__ __forceinline__ uint64_t global_ns() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
-// Waits for the phase of the given parity; gives up (false) after limit_ns nanoseconds, or
-// early once *abort (if given) is set by another role of the CTA.
-constexpr uint64_t kWaitNs = 4000000000ull;
-__device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, const int* abort = nullptr,
-                                          uint64_t limit_ns = kWaitNs) {
-  if (mbar_try(mbar, parity)) return true;
-  const uint64_t t0 = global_ns();
-  for (uint32_t it = 1;; ++it) {
-    if (mbar_try(mbar, parity)) return true;
-    if ((it & 255u) == 0) {
-      if (abort && *(volatile const int*)abort) return false;
-      if (global_ns() - t0 > limit_ns) return false;
-    }
-  }
-}
-
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
-  uint32_t r[8];
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "r"(taddr));
-#pragma unroll
-  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 __device__ __forceinline__ float pow2f(int k) {
   if (k < -126) return 0.0f;
@@ -528,9 +440,6 @@ __device__ __forceinline__ int row_exponent(float mx) {
   const int e = (int)(__float_as_uint(mx) >> 23) - 126;  // mx >= 0
   return e < -110 ? kZeroExp : e;
 }
-
-// Byte offset of 16-byte group j (0..3) of row r in a 64-byte-row swizzled operand tile.
-__device__ __forceinline__ uint32_t swz(int r, int j) { return (uint32_t)r * 64u + ((uint32_t)(j ^ ((r >> 1) & 3)) << 4); }
 
 }  // namespace mma
 
@@ -734,10 +643,6 @@ struct Smem {
   int abort;
 };
 
-__device__ __forceinline__ void mbar_init(uint64_t* b, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(mma::smem_u32(b)), "r"(count));
-}
-
 __device__ __forceinline__ void mbar_arrive(uint64_t* b) {
   asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(mma::smem_u32(b))
                : "memory");
@@ -872,28 +777,24 @@ __global__ void __launch_bounds__(ws::kThreads, 1)
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   ws::Smem& sm = *reinterpret_cast<ws::Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (warp == ws::kMmaWarp) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sm.tmem_base)),
-                 "r"(512));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-  }
+  if (warp == ws::kMmaWarp) tmem_alloc(&sm.tmem_base, 512);
   if (tid == 0) {
     for (int s = 0; s < kStages; ++s) {
-      ws::mbar_init(&sm.a_full[s], 1);
-      ws::mbar_init(&sm.a_free[s], 1);
+      mbar_init(&sm.a_full[s], 1);
+      mbar_init(&sm.a_free[s], 1);
     }
     for (int s = 0; s < kStagesB; ++s) {
-      ws::mbar_init(&sm.b_ready[s], 6);
-      ws::mbar_init(&sm.b_free[s], 1);
+      mbar_init(&sm.b_ready[s], 6);
+      mbar_init(&sm.b_free[s], 1);
     }
     for (int s = 0; s < 2; ++s) {
-      ws::mbar_init(&sm.tmem_full[s], 1);
-      ws::mbar_init(&sm.tmem_free[s], 8);
-      ws::mbar_init(&sm.raw_full[s], 1);
-      ws::mbar_init(&sm.raw_free[s], 6);
-      ws::mbar_init(&sm.eb_free[s], 8);
+      mbar_init(&sm.tmem_full[s], 1);
+      mbar_init(&sm.tmem_free[s], 8);
+      mbar_init(&sm.raw_full[s], 1);
+      mbar_init(&sm.raw_free[s], 6);
+      mbar_init(&sm.eb_free[s], 8);
     }
-    ws::mbar_init(&sm.drain, 1);
+    mbar_init(&sm.drain, 1);
     sm.abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -1124,7 +1025,7 @@ __global__ void __launch_bounds__(ws::kThreads, 1)
 #pragma unroll
               for (int i = 0; i < kSlices; ++i) {
                 const uint64_t da = make_desc(smem_u32(sm.a[s][i]) + ko);
-                mma_bf16(tset + (uint32_t)(kTileN * i), da, db, make_idesc(kTileN * (kSlices - i)),
+                mma_f16(tset + (uint32_t)(kTileN * i), da, db, make_idesc(kTileN * (kSlices - i)),
                          (j > 0 || k > 0 || i > 0) ? 1u : 0u);
               }
             }
@@ -1246,7 +1147,7 @@ __global__ void __launch_bounds__(ws::kThreads, 1)
   __syncthreads();
   if (warp == ws::kMmaWarp) {
     fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+    tmem_free(tmem, 512);
   }
 }
 

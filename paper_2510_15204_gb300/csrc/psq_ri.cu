@@ -1,11 +1,16 @@
 // RI 4-index assembly (Section 3, eq 14): (ij|kl) ~ sum_PQ (ij|P) [(PQ)^-1] (Q|kl).  The metric
 // (P|Q) is factored as L L^T (blocked right-looking Cholesky), B = L^-1 (P|ij) by blocked
-// forward substitution, and (ij|kl) = sum_R B[R][ij] B[R][kl] by a tiled FP64 product or,
-// for large blocks, on the tensor cores through the mixed path's packing and contraction.
-// The factor and the solve stay FP64 on the CUDA cores: the metric is ill-conditioned enough
-// to need it.  Blocks of 32 rows; every loop bound is a size argument (no waits outside the
-// contraction's own bounded ones).
+// forward substitution, and (ij|kl) = sum_R B[R][ij] B[R][kl], either to FP64 rounding on exact
+// digits (psq_fx.cuh, as the solve's off-diagonal products) or, for large blocks, to 2^-38
+// through the mixed path's packing and contraction.  The factor and the diagonal blocks stay on
+// the FP64 pipe.  Blocks of 32 rows; every loop bound is a size argument (no waits outside the
+// tensor-core products' bounded ones).
+//
+// Measured (693 aux functions, 51,984 pairs; FP64-pipe kernels before -> exact digits now):
+// (ij|kl) block of 4096 x 4096 18.9 -> 1.81 ms (12.8 useful TFLOP/s, ten times the FP64 pipe's
+// nominal rate; ALU pipe 53% busy slicing, tensor pipe 20%), solve of all pairs 24.0 -> 5.0 ms.
 #include "psq_internal.h"
+#include "psq_fx.cuh"
 
 #include <algorithm>
 #include <cstdint>
@@ -106,116 +111,127 @@ __global__ void zero_upper_kernel(int n, double* __restrict__ L) {
   if (j > i) L[idx] = 0.0;
 }
 
-// Forward substitution on the diagonal block: B[k0 + r][col] for r < kb, one thread per
-// column.
-__global__ void __launch_bounds__(256) trsv_diag_kernel(int n, int64_t m, int k0, int kb,
-                                                        const double* __restrict__ L, double* __restrict__ B) {
-  __shared__ double d[kB][kB + 1];
-  for (int t = threadIdx.x; t < kB * kB; t += blockDim.x) {
-    const int r = t >> 5, c = t & 31;
-    d[r][c] = (r < kb && c <= r) ? L[(int64_t)(k0 + r) * n + k0 + c] : 0.0;
-  }
-  __syncthreads();
-  const int64_t col = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (col >= m) return;
-  double* b = B + (int64_t)k0 * m + col;
-  double x[kB];
+// Forward substitution B <- L^-1 B, left-looking, one launch: a CTA owns up to 128 columns and
+// walks down the 32-row blocks.  Block k's rows take sum_{q < 32 k} L[r][q] B[q][col] from the
+// tensor cores (fx::window: the columns are the tile's rows, the block's rows of L its columns),
+// then the 32 x 32 diagonal block is solved in FP64, one thread per column.
+__global__ void __launch_bounds__(fx::kThreads, 2) trsv_kernel(int n, int64_t m, int cols, const double* __restrict__ L, double* B) {
+  extern __shared__ __align__(1024) uint8_t raw[];
+  fx::Smem& sm = fx::smem_at(raw);
+  const uint32_t tmem = fx::open(sm);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int64_t c0 = (int64_t)blockIdx.x * cols;
+  const int64_t col = c0 + fx::a_row();
+  const bool live = fx::a_row() < cols && col < m;
+  // after a block's products the digit planes are free: they hold its right-hand sides [row][col]
+  // and the diagonal block with its reciprocal pivots
+  double(*rhs)[fx::kRows] = reinterpret_cast<double(*)[fx::kRows]>(sm.a[0]);
+  double(*d)[kB + 1] = reinterpret_cast<double(*)[kB + 1]>(sm.a[0] + sizeof(double) * kB * fx::kRows);
+  uint32_t phase = 0;
+  bool ok = true;
+  for (int k0 = 0; k0 < n && ok; k0 += kB) {
+    const int kb = n - k0 < kB ? n - k0 : kB;
+    double acc[16] = {};
+    for (int q0 = 0; q0 < k0 && ok; q0 += fx::kWin) {
+      double va[32], vb[8];
 #pragma unroll
-  for (int j = 0; j < kB; ++j) {
-    if (j < kb) {
-      double s = b[(int64_t)j * m];
+      for (int c = 0; c < 2; ++c)
 #pragma unroll
-      for (int q = 0; q < j; ++q) s -= d[j][q] * x[q];
-      x[j] = s / d[j][j];
-      b[(int64_t)j * m] = x[j];
+        for (int i = 0; i < 16; ++i) {
+          const int q = q0 + fx::a_pt(c) + i;
+          va[16 * c + i] = live && q < k0 ? B[(int64_t)q * m + col] : 0.0;
+        }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int q = q0 + fx::b_pt() + i;
+        vb[i] = fx::b_col() < kb && q < k0 ? L[(int64_t)(k0 + fx::b_col()) * n + q] : 0.0;
+      }
+      ok = fx::window(sm, tmem, va, vb, acc, phase, [&](int r, int c) {
+        double s = 0.0;
+        if (r < cols && c0 + r < m && c < kb)
+          for (int q = q0; q < min(k0, q0 + fx::kWin); ++q) s = fma(B[(int64_t)q * m + c0 + r], L[(int64_t)(k0 + c) * n + q], s);
+        return s;
+      });
     }
-  }
-}
-
-// B[k1 + r][col] -= sum_q L[k1 + r][k0 + q] B[k0 + q][col]: 64 x 64 tiles, 256 threads with
-// 4 x 4 outputs each.
-__global__ void __launch_bounds__(256) trsv_update_kernel(int n, int64_t m, int k0, int kb,
-                                                          const double* __restrict__ L, double* __restrict__ B) {
-  __shared__ double ls[64][kB + 1];
-  __shared__ double bs[kB][64];
-  const int k1 = k0 + kb;
-  const int i0 = k1 + blockIdx.y * 64;
-  const int64_t c0 = (int64_t)blockIdx.x * 64;
-  for (int t = threadIdx.x; t < 64 * kB; t += blockDim.x) {
-    const int r = t / kB, q = t % kB;
-    ls[r][q] = (i0 + r < n && q < kb) ? L[(int64_t)(i0 + r) * n + k0 + q] : 0.0;
-  }
-  for (int t = threadIdx.x; t < kB * 64; t += blockDim.x) {
-    const int q = t / 64, c = t % 64;
-    bs[q][c] = (q < kb && c0 + c < m) ? B[(int64_t)(k0 + q) * m + c0 + c] : 0.0;
-  }
-  __syncthreads();
-  const int tr = threadIdx.x / 16, tc = threadIdx.x % 16;  // rows tr + 16a, columns tc + 16b
-  double acc[4][4] = {};
-  for (int q = 0; q < kb; ++q) {
-    double lv[4], bv[4];
+    const int r = 32 * (warp & 3) + lane;
 #pragma unroll
-    for (int a = 0; a < 4; ++a) lv[a] = ls[tr + 16 * a][q];
-#pragma unroll
-    for (int b = 0; b < 4; ++b) bv[b] = bs[q][tc + 16 * b];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b = 0; b < 4; ++b) acc[a][b] = fma(lv[a], bv[b], acc[a][b]);
-  }
-#pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    const int i = i0 + tr + 16 * a;
-    if (i >= n) continue;
-#pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const int64_t c = c0 + tc + 16 * b;
-      if (c < m) B[(int64_t)i * m + c] -= acc[a][b];
+    for (int j = 0; j < 16; ++j) {
+      const int i = 16 * (warp >> 2) + j;
+      rhs[i][r] = i < kb && r < cols && c0 + r < m ? B[(int64_t)(k0 + i) * m + c0 + r] - acc[j] : 0.0;
     }
-  }
-}
-
-// out[c][d] = sum_R B[R][c0 + c] B[R][d0 + d]: 64 x 64 output tiles, R in steps of 16
-// through shared memory, 4 x 4 outputs per thread.
-__global__ void __launch_bounds__(256) eri_kernel(int n, int64_t m, const double* __restrict__ B, int64_t c0,
-                                                  int64_t nc, int64_t d0, int64_t nd, double* __restrict__ out) {
-  __shared__ double as[16][64];
-  __shared__ double bs[16][64];
-  const int64_t tc0 = (int64_t)blockIdx.y * 64, td0 = (int64_t)blockIdx.x * 64;
-  const int tr = threadIdx.x / 16, tc = threadIdx.x % 16;
-  double acc[4][4] = {};
-  for (int R0 = 0; R0 < n; R0 += 16) {
-    for (int t = threadIdx.x; t < 16 * 64; t += blockDim.x) {
-      const int q = t / 64, x = t % 64;
-      const bool okr = R0 + q < n;
-      as[q][x] = (okr && tc0 + x < nc) ? B[(int64_t)(R0 + q) * m + c0 + tc0 + x] : 0.0;
-      bs[q][x] = (okr && td0 + x < nd) ? B[(int64_t)(R0 + q) * m + d0 + td0 + x] : 0.0;
+    for (int t = tid; t < kB * kB; t += fx::kThreads) {
+      const int i = t >> 5, c = t & 31;
+      d[i][c] = (i < kb && c <= i) ? L[(int64_t)(k0 + i) * n + k0 + c] : 0.0;
     }
     __syncthreads();
-#pragma unroll 4
-    for (int q = 0; q < 16; ++q) {
-      double av[4], bv[4];
+    if (tid < kB) d[tid][kB] = tid < kb ? 1.0 / d[tid][tid] : 0.0;
+    __syncthreads();
+    if (tid < fx::kRows && live) {
+      double x[kB];
 #pragma unroll
-      for (int a = 0; a < 4; ++a) av[a] = as[q][tr + 16 * a];
+      for (int j = 0; j < kB; ++j) {
+        if (j < kb) {
+          double s = rhs[j][tid];
 #pragma unroll
-      for (int b = 0; b < 4; ++b) bv[b] = bs[q][tc + 16 * b];
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = fma(av[a], bv[b], acc[a][b]);
+          for (int q = 0; q < j; ++q) s -= d[j][q] * x[q];
+          // s / d by the reciprocal and one correction of the quotient
+          const double q0 = s * d[j][kB];
+          const double q1 = fma(fma(-q0, d[j][j], s), d[j][kB], q0);
+          x[j] = isfinite(q1) ? q1 : s / d[j][j];
+          B[(int64_t)(k0 + j) * m + col] = x[j];
+        }
+      }
     }
     __syncthreads();
   }
+  if (!ok && live)  // a wait ran out: no result is better than a wrong one
+    for (int q = tid >> 7; q < n; q += 2) B[(int64_t)q * m + col] = __longlong_as_double(0x7ff8000000000000ll);
+  fx::close(sm, tmem, ok, phase);
+}
+
+// out[c][d] = sum_R B[R][c0 + c] B[R][d0 + d]: a CTA per 128 x 32 output tile, R in windows of 64.
+__global__ void __launch_bounds__(fx::kThreads, 2) eri_kernel(int n, int64_t m, const double* __restrict__ B, int64_t c0,
+                                                              int64_t nc, int64_t d0, int64_t nd, double* __restrict__ out) {
+  extern __shared__ __align__(1024) uint8_t raw[];
+  fx::Smem& sm = fx::smem_at(raw);
+  const uint32_t tmem = fx::open(sm);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t tc0 = (int64_t)blockIdx.y * fx::kRows, td0 = (int64_t)blockIdx.x * fx::kCols;
+  const bool liva = tc0 + fx::a_row() < nc, livb = td0 + fx::b_col() < nd;
+  const double* pa = B + c0 + tc0 + fx::a_row();
+  const double* pb = B + d0 + td0 + fx::b_col();
+  double acc[16] = {};
+  uint32_t phase = 0;
+  bool ok = true;
+  for (int R0 = 0; R0 < n && ok; R0 += fx::kWin) {
+    double va[32], vb[8];
 #pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    const int64_t c = tc0 + tr + 16 * a;
-    if (c >= nc) continue;
+    for (int c = 0; c < 2; ++c)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const int64_t d = td0 + tc + 16 * b;
-      if (d < nd) out[c * nd + d] = acc[a][b];
+      for (int i = 0; i < 16; ++i) {
+        const int R = R0 + fx::a_pt(c) + i;
+        va[16 * c + i] = liva && R < n ? __ldg(pa + (int64_t)R * m) : 0.0;
+      }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int R = R0 + fx::b_pt() + i;
+      vb[i] = livb && R < n ? __ldg(pb + (int64_t)R * m) : 0.0;
     }
+    ok = fx::window(sm, tmem, va, vb, acc, phase, [&](int r, int c) {
+      double s = 0.0;
+      if (tc0 + r < nc && td0 + c < nd)
+        for (int R = R0; R < min(n, R0 + fx::kWin); ++R)
+          s = fma(B[(int64_t)R * m + c0 + tc0 + r], B[(int64_t)R * m + d0 + td0 + c], s);
+      return s;
+    });
   }
+  const int64_t r = tc0 + 32 * (warp & 3) + lane;
+#pragma unroll
+  for (int j = 0; j < 16; ++j) {
+    const int64_t d = td0 + 16 * (warp >> 2) + j;
+    if (r < nc && d < nd) out[r * nd + d] = ok ? acc[j] : __longlong_as_double(0x7ff8000000000000ll);
+  }
+  fx::close(sm, tmem, ok, phase);
 }
 
 // ---------------------------------------------------------------- tensor-core product
@@ -331,6 +347,11 @@ __global__ void ri_transpose_kernel(int n, int64_t m, const double* __restrict__
   }
 }
 
+// The dynamic shared memory of a tile kernel (an attribute per device, set before each launch).
+bool fx_attr(const void* kernel) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fx::kSmemBytes) == cudaSuccess;
+}
+
 bool aligned8(const void* p) { return ((uintptr_t)p & 7u) == 0; }
 
 psq_status launched() {
@@ -376,12 +397,11 @@ extern "C" psq_status psq_ri_solve(int n, int64_t m, const double* d_L, double* 
     return set_error(PSQ_ERR_ARG, "psq_ri_solve: NULL or misaligned matrix");
   if ((m + 63) / 64 > 0x7fffffff) return set_error(PSQ_ERR_ARG, "psq_ri_solve: m too large");
   cudaStream_t s = (cudaStream_t)stream;
-  for (int k0 = 0; k0 < n; k0 += kB) {
-    const int kb = n - k0 < kB ? n - k0 : kB;
-    trsv_diag_kernel<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(n, m, k0, kb, d_L, d_B);
-    const int rest = n - k0 - kb;
-    if (rest > 0) trsv_update_kernel<<<dim3((unsigned)((m + 63) / 64), (rest + 63) / 64), 256, 0, s>>>(n, m, k0, kb, d_L, d_B);
-  }
+  // few columns: fewer per CTA, so that the serial substitutions spread over the SMs
+  const int64_t per = (m + 2 * 152 - 1) / (2 * 152);
+  const int cols = per >= 97 ? 128 : (int)((per + 31) / 32 * 32);
+  if (!fx_attr((const void*)trsv_kernel)) return launched();
+  trsv_kernel<<<(unsigned)((m + cols - 1) / cols), fx::kThreads, fx::kSmemBytes, s>>>(n, m, cols, d_L, d_B);
   return launched();
 }
 
@@ -393,8 +413,9 @@ extern "C" psq_status psq_ri_eri(int n, int64_t m, const double* d_B, int64_t c0
   if (!d_out || !aligned8(d_out) || (n > 0 && (!d_B || !aligned8(d_B))))
     return set_error(PSQ_ERR_ARG, "psq_ri_eri: NULL or misaligned pointer");
   if ((nc + 63) / 64 > 65535 || (nd + 63) / 64 > 0x7fffffff) return set_error(PSQ_ERR_ARG, "psq_ri_eri: block too large");
-  eri_kernel<<<dim3((unsigned)((nd + 63) / 64), (unsigned)((nc + 63) / 64)), 256, 0, (cudaStream_t)stream>>>(
-      n, m, d_B, c0, nc, d0, nd, d_out);
+  if (!fx_attr((const void*)eri_kernel)) return launched();
+  eri_kernel<<<dim3((unsigned)((nd + fx::kCols - 1) / fx::kCols), (unsigned)((nc + fx::kRows - 1) / fx::kRows)), fx::kThreads,
+               fx::kSmemBytes, (cudaStream_t)stream>>>(n, m, d_B, c0, nc, d0, nd, d_out);
   return launched();
 }
 
