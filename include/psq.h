@@ -62,7 +62,9 @@ typedef struct { int atom, n, l; double zeta; } psq_shell;      /* n > l >= 0, z
 typedef struct { int n_mu, n_nu, n_phi, q_mu, q_nu, q_phi, n_sp; } psq_grid_spec;
 
 typedef enum {
-  PSQ_FP64 = 0,  /* plain path: every step in FP64 */
+  PSQ_FP64 = 0,  /* plain path: FP64 values throughout.  The (P|Q) and (P|ij) sums run on the tensor
+                    cores on exact integer digits of the FP64 values (63 bits of each 64-point
+                    window's largest), one FP64 rounding per window; the other sums are FP64 FMAs */
   PSQ_MIXED = 1  /* FP64 node tables, third-centre offsets, row constants and range sums;
                     double-float (FP32 hi + lo, ~48 bits) weights, STO values and aux
                     potentials; contraction on tcgen05 tensor cores: five 8-bit integer slices
@@ -129,7 +131,8 @@ psq_status psq_job_autotune(psq_job* job, unsigned mask, void* d_workspace, size
  * measure a tensor-pipe roofline counts; no paper counterpart).  PSQ_MIXED: every tensor-core
  * MMA of the 8-bit slice products, tiles of 128 rows x 48 columns whatever their fill, 15
  * slice products per 32-point chunk, each M x N x K MMA counting 2MNK.  PSQ_FP64: 2 x rows x cols x
- * points summed over the computed blocks.  Errors: PSQ_ERR_ARG for NULL pointers or unknown
+ * points summed over the computed blocks (a symmetric block's elements once), whichever pipe they
+ * run on.  Errors: PSQ_ERR_ARG for NULL pointers or unknown
  * mask bits. */
 psq_status psq_job_issued_flops(const psq_job* job, unsigned mask, double* flops);
 

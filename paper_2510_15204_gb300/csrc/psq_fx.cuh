@@ -5,15 +5,15 @@
 // GB300's FP64 pipe does two FMAs per clock and SM (1.25 TFLOP/s), its tensor cores 4096 16-bit
 // ones.  So every value is cut, without rounding error, into integer digits (the error-free split
 // of Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59 (2012), here with one power-of-two scale
-// per row and window).  With |v| < 2^e over the window, X = trunc(v 2^(62-e)) is a 63-bit integer,
-// written as eight balanced base-256 digits d_k in [-128, 127] (|d_0| <= 64), exact in FP16.
-// The products of orders i + j = 0..7 (36 of 64) accumulate per order in FP32: an order's sum over
-// 64 points stays below 64 x 8 x 2^14 = 2^23, so the accumulation is exact.  The order sums join
-// in one 64-bit integer T with unit 2^(ea+eb-52), and the FP64 accumulator of an element takes
-// T by one FMA per window: where a chain of FP64 FMAs rounds 64 times, this rounds once.  What is
-// dropped (the truncation of X, orders above 7, the fraction of orders 6 and 7 below T's unit)
-// stays below two units per window, 2^-51 of the largest |a| times the largest |b|, against 2^-53
-// of the running sum per FMA of the chain.
+// per row and window).  With |v| < 2^e over the window, X = trunc(v 2^(63-e)) is a 64-bit integer
+// (exact for values above 2^-10 of the window's largest), written as eight balanced base-256
+// digits d_k in [-128, 127], exact in FP16.  The products of orders i + j = 0..7 (36 of 64)
+// accumulate per order in FP32: an order's sum over 64 points stays within 64 x 8 x 2^14 = 2^23,
+// so the accumulation is exact.  The order sums join in one 64-bit integer T and the FP64
+// accumulator of an element takes T by one FMA per window: where a chain of FP64 FMAs rounds 64
+// times, this rounds once.  What is dropped (the truncation of small values, orders above 7) stays
+// below about 2^-59 of the largest |a| times the largest |b| per window, against 2^-53 of the
+// running sum per FMA of the chain.
 //
 // Rows whose window lies below 2^-958 count as zeros.  Rows that hold an infinity, a NaN or a value of 2^478 and above take the plain FP64 chain for the
 // window (their products with the other operand may leave the range of the integer path).
@@ -41,13 +41,12 @@ constexpr int kBigField = 1500;         // exponent field from which a row takes
 struct Smem {
   alignas(1024) uint8_t a[kDigits][kRows * 64];
   alignas(1024) uint8_t b[kDigits][kCols * 64];
-  int ma[2][kRows];  // largest |high word| of the two threads of a row
-  int mb[8][kCols];  // and of the eight threads of a column
-  int ea[kRows], eb[kCols];  // exponent fields of the window
+  int ea[2][kRows], eb[2][kCols];  // exponent fields, of even and odd windows
   alignas(8) uint64_t done;
   uint32_t tmem;
 };
 constexpr size_t kSmemBytes = sizeof(Smem) + 1024;
+static_assert(3 * (kSmemBytes + 1024) > 228 * 1024, "a third CTA per SM would wait for TMEM columns");
 
 // Instruction descriptor: kind::f16, A = B = F16, D = F32, both K-major, M = 128, N = n.
 __device__ __forceinline__ uint32_t idesc(int n) {
@@ -80,13 +79,13 @@ __device__ __forceinline__ void close(Smem& sm, uint32_t tmem, bool ok, uint32_t
   }
 }
 
-// The operand values a thread brings to a window: row threadIdx.x % 128, points
-// 32 c + 16 (threadIdx.x / 128) + i of chunk c (a[16 c + i]); column threadIdx.x % 32, points
-// 8 (threadIdx.x / 32) + i (b[i]).
-__device__ __forceinline__ int a_row() { return threadIdx.x & (kRows - 1); }
-__device__ __forceinline__ int a_pt(int c) { return 32 * c + 16 * (threadIdx.x >> 7); }
-__device__ __forceinline__ int b_col() { return threadIdx.x & (kCols - 1); }
-__device__ __forceinline__ int b_pt() { return 8 * (threadIdx.x >> 5); }
+// The operand values a thread brings to a window.  A: rows a_row(u), u = 0, 1; of chunk c (32
+// points) the eight points from a_pt(c): va[2 c + u][i].  B: column b_col(); of chunk c the four
+// points from b_pt(c): vb[c][i].  A row's 64 points are in four lanes, a column's in eight.
+__device__ __forceinline__ int a_row(int u) { return 64 * u + 8 * (threadIdx.x >> 5) + ((threadIdx.x & 31) >> 2); }
+__device__ __forceinline__ int a_pt(int c) { return 32 * c + 8 * (threadIdx.x & 3); }
+__device__ __forceinline__ int b_col() { return 4 * (threadIdx.x >> 5) + ((threadIdx.x & 31) >> 3); }
+__device__ __forceinline__ int b_pt(int c) { return 32 * c + 4 * (threadIdx.x & 7); }
 
 // Biased digits of v (byte k of the result = digit 7 - k plus 128) in a window whose largest
 // exponent field is E (E = 4000: a row of zeros).
@@ -94,72 +93,90 @@ __device__ __forceinline__ uint64_t digits(double v, int E) {
   const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
   const int t = min(E - (int)((hi >> 20) & 0x7ffu), 63);
   const uint64_t m = ((uint64_t)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
-  const uint64_t x = (m << 9) >> t;
+  const uint64_t x = (m << 10) >> t;
   const uint64_t s = (uint64_t)((int64_t)(int32_t)hi >> 63);
-  return ((x ^ s) - s) + 0x8080808080808080ull;
+  return (x ^ s) + (0x8080808080808080ull - s);
 }
 
-// Eight consecutive points of one row or column into its 16-byte group of every plane.
-__device__ __forceinline__ void store_group(uint8_t* planes, uint32_t plane_bytes, uint32_t off, const double* v, int E) {
+// Digit plane k of the biased digits y0, y1 as two FP16 numbers: 1024 + byte, minus 1152.
+__device__ __forceinline__ uint32_t plane(uint64_t y0, uint64_t y1, int k) {
+  const uint32_t u0 = k < 4 ? (uint32_t)(y0 >> 32) : (uint32_t)y0, u1 = k < 4 ? (uint32_t)(y1 >> 32) : (uint32_t)y1;
+  const uint32_t by = 3 - (k & 3);
+  const uint32_t x = (__byte_perm(u0, u1, by | (by << 4) | ((4 + by) << 8) | ((4 + by) << 12)) & 0x00ff00ffu) | 0x64006400u;
+  const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&x), __half2half2(__ushort_as_half(0x6480)));
+  return *reinterpret_cast<const uint32_t*>(&d);
+}
+
+// Eight consecutive points of a row into its 16-byte group of every plane (offset off).
+__device__ __forceinline__ void store_a(Smem& sm, uint32_t off, const double (&v)[8], int E) {
   uint64_t y[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) y[i] = digits(v[i], E);
-  const __half2 bias = __half2half2(__ushort_as_half(0x6480));  // 1024 + 128
 #pragma unroll
-  for (int k = 0; k < kDigits; ++k) {
-    uint32_t w[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const uint32_t u0 = k < 4 ? (uint32_t)(y[2 * q] >> 32) : (uint32_t)y[2 * q];
-      const uint32_t u1 = k < 4 ? (uint32_t)(y[2 * q + 1] >> 32) : (uint32_t)y[2 * q + 1];
-      const uint32_t by = 3 - (k & 3);
-      // 1024 + byte in both halves, then minus 1152: the digit, exact in FP16
-      const uint32_t x = (__byte_perm(u0, u1, by | (by << 4) | ((4 + by) << 8) | ((4 + by) << 12)) & 0x00ff00ffu) | 0x64006400u;
-      const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&x), bias);
-      w[q] = *reinterpret_cast<const uint32_t*>(&d);
-    }
-    *reinterpret_cast<uint4*>(planes + k * plane_bytes + off) = make_uint4(w[0], w[1], w[2], w[3]);
-  }
+  for (int k = 0; k < kDigits; ++k)
+    *reinterpret_cast<uint4*>(sm.a[k] + off) =
+        make_uint4(plane(y[0], y[1], k), plane(y[2], y[3], k), plane(y[4], y[5], k), plane(y[6], y[7], k));
 }
+
+// Four consecutive points of a column into their half group.
+__device__ __forceinline__ void store_b(Smem& sm, uint32_t off, const double (&v)[4], int E) {
+  uint64_t y[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) y[i] = digits(v[i], E);
+#pragma unroll
+  for (int k = 0; k < kDigits; ++k)
+    *reinterpret_cast<uint2*>(sm.b[k] + off) = make_uint2(plane(y[0], y[1], k), plane(y[2], y[3], k));
+}
+
+// The exponent field a window is scaled by, from its largest |high word|: one more where the largest
+// value is within 2^-7 of the next power of two (its leading digit would round up to 128).
+__device__ __forceinline__ int field(int mx) { return (mx + 0x2040) >> 20; }
 
 __device__ __forceinline__ int hi_abs(double v) { return __double2hiint(v) & 0x7fffffff; }
 
 // One window: the tile's accumulators (element row 32 (warp % 4) + lane, columns 16 (warp / 4) + j,
-// acc[j]) take sum_p a_r(p) b_c(p).  phase: the parity of sm.done, kept by the caller from 0.
-// chain(row, col): the plain FP64 sum of the window for a row or column out of the integer
-// path's range.  Returns false (for every thread) when a wait ran out.
+// acc[j]) take sum_p a_r(p) b_c(p).  Only the first `rows` rows and `cols` columns are kept up
+// (8-row groups and 4-column groups past them are left out).  win: the windows done so far by this
+// CTA.  chain(row, col): the plain FP64 sum of the window for a row or column out of the integer
+// path's range.  ok turns false when a wait ran out (the caller ends its loop when the return
+// value, the same for all threads, is false, and asks all threads once more at the end).
 template <typename Chain>
-__device__ __forceinline__ bool window(Smem& sm, uint32_t tmem, const double (&va)[32], const double (&vb)[8],
-                                       double (&acc)[16], uint32_t& phase, Chain chain) {
+__device__ __forceinline__ bool window(Smem& sm, uint32_t tmem, const double (&va)[4][8], const double (&vb)[2][4],
+                                       double (&acc)[16], uint32_t& phase, uint32_t win, int rows, int cols, bool& ok,
+                                       Chain chain) {
+  constexpr unsigned kFull = 0xffffffffu;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  int ma = 0, mb = 0;
+  const int set = win & 1;
+  int E[2], Eb = 0;
 #pragma unroll
-  for (int i = 0; i < 32; ++i) ma = max(ma, hi_abs(va[i]));
+  for (int u = 0; u < 2; ++u) {
+    int mx = 0;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) mb = max(mb, hi_abs(vb[i]));
-  sm.ma[tid >> 7][tid & 127] = ma;
-  sm.mb[warp][lane] = mb;
-  __syncthreads();
-  const int Ea = max(sm.ma[0][tid & 127], sm.ma[1][tid & 127]) >> 20;
-  int Eb = 0;
+    for (int c = 0; c < 2; ++c)
 #pragma unroll
-  for (int i = 0; i < 8; ++i) Eb = max(Eb, sm.mb[i][lane]);
-  Eb >>= 20;
-  if (tid < kRows) sm.ea[tid] = Ea;
-  if (tid < kCols) sm.eb[tid] = Eb;
-  // rows below 2^-958 count as zeros (a zero's own field, 0, is then at least 64 below E)
-  const int Sa = Ea >= 64 ? Ea : 4000, Sb = Eb >= 64 ? Eb : 4000;
-  bool ok = true;
+      for (int i = 0; i < 8; ++i) mx = max(mx, hi_abs(va[2 * c + u][i]));
+    mx = max(mx, __shfl_xor_sync(kFull, mx, 1));
+    E[u] = field(max(mx, __shfl_xor_sync(kFull, mx, 2)));
+    if ((lane & 3) == 0) sm.ea[set][a_row(u)] = E[u];
+    if (E[u] < 64) E[u] = 4000;  // a zero's own field, 0, must be 63 below that of a row that counts
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) Eb = max(Eb, max(hi_abs(vb[0][i]), hi_abs(vb[1][i])));
+#pragma unroll
+  for (int o = 1; o < 8; o <<= 1) Eb = max(Eb, __shfl_xor_sync(kFull, Eb, o));
+  Eb = field(Eb);
+  if ((lane & 7) == 0) sm.eb[set][b_col()] = Eb;
+  if (Eb < 64) Eb = 4000;
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
-    if (c == 1) {
+    if (c == 1 && ok) {
       ok = mma::mbar_wait(mma::smem_u32(&sm.done), phase & 1);
       phase += ok ? 1u : 0u;
     }
-    const int g = 2 * (tid >> 7);
-    store_group(sm.a[0], kRows * 64, mma::swz(a_row(), g), va + 16 * c, Sa);
-    store_group(sm.a[0], kRows * 64, mma::swz(a_row(), g + 1), va + 16 * c + 8, Sa);
-    if ((warp >> 2) == c) store_group(sm.b[0], kCols * 64, mma::swz(b_col(), warp & 3), vb, Sb);
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+      if (64 * u + 8 * warp < rows) store_a(sm, mma::swz(a_row(u), lane & 3), va[2 * c + u], E[u]);
+    if (4 * warp < cols) store_b(sm, mma::swz(b_col(), (lane & 7) >> 1) + 8u * (lane & 1), vb[c], Eb);
     mma::fence_async_smem();
     mma::fence_before();
     if (!__syncthreads_and(ok)) return false;
@@ -178,36 +195,45 @@ __device__ __forceinline__ bool window(Smem& sm, uint32_t tmem, const double (&v
   }
   ok = mma::mbar_wait(mma::smem_u32(&sm.done), phase & 1);
   phase += ok ? 1u : 0u;
-  if (!__syncthreads_and(ok)) return false;
+  if (!__all_sync(kFull, ok)) { ok = false; return true; }
   mma::fence_after();
   // fold: order sums -> T -> FP64
   const int row = 32 * (warp & 3) + lane, c0 = 16 * (warp >> 2);
-  const uint32_t base = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0;
-  const int er = sm.ea[row];
+  if (32 * (warp & 3) < rows) {
+    const uint32_t base = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0;
+    const int er = sm.ea[set][row];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    float o[kDigits][4];
+    for (int q = 0; q < 4; ++q) {
+      if (c0 + 4 * q >= cols) break;
+      float o[kDigits][4];
 #pragma unroll
-    for (int k = 0; k < kDigits; ++k) mma::tmem_ld4(base + (uint32_t)(kCols * k + 4 * q), o[k]);
-    mma::tmem_wait_ld();
+      for (int k = 0; k < kDigits; ++k) mma::tmem_ld4(base + (uint32_t)(kCols * k + 4 * q), o[k]);
+      mma::tmem_wait_ld();
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int ec = sm.eb[c0 + 4 * q + j];
-      // orders 0..4 are integers of at most 2^22: their low bits by the magic number 1.5 x 2^23
-      int s[5];
+      for (int j = 0; j < 4; ++j) {
+        const int ec = sm.eb[set][c0 + 4 * q + j];
+        // orders 0..3 are integers of at most 2^22: their low bits by the magic number 1.5 x 2^23
+        int s[6];
 #pragma unroll
-      for (int k = 0; k < 5; ++k) s[k] = __float_as_int(__fadd_rn(o[k][j], 12582912.0f)) - 0x4B400000;
-      const int s5 = __float2int_rn(fmaf(o[6][j], 0.00390625f, fmaf(o[7][j], 1.52587890625e-5f, o[5][j])));
-      const int64_t t = (int64_t)(s[2] * 256 + s[3]) * 65536 + (s[4] * 256 + s5) + ((int64_t)(s[0] * 256 + s[1]) << 32);
-      const int f = er + ec - 2044 - 52 + 1023;  // exponent field of T's unit
-      double& r = acc[4 * q + j];
-      if (er >= kBigField || ec >= kBigField)
-        r += chain(row, c0 + 4 * q + j);
-      else
-        r = fma(__ll2double_rn(t), __hiloint2double(f > 0 ? f << 20 : 0, 0), r);
+        for (int k = 0; k < 4; ++k) s[k] = __float_as_int(__fadd_rn(o[k][j], 12582912.0f)) - 0x4B400000;
+        s[4] = __float2int_rn(o[4][j]);
+        s[5] = __float2int_rn(o[5][j]);
+        // orders 0..5 in units of order 5 (at most 2^61); orders 6 and 7 join in those units where
+        // the sum is large, in 1/128 of them where it is below 2^54 (a sum of cancelling terms)
+        int64_t t = (int64_t)(s[2] * 256 + s[3]) * 65536 + (s[4] * 256 + s[5]) + ((int64_t)(s[0] * 256 + s[1]) << 32);
+        const bool small = (uint32_t)((int)(t >> 32) + (1 << 22)) < (1u << 23);
+        t = (small ? t << 7 : t) +
+            __float2int_rn(fmaf(o[6][j], 0.00390625f, o[7][j] * 1.52587890625e-5f) * (small ? 128.0f : 1.0f));
+        const int f = er + ec - 2044 - 54 + 1023 - (small ? 7 : 0);  // exponent field of t's unit
+        double& r = acc[4 * q + j];
+        if (er >= kBigField || ec >= kBigField)
+          r += chain(row, c0 + 4 * q + j);
+        else
+          r = fma(__ll2double_rn(t), __hiloint2double(f > 0 ? f << 20 : 0, 0), r);
+      }
     }
   }
-  mma::fence_before();  // the next window's MMAs come after the caller's next barrier
+  mma::fence_before();  // the next window's MMAs come after its first barrier
   return true;
 }
 

@@ -55,7 +55,6 @@ psq_status fail(psq_status s, const char* fmt, ...) {
 
 constexpr double kOnAxisTol = 1e-10;  // a third centre this close (x a) to the axis is on it
 constexpr int kPointsPerBlock = 128;
-constexpr int64_t kMaxChunkPoints = 32768;  // FP64 path: points per sequential partial sum
 constexpr int kSmCount = 152;
 constexpr size_t kDefaultWaveBytes = (size_t)6 << 30;  // mixed path: operand + packed bytes per wave
 
@@ -448,7 +447,8 @@ psq_status make_plan(psq_job* j, unsigned mask, Plan& P) {
       if (mask & PSQ_J3) { g.row_U = rows; rows += g.nG; }
     }
     g.row_W = rows;
-    rows += 4;
+    if (!P.mixed) g.n_W = mask & PSQ_V ? (refined ? 1 : 3) : 0;
+    rows += P.mixed ? 4 : g.n_W;
     g.ld = (int64_t)align_up((size_t)g.K, 128);
     g.op_off = ops;
     ops += (int64_t)rows * g.ld;
@@ -462,140 +462,207 @@ psq_status make_plan(psq_job* j, unsigned mask, Plan& P) {
   P.j3.assign((size_t)nat * nat * nat, J3Src{0, 0, 0, 0, 0, 0, 0});
   auto J3at = [&](int X, int Y, int W) -> J3Src& { return P.j3[((size_t)X * nat + Y) * nat + W]; };
   if (!P.mixed) {
-    // FP64 path: one block per (grid, class) and per (grid, aux atom, basis atom pair)
-    // On a pair grid (A < B) only the blocks that some element reads: S the A x B block (the
-    // one-centre S and T come from their closed forms); T the A x B block and its mirror
-    // (B rows against A's kinetic columns), averaged; (P|Q) the A x B block and its mirror, and
-    // the A x A (B x B) block where the grid is A's (B's) one-centre grid; V_ne of nucleus A the
-    // A x B block, the B x B block (B's functions in A's field) and the A x A block where the
-    // grid is A's one-centre grid (and likewise for nucleus B).
-    struct Fp2 { int64_t ab = -1, ba = -1, aa = -1, bb = -1; };
-    std::vector<int64_t> s_loc(P.grids.size(), -1), vc_loc(P.grids.size(), -1);
-    std::vector<Fp2> t_loc(P.grids.size()), j2_loc(P.grids.size()), va_loc(P.grids.size()), vb_loc(P.grids.size());
+    // FP64 path.  On a pair grid (A < B) only the blocks that some element reads, operand rows that
+    // meet the same columns stacked into one block:
+    //   [lap chi_A | chi_A | zAB chi_A] x chi_B (T, S, V_ne of A x B), lap chi_B x chi_A (T's mirror),
+    //   chi_A x zAA chi_A and chi_B x zBB chi_B (V_ne of A x A and B x B, symmetric, the square root of
+    //   the weight on both sides); zAB, zAA, zBB are the nuclear weights summed over the nuclei, w is in the rows (eval_fp64_kernel);
+    //   [V^A | V^B on B's one-centre grid] x aux chi_B, and likewise x aux chi_A ((P|Q) and its
+    //   mirror);
+    //   the pair products chi_i chi_j of the classes whose (P|ij) this grid integrates x V^X.
+    // On a refined grid: zC chi_A x chi_B; the A x B pair products x V^C.
+    // (One-centre S and T come from their closed forms.)
+    // result offsets of the one-electron blocks and the first rows of T, S, V in the A x B block
+    struct Fp1e { int64_t ab = -1, ba = -1, aa = -1, bb = -1; int T = -1, S = -1, V = -1; };
+    struct FpJ2 { int64_t onB = -1, onA = -1; int BB = -1, AA = -1; };  // columns of B, of A; row of the own block
+    std::vector<Fp1e> e_loc(P.grids.size());
+    std::vector<FpJ2> j2_loc(P.grids.size());
     auto own_grid = [&](const DevGrid& g, int X) {
       const GridKey k = grid_for(j, X, X, X);
       return k.A == g.A && k.B == g.B && k.C == -1;
     };
-    auto add_block = [&](int g, int a_row, int m, int b_row, int n, int b_mode, int pair_off, int d_row) {
+    auto add_rows = [&](int row0, int n, int w) {
+      for (int i = 0; i < n; ++i) P.pairs.push_back(make_short2(row0 + i, w));
+    };
+    auto add_block = [&](int g, int kind, int a_off, int m, int b_off, int n) {
       GemmBlock b{};
-      b.grid = g; b.a_row = a_row; b.m = m; b.b_row = b_row; b.n = n; b.b_mode = b_mode;
-      b.pair_off = pair_off; b.d_row = d_row; b.res_off = res;
+      b.grid = g; b.kind = kind; b.a_off = a_off; b.m = m; b.b_off = b_off; b.n = n; b.res_off = res;
       res += (int64_t)m * n;
       P.gblocks.push_back(b);
       return b.res_off;
     };
     for (size_t gi = 0; gi < P.grids.size(); ++gi) {
       DevGrid& g = P.grids[gi];
-      const int nl = g.nFA + g.nFB;
-      const int w = g.row_W;
-      const int gint = (int)gi;
+      g.zA = j->atoms[g.A].Z;
+      g.zB = j->atoms[g.B].Z;
+      g.zC = g.C >= 0 ? j->atoms[g.C].Z : 0.0;
+      g.own_A = g.C < 0 && own_grid(g, g.A);
+      g.own_B = g.C < 0 && own_grid(g, g.B);
+      const int W = g.row_W, gint = (int)gi, nA = g.nFA, nB = g.nFB;
+      const int FA = g.row_F, FB = g.row_F + nA;
+      auto list = [&]() { return (int)P.pairs.size(); };
       if (g.C < 0) {
-        if (g.nFA > 0 && g.nFB > 0) {
-          if (mask & PSQ_S) s_loc[gi] = add_block(gint, g.row_F, g.nFA, g.row_F + g.nFA, g.nFB, 0, 0, w);
+        Fp1e& e = e_loc[gi];
+        auto sym_block = [&](int row0, int n, int w) {
+          const int a_off = list();
+          add_rows(row0, n, w);
+          return add_block(gint, kFpFmaSym, a_off, n, a_off, n);
+        };
+        if ((mask & (PSQ_S | PSQ_T | PSQ_V)) && nA > 0 && nB > 0) {
+          const int a_off = list();
+          if (mask & PSQ_T) { e.T = list() - a_off; add_rows(g.row_L, nA, -1); }
+          if (mask & PSQ_S) { e.S = list() - a_off; add_rows(FA, nA, -1); }
+          if (mask & PSQ_V) { e.V = list() - a_off; add_rows(FA, nA, W); }
+          const int m = list() - a_off, b_off = list();
+          add_rows(FB, nB, -1);
+          e.ab = add_block(gint, kFpFma, a_off, m, b_off, nB);
           if (mask & PSQ_T) {
-            t_loc[gi].ab = add_block(gint, g.row_F, g.nFA, g.row_L + g.nFA, g.nFB, 0, 0, w);
-            t_loc[gi].ba = add_block(gint, g.row_F + g.nFA, g.nFB, g.row_L, g.nFA, 0, 0, w);
+            const int l_off = list();
+            add_rows(g.row_L + nA, nB, -1);
+            const int f_off = list();
+            add_rows(FA, nA, -1);
+            e.ba = add_block(gint, kFpFma, l_off, nB, f_off, nA);
           }
         }
-        if (mask & PSQ_V) {
-          const bool oA = own_grid(g, g.A), oB = own_grid(g, g.B);
-          for (int c = 0; c < 2; ++c) {  // nucleus A (weight row w + 1), nucleus B (w + 2)
-            Fp2& v = c == 0 ? va_loc[gi] : vb_loc[gi];
-            if (g.nFA > 0 && g.nFB > 0) v.ab = add_block(gint, g.row_F, g.nFA, g.row_F + g.nFA, g.nFB, 0, 0, w + 1 + c);
-            if (g.nFA > 0 && (c == 1 || oA)) v.aa = add_block(gint, g.row_F, g.nFA, g.row_F, g.nFA, 0, 0, w + 1 + c);
-            if (g.nFB > 0 && (c == 0 || oB))
-              v.bb = add_block(gint, g.row_F + g.nFA, g.nFB, g.row_F + g.nFA, g.nFB, 0, 0, w + 1 + c);
-          }
-        }
+        if ((mask & PSQ_V) && nA > 0) e.aa = sym_block(FA, nA, W + 1);
+        if ((mask & PSQ_V) && nB > 0) e.bb = sym_block(FB, nB, W + 2);
+        const int naA = j->na[g.A], naB = j->na[g.B];
         if (mask & PSQ_J2) {
-          const int naA = j->na[g.A], naB = j->na[g.B];
-          if (naA > 0 && naB > 0) {
-            j2_loc[gi].ab = add_block(gint, g.row_U, naA, g.row_G + naA, naB, 0, 0, w);
-            j2_loc[gi].ba = add_block(gint, g.row_U + naA, naB, g.row_G, naA, 0, 0, w);
+          FpJ2& q = j2_loc[gi];
+          for (int side = 0; side < 2; ++side) {  // columns of B, then of A
+            const int nc = side == 0 ? naB : naA, nr = side == 0 ? naA : naB;
+            const bool own = side == 0 ? g.own_B : g.own_A;
+            if (nc == 0 || (nr == 0 && !own)) continue;
+            const int a_off = list();
+            add_rows(side == 0 ? g.row_U : g.row_U + naA, nr, -1);
+            if (own) {
+              (side == 0 ? q.BB : q.AA) = nr;
+              add_rows(side == 0 ? g.row_U + naA : g.row_U, nc, -1);
+            }
+            const int m = list() - a_off, b_off = list();
+            add_rows(side == 0 ? g.row_G + naA : g.row_G, nc, -1);
+            (side == 0 ? q.onB : q.onA) = add_block(gint, kFpDigits, a_off, m, b_off, nc);
           }
-          if (naA > 0 && own_grid(g, g.A)) j2_loc[gi].aa = add_block(gint, g.row_U, naA, g.row_G, naA, 0, 0, w);
-          if (naB > 0 && own_grid(g, g.B))
-            j2_loc[gi].bb = add_block(gint, g.row_U + naA, naB, g.row_G + naA, naB, 0, 0, w);
         }
         if (mask & PSQ_J3) {
           const int atoms2[2] = {g.A, g.B};
           for (int xi = 0; xi < 2; ++xi) {
             const int X = atoms2[xi];
             if (j->na[X] == 0) continue;
-            const int aoff = xi == 0 ? 0 : j->na[g.A];
+            const int a_off = list();
             const int yw[3][2] = {{g.A, g.A}, {g.A, g.B}, {g.B, g.B}};
-            for (auto& pq : yw) {
-              const int Y = pq[0], W = pq[1];
-              if (j->nb[Y] == 0 || j->nb[W] == 0) continue;
-              const GridKey k = grid_for(j, Y, W, X);
+            int first[3] = {-1, -1, -1};
+            for (int c = 0; c < 3; ++c) {
+              const int Y = yw[c][0], Wt = yw[c][1];
+              if (j->nb[Y] == 0 || j->nb[Wt] == 0) continue;
+              const GridKey k = grid_for(j, Y, Wt, X);
               if (k.A != g.A || k.B != g.B || k.C != -1) continue;
-              const int yoff = Y == g.A ? 0 : g.nFA, woff = W == g.A ? 0 : g.nFA;
-              const int pair_off = (int)P.pairs.size();
-              if (Y != W) {
-                for (int i = 0; i < j->nb[Y]; ++i)
-                  for (int jj = 0; jj < j->nb[W]; ++jj) P.pairs.push_back(make_short2(yoff + i, woff + jj));
-              } else {
-                for (int i = 0; i < j->nb[Y]; ++i)
-                  for (int jj = i; jj < j->nb[Y]; ++jj) P.pairs.push_back(make_short2(yoff + i, yoff + jj));
-              }
-              const int np = (int)P.pairs.size() - pair_off;
-              const int64_t off = add_block(gint, g.row_U + aoff, j->na[X], g.row_F, np, 1, pair_off, w);
-              J3at(X, Y, W) = J3Src{off, 1, np, Y == W ? 1 : 0, Y == W ? j->nb[Y] : j->nb[W], 0, 0};
+              first[c] = list() - a_off;
+              const int y0 = Y == g.A ? FA : FB, w0 = Wt == g.A ? FA : FB;
+              for (int i = 0; i < j->nb[Y]; ++i)
+                for (int jj = Y == Wt ? i : 0; jj < j->nb[Wt]; ++jj) P.pairs.push_back(make_short2(y0 + i, w0 + jj));
             }
+            const int m = list() - a_off, b_off = list();
+            if (m == 0) continue;
+            const int nx = j->na[X];
+            add_rows(g.row_U + (xi == 0 ? 0 : naA), nx, -1);
+            const int64_t off = add_block(gint, kFpDigits, a_off, m, b_off, nx);
+            for (int c = 0; c < 3; ++c)
+              if (first[c] >= 0)
+                J3at(X, yw[c][0], yw[c][1]) = J3Src{off + (int64_t)first[c] * nx, nx, 1, yw[c][0] == yw[c][1] ? 1 : 0, j->nb[yw[c][1]], 0, 0};
           }
         }
-      } else {
-        if ((mask & PSQ_V) && g.nFA > 0 && g.nFB > 0)
-          vc_loc[gi] = add_block(gint, g.row_F, g.nFA, g.row_F + g.nFA, g.nFB, 0, 0, w + 3);
-        if ((mask & PSQ_J3) && j->na[g.C] > 0 && g.nFA > 0 && g.nFB > 0) {
-          const int pair_off = (int)P.pairs.size();
-          for (int i = 0; i < g.nFA; ++i)
-            for (int jj = 0; jj < g.nFB; ++jj) P.pairs.push_back(make_short2(i, g.nFA + jj));
-          const int np = g.nFA * g.nFB;
-          const int64_t off = add_block(gint, g.row_U, j->na[g.C], g.row_F, np, 1, pair_off, w);
-          J3at(g.C, g.A, g.B) = J3Src{off, 1, np, 0, g.nFB, 0, 0};
+      } else if (nA > 0 && nB > 0) {
+        if (mask & PSQ_V) {
+          const int a_off = list();
+          add_rows(FA, nA, W);
+          const int b_off = list();
+          add_rows(FB, nB, -1);
+          e_loc[gi].ab = add_block(gint, kFpFma, a_off, nA, b_off, nB);
+        }
+        if ((mask & PSQ_J3) && j->na[g.C] > 0) {
+          const int a_off = list(), nx = j->na[g.C];
+          for (int i = 0; i < nA; ++i)
+            for (int jj = 0; jj < nB; ++jj) P.pairs.push_back(make_short2(FA + i, FB + jj));
+          const int b_off = list();
+          add_rows(g.row_U, nx, -1);
+          const int64_t off = add_block(gint, kFpDigits, a_off, nA * nB, b_off, nx);
+          J3at(g.C, g.A, g.B) = J3Src{off, nx, 1, 0, nB, 0, 0};
         }
       }
     }
-    // chunking: enough CTAs for several waves, chunks of at least 2048 points
-    int64_t tiles = 0;
-    // output tile per block: balanced row tiles of <= 64 rows, then balanced column tiles of
-    // <= min(256, 1024 / rows) columns (little padding; no FP64 operation on padding)
-    for (auto& b : P.gblocks) {
-      const int ntm = (b.m + kFpTileRows - 1) / kFpTileRows;
-      b.tile_m = std::max(1, (b.m + ntm - 1) / ntm);
-      const int tn_max = std::max(1, std::min(kFpTileCols, kFpTileOut / b.tile_m));
-      const int ntn = (b.n + tn_max - 1) / tn_max;
-      b.tile_n = std::max(1, (b.n + ntn - 1) / ntn);
-      tiles += (int64_t)ntm * ntn;
+    // Output tiles: 128 x 32 on the tensor cores; for the FMAs balanced tiles of at most 32 (lanes) x 16
+    // (registers, in steps of two), whichever side of the block on the lanes costs less; a symmetric
+    // block of at most 31 rows whole, else in square tiles of at most 16.
+    // Cost of a tile's window in SM cycles: a warp's FP64 FMA takes 16; the digits part slices its rows
+    // and columns and folds (measured about 12,000 for a full 128 x 32 tile).
+    auto even = [](int n, int most) { const int t = (n + most - 1) / most; return (n + t - 1) / t; };
+    auto ntm = [](const GemmBlock& b) { return (b.m + b.tile_m - 1) / b.tile_m; };
+    auto ntn = [](const GemmBlock& b) { return (b.n + b.tile_n - 1) / b.tile_n; };
+    auto tile_cost = [](const GemmBlock& b, int x, int y) {
+      const int r = std::min(b.tile_m, b.m - x * b.tile_m), c = std::min(b.tile_n, b.n - y * b.tile_n);
+      if (b.kind == kFpDigits) return 2000.0 + 60.0 * (r + c);
+      const int lanes = b.swap ? r : c, regs = b.swap ? c : r;
+      const double one = 16.0 * kFpWin / (lanes < 4 ? 8 : (lanes < 8 ? 4 : (lanes < 16 ? 2 : 1)));  // point groups
+      if (b.kind == kFpFmaSym && y <= x) return y < x ? 0.0 : one * ((r + 1) / 2);
+      return one * ((regs + 1) / 2 * 2);
+    };
+    for (GemmBlock& b : P.gblocks) {
+      if (b.kind == kFpDigits) {
+        b.tile_m = kFpDigitRows;
+        b.tile_n = kFpDigitCols;
+      } else if (b.kind == kFpFmaSym) {
+        b.tile_m = b.tile_n = b.m < kFpFmaLanes ? b.m : even(b.m, kFpFmaRegs);
+      } else {
+        double cost[2];
+        for (int sw = 1; sw >= 0; --sw) {
+          b.swap = sw;
+          b.tile_m = even(b.m, sw ? kFpFmaLanes : kFpFmaRegs);
+          b.tile_n = even(b.n, sw ? kFpFmaRegs : kFpFmaLanes);
+          cost[sw] = tile_cost(b, 0, 0) * ntm(b) * ntn(b);
+        }
+        if (cost[1] < cost[0]) {
+          b.swap = 1;
+          b.tile_m = even(b.m, kFpFmaLanes);
+          b.tile_n = even(b.n, kFpFmaRegs);
+        }
+      }
     }
-    const int64_t want = 2LL * kSmCount * P.work_split;
-    const int cglob = (int)std::max<int64_t>(1, tiles > 0 ? (want + tiles - 1) / tiles : 1);
+    auto windows = [&](const GemmBlock& b) { return (P.grids[b.grid].K + kFpWin - 1) / kFpWin; };
+    double total = 0;
+    for (const GemmBlock& b : P.gblocks)
+      for (int x = 0; x < ntm(b); ++x)
+        for (int y = 0; y < ntn(b); ++y) total += windows(b) * tile_cost(b, x, y);
+    // work items: tiles x ranges of windows of about the same cost, work_split items per SM, ranges of
+    // at least 8 windows (512 points)
+    // (and partial sums of at most 1/40 of the operand rows: coarser ranges beyond)
+    auto split = [&](double target) {
+      int64_t p = 0;
+      for (GemmBlock& b : P.gblocks) {
+        const int64_t nwin = windows(b);
+        const int64_t n = std::max<int64_t>(1, std::min<int64_t>((int64_t)std::ceil(nwin * tile_cost(b, 0, 0) / target), nwin / 8));
+        b.win_per = (int)((nwin + n - 1) / n);
+        b.n_chunks = (int)((nwin + b.win_per - 1) / b.win_per);
+        b.part_off = p;
+        p += (int64_t)b.n_chunks * b.m * b.n;
+      }
+      return p;
+    };
+    double target = std::max(1.0, total / ((double)kSmCount * P.work_split));
+    part = split(target);
+    while (part > ops / 40 && target < total) part = split(target *= 1.5);
     for (size_t bi = 0; bi < P.gblocks.size(); ++bi) {
-      GemmBlock& b = P.gblocks[bi];
-      const int64_t K = P.grids[b.grid].K;
-      // at most kMaxChunkPoints per sequential partial sum (bounded rounding growth), and
-      // more chunks where the grid has too few tiles to fill the GPU
-      b.n_chunks = (int)std::max<int64_t>((K + kMaxChunkPoints - 1) / kMaxChunkPoints,
-                                          std::min<int64_t>(cglob, (K + 2047) / 2048));
-      b.n_chunks = std::max(1, b.n_chunks);
-      b.part_off = part;
-      part += (int64_t)b.n_chunks * b.m * b.n;
-      const int tm = (b.m + b.tile_m - 1) / b.tile_m, tn = (b.n + b.tile_n - 1) / b.tile_n;
+      const GemmBlock& b = P.gblocks[bi];
       for (int c = 0; c < b.n_chunks; ++c)
-        for (int x = 0; x < tm; ++x)
-          for (int y = 0; y < tn; ++y) P.items.push_back(GemmItem{(int)bi, x, y, c});
+        for (int x = 0; x < ntm(b); ++x)
+          for (int y = b.kind == kFpFmaSym ? x : 0; y < ntn(b); ++y) P.items.push_back(GemmItem{(int)bi, x, y, c});
     }
-    // Largest items first (outputs x points, a formed pair column costing one more product per
-    // point): the CTA scheduler hands out blocks in index order, so the last wave holds the
-    // small items and the tail of the launch is short.
+    // Largest items first: the CTA scheduler hands out blocks in index order, so the last wave holds
+    // the small items.
     auto fp_cost = [&](const GemmItem& it) {
       const GemmBlock& b = P.gblocks[it.block];
-      const int64_t K = P.grids[b.grid].K;
-      const int64_t csz = (K + b.n_chunks - 1) / b.n_chunks;
-      const int64_t pts = std::max<int64_t>(0, std::min<int64_t>(K, (int64_t)it.chunk * csz + csz) - (int64_t)it.chunk * csz);
-      const int rows = std::min(b.tile_m, b.m - it.tm * b.tile_m), cols = std::min(b.tile_n, b.n - it.tn * b.tile_n);
-      return (double)pts * ((double)rows * cols + rows + (b.b_mode == 1 ? 2.0 : 1.0) * cols);
+      return tile_cost(b, it.tm, it.tn) *
+             (double)(std::min<int64_t>(windows(b), (int64_t)(it.chunk + 1) * b.win_per) - (int64_t)it.chunk * b.win_per);
     };
     std::stable_sort(P.items.begin(), P.items.end(),
                      [&](const GemmItem& x, const GemmItem& y) { return fp_cost(x) > fp_cost(y); });
@@ -603,42 +670,46 @@ psq_status make_plan(psq_job* j, unsigned mask, Plan& P) {
     P.elem_begin[0] = 0;
     for (size_t bi = 0; bi < P.gblocks.size(); ++bi)
       P.elem_begin[bi + 1] = P.elem_begin[bi] + (int64_t)P.gblocks[bi].m * P.gblocks[bi].n;
-    for (const GemmBlock& b : P.gblocks) P.issued_flops += 2.0 * b.m * b.n * (double)P.grids[b.grid].K;
+    for (const GemmBlock& b : P.gblocks)
+      P.issued_flops += (b.kind == kFpFmaSym ? (double)b.m * (b.m + 1) : 2.0 * b.m * b.n) * (double)P.grids[b.grid].K;
     for (int X = 0; X < nat; ++X) {
       for (int Y = 0; Y < nat; ++Y) {
         for (int c = 0; c < 4; ++c) P.src_ptr[c][X * nat + Y] = (int)P.src[c].size();
         if (X > Y || mask == 0) continue;
         const int gb = gidx[grid_for(j, X, Y, X)];
         const DevGrid& G = P.grids[gb];
+        const Fp1e& e = e_loc[gb];
         // X < Y: the grid of (X, Y) is the pair grid with A = X, B = Y; X == Y: closed forms
         // for S and T (no source), (P|Q) from the one-centre grid's own block
-        if (X < Y && (mask & PSQ_S) && s_loc[gb] >= 0)
-          P.src[0].push_back(SrcEntry{s_loc[gb], G.nFB, 0, 0, 0, 0, 0, 0, 0, 1.0, 0, 0});
-        if (X < Y && (mask & PSQ_T) && t_loc[gb].ab >= 0)
-          P.src[1].push_back(SrcEntry{t_loc[gb].ab, G.nFB, 0, 0, 0, 0, 0, 0, 0, 1.0, t_loc[gb].ba, G.nFA});
+        if (X < Y && e.S >= 0) P.src[0].push_back(SrcEntry{e.ab, G.nFB, e.S, 0, 0, 0, 0, 0, 0, 1.0, 0, 0});
+        if (X < Y && e.T >= 0) P.src[1].push_back(SrcEntry{e.ab, G.nFB, e.T, 0, 0, 0, 0, 0, 0, 1.0, e.ba, G.nFA});
         if (mask & PSQ_V) {
-          for (int C = 0; C < nat; ++C) {
-            const GridKey k = grid_for(j, X, Y, C);
-            const int gv = gidx[k];
-            const DevGrid& H = P.grids[gv];
-            const double z = -(double)j->atoms[C].Z;
-            if (k.C >= 0) {
-              P.src[2].push_back(SrcEntry{vc_loc[gv], H.nFB, 0, 0, 0, 0, 0, 0, 0, z});
-            } else {
-              // C is A or B of the pair grid; X < Y: (X, Y) = (A, B), the A x B block; X == Y:
-              // the X x X block
-              const Fp2& v = C == H.A ? va_loc[gv] : vb_loc[gv];
-              const int64_t off = X < Y ? v.ab : (X == H.A ? v.aa : v.bb);
-              P.src[2].push_back(SrcEntry{off, j->nb[Y], 0, 0, 0, 0, 0, 0, 0, z, 0, 0});
+          if (X < Y) {  // both nuclei of the pair at once, then each third nucleus
+            if (e.V >= 0) P.src[2].push_back(SrcEntry{e.ab, G.nFB, e.V, 0, 0, 0, 0, 0, 0, -1.0, 0, 0});
+            for (int C = 0; C < nat; ++C) {
+              if (C == X || C == Y) continue;
+              const int gv = gidx[grid_for(j, X, Y, C)];
+              if (e_loc[gv].ab >= 0) P.src[2].push_back(SrcEntry{e_loc[gv].ab, P.grids[gv].nFB, 0, 0, 0, 0, 0, 0, 0, -1.0, 0, 0});
+            }
+          } else if (j->nb[X] > 0) {
+            // nucleus C (and X's own on its one-centre grid) on the grid of (X, C)
+            for (int C = 0; C < nat; ++C) {
+              if (C == X) continue;
+              const int gv = gidx[grid_for(j, X, X, C)];
+              const int64_t off = X == P.grids[gv].A ? e_loc[gv].aa : e_loc[gv].bb;
+              P.src[2].push_back(SrcEntry{off, j->nb[X], 0, 0, 0, 0, 0, 0, 0, -1.0, 0, 0});
             }
           }
         }
         if (mask & PSQ_J2) {
-          const Fp2& b = j2_loc[gb];
-          if (X < Y && b.ab >= 0)
-            P.src[3].push_back(SrcEntry{b.ab, j->na[Y], 0, 0, 0, 0, 0, 0, 0, 1.0, b.ba, j->na[X]});
-          const int64_t own = X == G.A ? b.aa : b.bb;
-          if (X == Y && own >= 0) P.src[3].push_back(SrcEntry{own, j->na[X], 0, 0, 0, 0, 0, 0, 0, 1.0, 0, 0});
+          const FpJ2& q = j2_loc[gb];
+          if (X < Y && q.onB >= 0 && q.onA >= 0)
+            P.src[3].push_back(SrcEntry{q.onB, j->na[Y], 0, 0, 0, 0, 0, 0, 0, 1.0, q.onA, j->na[X]});
+          if (X == Y && j->na[X] > 0) {
+            const bool isA = X == G.A;
+            const int row = isA ? q.AA : q.BB;
+            P.src[3].push_back(SrcEntry{isA ? q.onA : q.onB, j->na[X], row, 0, row, 0, 0, 0, 0, 1.0, 0, 0});
+          }
         }
       }
     }
@@ -1352,6 +1423,7 @@ psq_status psq_context_create(int device, psq_context** out) {
   upload_gl_tables(x, w, klm);
   upload_mixed_tables(x, w, klm);
   CUDA_TRY(prepare_kernels());
+  CUDA_TRY(prepare_kernels_fp64());
   CUDA_TRY(cudaGetLastError());
   int sms = 0;
   CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device));

@@ -34,7 +34,9 @@ struct DevGrid {
   // Operand matrices of this grid: rows of ld doubles (or floats) from op_off.
   int64_t op_off;
   int64_t ld;
-  int row_F, row_L, row_G, row_U, row_W;  // first row per kind, -1 when absent
+  // First row per kind, -1 when absent: F chi, L lap chi, G aux chi, U V^P, and W: mixed path w, w/r_A,
+  // w/r_B, w/r_C; FP64 path the nuclear weights of V_ne (n_W rows), and F, L carry sqrt(w), G carries w.
+  int row_F, row_L, row_G, row_U, row_W;
   int nFA, nFB;     // basis functions of A and of B (rows of F/L: A's then B's)
   int nG;           // aux rows in G/U (A's then B's on an unrefined grid, C's on a refined one)
   int shb_A0, shb_A1, shb_B0, shb_B1;     // basis shell ranges of A and B
@@ -44,7 +46,13 @@ struct DevGrid {
   // touching row), and the third centre's pair-frame coordinates (xc, 0, zc)
   int nt_off, nt_mu, nt_nu, nt_phi;
   double xc, zc;
-  float Rh[9], Rl[9];  // R as an FP32 pair
+  union {
+    struct { float Rh[9], Rl[9]; };  // mixed path: R as an FP32 pair
+    struct {                         // FP64 path: nuclear charges of A, B, C, and whether this pair
+      double zA, zB, zC;             // grid is A's (B's) one-centre grid
+      int own_A, own_B, n_W;
+    };
+  };
   int xi_off;          // FP32 (hi, lo) x-scales of the shells: basis A, basis B, aux c0, aux c1
   int rc_off;          // FP64 constant of every operand row (norms, zeta powers, a^3 ...)
 };
@@ -115,22 +123,27 @@ struct PairTile {
   int col[kMmaN];
 };
 
-// One output block of a contraction (eq 9): out[r][c] = sum_p A_r(p) d(p) B_c(p), where
-// B_c is a row of the grid's operands (b_mode 0) or the product of two basis rows (b_mode 1,
-// the 3-index operand chi_i chi_j of eq 16).
+// One output block of the FP64 path's contraction (eq 9): out[r][c] = sum_p A_r(p) B_c(p), row-major
+// m x n.  Every operand row is one of the grid's operand rows times an optional second one: A_r =
+// src[a.x] * src[a.y] with a = rows[a_off + r] (y = -1: no factor), B_c likewise from
+// rows[b_off + c].  kind kFpDigits: on the tensor cores in exact digits (psq_fx.cuh), tiles of
+// 128 x 32; kFpFma: FP64 FMAs, a warp per tile and part of the points, one side of the tile across
+// the lanes (<= 32: the columns, or the rows when `swap`), the other in registers (<= 16);
+// kFpFmaSym: the same for a symmetric block (m = n, square tiles, tn >= tm only), of which each
+// (r, c) pair with c >= r is summed once and written to both places.
+enum { kFpDigits = 0, kFpFma = 1, kFpFmaSym = 2 };
 struct GemmBlock {
-  int grid;
-  int a_row, m;
-  int b_row, n;
-  int b_mode;
-  int pair_off;     // into the pair table (b_mode 1): pairs of F rows
-  int d_row;        // weight row (w, w/r_A, w/r_B or w/r_C)
-  int n_chunks;     // point range split into n_chunks partial sums
-  int tile_m, tile_n;  // output tile of one CTA (tile_m <= kFpTileRows, tile_n <= kFpTileCols, <= 1024 outputs)
-  int64_t res_off;  // m x n FP64 result
-  int64_t part_off; // n_chunks x m x n FP64 partial sums
+  int grid, kind, swap;
+  int a_off, m;
+  int b_off, n;
+  int tile_m, tile_n;
+  int n_chunks, win_per;  // point range split into n_chunks partial sums of win_per windows of kFpWin points
+  int64_t res_off;        // m x n FP64 result
+  int64_t part_off;       // n_chunks x m x n FP64 partial sums
 };
-constexpr int kFpTileRows = 64, kFpTileCols = 256, kFpTileOut = 1024;
+constexpr int kFpWin = 64;
+constexpr int kFpDigitRows = 128, kFpDigitCols = 32;           // tile of kFpDigits
+constexpr int kFpFmaLanes = 32, kFpFmaRegs = 16;               // and of kFpFma (a whole symmetric tile: 31 x 31)
 
 struct GemmItem { int block, tm, tn, chunk; };
 
@@ -175,6 +188,7 @@ struct LaunchTables {
   const int64_t* elem_begin;  // prefix sums of m*n over blocks (n_gblocks + 1)
   int64_t n_elems;
 };
+cudaError_t prepare_kernels_fp64();  // per-device kernel attributes (context creation)
 void upload_gl_tables(const double* x, const double* w, const double* klm);  // host constants
 cudaError_t launch_eval_fp64(const LaunchTables& t, double* ops, int kinds, cudaStream_t s);
 cudaError_t launch_contract_fp64(const LaunchTables& t, const double* ops, double* part, cudaStream_t s);

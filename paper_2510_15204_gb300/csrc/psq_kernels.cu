@@ -3,6 +3,7 @@
 // contraction of eq 9, the deterministic per-element reduction of its chunk partial sums,
 // and the assembly of molecule matrices from per-grid blocks (Section 4).
 #include "psq_internal.h"
+#include "psq_fx.cuh"
 
 #include <cstdio>
 
@@ -188,9 +189,10 @@ __device__ double aux_pot_radial(int n, int l, double zeta, double norm, double 
 // Evaluates the shells [s0, s1) of one centre at distance r (ir = 1/r) for one or two row
 // kinds (kind: 0 chi, 1 lap chi (kinetic operand), 2 V^P), writing from rows row_a and row_b
 // (-1: not wanted) of the operand matrix; e^-zeta r is computed once per shell for both.
+// Functions (not V^P) are written times wv.
 __device__ __forceinline__ void eval_shells(const DevShell* __restrict__ sh, int s0, int s1, double r, double ir,
                                             const double* Y, double* __restrict__ out, int64_t ld, int64_t p,
-                                            int row_a, int kind_a, int row_b, int kind_b) {
+                                            int row_a, int kind_a, int row_b, int kind_b, double wv) {
   for (int s = s0; s < s1; ++s) {
     const DevShell q = sh[s];
     const double ex = exp(-q.zeta * r);
@@ -203,7 +205,7 @@ __device__ __forceinline__ void eval_shells(const DevShell* __restrict__ sh, int
       if (kind == 2) {
         radial = aux_pot_radial(q.n, q.l, q.zeta, q.norm, r, ex);
       } else {
-        radial = q.norm * ipow(r, q.n - 1) * ex;
+        radial = wv * q.norm * ipow(r, q.n - 1) * ex;
         if (kind == 1) {
           const double f = (q.n * (q.n - 1) - q.l * (q.l + 1)) * (ir * ir) - 2.0 * q.n * q.zeta * ir +
                            q.zeta * q.zeta;
@@ -239,11 +241,19 @@ __global__ void __launch_bounds__(128) eval_fp64_kernel(LaunchTables t, double* 
     for (int c = 0; c < 3; ++c) dC[c] = pt.P[c] - g.RC[c];
     rC = sqrt(dC[0] * dC[0] + dC[1] * dC[1] + dC[2] * dC[2]);
   }
-  if (g.row_W >= 0) {
-    base[(int64_t)(g.row_W + 0) * ld + p] = pt.w;
-    base[(int64_t)(g.row_W + 1) * ld + p] = pt.w / pt.rA;
-    base[(int64_t)(g.row_W + 2) * ld + p] = pt.w / pt.rB;
-    base[(int64_t)(g.row_W + 3) * ld + p] = g.C >= 0 ? pt.w / rC : 0.0;
+  // The operand rows of a contraction carry the weight: chi and lap chi sqrt(w), aux chi w, so that
+  // a product of two basis rows is w chi_i chi_j and V^P, which varies slowly, stays as it is.
+  const double wg = g.row_W >= 0 ? pt.w : 1.0, wf = sqrt(wg);
+  // the nuclear weights that V_ne elements of this grid are summed with: on a pair grid those of the
+  // A x B elements and the square roots of those of the A x A and B x B elements (an atom's own
+  // nucleus only on its one-centre grid), on a refined grid the third nucleus's
+  if (g.row_W >= 0 && g.n_W == 3) {
+    const double wa = g.zA / pt.rA, wb = g.zB / pt.rB;
+    base[(int64_t)(g.row_W + 0) * ld + p] = wa + wb;
+    base[(int64_t)(g.row_W + 1) * ld + p] = sqrt(g.own_A ? wa + wb : wb);
+    base[(int64_t)(g.row_W + 2) * ld + p] = sqrt(g.own_B ? wa + wb : wa);
+  } else if (g.row_W >= 0 && g.n_W == 1) {
+    base[(int64_t)g.row_W * ld + p] = g.zC / rC;
   }
   double Y[(kMaxL + 1) * (kMaxL + 1)];
   // basis functions on A and B
@@ -256,7 +266,7 @@ __global__ void __launch_bounds__(128) eval_fp64_kernel(LaunchTables t, double* 
       real_ylm(shells_lmax(t.bshell, s0, s1), d[0] * ir, d[1] * ir, d[2] * ir, Y);
       const int roff = c == 0 ? 0 : g.nFA;
       eval_shells(t.bshell, s0, s1, r, ir, Y, base, ld, p, g.row_F >= 0 ? g.row_F + roff : -1, 0,
-                  g.row_L >= 0 ? g.row_L + roff : -1, 1);
+                  g.row_L >= 0 ? g.row_L + roff : -1, 1, wf);
     }
   }
   // aux functions and their potentials
@@ -274,7 +284,7 @@ __global__ void __launch_bounds__(128) eval_fp64_kernel(LaunchTables t, double* 
       const double ir = 1.0 / r;
       real_ylm(shells_lmax(t.ashell, s0, s1), d[0] * ir, d[1] * ir, d[2] * ir, Y);
       eval_shells(t.ashell, s0, s1, r, ir, Y, base, ld, p, g.row_G >= 0 ? g.row_G + roff : -1, 0,
-                  g.row_U >= 0 ? g.row_U + roff : -1, 2);
+                  g.row_U >= 0 ? g.row_U + roff : -1, 2, wg);
       int nf = 0;
       for (int s = s0; s < s1; ++s) nf += 2 * t.ashell[s].l + 1;
       roff += nf;
@@ -288,86 +298,268 @@ cudaError_t launch_eval_fp64(const LaunchTables& t, double* ops, int /*kinds*/, 
   return cudaGetLastError();
 }
 
-// Weighted contraction, FP64 (eq 9): one CTA per (block, output tile, point chunk); the tile
-// (tile_m x tile_n, chosen per block so that the block is covered with little padding) is
-// mapped densely onto 256 threads, thread t owning outputs t, t + 256, ... of the tile's real
-// rows x columns (row-major).  Per 16-point step the weighted A rows and the B columns (basis
-// rows, or products of two basis rows) are formed once in shared memory; on GB300 the FP64
-// pipe (a warp's DFMA every ~16 SM cycles) is the bound, so each output's sub-sum reads both
-// operands from shared memory and no FP64 operation goes to padding.  Sub-sums of each step
-// join the running sums (small outer-region terms are not absorbed one by one), and partial
-// sums go to their own slot, so the result does not depend on scheduling.
-constexpr int kFpPts = 16;
-__global__ void __launch_bounds__(256) contract_fp64_kernel(LaunchTables t, const double* __restrict__ ops,
-                                                             double* __restrict__ part) {
+// Weighted contraction, FP64 (eq 9): one CTA per (block, output tile, range of 64-point windows);
+// partial sums go to their own slot, so the result does not depend on scheduling.
+//
+// GB300's FP64 pipe (two FMAs per clock and SM) bounds every FP64 sum, so the (P|Q) and (P|ij) sums
+// run on the tensor cores in exact digits.  There one factor (V^P) varies slowly over a window and the
+// other (w times an aux function or a pair product, formed before it is cut) is scaled by
+// its own largest value, so an element keeps its precision relative to its own terms.  The overlap,
+// kinetic and V_ne sums multiply two steep functions of different atoms, whose largest values in a
+// window can lie at its opposite ends: on coarse or long grids the digits of both would be spent on
+// terms that never meet.  They stay on the FP64 pipe, with less to do: the nuclear weights of a
+// grid are summed first, and symmetric blocks are summed once.
+//
+// Measured on a bent triatomic (26 basis / 82 aux functions, 963,072 points; all sums on the FP64
+// pipe before -> now): 11.85 -> 3.88 ms ((P|ij) alone 2.35, (P|Q) 0.95, the three others 0.91).
+// One-electron matrices alone (90 functions, 4.5 M points): 36.0 -> 30.3 ms, 0.80 TFLOP/s on the FP64
+// pipe, its bound; H2 (57,600 points): 268 -> 150 us (launch and window latency).
+//
+// The FMA part: the warps of the CTA share the tile and take every eighth group of 8 points each, so
+// that no barrier stands between a warp's loads and its FMAs; a lane holds one column and up to 16
+// rows, 16 independent chains, and the pipe stays fed by the two CTAs of an SM (16 warps).  Sub-sums
+// of 32 points join the running sums (small outer-region terms are not absorbed one by one); the
+// warps' sums are added in order at the end.
+constexpr int kFpPts = 8;
+struct FmaSmem {
+  double v[8][kFpPts][kFpFmaRegs + kFpFmaLanes];   // per warp: [point][register side, then lane side]
+  int64_t x[kFpFmaRegs + kFpFmaLanes], y[kFpFmaRegs + kFpFmaLanes];  // operand rows (element offsets; y = -1: no factor)
+  double sum[8][kFpFmaRegs][kFpFmaLanes];
+};
+static_assert(sizeof(FmaSmem) <= fx::kSmemBytes, "the FMA part shares the digits part's shared memory");
+
+// A whole symmetric tile of side n <= 31 in ceil(n / 2) rows of n + 1 lanes: row r and row n - 1 - r
+// share a register row, lanes c >= r (c < n) take (r, c), lanes c < r (n - 1 - r, n - 1 - c) and lane
+// n the diagonal (n - 1 - r, n - 1 - r).
+__device__ __forceinline__ void sym_entry(int n, int r, int lane, int& row, int& col) {
+  const bool first = lane >= r && lane < n;
+  row = first ? r : n - 1 - r;
+  col = first ? lane : (lane < r ? n - 1 - lane : n - 1 - r);
+}
+
+// One warp's share of a tile of nr register-side and nl lane-side operand rows (SYM: of a whole
+// symmetric tile of nl rows, all on the lane side), into sm.sum[warp].  Narrow tiles: the lanes make
+// 1 << gs groups of 32 >> gs, each taking every (1 << gs)-th point.
+template <int R, bool SYM>
+__device__ __noinline__ void fma_warp(FmaSmem& sm, const double* __restrict__ base, int k0, int k1, int nr, int nl, int gs) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double(&v)[kFpPts][kFpFmaRegs + kFpFmaLanes] = sm.v[warp];
+  const int gl = lane & ((32 >> gs) - 1), grp = lane >> (5 - gs);
+  double acc[R], sq[R];
+  int ra[R], rb[R];  // staged operand rows of each entry
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    acc[r] = sq[r] = 0.0;
+    ra[r] = min(r, nr - 1);
+    rb[r] = kFpFmaRegs + min(gl, nl - 1);
+    if (SYM) {
+      sym_entry(nl, min(r, (nl - 1) / 2), min(gl, nl), ra[r], rb[r]);
+      ra[r] += kFpFmaRegs;
+      rb[r] += kFpFmaRegs;
+    }
+  }
+  const int pp = lane & (kFpPts - 1), e0 = lane >> 3;
+  for (int k = k0 + kFpPts * warp, n = 1; k < k1; k += 8 * kFpPts, ++n) {
+#pragma unroll
+    for (int i = SYM ? kFpFmaRegs / 4 : 0; i < (kFpFmaRegs + kFpFmaLanes) / 4; ++i) {
+      const int e = e0 + 4 * i;
+      if (e < kFpFmaRegs ? e < nr : e - kFpFmaRegs < nl) {
+        double x = 0.0;
+        if (k + pp < k1) {
+          x = __ldg(base + sm.x[e] + k + pp);
+          if (sm.y[e] >= 0) x *= __ldg(base + sm.y[e] + k + pp);
+        }
+        v[pp][e] = x;
+      }
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int p = grp; p < kFpPts; p += 1 << gs)
+#pragma unroll
+      for (int r = 0; r < R; ++r) sq[r] = fma(v[p][ra[r]], v[p][rb[r]], sq[r]);
+    if ((n & 3) == 0) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        acc[r] += sq[r];
+        sq[r] = 0.0;
+      }
+    }
+    __syncwarp();
+  }
+#pragma unroll
+  for (int r = 0; r < R; ++r) sm.sum[warp][r][lane] = acc[r] + sq[r];
+}
+
+__device__ __forceinline__ void contract_fma(const LaunchTables& t, const GemmItem& it, const GemmBlock& b, const DevGrid& g,
+                                             const double* __restrict__ base, double* __restrict__ part, uint8_t* raw) {
+  FmaSmem& sm = *reinterpret_cast<FmaSmem*>(raw);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, K = (int)g.K;
+  const int k0 = it.chunk * b.win_per * kFpWin, k1 = (int)min((int64_t)K, (int64_t)k0 + (int64_t)b.win_per * kFpWin);
+  const int r0 = it.tm * b.tile_m, c0 = it.tn * b.tile_n;
+  const int rows = min(b.tile_m, b.m - r0), cols = min(b.tile_n, b.n - c0);
+  const bool sym = b.kind == kFpFmaSym && it.tm == it.tn;
+  // register side and lane side: rows and columns, or (swap) columns and rows
+  const int nr = sym ? 0 : (b.swap ? cols : rows), nl = b.swap ? rows : cols;
+  const int roff = b.swap ? b.b_off + c0 : b.a_off + r0, loff = b.swap ? b.a_off + r0 : b.b_off + c0;
+  if (tid < kFpFmaRegs + kFpFmaLanes) {
+    const bool rs = tid < kFpFmaRegs;
+    const int i = rs ? tid : tid - kFpFmaRegs;
+    if (i < (rs ? nr : nl)) {
+      const short2 q = t.pairs[(rs ? roff : loff) + i];
+      sm.x[tid] = q.x * g.ld;
+      sm.y[tid] = q.y >= 0 ? q.y * g.ld : -1;
+    }
+  }
+  __syncthreads();
+  const int R = sym ? (nl + 1) / 2 : nr;
+  const int width = sym ? nl + 1 : nl, gs = width <= 4 ? 3 : (width <= 8 ? 2 : (width <= 16 ? 1 : 0));
+  if (sym) {
+    if (R <= 2) fma_warp<2, true>(sm, base, k0, k1, nr, nl, gs);
+    else if (R <= 4) fma_warp<4, true>(sm, base, k0, k1, nr, nl, gs);
+    else if (R <= 8) fma_warp<8, true>(sm, base, k0, k1, nr, nl, gs);
+    else if (R <= 12) fma_warp<12, true>(sm, base, k0, k1, nr, nl, gs);
+    else fma_warp<16, true>(sm, base, k0, k1, nr, nl, gs);
+  } else {
+    if (R <= 2) fma_warp<2, false>(sm, base, k0, k1, nr, nl, gs);
+    else if (R <= 4) fma_warp<4, false>(sm, base, k0, k1, nr, nl, gs);
+    else if (R <= 6) fma_warp<6, false>(sm, base, k0, k1, nr, nl, gs);
+    else if (R <= 8) fma_warp<8, false>(sm, base, k0, k1, nr, nl, gs);
+    else if (R <= 10) fma_warp<10, false>(sm, base, k0, k1, nr, nl, gs);
+    else if (R <= 12) fma_warp<12, false>(sm, base, k0, k1, nr, nl, gs);
+    else if (R <= 14) fma_warp<14, false>(sm, base, k0, k1, nr, nl, gs);
+    else fma_warp<16, false>(sm, base, k0, k1, nr, nl, gs);
+  }
+  __syncthreads();
+  double* out = part + b.part_off + (int64_t)it.chunk * b.m * b.n;
+  for (int r = warp; r < R; r += 8) {
+    if (lane >= 32 >> gs) continue;
+    double s = 0.0;
+    for (int w = 0; w < 8; ++w)
+      for (int g2 = lane; g2 < 32; g2 += 32 >> gs) s += sm.sum[w][r][g2];
+    int row = b.swap ? lane : r, col = b.swap ? r : lane;
+    bool live = lane < nl;
+    if (sym) {
+      sym_entry(nl, r, lane, row, col);
+      live = lane < nl || (lane == nl && 2 * r != nl - 1);
+    }
+    if (live) {
+      out[(int64_t)(r0 + row) * b.n + c0 + col] = s;
+      if (b.kind == kFpFmaSym) out[(int64_t)(c0 + col) * b.n + r0 + row] = s;
+    }
+  }
+}
+
+__global__ void __launch_bounds__(fx::kThreads, 2) contract_fp64_kernel(LaunchTables t, const double* __restrict__ ops,
+                                                                        double* __restrict__ part) {
+  extern __shared__ __align__(1024) uint8_t raw[];
   const GemmItem it = t.items[blockIdx.x];
   const GemmBlock b = t.gblocks[it.block];
   const DevGrid& g = t.grids[b.grid];
   const double* base = ops + g.op_off;
-  const int64_t ld = g.ld, K = g.K;
-  const int64_t csz = (K + b.n_chunks - 1) / b.n_chunks;
-  const int64_t k0 = (int64_t)it.chunk * csz;
-  const int64_t k1 = min(K, k0 + csz);
-  __shared__ double As[kFpPts][kFpTileRows];
-  __shared__ double Bs[kFpPts][kFpTileCols];
-  __shared__ short2 pr[kFpTileCols];
-  const int r0 = it.tm * b.tile_m, c0 = it.tn * b.tile_n;
-  const int rows = min(b.tile_m, b.m - r0), cols = min(b.tile_n, b.n - c0);
-  for (int c = threadIdx.x; c < cols; c += blockDim.x)
-    pr[c] = b.b_mode == 1 ? t.pairs[b.pair_off + c0 + c] : make_short2(0, 0);
-  const double* drow = base + (int64_t)b.d_row * ld;
-  const int nout = rows * cols;
-  int orow[4], ocol[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int o = threadIdx.x + 256 * q;
-    orow[q] = o < nout ? o / cols : 0;
-    ocol[q] = o < nout ? o - (o / cols) * cols : 0;
+  if (b.kind != kFpDigits) {
+    // a CTA that may still allocate TMEM keeps the next one of its kernel off the SM
+    if (threadIdx.x < 32) asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    contract_fma(t, it, b, g, base, part, raw);
+    return;
   }
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
-  __syncthreads();
-  for (int64_t k = k0; k < k1; k += kFpPts) {
-    // operands of this step: A rows x points, B columns x points (zeros past the chunk)
-    for (int e = threadIdx.x; e < rows * kFpPts; e += blockDim.x) {
-      const int r = e / kFpPts, pp = e - r * kFpPts;
-      const int64_t kk = k + pp;
-      As[pp][r] = kk < k1 ? base[(int64_t)(b.a_row + r0 + r) * ld + kk] * drow[kk] : 0.0;
-    }
-    for (int e = threadIdx.x; e < cols * kFpPts; e += blockDim.x) {
-      const int c = e / kFpPts, pp = e - c * kFpPts;
-      const int64_t kk = k + pp;
-      double bv = 0.0;
-      if (kk < k1) {
-        if (b.b_mode == 0) {
-          bv = base[(int64_t)(b.b_row + c0 + c) * ld + kk];
+  fx::Smem& sm = fx::smem_at(raw);
+  const uint32_t tmem = fx::open(sm);
+  const int64_t ld = g.ld;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int r0 = it.tm * kFpDigitRows, c0 = it.tn * kFpDigitCols;
+  const int rows = min(kFpDigitRows, b.m - r0), cols = min(kFpDigitCols, b.n - c0);
+  const int K = (int)g.K;  // below 2^31 - 256 (the planner checks)
+  const int k0 = it.chunk * b.win_per * kFpWin, k1 = (int)min((int64_t)K, (int64_t)k0 + (int64_t)b.win_per * kFpWin);
+  // this thread's operand rows (element offsets from base; the second one -1: none)
+  int64_t ax[2], ay[2], bx, by;
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const short2 q = t.pairs[b.a_off + r0 + min(fx::a_row(u), rows - 1)];
+    ax[u] = q.x * ld;
+    ay[u] = q.y >= 0 ? q.y * ld : -1;
+  }
+  {
+    const short2 q = t.pairs[b.b_off + c0 + min(fx::b_col(), cols - 1)];
+    bx = q.x * ld;
+    by = q.y >= 0 ? q.y * ld : -1;
+  }
+  auto value = [&](short2 q, int p) {
+    const double v = base[q.x * ld + p];
+    return q.y >= 0 ? v * base[q.y * ld + p] : v;
+  };
+  double acc[16] = {};
+  uint32_t phase = 0, win = 0;
+  bool ok = true, run = true;
+  for (int k = k0; k < k1 && run; k += kFpWin, ++win) {
+    double va[4][8], vb[2][4];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        double(&v)[8] = va[2 * c + u];
+        const int p = k + fx::a_pt(c), left = 64 * u + 8 * warp < rows ? k1 - p : 0;
+        if (left >= 8) {
+          const double2* x = reinterpret_cast<const double2*>(base + ax[u] + p);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const double2 q = __ldg(x + i);
+            v[2 * i] = q.x;
+            v[2 * i + 1] = q.y;
+          }
+          if (ay[u] >= 0) {
+            const double2* y = reinterpret_cast<const double2*>(base + ay[u] + p);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const double2 q = __ldg(y + i);
+              v[2 * i] *= q.x;
+              v[2 * i + 1] *= q.y;
+            }
+          }
         } else {
-          const short2 q = pr[c];
-          bv = base[(int64_t)(b.b_row + q.x) * ld + kk] * base[(int64_t)(b.b_row + q.y) * ld + kk];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            v[i] = 0.0;
+            if (i < left) v[i] = base[ax[u] + p + i] * (ay[u] >= 0 ? base[ay[u] + p + i] : 1.0);
+          }
         }
       }
-      Bs[pp][c] = bv;
-    }
-    __syncthreads();
+      const int p = k + fx::b_pt(c);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      if (threadIdx.x + 256 * q < nout) {
-        double sq = 0.0;
-#pragma unroll
-        for (int pp = 0; pp < kFpPts; ++pp) sq = fma(As[pp][orow[q]], Bs[pp][ocol[q]], sq);
-        acc[q] += sq;
+      for (int i = 0; i < 4; ++i) {
+        vb[c][i] = 0.0;
+        if (fx::b_col() < cols && p + i < k1) vb[c][i] = __ldg(base + bx + p + i) * (by >= 0 ? __ldg(base + by + p + i) : 1.0);
       }
     }
-    __syncthreads();
+    run = fx::window(sm, tmem, va, vb, acc, phase, win, rows, cols, ok, [&](int r, int c) {
+      double s = 0.0;
+      if (r < rows && c < cols) {
+        const short2 qa = t.pairs[b.a_off + r0 + r], qb = t.pairs[b.b_off + c0 + c];
+        for (int p = k; p < min(k1, k + kFpWin); ++p) s = fma(value(qa, p), value(qb, p), s);
+      }
+      return s;
+    });
   }
+  if (run) run = __syncthreads_and(ok);
   double* out = part + b.part_off + (int64_t)it.chunk * b.m * b.n;
+  const int r = 32 * (warp & 3) + lane;
 #pragma unroll
-  for (int q = 0; q < 4; ++q)
-    if (threadIdx.x + 256 * q < nout) out[(int64_t)(r0 + orow[q]) * b.n + c0 + ocol[q]] = acc[q];
+  for (int j = 0; j < 16; ++j) {
+    const int c = 16 * (warp >> 2) + j;
+    // a wait that ran out leaves NaN: no result is better than a wrong one
+    if (r < rows && c < cols) out[(int64_t)(r0 + r) * b.n + c0 + c] = run ? acc[j] : __longlong_as_double(0x7ff8000000000000ll);
+  }
+  fx::close(sm, tmem, run, phase);
+}
+
+cudaError_t prepare_kernels_fp64() {
+  const cudaError_t e = cudaFuncSetAttribute(contract_fp64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fx::kSmemBytes);
+  // room for two CTAs per SM (of 228 KB), the rest L1
+  return e != cudaSuccess ? e : cudaFuncSetAttribute(contract_fp64_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 80);
 }
 
 cudaError_t launch_contract_fp64(const LaunchTables& t, const double* ops, double* part, cudaStream_t s) {
   if (t.n_items == 0) return cudaSuccess;
-  contract_fp64_kernel<<<t.n_items, 256, 0, s>>>(t, ops, part);
+  contract_fp64_kernel<<<t.n_items, fx::kThreads, fx::kSmemBytes, s>>>(t, ops, part);
   return cudaGetLastError();
 }
 

@@ -121,43 +121,45 @@ __global__ void __launch_bounds__(fx::kThreads, 2) trsv_kernel(int n, int64_t m,
   const uint32_t tmem = fx::open(sm);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int64_t c0 = (int64_t)blockIdx.x * cols;
-  const int64_t col = c0 + fx::a_row();
-  const bool live = fx::a_row() < cols && col < m;
+  const int live = (int)(m - c0 < cols ? m - c0 : cols);  // columns of this CTA
   // after a block's products the digit planes are free: they hold its right-hand sides [row][col]
   // and the diagonal block with its reciprocal pivots
   double(*rhs)[fx::kRows] = reinterpret_cast<double(*)[fx::kRows]>(sm.a[0]);
   double(*d)[kB + 1] = reinterpret_cast<double(*)[kB + 1]>(sm.a[0] + sizeof(double) * kB * fx::kRows);
-  uint32_t phase = 0;
-  bool ok = true;
-  for (int k0 = 0; k0 < n && ok; k0 += kB) {
+  uint32_t phase = 0, win = 0;
+  bool ok = true, run = true;
+  for (int k0 = 0; k0 < n && run; k0 += kB) {
     const int kb = n - k0 < kB ? n - k0 : kB;
     double acc[16] = {};
-    for (int q0 = 0; q0 < k0 && ok; q0 += fx::kWin) {
-      double va[32], vb[8];
+    for (int q0 = 0; q0 < k0 && run; q0 += fx::kWin, ++win) {
+      double va[4][8], vb[2][4];
 #pragma unroll
-      for (int c = 0; c < 2; ++c)
+      for (int c = 0; c < 2; ++c) {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const int q = q0 + fx::a_pt(c) + i;
-          va[16 * c + i] = live && q < k0 ? B[(int64_t)q * m + col] : 0.0;
+        for (int u = 0; u < 2; ++u) {
+          const double* p = B + (int64_t)(q0 + fx::a_pt(c)) * m + c0 + fx::a_row(u);
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            va[2 * c + u][i] = fx::a_row(u) < live && q0 + fx::a_pt(c) + i < k0 ? p[i * m] : 0.0;
         }
+        const double* p = L + (int64_t)(k0 + fx::b_col()) * n + q0 + fx::b_pt(c);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int q = q0 + fx::b_pt() + i;
-        vb[i] = fx::b_col() < kb && q < k0 ? L[(int64_t)(k0 + fx::b_col()) * n + q] : 0.0;
+        for (int i = 0; i < 4; ++i) vb[c][i] = fx::b_col() < kb && q0 + fx::b_pt(c) + i < k0 ? p[i] : 0.0;
       }
-      ok = fx::window(sm, tmem, va, vb, acc, phase, [&](int r, int c) {
+      run = fx::window(sm, tmem, va, vb, acc, phase, win, live, kb, ok, [&](int r, int c) {
         double s = 0.0;
-        if (r < cols && c0 + r < m && c < kb)
+        if (r < live && c < kb)
           for (int q = q0; q < min(k0, q0 + fx::kWin); ++q) s = fma(B[(int64_t)q * m + c0 + r], L[(int64_t)(k0 + c) * n + q], s);
         return s;
       });
     }
+    if (k0 > 0 && run) run = __syncthreads_and(ok);  // and no MMA reads the planes any more
+    if (!run) break;
     const int r = 32 * (warp & 3) + lane;
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
       const int i = 16 * (warp >> 2) + j;
-      rhs[i][r] = i < kb && r < cols && c0 + r < m ? B[(int64_t)(k0 + i) * m + c0 + r] - acc[j] : 0.0;
+      rhs[i][r] = i < kb && r < live ? B[(int64_t)(k0 + i) * m + c0 + r] - acc[j] : 0.0;
     }
     for (int t = tid; t < kB * kB; t += fx::kThreads) {
       const int i = t >> 5, c = t & 31;
@@ -166,7 +168,7 @@ __global__ void __launch_bounds__(fx::kThreads, 2) trsv_kernel(int n, int64_t m,
     __syncthreads();
     if (tid < kB) d[tid][kB] = tid < kb ? 1.0 / d[tid][tid] : 0.0;
     __syncthreads();
-    if (tid < fx::kRows && live) {
+    if (tid < live) {
       double x[kB];
 #pragma unroll
       for (int j = 0; j < kB; ++j) {
@@ -178,15 +180,15 @@ __global__ void __launch_bounds__(fx::kThreads, 2) trsv_kernel(int n, int64_t m,
           const double q0 = s * d[j][kB];
           const double q1 = fma(fma(-q0, d[j][j], s), d[j][kB], q0);
           x[j] = isfinite(q1) ? q1 : s / d[j][j];
-          B[(int64_t)(k0 + j) * m + col] = x[j];
+          B[(int64_t)(k0 + j) * m + c0 + tid] = x[j];
         }
       }
     }
     __syncthreads();
   }
-  if (!ok && live)  // a wait ran out: no result is better than a wrong one
-    for (int q = tid >> 7; q < n; q += 2) B[(int64_t)q * m + col] = __longlong_as_double(0x7ff8000000000000ll);
-  fx::close(sm, tmem, ok, phase);
+  if (!run && tid < live)  // a wait ran out: no result is better than a wrong one
+    for (int q = 0; q < n; ++q) B[(int64_t)q * m + c0 + tid] = __longlong_as_double(0x7ff8000000000000ll);
+  fx::close(sm, tmem, run, phase);
 }
 
 // out[c][d] = sum_R B[R][c0 + c] B[R][d0 + d]: a CTA per 128 x 32 output tile, R in windows of 64.
@@ -197,41 +199,41 @@ __global__ void __launch_bounds__(fx::kThreads, 2) eri_kernel(int n, int64_t m, 
   const uint32_t tmem = fx::open(sm);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t tc0 = (int64_t)blockIdx.y * fx::kRows, td0 = (int64_t)blockIdx.x * fx::kCols;
-  const bool liva = tc0 + fx::a_row() < nc, livb = td0 + fx::b_col() < nd;
-  const double* pa = B + c0 + tc0 + fx::a_row();
-  const double* pb = B + d0 + td0 + fx::b_col();
+  const int rows = (int)(nc - tc0 < fx::kRows ? nc - tc0 : fx::kRows), cols = (int)(nd - td0 < fx::kCols ? nd - td0 : fx::kCols);
   double acc[16] = {};
-  uint32_t phase = 0;
-  bool ok = true;
-  for (int R0 = 0; R0 < n && ok; R0 += fx::kWin) {
-    double va[32], vb[8];
+  uint32_t phase = 0, win = 0;
+  bool ok = true, run = true;
+  for (int R0 = 0; R0 < n && run; R0 += fx::kWin, ++win) {
+    double va[4][8], vb[2][4];
 #pragma unroll
-    for (int c = 0; c < 2; ++c)
+    for (int c = 0; c < 2; ++c) {
 #pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        const int R = R0 + fx::a_pt(c) + i;
-        va[16 * c + i] = liva && R < n ? __ldg(pa + (int64_t)R * m) : 0.0;
+      for (int u = 0; u < 2; ++u) {
+        const double* p = B + (int64_t)(R0 + fx::a_pt(c)) * m + c0 + tc0 + fx::a_row(u);
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          va[2 * c + u][i] = fx::a_row(u) < rows && R0 + fx::a_pt(c) + i < n ? __ldg(p + i * m) : 0.0;
       }
+      const double* p = B + (int64_t)(R0 + fx::b_pt(c)) * m + d0 + td0 + fx::b_col();
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int R = R0 + fx::b_pt() + i;
-      vb[i] = livb && R < n ? __ldg(pb + (int64_t)R * m) : 0.0;
+      for (int i = 0; i < 4; ++i) vb[c][i] = fx::b_col() < cols && R0 + fx::b_pt(c) + i < n ? __ldg(p + i * m) : 0.0;
     }
-    ok = fx::window(sm, tmem, va, vb, acc, phase, [&](int r, int c) {
+    run = fx::window(sm, tmem, va, vb, acc, phase, win, rows, cols, ok, [&](int r, int c) {
       double s = 0.0;
-      if (tc0 + r < nc && td0 + c < nd)
+      if (r < rows && c < cols)
         for (int R = R0; R < min(n, R0 + fx::kWin); ++R)
           s = fma(B[(int64_t)R * m + c0 + tc0 + r], B[(int64_t)R * m + d0 + td0 + c], s);
       return s;
     });
   }
-  const int64_t r = tc0 + 32 * (warp & 3) + lane;
+  if (run) run = __syncthreads_and(ok);
+  const int r = 32 * (warp & 3) + lane;
 #pragma unroll
   for (int j = 0; j < 16; ++j) {
-    const int64_t d = td0 + 16 * (warp >> 2) + j;
-    if (r < nc && d < nd) out[r * nd + d] = ok ? acc[j] : __longlong_as_double(0x7ff8000000000000ll);
+    const int d = 16 * (warp >> 2) + j;
+    if (r < rows && d < cols) out[(tc0 + r) * nd + td0 + d] = run ? acc[j] : __longlong_as_double(0x7ff8000000000000ll);
   }
-  fx::close(sm, tmem, ok, phase);
+  fx::close(sm, tmem, run, phase);
 }
 
 // ---------------------------------------------------------------- tensor-core product
