@@ -54,7 +54,6 @@ psq_status fail(psq_status s, const char* fmt, ...) {
   } while (0)
 
 constexpr double kOnAxisTol = 1e-10;  // a third centre this close (x a) to the axis is on it
-constexpr int kPointsPerBlock = 128;
 constexpr int kSmCount = 152;
 constexpr size_t kDefaultWaveBytes = (size_t)6 << 30;  // mixed path: operand + packed bytes per wave
 
@@ -392,6 +391,30 @@ void row_constants(const psq_job* j, const DevGrid& g, int kind, std::vector<dou
                                 : d.norm * klm_norm(d.l, m) * std::pow(d.zeta, -(d.n - 1)));
     }
   }
+}
+
+// The evaluation CTAs of grid g: all node pairs of a column and all its phi rows where their tables
+// fit the CTA's shared memory, else fewer pairs, then fewer phi rows; the phi rows in at least `split`
+// parts (as far as there are rows).
+void point_blocks(int gi, const DevGrid& g, int split, std::vector<PointBlock>& out) {
+  const bool third = g.C >= 0;
+  const int pair_entries = 2 * ((g.shb_A1 - g.shb_A0) + (g.shb_B1 - g.shb_B0) +
+                                (third ? 0 : (g.sha_1 - g.sha_0) + (g.sha_3 - g.sha_2)));
+  const int node_entries = third ? g.sha_1 - g.sha_0 + 1 : 0;  // per phi node (and its distance from the centre)
+  const int budget = kEvalTabBytes / 8, np = g.q_mu * g.q_nu;
+  int npb = np;
+  while (npb > 1 && (pair_entries + g.q_phi * node_entries) * npb > budget) npb = (npb + 1) / 2;
+  auto column = [&](int col, int rows) {
+    const int half = (rows + 1) / 2;
+    int hc = std::min((half + split - 1) / split, std::max(1, kEvalMaxNodes / g.q_phi));
+    if (node_entries) hc = std::max(1, std::min(hc, (budget / npb - pair_entries) / (g.q_phi * node_entries)));
+    for (int u = 0; u < half; u += hc)
+      for (int q = 0; q < np; q += npb)
+        out.push_back(PointBlock{gi, col, u, std::min(half, u + hc), (short)q, (short)std::min(np, q + npb)});
+  };
+  for (int c = 0; c < g.n_mu * g.n_nu; ++c) column(c, g.n_phi);
+  if (g.n_touch > 0)
+    for (int c = 0; c < g.nt_mu * g.nt_nu * g.n_sp * g.n_sp; ++c) column(g.n_mu * g.n_nu + c, g.nt_phi * g.n_sp);
 }
 
 psq_status make_plan(psq_job* j, unsigned mask, Plan& P) {
@@ -1192,14 +1215,18 @@ psq_status make_plan(psq_job* j, unsigned mask, Plan& P) {
       P.max_node_entries = std::max(P.max_node_entries, n);
     }
   }
-  for (size_t gi = 0; gi < P.grids.size(); ++gi)
-    for (int64_t p0 = 0; p0 < P.grids[gi].K; p0 += kPointsPerBlock) P.pblocks.push_back(PointBlock{(int)gi, 0, p0});
+  // evaluation CTAs: at least about four rounds of the four that an SM holds where there are few columns
+  int64_t columns = 0;
+  for (const DevGrid& g : P.grids) columns += (int64_t)g.n_mu * g.n_nu;
+  const int split = (int)std::min<int64_t>(64, columns > 0 ? (16LL * kSmCount + columns - 1) / columns : 1);
+  for (size_t gi = 0; gi < P.grids.size(); ++gi) point_blocks((int)gi, P.grids[gi], split, P.pblocks);
   for (Plan::Wave& wv : P.waves) {
-    wv.pb0 = wv.pb1 = (int)P.pblocks.size();
-    for (int k = 0; k < (int)P.pblocks.size(); ++k) {
-      if (P.pblocks[k].grid >= wv.g0 && wv.pb0 == (int)P.pblocks.size()) wv.pb0 = k;
-      if (P.pblocks[k].grid >= wv.g1) { wv.pb1 = k; break; }
-    }
+    auto first = [&](int g) {  // the blocks are in grid order
+      return (int)(std::lower_bound(P.pblocks.begin(), P.pblocks.end(), g,
+                                    [](const PointBlock& b, int v) { return b.grid < v; }) - P.pblocks.begin());
+    };
+    wv.pb0 = first(wv.g0);
+    wv.pb1 = first(wv.g1);
   }
   // useful contractions: for every molecule-matrix block, rows x cols x the live points of
   // the one grid that integrates it (same-atom blocks count i <= j once)
@@ -1518,6 +1545,7 @@ psq_status psq_job_create(psq_context* ctx, const psq_atom* atoms, int n_atoms, 
       d.fn0 = cnt[X];
       d.zeta = sh[i].zeta;
       d.norm = std::pow(2.0 * sh[i].zeta, sh[i].n + 0.5) / std::sqrt(factorial(2 * sh[i].n));
+      d.vnorm = 4.0 * M_PI / (2 * d.l + 1) * d.norm * std::pow(d.zeta, -(d.n + 1));
       dsh.push_back(d);
       for (int m = 0; m < 2 * sh[i].l + 1; ++m) {
         fatom.push_back(X);
@@ -2003,7 +2031,7 @@ psq_status psq_job_grid_functions(psq_job* job, int g, int kind, void* d_workspa
   if (rows) *rows = nrows;
   const bool mixed = job->prec == PSQ_MIXED;
   std::vector<PointBlock> pb;
-  for (int64_t p0 = 0; p0 < G.K; p0 += kPointsPerBlock) pb.push_back(PointBlock{0, 0, p0});
+  point_blocks(0, G, 1, pb);
   // mixed path: node table of this grid, the FP64 row constants and the hi/lo operand rows
   const int n_nodes = (G.n_mu + G.nt_mu * G.n_sp) * G.q_mu + (G.n_nu + G.nt_nu * G.n_sp) * G.q_nu +
                       (G.n_phi + G.nt_phi * G.n_sp) * G.q_phi;

@@ -16,6 +16,7 @@ constexpr int kMaxQ = 16;   // Gauss-Legendre points per dimension
 struct DevShell {
   int n, l, atom, fn0;   // fn0: first function index of the shell within its atom
   double zeta, norm;     // norm = (2 zeta)^(n+1/2) / sqrt((2n)!)
+  double vnorm;          // of V^P as a function of zeta r: 4 pi/(2l+1) norm zeta^-(n+1)
 };
 
 // One PS grid: a pair (A, B) with A at (0,0,+a) of its own frame, optionally refined around
@@ -166,7 +167,18 @@ struct SrcEntry {
 // offW+lj.
 struct J3Src { int64_t off; int s_pair, s_aux, mode, nloc, offY, offW; };
 
-struct PointBlock { int grid; int pad; int64_t p0; };  // evaluation: 128 points (one window) of one grid
+// Evaluation: one CTA's points.  A column of a grid is one (mu, nu) volume-element row pair with all
+// its phi rows (columns 0 .. n_mu n_nu - 1: the volume elements; then the (mu, nu) sub-row pairs of
+// the split ones).  The CTA takes the (mu, nu) node pairs [pr0, pr1) of the column (pair = i q_nu + j)
+// and the phi rows [u0, u1) of the first half with their mirror rows: the grid is symmetric under
+// phi -> -phi, and so is the distance from a third centre (which lies at phi = 0).
+struct PointBlock {
+  int grid, col, u0, u1;
+  short pr0, pr1;
+};
+// Shared memory of an evaluation CTA: values kept per (node pair, shell and kind) and, for a third
+// centre, per (node pair, phi node, shell).
+constexpr int kEvalThreads = 256, kEvalTabBytes = 48 << 10, kEvalMaxNodes = 256;  // phi nodes of [u0, u1)
 
 }  // namespace psq
 

@@ -121,30 +121,37 @@ __device__ __forceinline__ void ps_point(const DevGrid& g, const double* __restr
 
 // Real orthonormal spherical harmonics Y_lm(u), |u| = 1, l <= lmax, index l*l + l + m:
 // Y_lm = K_lm Q_l^|m|(u_z) {Re, Im}(u_x + i u_y)^|m|, with Q_m^m = (2m-1)!!,
-// Q_{m+1}^m = (2m+1) u_z Q_m^m, (l-m) Q_l^m = (2l-1) u_z Q_{l-1}^m - (l+m-1) Q_{l-2}^m.
+// Q_{m+1}^m = (2m+1) u_z Q_m^m, (l-m) Q_l^m = (2l-1) u_z Q_{l-1}^m - (l+m-1) Q_{l-2}^m (unrolled: the
+// coefficients are constants, a conversion or division would run on the FP64 pipe).
 __device__ __forceinline__ void real_ylm(int lmax, double ux, double uy, double uz, double* Y) {
-  double C[kMaxL + 1], S[kMaxL + 1];
-  C[0] = 1.0; S[0] = 0.0;
-  for (int m = 1; m <= lmax; ++m) {
-    C[m] = ux * C[m - 1] - uy * S[m - 1];
-    S[m] = ux * S[m - 1] + uy * C[m - 1];
-  }
-  double dfact = 1.0;  // (2m-1)!!
-  for (int m = 0; m <= lmax; ++m) {
-    if (m > 0) dfact *= (2 * m - 1);
+  double C = 1.0, S = 0.0, dfact = 1.0;  // Re, Im of (u_x + i u_y)^m; (2m-1)!!
+#pragma unroll
+  for (int m = 0; m <= kMaxL; ++m) {
+    if (m > lmax) break;
+    if (m > 0) {
+      const double c = ux * C - uy * S;
+      S = ux * S + uy * C;
+      C = c;
+      dfact *= 2 * m - 1;
+    }
     double q2 = 0.0, q1 = dfact;  // Q_{l-2}, Q_{l-1} as l climbs
-    for (int l = m; l <= lmax; ++l) {
-      double q;
-      if (l == m) q = dfact;
-      else if (l == m + 1) q = (2 * m + 1) * uz * dfact;
-      else q = ((2 * l - 1) * uz * q1 - (l + m - 1) * q2) / (l - m);
-      if (l > m) { q2 = q1; q1 = q; }
+#pragma unroll
+    for (int l = m; l <= kMaxL; ++l) {
+      if (l > lmax) break;
+      double q = dfact;
+      if (l > m) {
+        q = l == m + 1 ? (double)(2 * m + 1) * dfact * uz
+                       : ((double)(2 * l - 1) / (l - m)) * (uz * q1) - ((double)(l + m - 1) / (l - m)) * q2;
+        q2 = q1;
+        q1 = q;
+      }
       const int base = l * l + l;
+      const double kq = c_klm[base + m] * q;
       if (m == 0) {
-        Y[base] = c_klm[base] * q;
+        Y[base] = kq;
       } else {
-        Y[base + m] = c_klm[base + m] * q * C[m];
-        Y[base - m] = c_klm[base - m] * q * S[m];
+        Y[base + m] = kq * C;
+        Y[base - m] = kq * S;
       }
     }
   }
@@ -156,66 +163,47 @@ __device__ __forceinline__ double ipow(double x, int n) {
   return r;
 }
 
-// Radial factor of V^P (eq 16 written out by the Laplace expansion of 1/r12):
-// 4 pi/(2l+1) N [ gamma(n+l+2, zr)/(z^(n+l+2) r^(l+1)) + Gamma(n-l+1, zr) r^l / z^(n-l+1) ].
-// gamma by its positive series below x = k (no cancellation), by (k-1)! - Gamma above.
-__device__ double aux_pot_radial(int n, int l, double zeta, double norm, double r, double ex) {
-  const double x = zeta * r;  // ex = e^-x
+// 1 + x/a (1 + x/(a+1) (1 + ... x/b)): a finite exponential-type sum, from its last term.
+__device__ __forceinline__ double nested(double x, int a, int b) {
+  double s = 1.0;
+#pragma unroll 1
+  for (int j = b; j >= a; --j) s = fma(s, div_int(x, j), 1.0);
+  return s;
+}
+
+// Radial factor of V^P (eq 16 written out by the Laplace expansion of 1/r12) as a function of
+// x = zeta r, without its constant 4 pi/(2l+1) N zeta^-(n+1):
+// gamma(n+l+2, x)/x^(l+1) + Gamma(n-l+1, x) x^l, ex = e^-x.
+// gamma by its positive series below x = k (no cancellation), by (k-1)! - Gamma above; the number of
+// terms of the series comes from an FP32 run of it.
+__device__ __forceinline__ double aux_pot_radial(int n, int l, double x, double ex) {
   const int k1 = n + l + 2, k2 = n - l + 1;
   double inner;
   if (x < (double)k1) {
-    double term = c_rcpd[k1], sum = term;
+    const float xf = (float)x;
+    float t = 1.0f, s = 1.0f;
+    int m = 0;
 #pragma unroll 1
-    for (int i = 1; i < 1000; ++i) {
-      term *= div_int(x, k1 + i);
-      sum += term;
-      if (term <= 1e-17 * sum) break;
+    while (t > 3e-18f * s && m < kRcpD - 1 - k1) {
+      ++m;
+      t *= __fdividef(xf, (float)(k1 + m));
+      s += t;
     }
-    inner = ipow(r, n + 1) * ex * sum;  // x^k1 / (z^k1 r^(l+1)) = r^(n+1)
+    inner = ipow(x, n + 1) * ex * (c_rcpd[k1] * nested(x, k1 + 1, k1 + m));  // x^k1 / x^(l+1) = x^(n+1)
   } else {
-    double t = 1.0, s = 1.0;
-#pragma unroll 1
-    for (int j = 1; j < k1; ++j) { t *= div_int(x, j); s += t; }
     const double f = c_fact[k1 - 1];
-    inner = (f - f * ex * s) / (ipow(zeta, k1) * ipow(r, l + 1));
+    inner = (f - f * ex * nested(x, 1, k1 - 1)) * ipow(1.0 / x, l + 1);
   }
-  double t = 1.0, s = 1.0;
-#pragma unroll 1
-  for (int j = 1; j < k2; ++j) { t *= div_int(x, j); s += t; }
-  const double outer = c_fact[k2 - 1] * ex * s * ipow(r, l) / ipow(zeta, k2);
-  return 4.0 * M_PI / (2 * l + 1) * norm * (inner + outer);
+  return inner + c_fact[k2 - 1] * ex * nested(x, 1, k2 - 1) * ipow(x, l);
 }
 
-// Evaluates the shells [s0, s1) of one centre at distance r (ir = 1/r) for one or two row
-// kinds (kind: 0 chi, 1 lap chi (kinetic operand), 2 V^P), writing from rows row_a and row_b
-// (-1: not wanted) of the operand matrix; e^-zeta r is computed once per shell for both.
-// Functions (not V^P) are written times wv.
-__device__ __forceinline__ void eval_shells(const DevShell* __restrict__ sh, int s0, int s1, double r, double ir,
-                                            const double* Y, double* __restrict__ out, int64_t ld, int64_t p,
-                                            int row_a, int kind_a, int row_b, int kind_b, double wv) {
-  for (int s = s0; s < s1; ++s) {
-    const DevShell q = sh[s];
-    const double ex = exp(-q.zeta * r);
-    const int base = q.l * q.l + q.l;
-#pragma unroll 1
-    for (int h = 0; h < 2; ++h) {
-      const int row0 = h == 0 ? row_a : row_b, kind = h == 0 ? kind_a : kind_b;
-      if (row0 < 0) continue;
-      double radial;
-      if (kind == 2) {
-        radial = aux_pot_radial(q.n, q.l, q.zeta, q.norm, r, ex);
-      } else {
-        radial = wv * q.norm * ipow(r, q.n - 1) * ex;
-        if (kind == 1) {
-          const double f = (q.n * (q.n - 1) - q.l * (q.l + 1)) * (ir * ir) - 2.0 * q.n * q.zeta * ir +
-                           q.zeta * q.zeta;
-          radial *= f;
-        }
-      }
-      for (int m = -q.l; m <= q.l; ++m)
-        out[(int64_t)(row0 + q.fn0 + q.l + m) * ld + p] = radial * Y[base + m];
-    }
-  }
+// Radial factor of one row kind (0 chi, 1 lap chi (kinetic operand), 2 V^P) of a shell at distance
+// r: x = zeta r, ex = e^-x, ir = 1/r.
+__device__ __forceinline__ double radial_value(const DevShell& q, int kind, double r, double ir, double ex) {
+  if (kind == 2) return q.vnorm * aux_pot_radial(q.n, q.l, q.zeta * r, ex);
+  double v = q.norm * ipow(r, q.n - 1) * ex;
+  if (kind == 1) v *= (q.n * (q.n - 1) - q.l * (q.l + 1)) * (ir * ir) - 2.0 * q.n * q.zeta * ir + q.zeta * q.zeta;
+  return v;
 }
 
 __device__ __forceinline__ int shells_lmax(const DevShell* sh, int s0, int s1) {
@@ -224,77 +212,232 @@ __device__ __forceinline__ int shells_lmax(const DevShell* sh, int s0, int s1) {
   return l;
 }
 
-// One thread per point: the point (ps_point), its weight rows and the requested function
-// rows of the grid's centres.  Row layout: F/L rows are A's basis functions then B's
-// (fn0 counted within each atom), G/U rows the aux functions of the grid's aux centres.
-__global__ void __launch_bounds__(128) eval_fp64_kernel(LaunchTables t, double* __restrict__ ops) {
+// One row kind of a shell at one point: the radial value v times the harmonics.
+__device__ __forceinline__ void store_shell(const DevShell& q, double v, const double* Y, double* __restrict__ out, int64_t ld,
+                                            int64_t p, int row) {
+  const int base = q.l * q.l + q.l;
+  int64_t o = (int64_t)(row + q.fn0) * ld + p;
+  for (int m = -q.l; m <= q.l; ++m, o += ld) out[o] = v * Y[base + m];
+}
+
+// Evaluation, FP64: one CTA per PointBlock, the operand rows of its points (ps_point's forms of the
+// weight, the distances and the offsets).  GB300's FP64 pipe is the bound (two operations per clock
+// and SM), so nothing is computed twice on it: the trigonometric functions once per node, the radial
+// factors of A and B (exponentials, incomplete gamma series) once per (mu, nu) node pair for all phi,
+// those of a third centre for half of the phi nodes (phi -> -phi is a symmetry of the grid).  A point
+// is then its harmonics and one product per function.  Row layout: F/L rows are A's basis functions
+// then B's (fn0 counted within each atom), G/U rows the aux functions of the grid's aux centres.
+struct EvalNodes {
+  double mu[kMaxQ][4];             // sinh, cosh, sinh^2(v/2), weight
+  double nu[kMaxQ][5];             // sin, cos, sin^2(v/2), cos^2(v/2), weight
+  double ph[2 * kEvalMaxNodes][3];  // sin, cos, weight: the rows [u0, u1), then their mirrors
+  int meta[4];                     // lmax of A, B, C; functions of the first aux centre
+};
+constexpr int kEvalFp64Smem = (int)sizeof(EvalNodes) + kEvalTabBytes;
+
+__global__ void __launch_bounds__(kEvalThreads) eval_fp64_kernel(LaunchTables t, double* __restrict__ ops) {
+  extern __shared__ __align__(16) uint8_t raw[];
+  EvalNodes& nd = *reinterpret_cast<EvalNodes*>(raw);
+  const int tid = threadIdx.x;
   const PointBlock pb = t.pblocks[blockIdx.x];
   const DevGrid& g = t.grids[pb.grid];
-  const int64_t p = pb.p0 + threadIdx.x;
-  if (p >= g.K) return;
-  Pt pt;
-  ps_point(g, t.edges, p, pt);
-  double* base = ops + g.op_off;
-  const int64_t ld = g.ld;
-  double rC = 1.0, dC[3] = {0, 0, 0};
-  if (g.C >= 0) {
-    for (int c = 0; c < 3; ++c) dC[c] = pt.P[c] - g.RC[c];
-    rC = sqrt(dC[0] * dC[0] + dC[1] * dC[1] + dC[2] * dC[2]);
+  const bool third = g.C >= 0;
+  const int np = pb.pr1 - pb.pr0, nu = pb.u1 - pb.u0, nn = nu * g.q_phi;  // node pairs; phi rows, nodes of the half
+  const int nbA = g.shb_A1 - g.shb_A0, nbB = g.shb_B1 - g.shb_B0, na0 = g.sha_1 - g.sha_0, na1 = g.sha_3 - g.sha_2;
+  const bool basis = g.row_F >= 0 || g.row_L >= 0, aux = g.row_G >= 0 || g.row_U >= 0;
+  const int n_pair = nbA + nbB + (third ? 0 : na0 + na1);  // shells with a value per node pair
+  double* tp = reinterpret_cast<double*>(raw + sizeof(EvalNodes));  // [2 shell + kind][pair]
+  double* tr = tp + 2 * n_pair * np;                                // [phi node][pair]: distance from C
+  double* tc = tr + (third ? nn * np : 0);                          // [shell of C][phi node][pair]
+  // the column: its element rows, its points, its phi rows
+  const int nreg = g.n_mu * g.n_nu, ns = g.n_sp, q3 = g.q_mu * g.q_nu * g.q_phi;
+  const bool reg = pb.col < nreg;
+  int i, j, si = 0, sj = 0, nu_rows;
+  int64_t cell0, cell_s1, cell_s2 = 0;  // first point; point strides of phi cells and of their sub-rows
+  bool touch = false;
+  if (reg) {
+    i = pb.col / g.n_nu;
+    j = pb.col - i * g.n_nu;
+    nu_rows = g.n_phi;
+    cell0 = (int64_t)pb.col * g.n_phi * q3;
+    cell_s1 = q3;
+    touch = g.n_touch > 0 && i >= g.t_mu0 && i <= g.t_mu1 && j >= g.t_nu0 && j <= g.t_nu1;
+  } else {
+    const int c = pb.col - nreg, sub = c % (ns * ns), tij = c / (ns * ns);
+    i = g.t_mu0 + tij / g.nt_nu;
+    j = g.t_nu0 + tij % g.nt_nu;
+    si = sub / ns;
+    sj = sub - si * ns;
+    nu_rows = g.nt_phi * ns;
+    cell0 = g.K_reg + ((int64_t)tij * g.nt_phi * ns * ns * ns + (si * ns + sj) * ns) * q3;
+    cell_s1 = (int64_t)ns * ns * ns * q3;
+    cell_s2 = q3;
   }
-  // The operand rows of a contraction carry the weight: chi and lap chi sqrt(w), aux chi w, so that
-  // a product of two basis rows is w chi_i chi_j and V^P, which varies slowly, stays as it is.
-  const double wg = g.row_W >= 0 ? pt.w : 1.0, wf = sqrt(wg);
-  // the nuclear weights that V_ne elements of this grid are summed with: on a pair grid those of the
-  // A x B elements and the square roots of those of the A x A and B x B elements (an atom's own
-  // nucleus only on its one-centre grid), on a refined grid the third nucleus's
-  if (g.row_W >= 0 && g.n_W == 3) {
-    const double wa = g.zA / pt.rA, wb = g.zB / pt.rB;
-    base[(int64_t)(g.row_W + 0) * ld + p] = wa + wb;
-    base[(int64_t)(g.row_W + 1) * ld + p] = sqrt(g.own_A ? wa + wb : wb);
-    base[(int64_t)(g.row_W + 2) * ld + p] = sqrt(g.own_B ? wa + wb : wa);
-  } else if (g.row_W >= 0 && g.n_W == 1) {
-    base[(int64_t)g.row_W * ld + p] = g.zC / rC;
-  }
-  double Y[(kMaxL + 1) * (kMaxL + 1)];
-  // basis functions on A and B
-  if (g.row_F >= 0 || g.row_L >= 0) {
-    for (int c = 0; c < 2; ++c) {
-      const int s0 = c == 0 ? g.shb_A0 : g.shb_B0, s1 = c == 0 ? g.shb_A1 : g.shb_B1;
-      if (s1 <= s0) continue;
-      const double r = c == 0 ? pt.rA : pt.rB, ir = 1.0 / r;
-      const double* d = c == 0 ? pt.dA : pt.dB;
-      real_ylm(shells_lmax(t.bshell, s0, s1), d[0] * ir, d[1] * ir, d[2] * ir, Y);
-      const int roff = c == 0 ? 0 : g.nFA;
-      eval_shells(t.bshell, s0, s1, r, ir, Y, base, ld, p, g.row_F >= 0 ? g.row_F + roff : -1, 0,
-                  g.row_L >= 0 ? g.row_L + roff : -1, 1, wf);
+  // nodes: mu, nu, and the phi rows of the half and their mirrors
+  const double* emu = t.edges + g.edge_off;
+  const double* enu = emu + g.n_mu + 1;
+  const double* eph = enu + g.n_nu + 1;
+  for (int e = tid; e < g.q_mu + g.q_nu + 2 * nn; e += kEvalThreads) {
+    const int dim = e < g.q_mu ? 0 : (e < g.q_mu + g.q_nu ? 1 : 2);
+    int q, Q, s = 0;
+    double m0, m1;
+    if (dim == 0) {
+      q = e; Q = g.q_mu; s = si; m0 = emu[i]; m1 = emu[i + 1];
+    } else if (dim == 1) {
+      q = e - g.q_mu; Q = g.q_nu; s = sj; m0 = enu[j]; m1 = enu[j + 1];
+    } else {
+      const int f = e - g.q_mu - g.q_nu, ul = f / g.q_phi;
+      const int uh = pb.u0 + (ul < nu ? ul : ul - nu), u = ul < nu ? uh : nu_rows - 1 - uh;
+      q = f - ul * g.q_phi;
+      Q = g.q_phi;
+      int k = u;
+      if (!reg) {
+        s = u % ns;
+        k = u / ns;
+        if (!g.t_phi_all && k > 0) k = g.n_phi - 1;
+      }
+      m0 = eph[k]; m1 = eph[k + 1];
+    }
+    if (!reg) {
+      const double M0 = m0, M1 = m1;
+      m0 = M0 + (M1 - M0) * s / ns;
+      m1 = M0 + (M1 - M0) * (s + 1) / ns;
+    }
+    const double h = 0.5 * (m1 - m0), v = 0.5 * (m0 + m1) + h * c_glx[Q][q], w = h * c_glw[Q][q];
+    if (dim == 0) {
+      const double s2 = sinh(0.5 * v);
+      nd.mu[q][0] = sinh(v); nd.mu[q][1] = cosh(v); nd.mu[q][2] = s2 * s2; nd.mu[q][3] = w;
+    } else {
+      double sn, cs;
+      sincos(v, &sn, &cs);
+      if (dim == 1) {
+        double s2, c2;
+        sincos(0.5 * v, &s2, &c2);
+        nd.nu[q][0] = sn; nd.nu[q][1] = cs; nd.nu[q][2] = s2 * s2; nd.nu[q][3] = c2 * c2; nd.nu[q][4] = w;
+      } else {
+        double* d = nd.ph[e - g.q_mu - g.q_nu];
+        d[0] = sn; d[1] = cs; d[2] = w;
+      }
     }
   }
-  // aux functions and their potentials
-  if (g.row_G >= 0 || g.row_U >= 0) {
-    int roff = 0;
-    for (int c = 0; c < 2; ++c) {
-      const int s0 = c == 0 ? g.sha_0 : g.sha_2, s1 = c == 0 ? g.sha_1 : g.sha_3;
-      const int atom = c == 0 ? g.aux_c0 : g.aux_c1;
-      if (atom < 0 || s1 <= s0) continue;
-      const double* d;
-      double r;
-      if (atom == g.A) { d = pt.dA; r = pt.rA; }
-      else if (atom == g.B) { d = pt.dB; r = pt.rB; }
-      else { d = dC; r = rC; }
-      const double ir = 1.0 / r;
-      real_ylm(shells_lmax(t.ashell, s0, s1), d[0] * ir, d[1] * ir, d[2] * ir, Y);
-      eval_shells(t.ashell, s0, s1, r, ir, Y, base, ld, p, g.row_G >= 0 ? g.row_G + roff : -1, 0,
-                  g.row_U >= 0 ? g.row_U + roff : -1, 2, wg);
-      int nf = 0;
-      for (int s = s0; s < s1; ++s) nf += 2 * t.ashell[s].l + 1;
-      roff += nf;
+  if (tid == 0) {
+    nd.meta[0] = max(basis ? shells_lmax(t.bshell, g.shb_A0, g.shb_A1) : 0, aux && !third ? shells_lmax(t.ashell, g.sha_0, g.sha_1) : 0);
+    nd.meta[1] = max(basis ? shells_lmax(t.bshell, g.shb_B0, g.shb_B1) : 0, aux && !third ? shells_lmax(t.ashell, g.sha_2, g.sha_3) : 0);
+    nd.meta[2] = third && aux ? shells_lmax(t.ashell, g.sha_0, g.sha_1) : 0;
+    int nf = 0;
+    for (int s = g.sha_0; s < g.sha_1; ++s) nf += 2 * t.ashell[s].l + 1;
+    nd.meta[3] = nf;
+  }
+  __syncthreads();
+  const double a = g.a;
+  if (third)
+    for (int e = tid; e < nn * np; e += kEvalThreads) {
+      const int f = e / np, pr = pb.pr0 + e - f * np, qi = pr / g.q_nu, qj = pr - qi * g.q_nu;
+      const double ss = a * nd.mu[qi][0] * nd.nu[qj][0];
+      const double x = ss * nd.ph[f][1] - g.xc, y = ss * nd.ph[f][0], z = a * nd.mu[qi][1] * nd.nu[qj][1] - g.zc;
+      tr[e] = sqrt(x * x + y * y + z * z);
+    }
+  // radial factors per node pair
+  for (int e = tid; e < n_pair * np; e += kEvalThreads) {
+    const int s = e / np, pq = e - s * np, pr = pb.pr0 + pq, qi = pr / g.q_nu, qj = pr - qi * g.q_nu;
+    const bool isb = s < nbA + nbB, onA = isb ? s < nbA : s < nbA + nbB + na0;
+    if (isb ? !basis : !aux) continue;
+    const DevShell& q = isb ? t.bshell[s < nbA ? g.shb_A0 + s : g.shb_B0 + s - nbA]
+                            : t.ashell[onA ? g.sha_0 + s - nbA - nbB : g.sha_2 + s - nbA - nbB - na0];
+    const double r = 2.0 * a * (nd.mu[qi][2] + nd.nu[qj][onA ? 2 : 3]), ex = exp(-q.zeta * r), ir = 1.0 / r;
+    const bool ka = isb ? g.row_F >= 0 : g.row_G >= 0, kb = isb ? g.row_L >= 0 : g.row_U >= 0;
+    if (ka) tp[2 * s * np + pq] = radial_value(q, 0, r, ir, ex);
+    if (kb) tp[(2 * s + 1) * np + pq] = radial_value(q, isb ? 1 : 2, r, ir, ex);
+  }
+  if (third && aux) {
+    __syncthreads();
+    const int kind = g.row_U >= 0 ? 2 : 0;  // (a refined grid has one aux kind)
+    for (int e = tid; e < na0 * nn * np; e += kEvalThreads) {
+      const int s = e / (nn * np);
+      const DevShell& q = t.ashell[g.sha_0 + s];
+      const double r = tr[e - s * nn * np];
+      tc[e] = radial_value(q, kind, r, 0.0, exp(-q.zeta * r));
+    }
+  }
+  __syncthreads();
+  // the points: phi rows u0 .. u1 - 1 and their mirrors
+  double* base = ops + g.op_off;
+  const int64_t ld = g.ld;
+  const int per = np * g.q_phi;
+  double Y[(kMaxL + 1) * (kMaxL + 1)];
+  for (int e = tid; e < 2 * nu * per; e += kEvalThreads) {
+    const int c = e / per, r = e - c * per, pq = r / g.q_phi, qk = r - pq * g.q_phi;
+    const bool mirror = c >= nu;
+    const int uh = pb.u0 + (mirror ? c - nu : c), u = mirror ? nu_rows - 1 - uh : uh;
+    if (mirror && u == uh) continue;  // the middle row is its own mirror
+    const int pr = pb.pr0 + pq, qi = pr / g.q_nu, qj = pr - qi * g.q_nu;
+    const int f = (uh - pb.u0) * g.q_phi + (mirror ? g.q_phi - 1 - qk : qk);  // node of the half
+    const int64_t p = cell0 + (reg ? u * cell_s1 : (u / ns) * cell_s1 + (u % ns) * cell_s2) + (int64_t)pr * g.q_phi + qk;
+    const bool dead = touch && (g.t_phi_all || u == 0 || u == g.n_phi - 1);
+    const double sh = nd.mu[qi][0], ch = nd.mu[qi][1], s2m = nd.mu[qi][2];
+    const double sn = nd.nu[qj][0], cs = nd.nu[qj][1], s2n = nd.nu[qj][2], c2n = nd.nu[qj][3];
+    const double* ph = nd.ph[c * g.q_phi + qk];
+    const double rA = 2.0 * a * (s2m + s2n), rB = 2.0 * a * (s2m + c2n), rC = third ? tr[f * np + pq] : 1.0;
+    // The operand rows of a contraction carry the weight: chi and lap chi sqrt(w), aux chi w, so that
+    // a product of two basis rows is w chi_i chi_j and V^P, which varies slowly, stays as it is.
+    double wg = 1.0, wf = 1.0;
+    if (g.row_W >= 0) {
+      wg = dead ? 0.0 : nd.mu[qi][3] * nd.nu[qj][4] * ph[2] * (a * a * a) * sh * sn * (sh * sh + sn * sn);
+      wf = sqrt(wg);
+      // the nuclear weights that V_ne elements of this grid are summed with: on a pair grid those of the
+      // A x B elements and the square roots of those of the A x A and B x B elements (an atom's own
+      // nucleus only on its one-centre grid), on a refined grid the third nucleus's
+      if (g.n_W == 3) {
+        const double wa = g.zA / rA, wb = g.zB / rB;
+        base[(int64_t)(g.row_W + 0) * ld + p] = wa + wb;
+        base[(int64_t)(g.row_W + 1) * ld + p] = sqrt(g.own_A ? wa + wb : wb);
+        base[(int64_t)(g.row_W + 2) * ld + p] = sqrt(g.own_B ? wa + wb : wa);
+      } else if (g.n_W == 1) {
+        base[(int64_t)g.row_W * ld + p] = g.zC / rC;
+      }
+    }
+    const double x = a * sh * sn * ph[1], y = a * sh * sn * ph[0];
+#pragma unroll 1
+    for (int ctr = 0; ctr < 3; ++ctr) {  // A, B, C
+      const int b0 = ctr == 0 ? g.shb_A0 : g.shb_B0, b1 = ctr == 0 ? g.shb_A1 : g.shb_B1;
+      const int a0 = ctr == 1 ? g.sha_2 : g.sha_0, a1 = ctr == 1 ? g.sha_3 : g.sha_1;
+      const bool hb = basis && ctr < 2 && b1 > b0, ha = aux && (ctr == 2) == third && a1 > a0;
+      if (!hb && !ha) continue;
+      const double ir = 1.0 / (ctr == 0 ? rA : (ctr == 1 ? rB : rC));
+      const double dx = (ctr == 2 ? x - g.xc : x) * ir, dy = y * ir;
+      const double dz = (ctr == 0 ? 2.0 * a * (s2m * cs - s2n) : (ctr == 1 ? 2.0 * a * (s2m * cs + c2n) : a * ch * cs - g.zc)) * ir;
+      real_ylm(nd.meta[ctr], g.R[0] * dx + g.R[1] * dy + g.R[2] * dz, g.R[3] * dx + g.R[4] * dy + g.R[5] * dz,
+               g.R[6] * dx + g.R[7] * dy + g.R[8] * dz, Y);
+      if (hb) {
+        const int roff = ctr == 0 ? 0 : g.nFA, e0 = ctr == 0 ? 0 : nbA;
+        for (int s = b0; s < b1; ++s) {
+          const DevShell& q = t.bshell[s];
+          const double* tv = tp + 2 * (e0 + s - b0) * np + pq;
+          if (g.row_F >= 0) store_shell(q, wf * tv[0], Y, base, ld, p, g.row_F + roff);
+          if (g.row_L >= 0) store_shell(q, wf * tv[np], Y, base, ld, p, g.row_L + roff);
+        }
+      }
+      if (ha) {
+        const int roff = ctr == 1 ? nd.meta[3] : 0, e0 = nbA + nbB + (ctr == 1 ? na0 : 0);
+        for (int s = a0; s < a1; ++s) {
+          const DevShell& q = t.ashell[s];
+          if (ctr == 2) {
+            const double v = tc[((s - a0) * nn + f) * np + pq];
+            store_shell(q, g.row_U >= 0 ? v : wg * v, Y, base, ld, p, g.row_U >= 0 ? g.row_U : g.row_G);
+          } else {
+            const double* tv = tp + 2 * (e0 + s - a0) * np + pq;
+            if (g.row_G >= 0) store_shell(q, wg * tv[0], Y, base, ld, p, g.row_G + roff);
+            if (g.row_U >= 0) store_shell(q, tv[np], Y, base, ld, p, g.row_U + roff);
+          }
+        }
+      }
     }
   }
 }
 
 cudaError_t launch_eval_fp64(const LaunchTables& t, double* ops, int /*kinds*/, cudaStream_t s) {
   if (t.n_pblocks == 0) return cudaSuccess;
-  eval_fp64_kernel<<<t.n_pblocks, 128, 0, s>>>(t, ops);
+  eval_fp64_kernel<<<t.n_pblocks, kEvalThreads, kEvalFp64Smem, s>>>(t, ops);
   return cudaGetLastError();
 }
 
@@ -552,7 +695,9 @@ __global__ void __launch_bounds__(fx::kThreads, 2) contract_fp64_kernel(LaunchTa
 }
 
 cudaError_t prepare_kernels_fp64() {
-  const cudaError_t e = cudaFuncSetAttribute(contract_fp64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fx::kSmemBytes);
+  cudaError_t e = cudaFuncSetAttribute(eval_fp64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kEvalFp64Smem);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(contract_fp64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fx::kSmemBytes);
   // room for two CTAs per SM (of 228 KB), the rest L1
   return e != cudaSuccess ? e : cudaFuncSetAttribute(contract_fp64_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 80);
 }

@@ -148,47 +148,24 @@ using dfa::df;
 
 __device__ __forceinline__ df ld2(float2 v) { return df{v.x, v.y}; }
 
-// Rows of the shells [s0, s1) of one centre for one or two row kinds (chi with lap chi, or
-// chi with V^P: x, e^-x and 1/x are shared).  xi[k] is the (hi, lo) scale that turns rho into
-// x for shell s0 + k.  Values go to the hi and lo planes.
-__device__ __forceinline__ void eval_shells_df(const DevShell* __restrict__ sh, const float2* __restrict__ xi,
-                                               int s0, int s1, df rho, const df* Y, float* __restrict__ oh,
-                                               float* __restrict__ ol, int64_t ld, int64_t p, int row_a,
-                                               int kind_a, int row_b, int kind_b, const float2* etab) {
-#pragma unroll 1  // one shell at a time: unrolled copies only grow the code
-  for (int s = s0; s < s1; ++s) {
-    const DevShell q = sh[s];
-    const df x = dfa::mul(ld2(xi[s - s0]), rho);
-    const df ex = dfa::exp_neg(x, c_expc, etab);
-    const df ix = (kind_a != 0 || (row_b >= 0 && kind_b != 0)) ? dfa::rcp(x) : dfa::mk(0.0f);
-    const int base = q.l * q.l + q.l;
-    if (row_a >= 0) {
-      const df ra = dfa::radial(kind_a, q.n, q.l, x, ex, ix, c_factd, c_rcpf);
-#pragma unroll 1
-      for (int m = -q.l; m <= q.l; ++m) {
-        const df v = dfa::mul(ra, Y[base + m]);
-        const int64_t o = (int64_t)(row_a + q.fn0 + q.l + m) * ld + p;
-        oh[o] = v.h;
-        ol[o] = v.l;
-      }
-    }
-    if (row_b >= 0) {
-      const df rb = dfa::radial(kind_b, q.n, q.l, x, ex, ix, c_factd, c_rcpf);
-#pragma unroll 1
-      for (int m = -q.l; m <= q.l; ++m) {
-        const df v = dfa::mul(rb, Y[base + m]);
-        const int64_t o = (int64_t)(row_b + q.fn0 + q.l + m) * ld + p;
-        oh[o] = v.h;
-        ol[o] = v.l;
-      }
-    }
-  }
-}
-
+// Highest l and number of functions of the shells [s0, s1).
 __device__ __forceinline__ int shells_lmax_f(const DevShell* sh, int s0, int s1) {
   int l = 0;
   for (int s = s0; s < s1; ++s) l = max(l, sh[s].l);
   return l;
+}
+
+// One row kind of a shell at one point: the radial value times the harmonics, to the hi and lo planes.
+__device__ __forceinline__ void store_shell(const DevShell& q, df r, const df* Y, float* __restrict__ oh,
+                                            float* __restrict__ ol, int64_t ld, int64_t p, int row) {
+  const int base = q.l * q.l + q.l;
+  int64_t o = (int64_t)(row + q.fn0) * ld + p;
+#pragma unroll 1
+  for (int m = -q.l; m <= q.l; ++m, o += ld) {
+    const df v = dfa::mul(r, Y[base + m]);
+    oh[o] = v.h;
+    ol[o] = v.l;
+  }
 }
 
 // u = R v / len (R as a double-float matrix), the unit vector of the offset v of length len.
@@ -206,125 +183,189 @@ __device__ __forceinline__ df split_d(double v) {
   return df{hi, (float)(v - (double)hi)};
 }
 
-// One thread per point.  The weight w = a^3 [G G G sinh mu sin nu (sinh^2 mu + sin^2 nu)]
+// One CTA per PointBlock.  The weight w = a^3 [G G G sinh mu sin nu (sinh^2 mu + sin^2 nu)]
 // and r_A = 2a rho_A, r_B = 2a rho_B are written without their per-grid constants (a^3,
 // a^2/2), which are applied in FP64 after the contraction; functions likewise.  The offsets
 // from A and B (in units of a) are (sinh mu sin nu cos phi, sinh mu sin nu sin phi,
 // 2(sinh^2(mu/2) cos nu -+ {sin^2, cos^2}(nu/2))), of length 2 rho; the offset from a third
 // centre is formed in FP64 (it cancels near that centre).
-__global__ void __launch_bounds__(128) eval_mixed_kernel(LaunchTables t, const NodeEntry* __restrict__ tab,
-                                                         const float2* __restrict__ xi_tab,
-                                                         float* __restrict__ ops, float* __restrict__ ops_lo) {
+//
+// The radial factors (e^-x, powers, incomplete gamma series) are most of the arithmetic, and those of
+// A and B depend on (mu, nu) only: they are computed once per node pair and kept in shared memory for
+// all phi nodes (32 points share one on an 8-cell grid with Q = 4); those of a third centre are
+// computed for half of the phi nodes.  A point is then its harmonics and one product per function.
+__global__ void __launch_bounds__(kEvalThreads) eval_mixed_kernel(LaunchTables t, const NodeEntry* __restrict__ tab,
+                                                                  const float2* __restrict__ xi_tab,
+                                                                  float* __restrict__ ops, float* __restrict__ ops_lo) {
+  extern __shared__ __align__(16) uint8_t raw[];
   __shared__ float2 etab[64];
-  if (threadIdx.x < 64) etab[threadIdx.x] = c_exp_tab[threadIdx.x];
-  __syncthreads();
+  __shared__ int meta[5];  // lmax of A, B, C; functions of the first aux centre
+  const int tid = threadIdx.x;
+  if (tid < 64) etab[tid] = c_exp_tab[tid];
   const PointBlock pb = t.pblocks[blockIdx.x];
   const DevGrid& g = t.grids[pb.grid];
-  const int p = (int)pb.p0 + (int)threadIdx.x;  // K < 2^31 - 256 (the planner checks)
-  if (p >= g.K) return;
+  const bool third = g.C >= 0;
+  const int np = pb.pr1 - pb.pr0, nn = (pb.u1 - pb.u0) * g.q_phi;  // node pairs, phi nodes of the half
+  const int nbA = g.shb_A1 - g.shb_A0, nbB = g.shb_B1 - g.shb_B0, na0 = g.sha_1 - g.sha_0, na1 = g.sha_3 - g.sha_2;
+  const bool basis = g.row_F >= 0 || g.row_L >= 0, aux = g.row_G >= 0 || g.row_U >= 0;
+  const int n_pair = nbA + nbB + (third ? 0 : na0 + na1);  // shells with a value per node pair
+  float2* tp = reinterpret_cast<float2*>(raw);             // [2 shell + kind][pair]
+  float2* tr = tp + 2 * n_pair * np;                       // [phi node][pair]: distance from C
+  float2* tc = tr + (third ? nn * np : 0);                 // [shell of C][phi node][pair]
+  // the column's node rows
+  const int nreg = g.n_mu * g.n_nu, ns = g.n_sp;
+  const bool reg = pb.col < nreg;
+  int ri, rj, nu_rows;
+  int64_t cell0;       // first point of the column's phi row 0
+  int64_t cell_s1, cell_s2;  // point strides of phi cells and of their sub-rows
   const int q3 = g.q_mu * g.q_nu * g.q_phi;
-  int ri, rj, rk;
-  bool dead = false;
-  int pr;
-  if (p < g.K_reg) {
-    const int cell = p / q3;
-    pr = p - cell * q3;
-    const int cnp = cell / g.n_phi;
-    rk = cell - cnp * g.n_phi;
-    ri = cnp / g.n_nu;
-    rj = cnp - ri * g.n_nu;
-    if (g.n_touch > 0 && ri >= g.t_mu0 && ri <= g.t_mu1 && rj >= g.t_nu0 && rj <= g.t_nu1 &&
-        (g.t_phi_all || rk == 0 || rk == g.n_phi - 1))
-      dead = true;
+  bool touch = false;
+  if (reg) {
+    ri = pb.col / g.n_nu;
+    rj = pb.col - ri * g.n_nu;
+    nu_rows = g.n_phi;
+    cell0 = (int64_t)pb.col * g.n_phi * q3;
+    cell_s1 = q3;
+    cell_s2 = 0;
+    touch = g.n_touch > 0 && ri >= g.t_mu0 && ri <= g.t_mu1 && rj >= g.t_nu0 && rj <= g.t_nu1;
   } else {
-    const int pe = p - (int)g.K_reg;
-    const int s = pe / q3;
-    pr = pe - s * q3;
-    const int ns = g.n_sp, ns3 = ns * ns * ns;
-    const int tc = s / ns3, sub = s - tc * ns3;
-    const int ntp = g.nt_phi, nnu = g.nt_nu;
-    const int ti = tc / (nnu * ntp), tj = (tc / ntp) % nnu, tk = tc % ntp;
-    const int si = sub / (ns * ns), sj = (sub / ns) % ns, sk = sub % ns;
+    const int c = pb.col - nreg, sub = c % (ns * ns), tij = c / (ns * ns);
+    const int ti = tij / g.nt_nu, tj = tij - ti * g.nt_nu, si = sub / ns, sj = sub - si * ns;
     ri = g.n_mu + ti * ns + si;
     rj = g.n_nu + tj * ns + sj;
-    rk = g.n_phi + tk * ns + sk;
+    nu_rows = g.nt_phi * ns;
+    cell0 = g.K_reg + ((int64_t)tij * g.nt_phi * ns * ns * ns + (si * ns + sj) * ns) * q3;
+    cell_s1 = (int64_t)ns * ns * ns * q3;
+    cell_s2 = q3;
   }
-  const int qnp = pr / g.q_phi;
-  const int qk = pr - qnp * g.q_phi;
-  const int qi = qnp / g.q_nu;
-  const int qj = qnp - qi * g.q_nu;
-  const int nmu = (g.n_mu + g.nt_mu * g.n_sp) * g.q_mu;
-  const int nnu = (g.n_nu + g.nt_nu * g.n_sp) * g.q_nu;
-  const NodeEntry& Mu = tab[g.nt_off + ri * g.q_mu + qi];
-  const NodeEntry& Nu = tab[g.nt_off + nmu + rj * g.q_nu + qj];
-  const NodeEntry& Ph = tab[g.nt_off + nmu + nnu + rk * g.q_phi + qk];
-  const df sh = ld2(Mu.fs), s2m = ld2(Mu.fh2);
-  const df sn = ld2(Nu.fs), cs = ld2(Nu.fc), s2n = ld2(Nu.fh2), c2n = ld2(Nu.fg2);
-  const df sp = ld2(Ph.fs), cp = ld2(Ph.fc);
-  const df shsn = dfa::mul(sh, sn);
-  df w = dfa::mk(0.0f);
-  if (!dead) {
-    const df gw = dfa::mul(dfa::mul(ld2(Mu.fw), ld2(Nu.fw)), ld2(Ph.fw));
-    w = dfa::mul(dfa::mul(gw, shsn), dfa::add_same(dfa::mul(sh, sh), dfa::mul(sn, sn)));
+  const NodeEntry* Mu = tab + g.nt_off + ri * g.q_mu;
+  const NodeEntry* Nu = tab + g.nt_off + (g.n_mu + g.nt_mu * ns) * g.q_mu + rj * g.q_nu;
+  const NodeEntry* Ph = tab + g.nt_off + (g.n_mu + g.nt_mu * ns) * g.q_mu + (g.n_nu + g.nt_nu * ns) * g.q_nu +
+                        (reg ? 0 : g.n_phi * g.q_phi);  // rows of the column's phi rows, in order
+  if (tid == 0) {
+    const bool auxA = !third;
+    meta[0] = max(basis ? shells_lmax_f(t.bshell, g.shb_A0, g.shb_A1) : 0, aux && auxA ? shells_lmax_f(t.ashell, g.sha_0, g.sha_1) : 0);
+    meta[1] = max(basis ? shells_lmax_f(t.bshell, g.shb_B0, g.shb_B1) : 0, aux && auxA ? shells_lmax_f(t.ashell, g.sha_2, g.sha_3) : 0);
+    meta[2] = third && aux ? shells_lmax_f(t.ashell, g.sha_0, g.sha_1) : 0;
+    int nf = 0;
+    for (int s = g.sha_0; s < g.sha_1; ++s) nf += 2 * t.ashell[s].l + 1;
+    meta[3] = nf;
   }
-  const df rhoA = dfa::add_same(s2m, s2n), rhoB = dfa::add_same(s2m, c2n);
-  const df xs = dfa::mul(shsn, cp), ys = dfa::mul(shsn, sp);
-  const df s2mc = dfa::mul(s2m, cs);
-  df uA[3], uB[3], uC[3] = {dfa::mk(0.f), dfa::mk(0.f), dfa::mk(1.f)};
-  rotate_unit_df(g, xs, ys, dfa::scale2(dfa::sub(s2mc, s2n), 2.0f), dfa::rcp(dfa::scale2(rhoA, 2.0f)), uA);
-  rotate_unit_df(g, xs, ys, dfa::scale2(dfa::add(s2mc, c2n), 2.0f), dfa::rcp(dfa::scale2(rhoB, 2.0f)), uB);
-  df rC = dfa::mk(1.0f);
-  if (g.C >= 0) {
-    // offset from the third centre in the pair frame, FP64: it cancels near that centre
-    const double X = g.a * Mu.s * Nu.s * Ph.c - g.xc;
-    const double Yv = g.a * Mu.s * Nu.s * Ph.s;
-    const double Z = g.a * Mu.c * Nu.c - g.zc;
-    const df dX = split_d(X), dY = split_d(Yv), dZ = split_d(Z);
-    rC = dfa::sqrt(dfa::add_same(dfa::add_same(dfa::mul(dX, dX), dfa::mul(dY, dY)), dfa::mul(dZ, dZ)));
-    rotate_unit_df(g, dX, dY, dZ, dfa::rcp(rC), uC);
+  // third centre: distances at the phi nodes of the half, FP64 offsets
+  if (third) {
+    for (int e = tid; e < nn * np; e += kEvalThreads) {
+      const int f = e / np, pr = pb.pr0 + e - f * np, qi = pr / g.q_nu, qj = pr - qi * g.q_nu;
+      const NodeEntry &M = Mu[qi], &N = Nu[qj], &F = Ph[pb.u0 * g.q_phi + f];
+      const df dX = split_d(g.a * M.s * N.s * F.c - g.xc), dY = split_d(g.a * M.s * N.s * F.s), dZ = split_d(g.a * M.c * N.c - g.zc);
+      const df r = dfa::sqrt(dfa::add_same(dfa::add_same(dfa::mul(dX, dX), dfa::mul(dY, dY)), dfa::mul(dZ, dZ)));
+      tr[e] = make_float2(r.h, r.l);
+    }
   }
+  __syncthreads();
+  const float2* xi = xi_tab + g.xi_off;  // basis A, basis B, aux c0, aux c1 shells
+  for (int e = tid; e < n_pair * np; e += kEvalThreads) {
+    const int s = e / np, pq = e - s * np, pr = pb.pr0 + pq, qi = pr / g.q_nu, qj = pr - qi * g.q_nu;
+    const bool isb = s < nbA + nbB, onA = isb ? s < nbA : s < nbA + nbB + na0;
+    if (isb ? !basis : !aux) continue;
+    const DevShell& q = isb ? t.bshell[s < nbA ? g.shb_A0 + s : g.shb_B0 + s - nbA]
+                            : t.ashell[onA ? g.sha_0 + s - nbA - nbB : g.sha_2 + s - nbA - nbB - na0];
+    const df rho = dfa::add_same(ld2(Mu[qi].fh2), onA ? ld2(Nu[qj].fh2) : ld2(Nu[qj].fg2));
+    const df x = dfa::mul(ld2(xi[s]), rho), ex = dfa::exp_neg(x, c_expc, etab), ix = dfa::rcp(x);
+    const bool ka = isb ? g.row_F >= 0 : g.row_G >= 0, kb = isb ? g.row_L >= 0 : g.row_U >= 0;
+    if (ka) {
+      const df r = dfa::radial(0, q.n, q.l, x, ex, ix, c_factd, c_rcpf);
+      tp[2 * s * np + pq] = make_float2(r.h, r.l);
+    }
+    if (kb) {
+      const df r = dfa::radial(isb ? 1 : 2, q.n, q.l, x, ex, ix, c_factd, c_rcpf);
+      tp[(2 * s + 1) * np + pq] = make_float2(r.h, r.l);
+    }
+  }
+  if (third && aux) {
+    const int kind = g.row_U >= 0 ? 2 : 0;  // (a refined grid has one aux kind)
+    for (int e = tid; e < na0 * nn * np; e += kEvalThreads) {
+      const int s = e / (nn * np);
+      const DevShell& q = t.ashell[g.sha_0 + s];
+      const df x = dfa::mul(ld2(xi[nbA + nbB + s]), ld2(tr[e - s * nn * np]));
+      const df r = dfa::radial(kind, q.n, q.l, x, dfa::exp_neg(x, c_expc, etab), dfa::rcp(x), c_factd, c_rcpf);
+      tc[e] = make_float2(r.h, r.l);
+    }
+  }
+  __syncthreads();
+  // the points: phi rows u0 .. u1 - 1 and their mirrors
   float* bh = ops + g.op_off;
   float* bl = ops_lo + g.op_off;
   const int64_t ld = g.ld;
-  if (g.row_W >= 0) {
-    const df wv[4] = {w, dfa::div(w, rhoA), dfa::div(w, rhoB), g.C >= 0 ? dfa::div(w, rC) : dfa::mk(0.0f)};
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      bh[(int64_t)(g.row_W + k) * ld + p] = wv[k].h;
-      bl[(int64_t)(g.row_W + k) * ld + p] = wv[k].l;
-    }
-  }
-  const float2* xi = xi_tab + g.xi_off;  // basis A, basis B, aux c0, aux c1 shells
-  const int nbA = g.shb_A1 - g.shb_A0, nbB = g.shb_B1 - g.shb_B0, na0 = g.sha_1 - g.sha_0;
+  const int per = np * g.q_phi, nu = pb.u1 - pb.u0;
   df Y[(kMaxL + 1) * (kMaxL + 1)];
-  if (g.row_F >= 0 || g.row_L >= 0) {
-    for (int c = 0; c < 2; ++c) {
-      const int s0 = c == 0 ? g.shb_A0 : g.shb_B0, s1 = c == 0 ? g.shb_A1 : g.shb_B1;
-      if (s1 <= s0) continue;
-      const df* u = c == 0 ? uA : uB;
-      dfa::real_ylm(shells_lmax_f(t.bshell, s0, s1), u[0], u[1], u[2], Y, c_rcpf);
-      const int roff = c == 0 ? 0 : g.nFA;
-      eval_shells_df(t.bshell, xi + (c == 0 ? 0 : nbA), s0, s1, c == 0 ? rhoA : rhoB, Y, bh, bl, ld, p,
-                     g.row_F >= 0 ? g.row_F + roff : -1, 0, g.row_L >= 0 ? g.row_L + roff : -1, 1, etab);
+  for (int e = tid; e < 2 * nu * per; e += kEvalThreads) {
+    const int c = e / per, r = e - c * per, pq = r / g.q_phi, qk = r - pq * g.q_phi;
+    const bool mirror = c >= nu;
+    const int uh = pb.u0 + (mirror ? c - nu : c), u = mirror ? nu_rows - 1 - uh : uh;
+    if (mirror && u == uh) continue;  // the middle row is its own mirror
+    const int pr = pb.pr0 + pq, qi = pr / g.q_nu, qj = pr - qi * g.q_nu;
+    const int f = (uh - pb.u0) * g.q_phi + (mirror ? g.q_phi - 1 - qk : qk);  // node of the half
+    const int64_t p = cell0 + (reg ? u * cell_s1 : (u / ns) * cell_s1 + (u % ns) * cell_s2) + (int64_t)pr * g.q_phi + qk;
+    const bool dead = touch && (g.t_phi_all || u == 0 || u == g.n_phi - 1);
+    const NodeEntry &M = Mu[qi], &N = Nu[qj], &F = Ph[u * g.q_phi + qk];
+    const df sh = ld2(M.fs), s2m = ld2(M.fh2), sn = ld2(N.fs), s2n = ld2(N.fh2), c2n = ld2(N.fg2);
+    const df shsn = dfa::mul(sh, sn);
+    const df rhoA = dfa::add_same(s2m, s2n), rhoB = dfa::add_same(s2m, c2n);
+    df rC = dfa::mk(1.0f);
+    if (third) rC = ld2(tr[f * np + pq]);
+    if (g.row_W >= 0) {
+      df w = dfa::mk(0.0f);
+      if (!dead) {
+        const df gw = dfa::mul(dfa::mul(ld2(M.fw), ld2(N.fw)), ld2(F.fw));
+        w = dfa::mul(dfa::mul(gw, shsn), dfa::add_same(dfa::mul(sh, sh), dfa::mul(sn, sn)));
+      }
+      const df wv[4] = {w, dfa::div(w, rhoA), dfa::div(w, rhoB), third ? dfa::div(w, rC) : dfa::mk(0.0f)};
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        bh[(int64_t)(g.row_W + k) * ld + p] = wv[k].h;
+        bl[(int64_t)(g.row_W + k) * ld + p] = wv[k].l;
+      }
     }
-  }
-  if (g.row_G >= 0 || g.row_U >= 0) {
-    int roff = 0;
-    for (int c = 0; c < 2; ++c) {
-      const int s0 = c == 0 ? g.sha_0 : g.sha_2, s1 = c == 0 ? g.sha_1 : g.sha_3;
-      const int atom = c == 0 ? g.aux_c0 : g.aux_c1;
-      if (atom < 0 || s1 <= s0) continue;
-      const df* u;
-      df rho;
-      if (atom == g.A) { u = uA; rho = rhoA; }
-      else if (atom == g.B) { u = uB; rho = rhoB; }
-      else { u = uC; rho = rC; }
-      dfa::real_ylm(shells_lmax_f(t.ashell, s0, s1), u[0], u[1], u[2], Y, c_rcpf);
-      eval_shells_df(t.ashell, xi + nbA + nbB + (c == 0 ? 0 : na0), s0, s1, rho, Y, bh, bl, ld, p,
-                     g.row_G >= 0 ? g.row_G + roff : -1, 0, g.row_U >= 0 ? g.row_U + roff : -1, 2, etab);
-      int nf = 0;
-      for (int s = s0; s < s1; ++s) nf += 2 * t.ashell[s].l + 1;
-      roff += nf;
+    const df xs = dfa::mul(shsn, ld2(F.fc)), ys = dfa::mul(shsn, ld2(F.fs)), s2mc = dfa::mul(s2m, ld2(N.fc));
+#pragma unroll 1
+    for (int ctr = 0; ctr < 3; ++ctr) {  // A, B, C
+      const int b0 = ctr == 0 ? g.shb_A0 : g.shb_B0, b1 = ctr == 0 ? g.shb_A1 : g.shb_B1;
+      const int a0 = ctr == 1 ? g.sha_2 : g.sha_0, a1 = ctr == 1 ? g.sha_3 : g.sha_1;
+      const bool hb = basis && ctr < 2 && b1 > b0, ha = aux && (ctr == 2) == third && a1 > a0;
+      if (!hb && !ha) continue;
+      df u3[3];
+      if (ctr < 2) {
+        const df z = ctr == 0 ? dfa::sub(s2mc, s2n) : dfa::add(s2mc, c2n);
+        rotate_unit_df(g, xs, ys, dfa::scale2(z, 2.0f), dfa::rcp(dfa::scale2(ctr == 0 ? rhoA : rhoB, 2.0f)), u3);
+      } else {
+        rotate_unit_df(g, split_d(g.a * M.s * N.s * F.c - g.xc), split_d(g.a * M.s * N.s * F.s),
+                       split_d(g.a * M.c * N.c - g.zc), dfa::rcp(rC), u3);
+      }
+      dfa::real_ylm(meta[ctr], u3[0], u3[1], u3[2], Y, c_rcpf);
+      if (hb) {
+        const int roff = ctr == 0 ? 0 : g.nFA, e0 = ctr == 0 ? 0 : nbA;
+#pragma unroll 1
+        for (int s = b0; s < b1; ++s) {
+          const DevShell& q = t.bshell[s];
+          const float2* tv = tp + 2 * (e0 + s - b0) * np + pq;
+          if (g.row_F >= 0) store_shell(q, ld2(tv[0]), Y, bh, bl, ld, p, g.row_F + roff);
+          if (g.row_L >= 0) store_shell(q, ld2(tv[np]), Y, bh, bl, ld, p, g.row_L + roff);
+        }
+      }
+      if (ha) {
+        const int roff = ctr == 1 ? meta[3] : 0, e0 = nbA + nbB + (ctr == 1 ? na0 : 0);
+#pragma unroll 1
+        for (int s = a0; s < a1; ++s) {
+          const DevShell& q = t.ashell[s];
+          if (ctr == 2) {
+            store_shell(q, ld2(tc[((s - a0) * nn + f) * np + pq]), Y, bh, bl, ld, p, g.row_U >= 0 ? g.row_U : g.row_G);
+          } else {
+            const float2* tv = tp + 2 * (e0 + s - a0) * np + pq;
+            if (g.row_G >= 0) store_shell(q, ld2(tv[0]), Y, bh, bl, ld, p, g.row_G + roff);
+            if (g.row_U >= 0) store_shell(q, ld2(tv[np]), Y, bh, bl, ld, p, g.row_U + roff);
+          }
+        }
+      }
     }
   }
 }
@@ -1216,7 +1257,7 @@ cudaError_t launch_nodes(const DevGrid* grids, int n_grids, int max_entries, con
 cudaError_t launch_eval_mixed(const LaunchTables& t, const NodeEntry* tab, const float2* xi, float* ops,
                               float* ops_lo, cudaStream_t s) {
   if (t.n_pblocks == 0) return cudaSuccess;
-  eval_mixed_kernel<<<t.n_pblocks, 128, 0, s>>>(t, tab, xi, ops, ops_lo);
+  eval_mixed_kernel<<<t.n_pblocks, kEvalThreads, kEvalTabBytes, s>>>(t, tab, xi, ops, ops_lo);
   return cudaGetLastError();
 }
 
@@ -1225,6 +1266,8 @@ static_assert(sizeof(ws::Smem) + 1024 <= 232448, "contraction shared memory abov
 size_t ws_smem_bytes() { return sizeof(ws::Smem) + 1024; }
 
 cudaError_t prepare_kernels() {
+  const cudaError_t e = cudaFuncSetAttribute(eval_mixed_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kEvalTabBytes);
+  if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(contract_ws_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ws_smem_bytes());
 }
 
