@@ -474,6 +474,8 @@ psq_status make_plan(psq_job* j, unsigned mask, Plan& P) {
     rows += P.mixed ? 4 : g.n_W;
     g.ld = (int64_t)align_up((size_t)g.K, 128);
     g.op_off = ops;
+    g.rs = 128;
+    g.ws = 128 * (int64_t)rows;
     ops += (int64_t)rows * g.ld;
     P.n_points += g.K;
   }
@@ -778,7 +780,23 @@ psq_status make_plan(psq_job* j, unsigned mask, Plan& P) {
       const int first = (int)P.ptiles.size();
       PairTile t{};
       auto flush = [&]() {
-        if (t.ncols > 0) P.ptiles.push_back(t);
+        if (t.ncols > 0) {
+          // rows in ascending order: runs of consecutive rows are staged by one copy
+          int order[kPairTileRows], place[kPairTileRows];
+          for (int k = 0; k < t.nrows; ++k) order[k] = k;
+          std::sort(order, order + t.nrows, [&](int x, int y) { return t.rows[x] < t.rows[y]; });
+          short rows[kPairTileRows];
+          for (int k = 0; k < t.nrows; ++k) {
+            rows[k] = t.rows[order[k]];
+            place[order[k]] = k;
+          }
+          std::copy(rows, rows + t.nrows, t.rows);
+          for (int c = 0; c < t.ncols; ++c) {
+            t.dx[c] = (unsigned char)place[t.dx[c]];
+            t.dy[c] = (unsigned char)place[t.dy[c]];
+          }
+          P.ptiles.push_back(t);
+        }
         t = PairTile{};
       };
       auto slot = [&](int row) {
@@ -2038,6 +2056,8 @@ psq_status psq_job_grid_functions(psq_job* job, int g, int kind, void* d_workspa
   std::vector<double> rc;
   if (mixed) row_constants(job, G, kind, rc);
   G.ld = mixed ? (int64_t)align_up((size_t)G.K, 128) : G.K;
+  G.rs = G.ld;
+  G.ws = 128;
   if (mixed) G.nt_off = 0;
   const size_t o_grid = 0, o_pb = align_up(sizeof(DevGrid), 256);
   size_t need = o_pb + align_up(sizeof(PointBlock) * pb.size(), 256);

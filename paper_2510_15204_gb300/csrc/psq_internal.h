@@ -32,9 +32,12 @@ struct DevGrid {
   int edge_off;     // edges: mu[n_mu+1], nu[n_nu+1], phi[n_phi+1] from this offset
   int t_mu0, t_mu1, t_nu0, t_nu1, t_phi_all, n_touch;  // cells touching C (n_touch = 0: none)
   int64_t K, K_reg; // points; points of the regular cell block
-  // Operand matrices of this grid: rows of ld doubles (or floats) from op_off.
+  // Operand matrix of this grid, from op_off, in blocks of 128 points: point p of row r is element
+  // r * rs + (p / 128) * ws + p % 128.  A block holds its points of every row (rs = 128, ws = 128 x
+  // rows), so that the kernels, which take all rows of a few points, touch few DRAM and TLB pages
+  // (the diagnostics write plain rows: rs = ld, ws = 128).  ld: points rounded up to 128.
   int64_t op_off;
-  int64_t ld;
+  int64_t ld, rs, ws;
   // First row per kind, -1 when absent: F chi, L lap chi, G aux chi, U V^P, and W: mixed path w, w/r_A,
   // w/r_B, w/r_C; FP64 path the nuclear weights of V_ne (n_W rows), and F, L carry sqrt(w), G carries w.
   int row_F, row_L, row_G, row_U, row_W;

@@ -213,11 +213,11 @@ __device__ __forceinline__ int shells_lmax(const DevShell* sh, int s0, int s1) {
 }
 
 // One row kind of a shell at one point: the radial value v times the harmonics.
-__device__ __forceinline__ void store_shell(const DevShell& q, double v, const double* Y, double* __restrict__ out, int64_t ld,
+__device__ __forceinline__ void store_shell(const DevShell& q, double v, const double* Y, double* __restrict__ out, int64_t rs,
                                             int64_t p, int row) {
   const int base = q.l * q.l + q.l;
-  int64_t o = (int64_t)(row + q.fn0) * ld + p;
-  for (int m = -q.l; m <= q.l; ++m, o += ld) out[o] = v * Y[base + m];
+  int64_t o = (int64_t)(row + q.fn0) * rs + p;
+  for (int m = -q.l; m <= q.l; ++m, o += rs) out[o] = v * Y[base + m];
 }
 
 // Evaluation, FP64: one CTA per PointBlock, the operand rows of its points (ps_point's forms of the
@@ -362,7 +362,7 @@ __global__ void __launch_bounds__(kEvalThreads) eval_fp64_kernel(LaunchTables t,
   __syncthreads();
   // the points: phi rows u0 .. u1 - 1 and their mirrors
   double* base = ops + g.op_off;
-  const int64_t ld = g.ld;
+  const int64_t rs = g.rs;
   const int per = np * g.q_phi;
   double Y[(kMaxL + 1) * (kMaxL + 1)];
   for (int e = tid; e < 2 * nu * per; e += kEvalThreads) {
@@ -372,7 +372,8 @@ __global__ void __launch_bounds__(kEvalThreads) eval_fp64_kernel(LaunchTables t,
     if (mirror && u == uh) continue;  // the middle row is its own mirror
     const int pr = pb.pr0 + pq, qi = pr / g.q_nu, qj = pr - qi * g.q_nu;
     const int f = (uh - pb.u0) * g.q_phi + (mirror ? g.q_phi - 1 - qk : qk);  // node of the half
-    const int64_t p = cell0 + (reg ? u * cell_s1 : (u / ns) * cell_s1 + (u % ns) * cell_s2) + (int64_t)pr * g.q_phi + qk;
+    const int64_t pt = cell0 + (reg ? u * cell_s1 : (u / ns) * cell_s1 + (u % ns) * cell_s2) + (int64_t)pr * g.q_phi + qk;
+    const int64_t p = (pt >> 7) * g.ws + (pt & 127);  // its element in row 0
     const bool dead = touch && (g.t_phi_all || u == 0 || u == g.n_phi - 1);
     const double sh = nd.mu[qi][0], ch = nd.mu[qi][1], s2m = nd.mu[qi][2];
     const double sn = nd.nu[qj][0], cs = nd.nu[qj][1], s2n = nd.nu[qj][2], c2n = nd.nu[qj][3];
@@ -389,11 +390,11 @@ __global__ void __launch_bounds__(kEvalThreads) eval_fp64_kernel(LaunchTables t,
       // nucleus only on its one-centre grid), on a refined grid the third nucleus's
       if (g.n_W == 3) {
         const double wa = g.zA / rA, wb = g.zB / rB;
-        base[(int64_t)(g.row_W + 0) * ld + p] = wa + wb;
-        base[(int64_t)(g.row_W + 1) * ld + p] = sqrt(g.own_A ? wa + wb : wb);
-        base[(int64_t)(g.row_W + 2) * ld + p] = sqrt(g.own_B ? wa + wb : wa);
+        base[(int64_t)(g.row_W + 0) * rs + p] = wa + wb;
+        base[(int64_t)(g.row_W + 1) * rs + p] = sqrt(g.own_A ? wa + wb : wb);
+        base[(int64_t)(g.row_W + 2) * rs + p] = sqrt(g.own_B ? wa + wb : wa);
       } else if (g.n_W == 1) {
-        base[(int64_t)g.row_W * ld + p] = g.zC / rC;
+        base[(int64_t)g.row_W * rs + p] = g.zC / rC;
       }
     }
     const double x = a * sh * sn * ph[1], y = a * sh * sn * ph[0];
@@ -413,8 +414,8 @@ __global__ void __launch_bounds__(kEvalThreads) eval_fp64_kernel(LaunchTables t,
         for (int s = b0; s < b1; ++s) {
           const DevShell& q = t.bshell[s];
           const double* tv = tp + 2 * (e0 + s - b0) * np + pq;
-          if (g.row_F >= 0) store_shell(q, wf * tv[0], Y, base, ld, p, g.row_F + roff);
-          if (g.row_L >= 0) store_shell(q, wf * tv[np], Y, base, ld, p, g.row_L + roff);
+          if (g.row_F >= 0) store_shell(q, wf * tv[0], Y, base, rs, p, g.row_F + roff);
+          if (g.row_L >= 0) store_shell(q, wf * tv[np], Y, base, rs, p, g.row_L + roff);
         }
       }
       if (ha) {
@@ -423,11 +424,11 @@ __global__ void __launch_bounds__(kEvalThreads) eval_fp64_kernel(LaunchTables t,
           const DevShell& q = t.ashell[s];
           if (ctr == 2) {
             const double v = tc[((s - a0) * nn + f) * np + pq];
-            store_shell(q, g.row_U >= 0 ? v : wg * v, Y, base, ld, p, g.row_U >= 0 ? g.row_U : g.row_G);
+            store_shell(q, g.row_U >= 0 ? v : wg * v, Y, base, rs, p, g.row_U >= 0 ? g.row_U : g.row_G);
           } else {
             const double* tv = tp + 2 * (e0 + s - a0) * np + pq;
-            if (g.row_G >= 0) store_shell(q, wg * tv[0], Y, base, ld, p, g.row_G + roff);
-            if (g.row_U >= 0) store_shell(q, tv[np], Y, base, ld, p, g.row_U + roff);
+            if (g.row_G >= 0) store_shell(q, wg * tv[0], Y, base, rs, p, g.row_G + roff);
+            if (g.row_U >= 0) store_shell(q, tv[np], Y, base, rs, p, g.row_U + roff);
           }
         }
       }
@@ -484,7 +485,8 @@ __device__ __forceinline__ void sym_entry(int n, int r, int lane, int& row, int&
 // symmetric tile of nl rows, all on the lane side), into sm.sum[warp].  Narrow tiles: the lanes make
 // 1 << gs groups of 32 >> gs, each taking every (1 << gs)-th point.
 template <int R, bool SYM>
-__device__ __noinline__ void fma_warp(FmaSmem& sm, const double* __restrict__ base, int k0, int k1, int nr, int nl, int gs) {
+__device__ __noinline__ void fma_warp(FmaSmem& sm, const double* __restrict__ base, int64_t ws, int k0, int k1, int nr, int nl,
+                                      int gs) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   double(&v)[kFpPts][kFpFmaRegs + kFpFmaLanes] = sm.v[warp];
   const int gl = lane & ((32 >> gs) - 1), grp = lane >> (5 - gs);
@@ -503,14 +505,15 @@ __device__ __noinline__ void fma_warp(FmaSmem& sm, const double* __restrict__ ba
   }
   const int pp = lane & (kFpPts - 1), e0 = lane >> 3;
   for (int k = k0 + kFpPts * warp, n = 1; k < k1; k += 8 * kFpPts, ++n) {
+    const double* at = base + (int64_t)(k >> 7) * ws + (k & 127) + pp;
 #pragma unroll
     for (int i = SYM ? kFpFmaRegs / 4 : 0; i < (kFpFmaRegs + kFpFmaLanes) / 4; ++i) {
       const int e = e0 + 4 * i;
       if (e < kFpFmaRegs ? e < nr : e - kFpFmaRegs < nl) {
         double x = 0.0;
         if (k + pp < k1) {
-          x = __ldg(base + sm.x[e] + k + pp);
-          if (sm.y[e] >= 0) x *= __ldg(base + sm.y[e] + k + pp);
+          x = __ldg(at + sm.x[e]);
+          if (sm.y[e] >= 0) x *= __ldg(at + sm.y[e]);
         }
         v[pp][e] = x;
       }
@@ -549,28 +552,28 @@ __device__ __forceinline__ void contract_fma(const LaunchTables& t, const GemmIt
     const int i = rs ? tid : tid - kFpFmaRegs;
     if (i < (rs ? nr : nl)) {
       const short2 q = t.pairs[(rs ? roff : loff) + i];
-      sm.x[tid] = q.x * g.ld;
-      sm.y[tid] = q.y >= 0 ? q.y * g.ld : -1;
+      sm.x[tid] = q.x * g.rs;
+      sm.y[tid] = q.y >= 0 ? q.y * g.rs : -1;
     }
   }
   __syncthreads();
   const int R = sym ? (nl + 1) / 2 : nr;
   const int width = sym ? nl + 1 : nl, gs = width <= 4 ? 3 : (width <= 8 ? 2 : (width <= 16 ? 1 : 0));
   if (sym) {
-    if (R <= 2) fma_warp<2, true>(sm, base, k0, k1, nr, nl, gs);
-    else if (R <= 4) fma_warp<4, true>(sm, base, k0, k1, nr, nl, gs);
-    else if (R <= 8) fma_warp<8, true>(sm, base, k0, k1, nr, nl, gs);
-    else if (R <= 12) fma_warp<12, true>(sm, base, k0, k1, nr, nl, gs);
-    else fma_warp<16, true>(sm, base, k0, k1, nr, nl, gs);
+    if (R <= 2) fma_warp<2, true>(sm, base, g.ws, k0, k1, nr, nl, gs);
+    else if (R <= 4) fma_warp<4, true>(sm, base, g.ws, k0, k1, nr, nl, gs);
+    else if (R <= 8) fma_warp<8, true>(sm, base, g.ws, k0, k1, nr, nl, gs);
+    else if (R <= 12) fma_warp<12, true>(sm, base, g.ws, k0, k1, nr, nl, gs);
+    else fma_warp<16, true>(sm, base, g.ws, k0, k1, nr, nl, gs);
   } else {
-    if (R <= 2) fma_warp<2, false>(sm, base, k0, k1, nr, nl, gs);
-    else if (R <= 4) fma_warp<4, false>(sm, base, k0, k1, nr, nl, gs);
-    else if (R <= 6) fma_warp<6, false>(sm, base, k0, k1, nr, nl, gs);
-    else if (R <= 8) fma_warp<8, false>(sm, base, k0, k1, nr, nl, gs);
-    else if (R <= 10) fma_warp<10, false>(sm, base, k0, k1, nr, nl, gs);
-    else if (R <= 12) fma_warp<12, false>(sm, base, k0, k1, nr, nl, gs);
-    else if (R <= 14) fma_warp<14, false>(sm, base, k0, k1, nr, nl, gs);
-    else fma_warp<16, false>(sm, base, k0, k1, nr, nl, gs);
+    if (R <= 2) fma_warp<2, false>(sm, base, g.ws, k0, k1, nr, nl, gs);
+    else if (R <= 4) fma_warp<4, false>(sm, base, g.ws, k0, k1, nr, nl, gs);
+    else if (R <= 6) fma_warp<6, false>(sm, base, g.ws, k0, k1, nr, nl, gs);
+    else if (R <= 8) fma_warp<8, false>(sm, base, g.ws, k0, k1, nr, nl, gs);
+    else if (R <= 10) fma_warp<10, false>(sm, base, g.ws, k0, k1, nr, nl, gs);
+    else if (R <= 12) fma_warp<12, false>(sm, base, g.ws, k0, k1, nr, nl, gs);
+    else if (R <= 14) fma_warp<14, false>(sm, base, g.ws, k0, k1, nr, nl, gs);
+    else fma_warp<16, false>(sm, base, g.ws, k0, k1, nr, nl, gs);
   }
   __syncthreads();
   double* out = part + b.part_off + (int64_t)it.chunk * b.m * b.n;
@@ -607,7 +610,7 @@ __global__ void __launch_bounds__(fx::kThreads, 2) contract_fp64_kernel(LaunchTa
   }
   fx::Smem& sm = fx::smem_at(raw);
   const uint32_t tmem = fx::open(sm);
-  const int64_t ld = g.ld;
+  const int64_t rs = g.rs;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int r0 = it.tm * kFpDigitRows, c0 = it.tn * kFpDigitCols;
   const int rows = min(kFpDigitRows, b.m - r0), cols = min(kFpDigitCols, b.n - c0);
@@ -618,31 +621,33 @@ __global__ void __launch_bounds__(fx::kThreads, 2) contract_fp64_kernel(LaunchTa
 #pragma unroll
   for (int u = 0; u < 2; ++u) {
     const short2 q = t.pairs[b.a_off + r0 + min(fx::a_row(u), rows - 1)];
-    ax[u] = q.x * ld;
-    ay[u] = q.y >= 0 ? q.y * ld : -1;
+    ax[u] = q.x * rs;
+    ay[u] = q.y >= 0 ? q.y * rs : -1;
   }
   {
     const short2 q = t.pairs[b.b_off + c0 + min(fx::b_col(), cols - 1)];
-    bx = q.x * ld;
-    by = q.y >= 0 ? q.y * ld : -1;
+    bx = q.x * rs;
+    by = q.y >= 0 ? q.y * rs : -1;
   }
   auto value = [&](short2 q, int p) {
-    const double v = base[q.x * ld + p];
-    return q.y >= 0 ? v * base[q.y * ld + p] : v;
+    const double* at = base + (int64_t)(p >> 7) * g.ws + (p & 127);
+    return q.y >= 0 ? at[q.x * rs] * at[q.y * rs] : at[q.x * rs];
   };
   double acc[16] = {};
   uint32_t phase = 0, win = 0;
   bool ok = true, run = true;
   for (int k = k0; k < k1 && run; k += kFpWin, ++win) {
     double va[4][8], vb[2][4];
+    const double* win0 = base + (int64_t)(k >> 7) * g.ws + (k & 127);  // the window's first point (row 0)
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
         double(&v)[8] = va[2 * c + u];
-        const int p = k + fx::a_pt(c), left = 64 * u + 8 * warp < rows ? k1 - p : 0;
+        const int left = 64 * u + 8 * warp < rows ? k1 - k - fx::a_pt(c) : 0;
+        const double* at = win0 + fx::a_pt(c);
         if (left >= 8) {
-          const double2* x = reinterpret_cast<const double2*>(base + ax[u] + p);
+          const double2* x = reinterpret_cast<const double2*>(at + ax[u]);
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             const double2 q = __ldg(x + i);
@@ -650,7 +655,7 @@ __global__ void __launch_bounds__(fx::kThreads, 2) contract_fp64_kernel(LaunchTa
             v[2 * i + 1] = q.y;
           }
           if (ay[u] >= 0) {
-            const double2* y = reinterpret_cast<const double2*>(base + ay[u] + p);
+            const double2* y = reinterpret_cast<const double2*>(at + ay[u]);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
               const double2 q = __ldg(y + i);
@@ -662,15 +667,15 @@ __global__ void __launch_bounds__(fx::kThreads, 2) contract_fp64_kernel(LaunchTa
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
             v[i] = 0.0;
-            if (i < left) v[i] = base[ax[u] + p + i] * (ay[u] >= 0 ? base[ay[u] + p + i] : 1.0);
+            if (i < left) v[i] = at[ax[u] + i] * (ay[u] >= 0 ? at[ay[u] + i] : 1.0);
           }
         }
       }
-      const int p = k + fx::b_pt(c);
+      const double* at = win0 + fx::b_pt(c);
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         vb[c][i] = 0.0;
-        if (fx::b_col() < cols && p + i < k1) vb[c][i] = __ldg(base + bx + p + i) * (by >= 0 ? __ldg(base + by + p + i) : 1.0);
+        if (fx::b_col() < cols && k + fx::b_pt(c) + i < k1) vb[c][i] = __ldg(at + bx + i) * (by >= 0 ? __ldg(at + by + i) : 1.0);
       }
     }
     run = fx::window(sm, tmem, va, vb, acc, phase, win, rows, cols, ok, [&](int r, int c) {

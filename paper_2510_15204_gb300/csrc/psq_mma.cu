@@ -24,6 +24,7 @@
 #include "psq_internal.h"
 #include "psq_df.cuh"
 #include "psq_tc.cuh"
+#include "psq_f2.cuh"
 
 #include <cuda_bf16.h>
 
@@ -157,11 +158,11 @@ __device__ __forceinline__ int shells_lmax_f(const DevShell* sh, int s0, int s1)
 
 // One row kind of a shell at one point: the radial value times the harmonics, to the hi and lo planes.
 __device__ __forceinline__ void store_shell(const DevShell& q, df r, const df* Y, float* __restrict__ oh,
-                                            float* __restrict__ ol, int64_t ld, int64_t p, int row) {
+                                            float* __restrict__ ol, int64_t rs, int64_t p, int row) {
   const int base = q.l * q.l + q.l;
-  int64_t o = (int64_t)(row + q.fn0) * ld + p;
+  int64_t o = (int64_t)(row + q.fn0) * rs + p;
 #pragma unroll 1
-  for (int m = -q.l; m <= q.l; ++m, o += ld) {
+  for (int m = -q.l; m <= q.l; ++m, o += rs) {
     const df v = dfa::mul(r, Y[base + m]);
     oh[o] = v.h;
     ol[o] = v.l;
@@ -295,7 +296,7 @@ __global__ void __launch_bounds__(kEvalThreads) eval_mixed_kernel(LaunchTables t
   // the points: phi rows u0 .. u1 - 1 and their mirrors
   float* bh = ops + g.op_off;
   float* bl = ops_lo + g.op_off;
-  const int64_t ld = g.ld;
+  const int64_t rs = g.rs;
   const int per = np * g.q_phi, nu = pb.u1 - pb.u0;
   df Y[(kMaxL + 1) * (kMaxL + 1)];
   for (int e = tid; e < 2 * nu * per; e += kEvalThreads) {
@@ -305,7 +306,8 @@ __global__ void __launch_bounds__(kEvalThreads) eval_mixed_kernel(LaunchTables t
     if (mirror && u == uh) continue;  // the middle row is its own mirror
     const int pr = pb.pr0 + pq, qi = pr / g.q_nu, qj = pr - qi * g.q_nu;
     const int f = (uh - pb.u0) * g.q_phi + (mirror ? g.q_phi - 1 - qk : qk);  // node of the half
-    const int64_t p = cell0 + (reg ? u * cell_s1 : (u / ns) * cell_s1 + (u % ns) * cell_s2) + (int64_t)pr * g.q_phi + qk;
+    const int64_t pt = cell0 + (reg ? u * cell_s1 : (u / ns) * cell_s1 + (u % ns) * cell_s2) + (int64_t)pr * g.q_phi + qk;
+    const int64_t p = (pt >> 7) * g.ws + (pt & 127);  // its element in row 0
     const bool dead = touch && (g.t_phi_all || u == 0 || u == g.n_phi - 1);
     const NodeEntry &M = Mu[qi], &N = Nu[qj], &F = Ph[u * g.q_phi + qk];
     const df sh = ld2(M.fs), s2m = ld2(M.fh2), sn = ld2(N.fs), s2n = ld2(N.fh2), c2n = ld2(N.fg2);
@@ -322,8 +324,8 @@ __global__ void __launch_bounds__(kEvalThreads) eval_mixed_kernel(LaunchTables t
       const df wv[4] = {w, dfa::div(w, rhoA), dfa::div(w, rhoB), third ? dfa::div(w, rC) : dfa::mk(0.0f)};
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        bh[(int64_t)(g.row_W + k) * ld + p] = wv[k].h;
-        bl[(int64_t)(g.row_W + k) * ld + p] = wv[k].l;
+        bh[(int64_t)(g.row_W + k) * rs + p] = wv[k].h;
+        bl[(int64_t)(g.row_W + k) * rs + p] = wv[k].l;
       }
     }
     const df xs = dfa::mul(shsn, ld2(F.fc)), ys = dfa::mul(shsn, ld2(F.fs)), s2mc = dfa::mul(s2m, ld2(N.fc));
@@ -348,8 +350,8 @@ __global__ void __launch_bounds__(kEvalThreads) eval_mixed_kernel(LaunchTables t
         for (int s = b0; s < b1; ++s) {
           const DevShell& q = t.bshell[s];
           const float2* tv = tp + 2 * (e0 + s - b0) * np + pq;
-          if (g.row_F >= 0) store_shell(q, ld2(tv[0]), Y, bh, bl, ld, p, g.row_F + roff);
-          if (g.row_L >= 0) store_shell(q, ld2(tv[np]), Y, bh, bl, ld, p, g.row_L + roff);
+          if (g.row_F >= 0) store_shell(q, ld2(tv[0]), Y, bh, bl, rs, p, g.row_F + roff);
+          if (g.row_L >= 0) store_shell(q, ld2(tv[np]), Y, bh, bl, rs, p, g.row_L + roff);
         }
       }
       if (ha) {
@@ -358,11 +360,11 @@ __global__ void __launch_bounds__(kEvalThreads) eval_mixed_kernel(LaunchTables t
         for (int s = a0; s < a1; ++s) {
           const DevShell& q = t.ashell[s];
           if (ctr == 2) {
-            store_shell(q, ld2(tc[((s - a0) * nn + f) * np + pq]), Y, bh, bl, ld, p, g.row_U >= 0 ? g.row_U : g.row_G);
+            store_shell(q, ld2(tc[((s - a0) * nn + f) * np + pq]), Y, bh, bl, rs, p, g.row_U >= 0 ? g.row_U : g.row_G);
           } else {
             const float2* tv = tp + 2 * (e0 + s - a0) * np + pq;
-            if (g.row_G >= 0) store_shell(q, ld2(tv[0]), Y, bh, bl, ld, p, g.row_G + roff);
-            if (g.row_U >= 0) store_shell(q, ld2(tv[np]), Y, bh, bl, ld, p, g.row_U + roff);
+            if (g.row_G >= 0) store_shell(q, ld2(tv[0]), Y, bh, bl, rs, p, g.row_G + roff);
+            if (g.row_U >= 0) store_shell(q, ld2(tv[np]), Y, bh, bl, rs, p, g.row_U + roff);
           }
         }
       }
@@ -378,7 +380,8 @@ constexpr int kM = kMmaM;
 constexpr int kTileN = kMmaN;
 constexpr int kChunk = kChunkPts;
 constexpr int kRowB = 2 * kChunkPts;            // bytes of one operand row of a stage (64)
-constexpr int kStages = 3;                      // A ring depth (chunks, 40 KB each)
+constexpr int kARingBytes = 147456;             // A ring: 3 chunks of 128 rows (40 KB each), more of fewer rows
+constexpr int kMaxStages = 8;
 constexpr int kStagesB = 3;                     // B ring depth (chunks, 15 KB each)
 constexpr int kChunksPerWin = kWinPts / kChunkPts;
 
@@ -420,7 +423,7 @@ namespace mma {
 // |hi|: the join adds at most 1.5 to s2, which stays <= 130, and rounds at 2^-17 of s2's unit,
 // 2^-40 of the window's largest value).
 //
-// Each digit takes three full-rate FP32 instructions.  With M = 1.5 x 2^23 and |x| < 2^22,
+// Each digit takes three full-rate FP32 instructions (packed: for two values).  With M = 1.5 x 2^23 and |x| < 2^22,
 // t = x + M rounds x to its nearest integer s (ties to even): t lies in [2^23, 2^24), where the
 // spacing is 1, so t = M + s exactly.  Then fma(t, -256, 256 M) = -256 s and
 // fma(x, 256, -256 s) = 256 (x - s) are exact (|x - s| <= 1/2 is a multiple of x's spacing).
@@ -446,28 +449,28 @@ __device__ __forceinline__ void window_scales(int e, float& sc, float& scj) {
   scj = e == kZeroExp ? 0.0f : pow2f(7 - e + 8 * (JOIN + 1));
 }
 
+// The planes of eight consecutive points (a 16-byte group) given as four pairs; the values are sgn vh
+// + vl (sgn: the sign the hi words' scale sc carries).
 template <int JOIN>
-__device__ __forceinline__ void slice8_df(const float* vh, const float* vl, float sc, float scj, uint4* w) {
+__device__ __forceinline__ void slice8_f2(const f2 (&vh)[4], const f2 (&vl)[4], float sc, float scj, uint4 (&w)[kSlices]) {
   uint32_t o[kSlices][4];
-  const float sc256 = sc * 256.0f;  // at most 2^125
+  const f2 s0 = f2_both(sc), s256 = f2_both(sc * 256.0f), sj = f2_both(scj);  // |sc 256| at most 2^125
+  const f2 magic = f2_both(kRneMagic), magic256 = f2_both(kRneMagic256), m256 = f2_both(-256.0f), p256 = f2_both(256.0f);
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    float r0 = 0.0f, r1 = 0.0f;
-    const float l0 = vl[2 * q] * scj, l1 = vl[2 * q + 1] * scj;
+    f2 r{};
+    const f2 l = f2_mul(vl[q], sj);
 #pragma unroll
     for (int k = 0; k < kSlices; ++k) {
       // digit 0 rounds v sc (exact: sc is a power of two) inside its first FMA
-      const float t0 = k == 0 ? __fmaf_rn(vh[2 * q], sc, kRneMagic) : __fadd_rn(r0, kRneMagic);
-      const float t1 = k == 0 ? __fmaf_rn(vh[2 * q + 1], sc, kRneMagic) : __fadd_rn(r1, kRneMagic);
-      const float d0 = __fmaf_rn(t0, -256.0f, kRneMagic256), d1 = __fmaf_rn(t1, -256.0f, kRneMagic256);
+      const f2 t = k == 0 ? f2_fma(vh[q], s0, magic) : f2_add(r, magic);
+      const f2 d = f2_fma(t, m256, magic256);
+      float d0, d1;
+      f2_unpack(d, d0, d1);
       o[k][q] = pack_bf16_exact(d0, d1);
       if (k + 1 < kSlices) {
-        r0 = k == 0 ? __fmaf_rn(vh[2 * q], sc256, d0) : __fmaf_rn(r0, 256.0f, d0);
-        r1 = k == 0 ? __fmaf_rn(vh[2 * q + 1], sc256, d1) : __fmaf_rn(r1, 256.0f, d1);
-        if (k == JOIN) {
-          r0 = __fadd_rn(r0, l0);
-          r1 = __fadd_rn(r1, l1);
-        }
+        r = k == 0 ? f2_fma(vh[q], s256, d) : f2_fma(r, p256, d);
+        if (k == JOIN) r = f2_add(r, l);
       }
     }
   }
@@ -485,12 +488,11 @@ __device__ __forceinline__ int row_exponent(float mx) {
 }  // namespace mma
 
 // (xh + xl)(yh + yl) as hi = fl(xh yh) and the unnormalised lo = the exact error of that
-// product plus the cross terms (|lo| <= 3 2^-24 |hi|; the lo lo term, below 2^-48, dropped).
-__device__ __forceinline__ void prod_unnorm(float xh, float xl, float yh, float yl, float& h, float& l) {
-  h = __fmul_rn(xh, yh);
-  float e = __fmaf_rn(xh, yh, -h);
-  e = __fmaf_rn(xh, yl, e);
-  l = __fmaf_rn(xl, yh, e);
+// product plus the cross terms (|lo| <= 3 2^-24 |hi|; the lo lo term, below 2^-48, dropped).  The hi
+// words come negated (the error of a product is one FMA from its negative).
+__device__ __forceinline__ void prod_unnorm(f2 xh, f2 xl, f2 yh, f2 yl, f2& nh, f2& l) {
+  nh = f2_mul(xh, f2_mul(yh, f2_both(-1.0f)));
+  l = f2_fma(xl, yh, f2_fma(xh, yl, f2_fma(xh, yh, nh)));
 }
 
 // Decodes packing job `job` (panel, tile, window, 16-row group) for this thread: 8 threads per
@@ -529,13 +531,17 @@ __device__ __forceinline__ PackPos pack_pos(int64_t job, const Panel* __restrict
 }
 
 // The row's window exponent (the eight threads of the row share it) and the five planes of
-// this thread's 16 points.
-__device__ __forceinline__ void pack_store(const PackPos& P, const Panel& pn, const float* h, const float* l,
+// this thread's 16 points, sgn h + l (sgn = 1 or -1).
+__device__ __forceinline__ void pack_store(const PackPos& P, const Panel& pn, const f2 (&h)[2][4], const f2 (&l)[2][4], float sgn,
                                            uint8_t* __restrict__ packed) {
   using namespace mma;
   float mx = 0.0f;
 #pragma unroll
-  for (int i = 0; i < 16; ++i) mx = fmaxf(mx, fabsf(h[i]));
+  for (int i = 0; i < 8; ++i) {
+    float a, b;
+    f2_unpack(h[i >> 2][i & 3], a, b);
+    mx = fmaxf(mx, fmaxf(fabsf(a), fabsf(b)));
+  }
   const unsigned m8 = 0xffu << ((threadIdx.x & 31) & ~7u);
   mx = fmaxf(mx, __shfl_xor_sync(m8, mx, 1));
   mx = fmaxf(mx, __shfl_xor_sync(m8, mx, 2));
@@ -554,7 +560,7 @@ __device__ __forceinline__ void pack_store(const PackPos& P, const Panel& pn, co
 #pragma unroll
   for (int j = 0; j < 2; ++j) {
     uint4 wv[kSlices];
-    slice8_df<1>(h + 8 * j, l + 8 * j, sc, scj, wv);
+    slice8_f2<1>(h[j], l[j], sgn * sc, scj, wv);
 #pragma unroll
     for (int k = 0; k < kSlices; ++k) *reinterpret_cast<uint4*>(dst + k * plane + swz(P.r, 2 * (P.qq & 1) + j)) = wv[k];
   }
@@ -571,48 +577,51 @@ __global__ void __launch_bounds__(128) pack_kernel(const DevGrid* __restrict__ g
   const DevGrid& g = grids[pn.grid];
   const int row = P.t * pn.tr + P.r;
   const int64_t k0 = (int64_t)kWinPts * P.w + 16 * P.qq;
+  const int64_t blk = g.op_off + (int64_t)P.w * g.ws + 16 * P.qq;  // (kWinPts = 128: one block)
   int64_t src = -1, mul = -1;
   if (row < pn.nrows) {
     const short2 q = rows[pn.rows_off + row];
-    src = g.op_off + (int64_t)q.x * g.ld + k0;
-    if (q.y >= 0) mul = g.op_off + (int64_t)q.y * g.ld + k0;
+    src = blk + q.x * g.rs;
+    if (q.y >= 0) mul = blk + q.y * g.rs;
   }
   const int64_t left = src >= 0 ? g.K - k0 : 0;
-  float h[16], l[16];
+  f2 h[2][4], l[2][4];
 #pragma unroll
   for (int i4 = 0; i4 < 4; ++i4) {
-    float4 ah = make_float4(0.f, 0.f, 0.f, 0.f), al = ah, bh = make_float4(1.f, 1.f, 1.f, 1.f), bl = al;
+    ulonglong2 ah = make_ulonglong2(0, 0), al = ah, bh = ah, bl = ah;
     if (left >= 4 * i4 + 4) {
-      ah = __ldg(reinterpret_cast<const float4*>(ops + src) + i4);
-      al = __ldg(reinterpret_cast<const float4*>(ops_lo + src) + i4);
+      ah = __ldg(reinterpret_cast<const ulonglong2*>(ops + src) + i4);
+      al = __ldg(reinterpret_cast<const ulonglong2*>(ops_lo + src) + i4);
       if (mul >= 0) {
-        bh = __ldg(reinterpret_cast<const float4*>(ops + mul) + i4);
-        bl = __ldg(reinterpret_cast<const float4*>(ops_lo + mul) + i4);
+        bh = __ldg(reinterpret_cast<const ulonglong2*>(ops + mul) + i4);
+        bl = __ldg(reinterpret_cast<const ulonglong2*>(ops_lo + mul) + i4);
       }
     } else if (left > 4 * i4) {
-      float* ph = &ah.x; float* pl = &al.x; float* qh = &bh.x; float* ql = &bl.x;
+      float v[4][4] = {};
       for (int i = 0; i < 4 && 4 * i4 + i < left; ++i) {
-        ph[i] = ops[src + 4 * i4 + i];
-        pl[i] = ops_lo[src + 4 * i4 + i];
+        v[0][i] = ops[src + 4 * i4 + i];
+        v[1][i] = ops_lo[src + 4 * i4 + i];
         if (mul >= 0) {
-          qh[i] = ops[mul + 4 * i4 + i];
-          ql[i] = ops_lo[mul + 4 * i4 + i];
+          v[2][i] = ops[mul + 4 * i4 + i];
+          v[3][i] = ops_lo[mul + 4 * i4 + i];
         }
       }
+      ah = make_ulonglong2(f2_pack(v[0][0], v[0][1]).v, f2_pack(v[0][2], v[0][3]).v);
+      al = make_ulonglong2(f2_pack(v[1][0], v[1][1]).v, f2_pack(v[1][2], v[1][3]).v);
+      bh = make_ulonglong2(f2_pack(v[2][0], v[2][1]).v, f2_pack(v[2][2], v[2][3]).v);
+      bl = make_ulonglong2(f2_pack(v[3][0], v[3][1]).v, f2_pack(v[3][2], v[3][3]).v);
     }
-    const float xh[4] = {ah.x, ah.y, ah.z, ah.w}, xl[4] = {al.x, al.y, al.z, al.w};
-    const float yh[4] = {bh.x, bh.y, bh.z, bh.w}, yl[4] = {bl.x, bl.y, bl.z, bl.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      if (mul >= 0) {
-        prod_unnorm(xh[i], xl[i], yh[i], yl[i], h[4 * i4 + i], l[4 * i4 + i]);
-      } else {
-        h[4 * i4 + i] = xh[i];
-        l[4 * i4 + i] = xl[i];
-      }
+    f2 &h0 = h[i4 >> 1][2 * (i4 & 1)], &h1 = h[i4 >> 1][2 * (i4 & 1) + 1];
+    f2 &l0 = l[i4 >> 1][2 * (i4 & 1)], &l1 = l[i4 >> 1][2 * (i4 & 1) + 1];
+    if (mul >= 0) {
+      prod_unnorm(f2{ah.x}, f2{al.x}, f2{bh.x}, f2{bl.x}, h0, l0);
+      prod_unnorm(f2{ah.y}, f2{al.y}, f2{bh.y}, f2{bl.y}, h1, l1);
+    } else {
+      h0 = f2{ah.x}; h1 = f2{ah.y};
+      l0 = f2{al.x}; l1 = f2{al.y};
     }
   }
-  pack_store(P, pn, h, l, packed);
+  pack_store(P, pn, h, l, mul >= 0 ? -1.0f : 1.0f, packed);
 }
 
 // The same packed-panel image from FP64 operand rows (row-major, stride n): used for the
@@ -627,15 +636,21 @@ __global__ void __launch_bounds__(128) ri_pack_kernel(const Panel* __restrict__ 
   const double* src = P.pn ? srcB : srcA;
   const int row = P.t * pn.tr + P.r;
   const int k0 = kWinPts * P.w + 16 * P.qq;
-  float h[16], l[16];
+  f2 h[2][4], l[2][4];
 #pragma unroll
-  for (int i = 0; i < 16; ++i) {
-    double v = 0.0;
-    if (row < pn.nrows && k0 + i < n) v = src[(int64_t)row * n + k0 + i];
-    h[i] = (float)v;
-    l[i] = (float)(v - (double)h[i]);
+  for (int i = 0; i < 8; ++i) {
+    float hv[2], lv[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      double v = 0.0;
+      if (row < pn.nrows && k0 + 2 * i + k < n) v = src[(int64_t)row * n + k0 + 2 * i + k];
+      hv[k] = (float)v;
+      lv[k] = (float)(v - (double)hv[k]);
+    }
+    h[i >> 2][i & 3] = f2_pack(hv[0], hv[1]);
+    l[i >> 2][i & 3] = f2_pack(lv[0], lv[1]);
   }
-  pack_store(P, pn, h, l, packed);
+  pack_store(P, pn, h, l, 1.0f, packed);
 }
 
 // ------------------------------------------------------------------ warp-specialised contraction
@@ -643,8 +658,8 @@ __global__ void __launch_bounds__(128) ri_pack_kernel(const Panel* __restrict__ 
 // One persistent CTA per SM, 512 threads, working through tiles (128 A rows x <= 48 B
 // columns x a range of 128-point windows):
 //   warp 4       loader: two ordered streams of bulk copies, each served as soon as its next
-//                buffer is free: the packed A tile of every 32-point chunk into a three-stage
-//                A ring (and, for a packed B, its B tile into the B ring), and the staged basis
+//                buffer is free: the packed A tile of every 32-point chunk into the A ring
+//                of three to eight chunks (and, for a packed B, its B tile into the B ring), and the staged basis
 //                rows (hi and lo planes) of every formed window into two buffers;
 //   warps 0-3, 6, 7  producers: for a formed B, column c of the tile = product of two staged
 //                rows (a double-float product); each warp owns 8 columns, four lanes per
@@ -669,15 +684,18 @@ namespace ws {
 
 constexpr int kThreads = 512;
 constexpr int kLoadWarp = 4, kMmaWarp = 5, kFoldWarp0 = 8;
-constexpr int kRawStride = 132;  // floats per staged row: 128 points + 4 (bank spread)
+// Staged basis rows lie 512 bytes apart, as in memory, so that a run of consecutive rows is one copy (a
+// bulk copy takes the loader about 100 cycles to issue; rows spread over the banks, one copy each,
+// cost more than the two-way conflicts of this layout's reads).
+constexpr int kRawStride = kWinPts;
 
 struct Smem {
-  alignas(1024) uint8_t a[mma::kStages][kSlices][mma::kM * mma::kRowB];
+  alignas(1024) uint8_t a[mma::kARingBytes];
   alignas(1024) uint8_t b[mma::kStagesB][kSlices][mma::kTileN * mma::kRowB];
   alignas(16) float raw[2][2][kPairTileRows][kRawStride];  // [buffer][hi, lo][row][point]
   int eb[2][mma::kTileN];
-  float sbw[8][mma::kTileN];  // fold warp k: the column scales of the current window
-  alignas(8) uint64_t a_full[mma::kStages], a_free[mma::kStages], b_ready[mma::kStagesB], b_free[mma::kStagesB];
+  alignas(8) float sbw[8][mma::kTileN];  // fold warp k: the column scales of the current window
+  alignas(8) uint64_t a_full[mma::kMaxStages], a_free[mma::kMaxStages], b_ready[mma::kStagesB], b_free[mma::kStagesB];
   uint64_t tmem_full[2], tmem_free[2], raw_full[2], raw_free[2], eb_free[2];
   uint64_t drain;
   uint32_t tmem_base;
@@ -709,16 +727,37 @@ __device__ __forceinline__ bool wait(uint64_t* b, uint32_t parity, const int* ab
   return mma::mbar_wait(mma::smem_u32(b), parity, abort, limit_ns);
 }
 
-// Ring positions of chunk c: A stage c % kStages after c / kStages completed rounds, B stage
-// c % kStagesB after c / kStagesB rounds.
-__device__ __forceinline__ int stage_of(uint32_t c) { return (int)(c % mma::kStages); }
-__device__ __forceinline__ uint32_t round_of(uint32_t c) { return c / mma::kStages; }
+// The A ring.  A tile's chunk takes its real rows (rounded up to eight) times 64 bytes per plane, so a
+// tile of 72 rows has six chunks in flight where one of 128 rows has three: the ring must cover the
+// latency of the copies (2 us under load, about three chunks' MMAs).  The MMAs read 128 rows per
+// plane; what lies past the real ones (other planes, the B ring) only reaches result rows that are
+// never read.  Loader and MMA lane step through the stages alike; when the rows per tile change, the
+// loader waits for the ring to empty and both start again at stage 0.
+struct ARing {
+  uint32_t par;   // loader: parity of each stage's next a_free phase; MMA lane: of its next a_full phase
+  uint32_t used;  // loader: stages whose last use is not yet known to be over
+  int s, n, plane;  // stage, stages, bytes of a plane
+  __device__ __forceinline__ void open() { par = used = 0; s = n = plane = 0; }
+  __device__ __forceinline__ bool fits(int rows) const { return plane == ((rows + 7) & ~7) * mma::kRowB; }
+  __device__ __forceinline__ void layout(int rows) {
+    plane = ((rows + 7) & ~7) * mma::kRowB;
+    n = min(mma::kMaxStages, mma::kARingBytes / (kSlices * plane));
+    s = 0;
+  }
+  __device__ __forceinline__ uint32_t offset() const { return (uint32_t)(s * kSlices * plane); }
+  __device__ __forceinline__ void next() { s = s + 1 == n ? 0 : s + 1; }
+};
+// Stage k free again (loader)
+__device__ __forceinline__ bool wait_a_free(Smem& sm, ARing& r, int k, uint64_t ns) {
+  if (!((r.used >> k) & 1u)) return true;
+  if (!mma::mbar_wait(mma::smem_u32(&sm.a_free[k]), (r.par >> k) & 1u, &sm.abort, ns)) return false;
+  r.par ^= 1u << k;
+  r.used &= ~(1u << k);
+  return true;
+}
+// B stage of chunk c: c % kStagesB after c / kStagesB completed rounds
 __device__ __forceinline__ int bstage_of(uint32_t c) { return (int)(c % mma::kStagesB); }
 __device__ __forceinline__ uint32_t bround_of(uint32_t c) { return c / mma::kStagesB; }
-// A stage of chunk c free again (its MMAs of chunk c - kStages complete)
-__device__ __forceinline__ bool wait_a_free(Smem& sm, uint32_t c, uint64_t ns) {
-  return c < (uint32_t)mma::kStages || mma::mbar_wait(mma::smem_u32(&sm.a_free[stage_of(c)]), (round_of(c) - 1) & 1, &sm.abort, ns);
-}
 // B stage of chunk c free again (its MMAs of chunk c - kStagesB complete)
 __device__ __forceinline__ bool wait_b_free(Smem& sm, uint32_t c, uint64_t ns) {
   return c < (uint32_t)mma::kStagesB ||
@@ -766,7 +805,8 @@ __device__ __forceinline__ bool aborted(Smem& sm) { return *(volatile int*)&sm.a
 struct RowStream {
   int ii, ie, win, w1;  // current item, end, next window, the item's window end
   int nr;               // staged rows of the item's pair tile (<= kPairTileRows)
-  int64_t src;          // this lane's row (lane & 15) of plane (lane >> 4), window 0, in floats
+  unsigned runs;        // bit r: row r does not follow row r - 1 in memory
+  int64_t src, ws;      // this lane's row (lane & 15), window 0, in floats; window stride
   bool more;
 
   __device__ __forceinline__ void open(int i0, int i1, const GemmItem* items, const MmaBlock* blocks,
@@ -789,19 +829,35 @@ struct RowStream {
       win = q.w0;
       w1 = q.w1;
       nr = q.pt->nrows;
-      src = g.op_off + (int64_t)q.pt->rows[max(0, min(lane & 15, nr - 1))] * g.ld;
+      const int row = q.pt->rows[max(0, min(lane & 15, nr - 1))];
+      const int before = __shfl_up_sync(0xffffffffu, row, 1);
+      runs = __ballot_sync(0xffffffffu, lane < nr && (lane == 0 || row != before + 1));
+      src = g.op_off + row * g.rs;
+      ws = g.ws;
       more = win < w1;
       if (more) return;
     }
     more = false;
   }
-  // Bulk copies of the current window's rows (hi and lo planes, 512 bytes per row and plane)
-  // into raw buffer rb, completing on raw_full[rb]; one warp.
-  __device__ __forceinline__ void request(Smem& sm, int rb, const float* ops, const float* ops_lo, int lane) const {
-    if (lane == 0) mbar_expect_tx(&sm.raw_full[rb], (uint32_t)nr * 2u * 512u);
+  // Bulk copies of the current window's rows (hi and lo planes, 512 bytes per row and plane, one copy
+  // per run of consecutive rows) into raw buffer rb, completing on raw_full[rb]; one warp, one lane
+  // issuing on uniform addresses.
+  __device__ __forceinline__ void request(Smem& sm, int rb, const float* ops, const float* ops_lo) const {
+    const int n = __shfl_sync(0xffffffffu, nr, 0);
+    if (mma::elect_one()) mbar_expect_tx(&sm.raw_full[rb], (uint32_t)n * 2u * 512u);
     __syncwarp();
-    const int rr = lane & 15, pl = lane >> 4;
-    if (rr < nr) bulk_g2s(sm.raw[rb][pl][rr], (pl ? ops_lo : ops) + src + (int64_t)kWinPts * win, 512u, &sm.raw_full[rb]);
+    const int64_t w0 = ws * win;
+    for (unsigned m = runs; m != 0;) {
+      const int r = __ffs(m) - 1;
+      m &= m - 1;
+      const uint32_t bytes = (uint32_t)((m ? __ffs(m) - 1 : n) - r) * 512u;
+      const int64_t at = __shfl_sync(0xffffffffu, src, r) + w0;
+      if (mma::elect_one()) {
+        bulk_g2s(sm.raw[rb][0][r], ops + at, bytes, &sm.raw_full[rb]);
+        bulk_g2s(sm.raw[rb][1][r], ops_lo + at, bytes, &sm.raw_full[rb]);
+      }
+      __syncwarp();
+    }
   }
 };
 
@@ -817,10 +873,10 @@ __global__ void __launch_bounds__(ws::kThreads, 1)
   using namespace mma;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   ws::Smem& sm = *reinterpret_cast<ws::Smem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;  // (a warp-uniform index)
   if (warp == ws::kMmaWarp) tmem_alloc(&sm.tmem_base, 512);
   if (tid == 0) {
-    for (int s = 0; s < kStages; ++s) {
+    for (int s = 0; s < kMaxStages; ++s) {
       mbar_init(&sm.a_full[s], 1);
       mbar_init(&sm.a_free[s], 1);
     }
@@ -849,7 +905,10 @@ __global__ void __launch_bounds__(ws::kThreads, 1)
   if (warp == ws::kLoadWarp) {
     // ------------------------------------------------------------------ loader
     bool run = true;  // warp-uniform
-    int last_a = -1;  // last issued chunk (for the drain)
+    ws::ARing ar;
+    ar.open();
+    bool was_formed = false;
+    uint32_t loads = 0, loaded = 0;  // parity of each stage's loads so far; stages ever loaded (for the drain)
     if (hold) {
       // failure-detection test: a raised flag that nothing clears holds the first copy back
       // until the wait limit runs out
@@ -880,7 +939,7 @@ __global__ void __launch_bounds__(ws::kThreads, 1)
         int free_ = 1;
         if (lane == 0) free_ = rq < 2 || mbar_test(smem_u32(&sm.raw_free[rb]), ((rq - 2) >> 1) & 1);
         if (!__shfl_sync(kFull, free_, 0)) return;
-        rs.request(sm, rb, ops, ops_lo, lane);
+        rs.request(sm, rb, ops, ops_lo);
         ++rq;
         rs.seek(items, blocks, grids, ptiles, lane, true);
       }
@@ -891,31 +950,57 @@ __global__ void __launch_bounds__(ws::kThreads, 1)
       const MmaBlock& b = *q.blk;
       const Panel& pa = panels[b.a_panel];
       const Panel* pb = q.formed ? nullptr : panels + b.b_panel;
+      // the stored rows of the tiles, and their first chunk
+      const int ra = __shfl_sync(kFull, min(kM, pa.nrows - it.tm * kM), 0);
+      const int rbw = __shfl_sync(kFull, pb ? min(kTileN, pb->nrows - it.tn * kTileN) : 0, 0);
+      const uint8_t* pk_a = packed + __shfl_sync(kFull, pa.pack_off + (int64_t)it.tm * pa.nch * (kSlices * kM * kRowB), 0);
+      const uint8_t* pk_b = packed + __shfl_sync(kFull, pb ? pb->pack_off + (int64_t)it.tn * pb->nch * (kSlices * kTileN * kRowB) : 0, 0);
+      // The ring empties before another row count's layout, and before a packed B after formed ones (the
+      // B ring's phases are then known to be over up to this item's first chunk).
+      if (!ar.fits(ra) || (pb && was_formed)) {
+        bool ok = true;
+        for (int k = 0; k < kMaxStages && ok; ++k) ok = ws::wait_a_free(sm, ar, k, wait_ns);
+        run = __all_sync(kFull, ok);
+        if (!run) { ws::fail(sm, status, 4); break; }
+        if (!ar.fits(ra)) ar.layout(ra);
+      }
+      was_formed = !pb;
       for (int win = q.w0; win < q.w1 && run; ++win) {
         const int nck = ws::chunks_in(q, win);
         for (int j = 0; j < nck; ++j, ++c) {
           request_free();
-          const int s = ws::stage_of(c), sb = ws::bstage_of(c), ch = kChunksPerWin * win + j;
-          const bool ok = ws::wait_a_free(sm, c, wait_ns) && (!pb || ws::wait_b_free(sm, c, wait_ns));
+          const int s = ar.s, sb = ws::bstage_of(c), ch = kChunksPerWin * win + j;
+          const bool ok = ws::wait_a_free(sm, ar, s, wait_ns) && (!pb || ws::wait_b_free(sm, c, wait_ns));
           run = __all_sync(kFull, ok && !ws::aborted(sm));
           if (!run) { ws::fail(sm, status, 4); break; }
-          // the stored rows of the tiles, one bulk copy per plane (lanes 0-4: A, 5-9: B)
-          const int ra = min(kM, pa.nrows - it.tm * kM);
-          const int rbw = pb ? min(kTileN, pb->nrows - it.tn * kTileN) : 0;
-          if (lane == 0) ws::mbar_expect_tx(&sm.a_full[s], (uint32_t)(kSlices * kRowB * (ra + rbw)));
-          __syncwarp();
-          if (lane < kSlices) {
-            const uint8_t* src = packed + pa.pack_off + (int64_t)it.tm * pa.nch * (kSlices * kM * kRowB) +
-                                 (int64_t)ch * (kSlices * ra * kRowB) + (int64_t)lane * ra * kRowB;
-            ws::bulk_g2s(sm.a[s][lane], src, (uint32_t)(kRowB * ra), &sm.a_full[s]);
-          } else if (lane < 2 * kSlices && pb) {
-            const int k = lane - kSlices;
-            const uint8_t* src = packed + pb->pack_off + (int64_t)it.tn * pb->nch * (kSlices * kTileN * kRowB) +
-                                 (int64_t)ch * (kSlices * rbw * kRowB) + (int64_t)k * rbw * kRowB;
-            ws::bulk_g2s(sm.b[sb][k], src, (uint32_t)(kRowB * rbw), &sm.a_full[s]);
+          // one bulk copy, or one per plane, issued by one lane on uniform addresses
+          if (elect_one()) {
+            ws::mbar_expect_tx(&sm.a_full[s], (uint32_t)(kSlices * kRowB * (ra + rbw)));
+            const uint8_t* src = pk_a + (int64_t)ch * (kSlices * ra * kRowB);
+            uint8_t* dst = sm.a + ar.offset();
+            if (ar.plane == ra * kRowB) {  // whole groups of eight rows: the planes follow one another
+              ws::bulk_g2s(dst, src, (uint32_t)(kSlices * kRowB * ra), &sm.a_full[s]);
+            } else {
+#pragma unroll
+              for (int k = 0; k < kSlices; ++k)
+                ws::bulk_g2s(dst + k * ar.plane, src + k * (ra * kRowB), (uint32_t)(kRowB * ra), &sm.a_full[s]);
+            }
+            if (pb) {
+              const uint8_t* srcb = pk_b + (int64_t)ch * (kSlices * rbw * kRowB);
+              if (rbw == kTileN) {
+                ws::bulk_g2s(sm.b[sb][0], srcb, (uint32_t)(kSlices * kTileN * kRowB), &sm.a_full[s]);
+              } else {
+#pragma unroll
+                for (int k = 0; k < kSlices; ++k)
+                  ws::bulk_g2s(sm.b[sb][k], srcb + k * (rbw * kRowB), (uint32_t)(kRowB * rbw), &sm.a_full[s]);
+              }
+            }
           }
           __syncwarp();
-          last_a = (int)c;
+          ar.used |= 1u << s;
+          loads ^= 1u << s;
+          loaded |= 1u << s;
+          ar.next();
         }
       }
     }
@@ -930,8 +1015,8 @@ __global__ void __launch_bounds__(ws::kThreads, 1)
     // drain: nothing may still be copying into shared memory when the CTA exits (another
     // role may have given up after this loop ended; the phases waited for here are the last
     // ones issued on each barrier, complete at once when the copies were consumed)
-    for (int k = last_a; k >= 0 && k > last_a - kStages; --k)
-      ws::wait(&sm.a_full[ws::stage_of(k)], ws::round_of(k) & 1, nullptr, kWaitNs);
+    for (int k = 0; k < kMaxStages; ++k)
+      if ((loaded >> k) & 1u) ws::wait(&sm.a_full[k], ((loads >> k) & 1u) ^ 1u, nullptr, kWaitNs);
     for (int k = (int)rq - 1; k >= 0 && k > (int)rq - 3; --k)
       ws::wait(&sm.raw_full[k & 1], (k >> 1) & 1, nullptr, kWaitNs);
   } else if (warp < 4 || warp == 6 || warp == 7) {
@@ -966,39 +1051,41 @@ __global__ void __launch_bounds__(ws::kThreads, 1)
         bool ok = ws::wait(&sm.raw_full[rb], (rw >> 1) & 1, &sm.abort, wait_ns);
         run = __all_sync(kFull, ok && !ws::aborted(sm));
         if (!run) { ws::fail(sm, status, 5); break; }
-        const int64_t wleft = q.K - (int64_t)kWinPts * win;  // points of the window that exist
-        float vh[kChunksPerWin][8], vl[kChunksPerWin][8];
+        const int wleft = (int)(q.K - (int64_t)kWinPts * win);  // points of the window that exist
+        f2 vh[kChunksPerWin][4], vl[kChunksPerWin][4];  // products, hi words negated
         float mx = 0.0f;
 #pragma unroll
         for (int cc = 0; cc < kChunksPerWin; ++cc) {
           const int p0 = kChunk * cc + 8 * g;
-          const float* xh = sm.raw[rb][0][dx] + p0;
-          const float* xl = sm.raw[rb][1][dx] + p0;
-          const float* yh = sm.raw[rb][0][dy] + p0;
-          const float* yl = sm.raw[rb][1][dy] + p0;
-          const int64_t left = valid ? wleft - p0 : 0;
-          if (left >= 8) {
-            float a[8], al[8], bb[8], bl[8];
-            *reinterpret_cast<float4*>(a) = *reinterpret_cast<const float4*>(xh);
-            *reinterpret_cast<float4*>(a + 4) = *reinterpret_cast<const float4*>(xh + 4);
-            *reinterpret_cast<float4*>(al) = *reinterpret_cast<const float4*>(xl);
-            *reinterpret_cast<float4*>(al + 4) = *reinterpret_cast<const float4*>(xl + 4);
-            *reinterpret_cast<float4*>(bb) = *reinterpret_cast<const float4*>(yh);
-            *reinterpret_cast<float4*>(bb + 4) = *reinterpret_cast<const float4*>(yh + 4);
-            *reinterpret_cast<float4*>(bl) = *reinterpret_cast<const float4*>(yl);
-            *reinterpret_cast<float4*>(bl + 4) = *reinterpret_cast<const float4*>(yl + 4);
+          const ulonglong2* xh = reinterpret_cast<const ulonglong2*>(sm.raw[rb][0][dx] + p0);
+          const ulonglong2* xl = reinterpret_cast<const ulonglong2*>(sm.raw[rb][1][dx] + p0);
+          const ulonglong2* yh = reinterpret_cast<const ulonglong2*>(sm.raw[rb][0][dy] + p0);
+          const ulonglong2* yl = reinterpret_cast<const ulonglong2*>(sm.raw[rb][1][dy] + p0);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) prod_unnorm(a[i], al[i], bb[i], bl[i], vh[cc][i], vl[cc][i]);
-          } else {
+          for (int i = 0; i < 2; ++i) {
+            const ulonglong2 a = xh[i], al = xl[i], bb = yh[i], bl = yl[i];
+            prod_unnorm(f2{a.x}, f2{al.x}, f2{bb.x}, f2{bl.x}, vh[cc][2 * i], vl[cc][2 * i]);
+            prod_unnorm(f2{a.y}, f2{al.y}, f2{bb.y}, f2{bl.y}, vh[cc][2 * i + 1], vl[cc][2 * i + 1]);
+          }
+          const int left = valid ? wleft - p0 : 0;  // a short last window, or no such column: zeros
+          if (left < 8) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              vh[cc][i] = 0.0f;
-              vl[cc][i] = 0.0f;
-              if (i < left) prod_unnorm(xh[i], xl[i], yh[i], yl[i], vh[cc][i], vl[cc][i]);
+            for (int i = 0; i < 4; ++i) {
+              float h0, h1, l0, l1;
+              f2_unpack(vh[cc][i], h0, h1);
+              f2_unpack(vl[cc][i], l0, l1);
+              if (2 * i >= left) h0 = l0 = 0.0f;
+              if (2 * i + 1 >= left) h1 = l1 = 0.0f;
+              vh[cc][i] = f2_pack(h0, h1);
+              vl[cc][i] = f2_pack(l0, l1);
             }
           }
 #pragma unroll
-          for (int i = 0; i < 8; ++i) mx = fmaxf(mx, fabsf(vh[cc][i]));
+          for (int i = 0; i < 4; ++i) {
+            float h0, h1;
+            f2_unpack(vh[cc][i], h0, h1);
+            mx = fmaxf(mx, fmaxf(fabsf(h0), fabsf(h1)));
+          }
         }
         // the staged rows are read: release the buffer for the window after next
         __syncwarp();
@@ -1025,7 +1112,7 @@ __global__ void __launch_bounds__(ws::kThreads, 1)
               ws::fail(sm, status, 5);
             } else {
               uint4 wv[kSlices];
-              slice8_df<1>(vh[cc], vl[cc], sc, scj, wv);
+              slice8_f2<1>(vh[cc], vl[cc], -sc, scj, wv);
 #pragma unroll
               for (int k = 0; k < kSlices; ++k) *reinterpret_cast<uint4*>(sm.b[sb][k] + swz(col, g)) = wv[k];
               fence_async_smem();
@@ -1040,49 +1127,56 @@ __global__ void __launch_bounds__(ws::kThreads, 1)
     }
   } else if (warp == ws::kMmaWarp) {
     // ------------------------------------------------------------------ MMA issue
-    if (lane == 0) {
-      for (int ii = cta_begin[blockIdx.x], ie = cta_begin[blockIdx.x + 1]; ii < ie && !ws::aborted(sm); ++ii) {
-        const GemmItem it = items[ii];
-        const ws::Geo q = ws::geo(it, blocks, grids, ptiles);
-        bool ok = true;
-        for (int win = q.w0; win < q.w1 && ok; ++win, ++w) {
-          const int nck = ws::chunks_in(q, win);
-          const int set = w & 1;
-          if (w >= 2) ok = ws::wait(&sm.tmem_free[set], ((w - 2) >> 1) & 1, &sm.abort, wait_ns);
-          const uint32_t tset = tmem + (uint32_t)set * 256u;
-          for (int j = 0; j < nck && ok; ++j, ++c) {
-            const int s = ws::stage_of(c), sb = ws::bstage_of(c);
-            ok = ws::wait(&sm.a_full[s], ws::round_of(c) & 1, &sm.abort, wait_ns);
-            if (ok) ok = ws::wait(&sm.b_ready[sb], ws::bround_of(c) & 1, &sm.abort, wait_ns);
-            if (!ok) break;
-            fence_after();
-            // The B planes of a stage are contiguous (48 rows each), so plane i of A against
-            // planes 0..4-i of B is one MMA of N = 48 (5 - i) whose columns land on the order
-            // accumulators i..4 (order k at TMEM columns 48k..48k+47 of the set).
+    // The whole warp runs the loop on warp-uniform values and one lane issues: issued from a divergent
+    // branch, an MMA took about 90 cycles to issue, more than the smaller ones of a K step run.
+    bool ok = true;
+    ws::ARing ar;
+    ar.open();
+    for (int ii = cta_begin[blockIdx.x], ie = cta_begin[blockIdx.x + 1]; ii < ie && ok; ++ii) {
+      const GemmItem it = items[ii];
+      const ws::Geo q = ws::geo(it, blocks, grids, ptiles);
+      const int ra = __shfl_sync(kFull, min(kM, panels[q.blk->a_panel].nrows - it.tm * kM), 0);
+      if (!ar.fits(ra)) ar.layout(ra);
+      const int w0 = __shfl_sync(kFull, q.w0, 0), w1 = __shfl_sync(kFull, q.w1, 0), nch = __shfl_sync(kFull, q.nch, 0);
+      for (int win = w0; win < w1 && ok; ++win, ++w) {
+        const int nck = min(kChunksPerWin, nch - kChunksPerWin * win);
+        const int set = w & 1;
+        if (w >= 2) ok = ws::wait(&sm.tmem_free[set], ((w - 2) >> 1) & 1, &sm.abort, wait_ns);
+        const uint32_t tset = tmem + (uint32_t)set * 256u;
+        for (int j = 0; j < nck && ok; ++j, ++c) {
+          const uint32_t s = ar.s, sb = c % kStagesB;
+          ok = ws::wait(&sm.a_full[s], (ar.par >> s) & 1u, &sm.abort, wait_ns) &&
+               ws::wait(&sm.b_ready[sb], ws::bround_of(c) & 1, &sm.abort, wait_ns);
+          ok = __all_sync(kFull, ok);
+          if (!ok) break;
+          fence_after();
+          // The B planes of a stage are contiguous (48 rows each), so plane i of A against
+          // planes 0..4-i of B is one MMA of N = 48 (5 - i) whose columns land on the order
+          // accumulators i..4 (order k at TMEM columns 48k..48k+47 of the set).
+          const uint32_t da = desc_lo(smem_u32(sm.a)) + (ar.offset() >> 4), dp = (uint32_t)ar.plane >> 4;
+          const uint32_t db = desc_lo(smem_u32(sm.b[0][0])) + sb * (uint32_t)(sizeof(sm.b[0]) >> 4);
+          if (elect_one()) {
 #pragma unroll
-            for (int k = 0; k < kChunk / 16; ++k) {
-              const uint32_t ko = 32u * k;
-              const uint64_t db = make_desc(smem_u32(sm.b[sb][0]) + ko);
+            for (int k = 0; k < kChunk / 16; ++k)
 #pragma unroll
-              for (int i = 0; i < kSlices; ++i) {
-                const uint64_t da = make_desc(smem_u32(sm.a[s][i]) + ko);
-                mma_f16(tset + (uint32_t)(kTileN * i), da, db, make_idesc(kTileN * (kSlices - i)),
-                         (j > 0 || k > 0 || i > 0) ? 1u : 0u);
-              }
-            }
+              for (int i = 0; i < kSlices; ++i)
+                mma_f16_lo(tset + (uint32_t)(kTileN * i), da + i * dp + 2u * k, db + 2u * k,
+                           make_idesc(kTileN * (kSlices - i)), (j > 0 || k > 0 || i > 0) ? 1u : 0u);
             mma_commit(smem_u32(&sm.a_free[s]));
             mma_commit(smem_u32(&sm.b_free[sb]));
+            if (j + 1 == nck) mma_commit(smem_u32(&sm.tmem_full[set]));
           }
-          if (!ok) { ws::fail(sm, status, 6); break; }
-          mma_commit(smem_u32(&sm.tmem_full[set]));
+          __syncwarp();
+          ar.par ^= 1u << s;
+          ar.next();
         }
-        if (!ok) break;
       }
-      // drain: every issued MMA must be complete before the TMEM is released (also when
-      // another role gave up after this loop ended)
-      mma_commit(smem_u32(&sm.drain));
-      ws::wait(&sm.drain, 0, nullptr, kWaitNs);
     }
+    if (!ok) ws::fail(sm, status, 6);
+    // drain: every issued MMA must be complete before the TMEM is released (also when
+    // another role gave up after this loop ended)
+    if (elect_one()) mma_commit(smem_u32(&sm.drain));
+    ws::wait(&sm.drain, 0, nullptr, kWaitNs);
     __syncwarp();
   } else if (warp >= ws::kFoldWarp0) {
     // ------------------------------------------------------------------ fold
@@ -1099,9 +1193,9 @@ __global__ void __launch_bounds__(ws::kThreads, 1)
       const Panel& pa = panels[b.a_panel];
       const Panel* pb = q.formed ? nullptr : panels + b.b_panel;
       const int rows_valid = min(kM, b.m - it.tm * kM);  // real rows of the A tile
-      float H[24], L[24];
+      f2 H[12], L[12];  // pairs of columns
 #pragma unroll
-      for (int j = 0; j < 24; ++j) { H[j] = 0.0f; L[j] = 0.0f; }
+      for (int j = 0; j < 12; ++j) H[j] = L[j] = f2_both(0.0f);
       // the window's exponents (A rows from the packed panel; B columns from the packed panel,
       // one per lane for this warp's 24 columns, or from the producers), loaded one window ahead
       const int* ea_src = reinterpret_cast<const int*>(packed + pa.exp_off) + (int64_t)it.tm * pa.nwin * kM + row_in_tile;
@@ -1140,26 +1234,27 @@ __global__ void __launch_bounds__(ws::kThreads, 1)
               for (int k = 0; k < kSlices; ++k) tmem_ld8(lane_base + (uint32_t)(kTileN * k + c0), o[k]);
               tmem_wait_ld();
 #pragma unroll
-              for (int j = 0; j < 8; ++j) {
-                const int qq = 8 * gi + j;
-                const float sc = sa * sbw[c0 + j];  // 2^(e_a + e_b - 30)
-                // Order 1 splits exactly into q1, its nearest multiple of 2^24 (adding 1.5 x 2^47
-                // rounds at that spacing), and r1 = o1 - q1; q1 / 256 joins order 0 exactly
-                // (both multiples of 2^16 below 2^38).  That part, times the power of two sc,
-                // enters the double-float sum through one TwoSum; r1 / 256 and orders 2-4 (at
-                // most 2^-15 of order 0) join the lo word as one FP32 term, rounded at 2^-16 of
-                // order 0's unit (2^-37 of the window's largest possible sum).
-                const float q1 = __fsub_rn(__fadd_rn(o[1][j], 211106232532992.0f), 211106232532992.0f);
-                const float r1 = __fsub_rn(o[1][j], q1);
-                const df s0 = dfa::two_sum(H[qq], __fmaf_rn(q1, 0.00390625f, o[0][j]) * sc);
-                const float tail =
-                    fmaf(r1, 0.00390625f,
-                         fmaf(o[2][j], 1.52587890625e-5f, fmaf(o[4][j], 2.3283064365386963e-10f, o[3][j] * 5.9604644775390625e-8f))) *
-                    sc;
-                const float lo = L[qq] + (s0.l + tail);
-                const df r = dfa::fast_two_sum(s0.h, lo);
-                H[qq] = r.h;
-                L[qq] = r.l;
+              for (int j = 0; j < 4; ++j) {
+                f2 &h = H[4 * gi + j], &lo = L[4 * gi + j];
+                const f2 sc = f2_mul(f2_both(sa), *reinterpret_cast<const f2*>(sbw + c0 + 2 * j));  // 2^(e_a + e_b - 30)
+                const f2 o0 = f2_pack(o[0][2 * j], o[0][2 * j + 1]), o1 = f2_pack(o[1][2 * j], o[1][2 * j + 1]),
+                         o2 = f2_pack(o[2][2 * j], o[2][2 * j + 1]), o3 = f2_pack(o[3][2 * j], o[3][2 * j + 1]),
+                         o4 = f2_pack(o[4][2 * j], o[4][2 * j + 1]);
+                // Orders 0 and 1 as a sum t and its exact error e (Dekker's Fast2Sum on the FMA; the
+                // orders are multiples of 2^16 below 2^40, so o0 - t is exact also where o0 is the
+                // smaller); t, times the power of two sc, enters the double-float sum through one
+                // TwoSum; e and orders 2-4 (at most 2^-15 of order 0) join the lo word as one FP32
+                // term, rounded at 2^-16 of order 0's unit (2^-37 of the window's largest sum).
+                const f2 c8 = f2_both(0.00390625f);
+                const f2 t = f2_fma(o1, c8, o0);
+                const f2 e = f2_fma(o1, c8, f2_rsub(t, o0));
+                const f2 tail = f2_fma(f2_fma(f2_fma(o4, c8, o3), c8, o2), f2_both(1.52587890625e-5f), e);
+                const f2 p = f2_mul(t, sc);
+                const f2 s = f2_add(h, p), bb = f2_rsub(h, s);
+                const f2 er = f2_add(f2_rsub(f2_rsub(bb, s), h), f2_rsub(bb, p));
+                const f2 l2 = f2_add(lo, f2_fma(tail, sc, er));
+                h = f2_add(s, l2);
+                lo = f2_rsub(f2_rsub(s, h), l2);
               }
             }
           }
@@ -1174,11 +1269,17 @@ __global__ void __launch_bounds__(ws::kThreads, 1)
       if (grow < b.m) {
         float2* out = part + b.part_off + (int64_t)it.chunk * b.m * b.n + (int64_t)grow * b.n;
 #pragma unroll
-        for (int j = 0; j < 24; ++j) {
-          const int cc = 24 * half + j;
-          if (cc < q.nt) {
-            const int ocol = q.formed ? q.pt->col[cc] : it.tn * kTileN + cc;
-            out[ocol] = make_float2(H[j], L[j]);
+        for (int j = 0; j < 12; ++j) {
+          float h[2], l[2];
+          f2_unpack(H[j], h[0], h[1]);
+          f2_unpack(L[j], l[0], l[1]);
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            const int cc = 24 * half + 2 * j + k;
+            if (cc < q.nt) {
+              const int ocol = q.formed ? q.pt->col[cc] : it.tn * kTileN + cc;
+              out[ocol] = make_float2(h[k], l[k]);
+            }
           }
         }
       }

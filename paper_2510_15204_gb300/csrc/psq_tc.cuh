@@ -23,6 +23,21 @@ __device__ __forceinline__ uint64_t make_desc(uint32_t saddr) {
   return d;
 }
 
+// Low word of make_desc (the high word is the constant kDescHi): bytes further on in shared memory
+// add bytes / 16.
+constexpr uint32_t kDescHi = (512u >> 4) | (1u << 14) | (4u << 29);
+__device__ __forceinline__ uint32_t desc_lo(uint32_t saddr) { return ((saddr & 0x3FFFF) >> 4) | (1u << 16); }
+
+// One MMA of kind::f16 on descriptors given by their low words.
+__device__ __forceinline__ void mma_f16_lo(uint32_t tmem_d, uint32_t da, uint32_t db, uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "mov.b64 a, {%1, %5};\n\tmov.b64 b, {%2, %5};\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n\t}\n" ::"r"(tmem_d),
+      "r"(da), "r"(db), "r"(idesc), "r"(acc), "n"(kDescHi));
+}
+
 // One MMA of kind::f16 (the operand type is the instruction descriptor's: F16 or BF16).
 __device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
   asm volatile(
@@ -30,6 +45,14 @@ __device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint64_t da, uint64_t d
       "setp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem_d),
       "l"(da), "l"(db), "r"(idesc), "r"(acc));
+}
+
+// True in one lane of a converged warp.  The issuing code stays warp-uniform up to this branch, so that
+// descriptors and addresses live in uniform registers.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\tselp.u32 %0, 1, 0, e;\n\t}\n" : "=r"(p));
+  return p != 0;
 }
 
 __device__ __forceinline__ void mma_commit(uint32_t mbar) {
