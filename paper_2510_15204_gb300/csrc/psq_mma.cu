@@ -449,15 +449,14 @@ __device__ __forceinline__ void window_scales(int e, float& sc, float& scj) {
   scj = e == kZeroExp ? 0.0f : pow2f(7 - e + 8 * (JOIN + 1));
 }
 
-// The planes of eight consecutive points (a 16-byte group) given as four pairs; the values are sgn vh
-// + vl (sgn: the sign the hi words' scale sc carries).
-template <int JOIN>
-__device__ __forceinline__ void slice8_f2(const f2 (&vh)[4], const f2 (&vl)[4], float sc, float scj, uint4 (&w)[kSlices]) {
-  uint32_t o[kSlices][4];
+// The planes of 2 NP consecutive points (NP = 4: a 16-byte group) given as pairs, NP words each; the
+// values are sgn vh + vl (sgn: the sign the hi words' scale sc carries).
+template <int JOIN, int NP>
+__device__ __forceinline__ void slice_f2(const f2 (&vh)[NP], const f2 (&vl)[NP], float sc, float scj, uint32_t (&o)[kSlices][NP]) {
   const f2 s0 = f2_both(sc), s256 = f2_both(sc * 256.0f), sj = f2_both(scj);  // |sc 256| at most 2^125
   const f2 magic = f2_both(kRneMagic), magic256 = f2_both(kRneMagic256), m256 = f2_both(-256.0f), p256 = f2_both(256.0f);
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
+  for (int q = 0; q < NP; ++q) {
     f2 r{};
     const f2 l = f2_mul(vl[q], sj);
 #pragma unroll
@@ -474,8 +473,6 @@ __device__ __forceinline__ void slice8_f2(const f2 (&vh)[4], const f2 (&vl)[4], 
       }
     }
   }
-#pragma unroll
-  for (int k = 0; k < kSlices; ++k) w[k] = make_uint4(o[k][0], o[k][1], o[k][2], o[k][3]);
 }
 
 // Exponent e with mx < 2^e <= 2 mx (frexp's), read from the exponent bits, or kZeroExp for
@@ -559,10 +556,11 @@ __device__ __forceinline__ void pack_store(const PackPos& P, const Panel& pn, co
   const int plane = rt * kRowB;
 #pragma unroll
   for (int j = 0; j < 2; ++j) {
-    uint4 wv[kSlices];
-    slice8_f2<1>(h[j], l[j], sgn * sc, scj, wv);
+    uint32_t wv[kSlices][4];
+    slice_f2<1, 4>(h[j], l[j], sgn * sc, scj, wv);
 #pragma unroll
-    for (int k = 0; k < kSlices; ++k) *reinterpret_cast<uint4*>(dst + k * plane + swz(P.r, 2 * (P.qq & 1) + j)) = wv[k];
+    for (int k = 0; k < kSlices; ++k)
+      *reinterpret_cast<uint4*>(dst + k * plane + swz(P.r, 2 * (P.qq & 1) + j)) = make_uint4(wv[k][0], wv[k][1], wv[k][2], wv[k][3]);
   }
 }
 
@@ -1021,10 +1019,13 @@ __global__ void __launch_bounds__(ws::kThreads, 1)
       ws::wait(&sm.raw_full[k & 1], (k >> 1) & 1, nullptr, kWaitNs);
   } else if (warp < 4 || warp == 6 || warp == 7) {
     // ------------------------------------------------------------------ producers
+    // A lane forms columns col[0] and col[1], which mostly share their first row (the pairs of a tile
+    // are listed row by row), four points of each per chunk: its eight lanes read 128 contiguous bytes
+    // of a row, and the shared row once.
     const int pw = warp < 4 ? warp : warp - 2;  // 0..5
-    const int col = 8 * pw + (lane >> 2);       // 0..47: this lane's column of the tile
-    const int g = lane & 3;                     // 16-byte group of each chunk's row
-    const unsigned col_mask = 0xfu << (lane & 28);
+    const int col[2] = {8 * pw + (lane >> 3), 8 * pw + 4 + (lane >> 3)};
+    const int g = lane & 7;                     // points [4 g, 4 g + 4) of each chunk
+    const unsigned col_mask = 0xffu << (lane & 24);
     bool run = true;  // warp-uniform
     for (int ii = cta_begin[blockIdx.x], ie = cta_begin[blockIdx.x + 1]; ii < ie && run; ++ii) {
       const GemmItem it = items[ii];
@@ -1043,8 +1044,14 @@ __global__ void __launch_bounds__(ws::kThreads, 1)
         }
         continue;
       }
-      const bool valid = col < q.nt;
-      const int dx = valid ? q.pt->dx[col] : 0, dy = valid ? q.pt->dy[col] : 0;
+      int dx[2], dy[2];
+      bool valid[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        valid[u] = col[u] < q.nt;
+        dx[u] = valid[u] ? q.pt->dx[col[u]] : 0;
+        dy[u] = valid[u] ? q.pt->dy[col[u]] : 0;
+      }
       for (int win = q.w0; win < q.w1 && run; ++win, ++w, ++rw) {
         const int nck = ws::chunks_in(q, win);
         const int rb = rw & 1, set = w & 1;
@@ -1052,56 +1059,66 @@ __global__ void __launch_bounds__(ws::kThreads, 1)
         run = __all_sync(kFull, ok && !ws::aborted(sm));
         if (!run) { ws::fail(sm, status, 5); break; }
         const int wleft = (int)(q.K - (int64_t)kWinPts * win);  // points of the window that exist
-        f2 vh[kChunksPerWin][4], vl[kChunksPerWin][4];  // products, hi words negated
-        float mx = 0.0f;
+        f2 vh[kChunksPerWin][2][2], vl[kChunksPerWin][2][2];  // products, hi words negated
+        float mx[2] = {0.0f, 0.0f};
 #pragma unroll
         for (int cc = 0; cc < kChunksPerWin; ++cc) {
-          const int p0 = kChunk * cc + 8 * g;
-          const ulonglong2* xh = reinterpret_cast<const ulonglong2*>(sm.raw[rb][0][dx] + p0);
-          const ulonglong2* xl = reinterpret_cast<const ulonglong2*>(sm.raw[rb][1][dx] + p0);
-          const ulonglong2* yh = reinterpret_cast<const ulonglong2*>(sm.raw[rb][0][dy] + p0);
-          const ulonglong2* yl = reinterpret_cast<const ulonglong2*>(sm.raw[rb][1][dy] + p0);
+          const int p0 = kChunk * cc + 4 * g;
+          ulonglong2 a = *reinterpret_cast<const ulonglong2*>(sm.raw[rb][0][dx[0]] + p0);
+          ulonglong2 al = *reinterpret_cast<const ulonglong2*>(sm.raw[rb][1][dx[0]] + p0);
 #pragma unroll
-          for (int i = 0; i < 2; ++i) {
-            const ulonglong2 a = xh[i], al = xl[i], bb = yh[i], bl = yl[i];
-            prod_unnorm(f2{a.x}, f2{al.x}, f2{bb.x}, f2{bl.x}, vh[cc][2 * i], vl[cc][2 * i]);
-            prod_unnorm(f2{a.y}, f2{al.y}, f2{bb.y}, f2{bl.y}, vh[cc][2 * i + 1], vl[cc][2 * i + 1]);
-          }
-          const int left = valid ? wleft - p0 : 0;  // a short last window, or no such column: zeros
-          if (left < 8) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              float h0, h1, l0, l1;
-              f2_unpack(vh[cc][i], h0, h1);
-              f2_unpack(vl[cc][i], l0, l1);
-              if (2 * i >= left) h0 = l0 = 0.0f;
-              if (2 * i + 1 >= left) h1 = l1 = 0.0f;
-              vh[cc][i] = f2_pack(h0, h1);
-              vl[cc][i] = f2_pack(l0, l1);
+          for (int u = 0; u < 2; ++u) {
+            if (u == 1 && dx[1] != dx[0]) {
+              a = *reinterpret_cast<const ulonglong2*>(sm.raw[rb][0][dx[1]] + p0);
+              al = *reinterpret_cast<const ulonglong2*>(sm.raw[rb][1][dx[1]] + p0);
             }
-          }
+            const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(sm.raw[rb][0][dy[u]] + p0);
+            const ulonglong2 bl = *reinterpret_cast<const ulonglong2*>(sm.raw[rb][1][dy[u]] + p0);
+            prod_unnorm(f2{a.x}, f2{al.x}, f2{b.x}, f2{bl.x}, vh[cc][u][0], vl[cc][u][0]);
+            prod_unnorm(f2{a.y}, f2{al.y}, f2{b.y}, f2{bl.y}, vh[cc][u][1], vl[cc][u][1]);
+            const int left = valid[u] ? wleft - p0 : 0;  // a short last window, or no such column: zeros
+            if (left < 4) {
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            float h0, h1;
-            f2_unpack(vh[cc][i], h0, h1);
-            mx = fmaxf(mx, fmaxf(fabsf(h0), fabsf(h1)));
+              for (int i = 0; i < 2; ++i) {
+                float h0, h1, l0, l1;
+                f2_unpack(vh[cc][u][i], h0, h1);
+                f2_unpack(vl[cc][u][i], l0, l1);
+                if (2 * i >= left) h0 = l0 = 0.0f;
+                if (2 * i + 1 >= left) h1 = l1 = 0.0f;
+                vh[cc][u][i] = f2_pack(h0, h1);
+                vl[cc][u][i] = f2_pack(l0, l1);
+              }
+            }
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+              float h0, h1;
+              f2_unpack(vh[cc][u][i], h0, h1);
+              mx[u] = fmaxf(mx[u], fmaxf(fabsf(h0), fabsf(h1)));
+            }
           }
         }
         // the staged rows are read: release the buffer for the window after next
         __syncwarp();
         if (lane == 0) ws::mbar_arrive(&sm.raw_free[rb]);
-        // the column's window maximum over its four lanes
-        mx = fmaxf(mx, __shfl_xor_sync(col_mask, mx, 1));
-        mx = fmaxf(mx, __shfl_xor_sync(col_mask, mx, 2));
-        const int e = row_exponent(mx);
+        // the columns' window maxima over their eight lanes
+        int e[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+#pragma unroll
+          for (int o = 1; o < 8; o <<= 1) mx[u] = fmaxf(mx[u], __shfl_xor_sync(col_mask, mx[u], o));
+          e[u] = row_exponent(mx[u]);
+        }
         // the column exponents of this set were last read by the fold of window w - 2, which
         // releases them (eb_free) as soon as it has copied them: the fold stays off this path
         const bool okb = w < 2 || ws::wait(&sm.eb_free[set], ((w - 2) >> 1) & 1, &sm.abort, wait_ns);
         run = __all_sync(kFull, okb && !ws::aborted(sm));
         if (!run) { ws::fail(sm, status, 5); break; }
-        if (g == 0) sm.eb[set][col] = e;
-        float sc, scj;
-        window_scales<1>(e, sc, scj);
+        float sc[2], scj[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          if (g == 0) sm.eb[set][col[u]] = e[u];
+          window_scales<1>(e[u], sc[u], scj[u]);
+        }
 #pragma unroll
         for (int cc = 0; cc < kChunksPerWin; ++cc) {
           if (cc < nck && run) {
@@ -1111,10 +1128,14 @@ __global__ void __launch_bounds__(ws::kThreads, 1)
             if (!run) {
               ws::fail(sm, status, 5);
             } else {
-              uint4 wv[kSlices];
-              slice8_f2<1>(vh[cc], vl[cc], -sc, scj, wv);
 #pragma unroll
-              for (int k = 0; k < kSlices; ++k) *reinterpret_cast<uint4*>(sm.b[sb][k] + swz(col, g)) = wv[k];
+              for (int u = 0; u < 2; ++u) {
+                uint32_t wv[kSlices][2];
+                slice_f2<1, 2>(vh[cc][u], vl[cc][u], -sc[u], scj[u], wv);
+#pragma unroll
+                for (int k = 0; k < kSlices; ++k)
+                  *reinterpret_cast<uint2*>(sm.b[sb][k] + swz(col[u], g >> 1) + 8 * (g & 1)) = make_uint2(wv[k][0], wv[k][1]);
+              }
               fence_async_smem();
               __syncwarp();
               if (lane == 0) ws::mbar_arrive(&sm.b_ready[sb]);
