@@ -20,56 +20,108 @@ namespace {
 
 constexpr int kB = 32;  // block size of the factor and the solve
 
-// Factor of the kb x kb diagonal block at (k0, k0), in place in shared memory (one CTA of
-// 32 x 32 threads).  A pivot that is not positive records info = k0 + j + 1 (the first one
-// wins) and continues with 1 so that nothing divides by zero.
-__global__ void __launch_bounds__(1024) chol_diag_kernel(int n, int k0, int kb, double* __restrict__ L,
-                                                         int* __restrict__ info) {
-  __shared__ double a[kB][kB + 1];
-  const int r = threadIdx.x >> 5, c = threadIdx.x & 31;
-  if (r < kb && c <= r) a[r][c] = L[(int64_t)(k0 + r) * n + k0 + c];
-  __syncthreads();
-  for (int j = 0; j < kb; ++j) {
-    if (threadIdx.x == 0) {
-      double d = a[j][j];
-      if (!(d > 0.0)) {
-        atomicCAS(info, 0, k0 + j + 1);
-        d = 1.0;
-      }
-      a[j][j] = sqrt(d);
-    }
-    __syncthreads();
-    if (c == j && r > j && r < kb) a[r][j] /= a[j][j];
-    __syncthreads();
-    if (r > j && r < kb && c > j && c <= r) a[r][c] -= a[r][j] * a[c][j];
-    __syncthreads();
-  }
-  if (r < kb && c <= r) L[(int64_t)(k0 + r) * n + k0 + c] = a[r][c];
+// 1/sqrt(d), d > 0: one step of Halley's third-order iteration from the hardware's approximation (about
+// 22 bits).  A pivot's root heads a serial chain, and an FP64 operation takes 64 cycles here, dependent
+// or not: five of them, where sqrt and a division take 675 and 354 cycles.
+__device__ __forceinline__ double rsqrt_fast(double d) {
+  const int hi = __double2hiint(d);
+  if (hi < 0x03d00000 || hi > 0x7c200000) return 1.0 / sqrt(d);  // near the ends of the range
+  double r;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+  const double h = fma(-d * r, r, 1.0);
+  return fma(fma(0.375, h, 0.5), r * h, r);
 }
 
-// Panel below the diagonal block: row i >= k0 + kb gets x with x D^T = a (D the factored
-// diagonal block), one thread per row.
-__global__ void __launch_bounds__(128) chol_panel_kernel(int n, int k0, int kb, double* __restrict__ L) {
-  __shared__ double d[kB][kB + 1];
-  for (int t = threadIdx.x; t < kB * kB; t += blockDim.x) {
-    const int r = t >> 5, c = t & 31;
-    d[r][c] = (r < kb && c <= r) ? L[(int64_t)(k0 + r) * n + k0 + c] : 0.0;
+// One block column: the kb x kb diagonal block at (k0, k0) and the panel below it, a CTA per 32 rows.
+// Four lanes share a row (lane q its columns 4 i + q): one warp's FP64 instruction occupies its quarter
+// of the SM for 64 cycles, so the work is spread over four warps.  Every CTA factors the diagonal block
+// for itself from the lower triangle, which none of them may write in this launch: the first one parks
+// the factor in the matrix's free upper triangle (below the diagonal transposed, the diagonal in the
+// column after the block) until finish_factor_kernel.  Then a CTA's rows: row i gets x with x D^T = a, each x_j applied to
+// the rest of the row at once (no chain but x_0, x_1, ...).  Past kb the block is the identity.  A pivot
+// that is not positive records info = k0 + j + 1 (the first one wins) and continues with 1 so that
+// nothing divides by zero.
+// Measured with the update below: n = 693 from 2.55 ms (three launches per block column, roots and
+// divisions by one thread between barriers) to 1.10, n = 82 from 266 us to 129.
+__global__ void __launch_bounds__(128) chol_panel_kernel(int n, int k0, int kb, double* __restrict__ L, int* __restrict__ info) {
+  __shared__ double d[kB][kB + 1];  // column-wise: d[j][i] = D[i][j]
+  __shared__ double piv[2], inv[kB];  // reciprocal pivots
+  const int tid = threadIdx.x, row = tid >> 2, q = tid & 3, lane = tid & 31;
+  const int i0 = k0 + kb + (blockIdx.x - 1) * kB;  // block 0: the diagonal block alone
+  double a[kB / 4];                                // columns 4 i + q of this row
+#pragma unroll
+  for (int i = 0; i < kB / 4; ++i) {
+    const int c = 4 * i + q;
+    a[i] = row < kb && c < kb ? (c <= row ? L[(int64_t)(k0 + row) * n + k0 + c] : 0.0) : (c == row ? 1.0 : 0.0);
+  }
+  // column j = 4 jj + qq: jj unrolled (registers), qq rolled (code that runs once is bound by its fetch)
+#pragma unroll
+  for (int jj = 0; jj < kB / 4; ++jj)
+#pragma unroll 1
+    for (int qq = 0; qq < 4; ++qq) {
+      const int j = 4 * jj + qq;
+      if (row == j && q == qq) piv[qq & 1] = a[jj];
+      __syncthreads();
+      double p = piv[qq & 1];
+      const int hi = __double2hiint(p);
+      if (hi < 0 || hi >= 0x7ff00000 || (hi == 0 && __double2loint(p) == 0)) {  // not positive, or not a number
+        if (blockIdx.x == 0 && tid == 0 && !(p > 0.0)) atomicCAS(info, 0, k0 + j + 1);
+        if (!(p > 0.0)) p = 1.0;
+      }
+      const double y = rsqrt_fast(p);
+      if (q == qq) {
+        // the diagonal entry keeps the pivot itself for now (its root: below, all at once)
+        a[jj] = row > j ? a[jj] * y : (row == j ? p : 0.0);
+        d[j][row] = a[jj];
+      }
+      if (tid == 0) inv[j] = y;
+      __syncthreads();
+      const double l = -d[j][row];
+#pragma unroll
+      for (int i = jj; i < kB / 4; ++i)
+        if (i > jj || q > qq) a[i] = fma(l, d[j][4 * i + q], a[i]);
+    }
+  __syncthreads();
+  if (tid < kB) {  // the diagonal: sqrt(p) = p y, corrected by its residual
+    const double p = d[tid][tid], y = inv[tid], r = p * y;
+    const double t = fma(fma(-r, r, p), 0.5 * y, r);
+    d[tid][tid] = (__double2hiint(t) & 0x7ff00000) == 0x7ff00000 ? sqrt(p) : t;
   }
   __syncthreads();
-  const int i = k0 + kb + blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  double* row = L + (int64_t)i * n + k0;
-  double x[kB];
+  if (blockIdx.x == 0) {
 #pragma unroll
-  for (int j = 0; j < kB; ++j) {
-    if (j < kb) {
-      double s = row[j];
-#pragma unroll
-      for (int m = 0; m < j; ++m) s -= x[m] * d[j][m];
-      x[j] = s / d[j][j];
-      row[j] = x[j];
-    }
+    for (int i = 0; i < kB / 4; ++i)
+      if (const int c = 4 * i + q; row < kb && c <= row) {
+        const int r0 = k0 + row, c0 = k0 + c;
+        if (k0 + kb == n)  // the last block: no other CTA
+          L[(int64_t)r0 * n + c0] = c == row ? d[row][row] : a[i];
+        else if (c == row)
+          L[(int64_t)r0 * n + k0 + kB] = d[row][row];
+        else
+          L[(int64_t)c0 * n + r0] = a[i];
+      }
+    return;
   }
+#pragma unroll
+  for (int i = 0; i < kB / 4; ++i) a[i] = i0 + row < n && 4 * i + q < kb ? L[(int64_t)(i0 + row) * n + k0 + 4 * i + q] : 0.0;
+#pragma unroll
+  for (int jj = 0; jj < kB / 4; ++jj)
+#pragma unroll 1
+    for (int qq = 0; qq < 4; ++qq) {
+      const int j = 4 * jj + qq;
+      // a / d by the reciprocal and one correction of the quotient, in the column's lane
+      const double q0 = a[jj] * inv[j];
+      double x = fma(fma(-q0, d[j][j], a[jj]), inv[j], q0);
+      if ((__double2hiint(x) & 0x7ff00000) == 0x7ff00000) x = q0;  // an infinite pivot or quotient: no residual
+      x = __shfl_sync(0xffffffffu, x, (lane & ~3) | qq);
+      if (q == qq) a[jj] = x;
+#pragma unroll
+      for (int i = jj; i < kB / 4; ++i)
+        if (i > jj || q > qq) a[i] = fma(-x, d[j][4 * i + q], a[i]);
+    }
+#pragma unroll
+  for (int i = 0; i < kB / 4; ++i)
+    if (i0 + row < n && 4 * i + q < kb) L[(int64_t)(i0 + row) * n + k0 + 4 * i + q] = a[i];
 }
 
 // Trailing update L[i][j] -= sum_m L[i][k0+m] L[j][k0+m] for k1 = k0 + kb <= j <= i < n, one
@@ -104,11 +156,19 @@ __global__ void __launch_bounds__(256) chol_update_kernel(int n, int k0, int kb,
   }
 }
 
-__global__ void zero_upper_kernel(int n, double* __restrict__ L) {
+// The diagonal blocks' factors from where chol_panel_kernel parked them; zeros above the diagonal.  The
+// thread of a parked entry's lower element moves it, so that no other reads what it clears.
+__global__ void finish_factor_kernel(int n, double* __restrict__ L) {
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (int64_t)n * n) return;
-  const int i = (int)(idx / n), j = (int)(idx % n);
-  if (j > i) L[idx] = 0.0;
+  const int i = (int)(idx / n), j = (int)(idx % n), k1 = (i / kB + 1) * kB;  // the column after i's block
+  if (j > i) {
+    if (j > k1 || k1 >= n) L[idx] = 0.0;
+  } else if (j / kB == i / kB && k1 < n) {
+    const int64_t from = i == j ? (int64_t)i * n + k1 : (int64_t)j * n + i;
+    L[idx] = L[from];
+    L[from] = 0.0;
+  }
 }
 
 // Forward substitution B <- L^-1 B, left-looking, one launch: a CTA owns up to 128 columns and
@@ -379,16 +439,12 @@ extern "C" psq_status psq_ri_factor(int n, const double* d_J2, double* d_L, int*
     return launched();
   for (int k0 = 0; k0 < n; k0 += kB) {
     const int kb = n - k0 < kB ? n - k0 : kB;
-    chol_diag_kernel<<<1, 1024, 0, s>>>(n, k0, kb, d_L, d_info);
-    const int rest = n - k0 - kb;
-    if (rest > 0) {
-      chol_panel_kernel<<<(rest + 127) / 128, 128, 0, s>>>(n, k0, kb, d_L);
-      const int T = (rest + kB - 1) / kB;
-      chol_update_kernel<<<T * (T + 1) / 2, 256, 0, s>>>(n, k0, kb, d_L);
-    }
+    const int rest = n - k0 - kb, T = (rest + kB - 1) / kB;
+    chol_panel_kernel<<<1 + T, 128, 0, s>>>(n, k0, kb, d_L, d_info);
+    if (rest > 0) chol_update_kernel<<<T * (T + 1) / 2, 256, 0, s>>>(n, k0, kb, d_L);
   }
   const int64_t nn = (int64_t)n * n;
-  zero_upper_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(n, d_L);
+  finish_factor_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(n, d_L);
   return launched();
 }
 

@@ -76,3 +76,31 @@ def test_solve_is_backward_stable(P, n, m):
     X = P.ri_solve(torch.tensor(L, device="cuda"), torch.tensor(R, device="cuda")).cpu().numpy()
     res = np.abs((L.astype(np.longdouble) @ X.astype(np.longdouble) - R).astype(np.float64)) if n * m < 1e5 else np.abs(L @ X - R)
     assert np.all(res <= (n + 4) * 2.0 ** -52 * (np.abs(L) @ np.abs(X) + np.abs(R)))
+
+
+@pytest.mark.parametrize("n", [1, 3, 4, 31, 32, 33, 63, 64, 65, 97, 300, 693])
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** 1000, 2.0 ** -1000])
+def test_factor_residual(P, n, scale):
+    """|A - L L^T| <= gamma |L| |L|^T: a column sum has at most n products and a subtraction, the reciprocal
+    pivot and its use three more roundings, the diagonal's root one."""
+    import torch
+    rng = np.random.default_rng(n)
+    X = rng.standard_normal((n, n + 2)) * np.exp(rng.uniform(-2, 2, (n, 1)))
+    A = (X @ X.T + 1e-3 * np.eye(n)) * scale
+    A = np.tril(A) + np.tril(A, -1).T
+    L, info = P.ri_factor(torch.tensor(A, device="cuda"))
+    L = L.cpu().numpy()
+    assert int(info.item() if hasattr(info, "item") else info) == 0
+    assert np.array_equal(L, np.tril(L)) and np.all(np.diag(L) > 0)
+    Ll = (L / np.sqrt(scale)).astype(np.longdouble)
+    err = np.abs(Ll @ Ll.T - (A / scale).astype(np.longdouble))
+    assert np.all(err <= (n + 8) * 2.0 ** -53 * (np.abs(Ll) @ np.abs(Ll).T))
+
+
+@pytest.mark.parametrize("n,bad", [(1, 0), (40, 35), (65, 64), (97, 31)])
+def test_factor_names_the_first_bad_pivot(P, n, bad):
+    import torch
+    A = np.eye(n) + 0.01
+    A[bad, bad] = -1.0
+    _, info = P.ri_factor(torch.tensor(A, device="cuda"))
+    assert int(info.item() if hasattr(info, "item") else info) == bad + 1
