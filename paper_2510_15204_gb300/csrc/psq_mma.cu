@@ -956,9 +956,18 @@ __global__ void __launch_bounds__(ws::kThreads, 1)
       // The ring empties before another row count's layout, and before a packed B after formed ones (the
       // B ring's phases are then known to be over up to this item's first chunk).
       if (!ar.fits(ra) || (pb && was_formed)) {
-        bool ok = true;
-        for (int k = 0; k < kMaxStages && ok; ++k) ok = ws::wait_a_free(sm, ar, k, wait_ns);
-        run = __all_sync(kFull, ok);
+        // The rows of the formed windows still in the ring may have to be requested meanwhile: the
+        // ring holds up to eight chunks of as many windows, the staged buffers two windows.
+        const uint64_t t0 = global_ns();
+        for (int k = 0; k < kMaxStages && run; ++k) {
+          if (!((ar.used >> k) & 1u)) continue;
+          while (run && !__all_sync(kFull, mbar_test(smem_u32(&sm.a_free[k]), (ar.par >> k) & 1u))) {
+            request_free();
+            run = __all_sync(kFull, !ws::aborted(sm) && global_ns() - t0 <= wait_ns);
+          }
+          ar.par ^= 1u << k;
+          ar.used &= ~(1u << k);
+        }
         if (!run) { ws::fail(sm, status, 4); break; }
         if (!ar.fits(ra)) ar.layout(ra);
       }
@@ -1034,6 +1043,11 @@ __global__ void __launch_bounds__(ws::kThreads, 1)
         // packed B: the loader brings it; b_ready still completes one phase per chunk
         for (int win = q.w0; win < q.w1 && run; ++win, ++w) {
           const int nck = ws::chunks_in(q, win);
+          // every phase of eb_free is waited for, so that a formed window's wait cannot take an older
+          // phase of the same parity for its own where windows of one chunk follow one another
+          const bool oke = w < 2 || ws::wait(&sm.eb_free[w & 1], ((w - 2) >> 1) & 1, &sm.abort, wait_ns);
+          run = __all_sync(kFull, oke && !ws::aborted(sm));
+          if (!run) { ws::fail(sm, status, 5); break; }
           for (int j = 0; j < nck; ++j, ++c) {
             const int sb = ws::bstage_of(c);
             const bool ok = ws::wait_b_free(sm, c, wait_ns);
@@ -1162,7 +1176,7 @@ __global__ void __launch_bounds__(ws::kThreads, 1)
       for (int win = w0; win < w1 && ok; ++win, ++w) {
         const int nck = min(kChunksPerWin, nch - kChunksPerWin * win);
         const int set = w & 1;
-        if (w >= 2) ok = ws::wait(&sm.tmem_free[set], ((w - 2) >> 1) & 1, &sm.abort, wait_ns);
+        if (w >= 2) ok = __all_sync(kFull, ws::wait(&sm.tmem_free[set], ((w - 2) >> 1) & 1, &sm.abort, wait_ns));
         const uint32_t tset = tmem + (uint32_t)set * 256u;
         for (int j = 0; j < nck && ok; ++j, ++c) {
           const uint32_t s = ar.s, sb = c % kStagesB;
