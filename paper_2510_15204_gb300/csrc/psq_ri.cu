@@ -25,7 +25,7 @@ constexpr int kB = 32;  // block size of the factor and the solve
 // or not: five of them, where sqrt and a division take 675 and 354 cycles.
 __device__ __forceinline__ double rsqrt_fast(double d) {
   const int hi = __double2hiint(d);
-  if (hi < 0x03d00000 || hi > 0x7c200000) return 1.0 / sqrt(d);  // near the ends of the range
+  if (hi < ((1023 - 1000) << 20) || hi >= ((1023 + 1000) << 20)) return 1.0 / sqrt(d);  // outside [2^-1000, 2^1000)
   double r;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
   const double h = fma(-d * r, r, 1.0);
