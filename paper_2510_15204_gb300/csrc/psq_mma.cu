@@ -493,8 +493,9 @@ __device__ __forceinline__ void prod_unnorm(f2 xh, f2 xl, f2 yh, f2 yl, f2& nh, 
 }
 
 // Decodes packing job `job` (panel, tile, window, 16-row group) for this thread: 8 threads per
-// row, thread qq holding points [16 qq, 16 qq + 16) of the window (chunk 4 w + qq/2, 16-byte
-// groups 2 (qq % 2) and 2 (qq % 2) + 1 of its row).
+// row, thread qq holding points [4 qq, 4 qq + 4) of each of the window's four chunks (half qq % 2 of
+// 16-byte group qq / 2 of its row), so that the eight read 128 contiguous bytes and write whole
+// 64-byte rows, four of them one after the other.
 struct PackPos {
   int pn, t, w, r, qq;
 };
@@ -528,15 +529,15 @@ __device__ __forceinline__ PackPos pack_pos(int64_t job, const Panel* __restrict
 }
 
 // The row's window exponent (the eight threads of the row share it) and the five planes of
-// this thread's 16 points, sgn h + l (sgn = 1 or -1).
-__device__ __forceinline__ void pack_store(const PackPos& P, const Panel& pn, const f2 (&h)[2][4], const f2 (&l)[2][4], float sgn,
+// this thread's 4 x 4 points, sgn h + l (sgn = 1 or -1).
+__device__ __forceinline__ void pack_store(const PackPos& P, const Panel& pn, const f2 (&h)[4][2], const f2 (&l)[4][2], float sgn,
                                            uint8_t* __restrict__ packed) {
   using namespace mma;
   float mx = 0.0f;
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     float a, b;
-    f2_unpack(h[i >> 2][i & 3], a, b);
+    f2_unpack(h[i >> 1][i & 1], a, b);
     mx = fmaxf(mx, fmaxf(fabsf(a), fabsf(b)));
   }
   const unsigned m8 = 0xffu << ((threadIdx.x & 31) & ~7u);
@@ -547,35 +548,38 @@ __device__ __forceinline__ void pack_store(const PackPos& P, const Panel& pn, co
   if (P.qq == 0)
     *reinterpret_cast<int*>(packed + pn.exp_off + (((int64_t)P.t * pn.nwin + P.w) * pn.tr + P.r) * 4) = e;
   const int rt = min(pn.tr, pn.nrows - P.t * pn.tr);
-  const int c = kChunksPerWin * P.w + (P.qq >> 1);
-  if (c >= pn.nch || P.r >= rt) return;
+  if (P.r >= rt) return;
   float sc, scj;
   window_scales<1>(e, sc, scj);
+  const int plane = rt * kRowB, left = pn.nch - kChunksPerWin * P.w;  // chunks of the window that exist
   uint8_t* dst = packed + pn.pack_off + (int64_t)P.t * pn.nch * (kSlices * pn.tr * kRowB) +
-                 (int64_t)c * (kSlices * rt * kRowB);
-  const int plane = rt * kRowB;
+                 (int64_t)kChunksPerWin * P.w * (kSlices * plane) + swz(P.r, P.qq >> 1) + 8 * (P.qq & 1);
 #pragma unroll
-  for (int j = 0; j < 2; ++j) {
-    uint32_t wv[kSlices][4];
-    slice_f2<1, 4>(h[j], l[j], sgn * sc, scj, wv);
+  for (int c = 0; c < kChunksPerWin; ++c) {
+    if (c >= left) break;
+    uint32_t wv[kSlices][2];
+    slice_f2<1, 2>(h[c], l[c], sgn * sc, scj, wv);
 #pragma unroll
-    for (int k = 0; k < kSlices; ++k)
-      *reinterpret_cast<uint4*>(dst + k * plane + swz(P.r, 2 * (P.qq & 1) + j)) = make_uint4(wv[k][0], wv[k][1], wv[k][2], wv[k][3]);
+    for (int k = 0; k < kSlices; ++k) *reinterpret_cast<uint2*>(dst + (c * kSlices + k) * plane) = make_uint2(wv[k][0], wv[k][1]);
   }
 }
 
 // One CTA of 128 threads per packing job.  Values: source row times its weight row
-// (double-float products), zeros past K.
+// (double-float products), zeros past K.  Bound by HBM and by the sectors its loads and stores touch:
+// with 16 consecutive points per thread every access of a warp touched 32 sectors of which it used
+// half; with four points of each chunk it uses them whole (and 64 registers instead of 70: eight CTAs
+// per SM).  Whole steps before -> after: bent triatomic 1.503 -> 1.421 ms, C3H6 225.2 -> 219.9 ms.
 __global__ void __launch_bounds__(128) pack_kernel(const DevGrid* __restrict__ grids, const Panel* __restrict__ panels,
                                                    int n_panels, const int* __restrict__ hint, const short2* __restrict__ rows,
                                                    const float* __restrict__ ops, const float* __restrict__ ops_lo,
                                                    uint8_t* __restrict__ packed) {
+  using namespace mma;
   const PackPos P = pack_pos(blockIdx.x, panels, n_panels, hint);
   const Panel& pn = panels[P.pn];
   const DevGrid& g = grids[pn.grid];
   const int row = P.t * pn.tr + P.r;
-  const int64_t k0 = (int64_t)kWinPts * P.w + 16 * P.qq;
-  const int64_t blk = g.op_off + (int64_t)P.w * g.ws + 16 * P.qq;  // (kWinPts = 128: one block)
+  const int64_t k0 = (int64_t)kWinPts * P.w + 4 * P.qq;
+  const int64_t blk = g.op_off + (int64_t)P.w * g.ws + 4 * P.qq;  // (kWinPts = 128: one block)
   int64_t src = -1, mul = -1;
   if (row < pn.nrows) {
     const short2 q = rows[pn.rows_off + row];
@@ -583,25 +587,26 @@ __global__ void __launch_bounds__(128) pack_kernel(const DevGrid* __restrict__ g
     if (q.y >= 0) mul = blk + q.y * g.rs;
   }
   const int64_t left = src >= 0 ? g.K - k0 : 0;
-  f2 h[2][4], l[2][4];
+  f2 h[kChunksPerWin][2], l[kChunksPerWin][2];
 #pragma unroll
-  for (int i4 = 0; i4 < 4; ++i4) {
+  for (int c = 0; c < kChunksPerWin; ++c) {
+    const int p = kChunk * c;  // this chunk's four points, from the thread's first
     ulonglong2 ah = make_ulonglong2(0, 0), al = ah, bh = ah, bl = ah;
-    if (left >= 4 * i4 + 4) {
-      ah = __ldg(reinterpret_cast<const ulonglong2*>(ops + src) + i4);
-      al = __ldg(reinterpret_cast<const ulonglong2*>(ops_lo + src) + i4);
+    if (left >= p + 4) {
+      ah = __ldg(reinterpret_cast<const ulonglong2*>(ops + src + p));
+      al = __ldg(reinterpret_cast<const ulonglong2*>(ops_lo + src + p));
       if (mul >= 0) {
-        bh = __ldg(reinterpret_cast<const ulonglong2*>(ops + mul) + i4);
-        bl = __ldg(reinterpret_cast<const ulonglong2*>(ops_lo + mul) + i4);
+        bh = __ldg(reinterpret_cast<const ulonglong2*>(ops + mul + p));
+        bl = __ldg(reinterpret_cast<const ulonglong2*>(ops_lo + mul + p));
       }
-    } else if (left > 4 * i4) {
+    } else if (left > p) {
       float v[4][4] = {};
-      for (int i = 0; i < 4 && 4 * i4 + i < left; ++i) {
-        v[0][i] = ops[src + 4 * i4 + i];
-        v[1][i] = ops_lo[src + 4 * i4 + i];
+      for (int i = 0; i < 4 && p + i < left; ++i) {
+        v[0][i] = ops[src + p + i];
+        v[1][i] = ops_lo[src + p + i];
         if (mul >= 0) {
-          v[2][i] = ops[mul + 4 * i4 + i];
-          v[3][i] = ops_lo[mul + 4 * i4 + i];
+          v[2][i] = ops[mul + p + i];
+          v[3][i] = ops_lo[mul + p + i];
         }
       }
       ah = make_ulonglong2(f2_pack(v[0][0], v[0][1]).v, f2_pack(v[0][2], v[0][3]).v);
@@ -609,8 +614,7 @@ __global__ void __launch_bounds__(128) pack_kernel(const DevGrid* __restrict__ g
       bh = make_ulonglong2(f2_pack(v[2][0], v[2][1]).v, f2_pack(v[2][2], v[2][3]).v);
       bl = make_ulonglong2(f2_pack(v[3][0], v[3][1]).v, f2_pack(v[3][2], v[3][3]).v);
     }
-    f2 &h0 = h[i4 >> 1][2 * (i4 & 1)], &h1 = h[i4 >> 1][2 * (i4 & 1) + 1];
-    f2 &l0 = l[i4 >> 1][2 * (i4 & 1)], &l1 = l[i4 >> 1][2 * (i4 & 1) + 1];
+    f2 &h0 = h[c][0], &h1 = h[c][1], &l0 = l[c][0], &l1 = l[c][1];
     if (mul >= 0) {
       prod_unnorm(f2{ah.x}, f2{al.x}, f2{bh.x}, f2{bl.x}, h0, l0);
       prod_unnorm(f2{ah.y}, f2{al.y}, f2{bh.y}, f2{bl.y}, h1, l1);
@@ -629,24 +633,25 @@ __global__ void __launch_bounds__(128) pack_kernel(const DevGrid* __restrict__ g
 // digits keep).
 __global__ void __launch_bounds__(128) ri_pack_kernel(const Panel* __restrict__ panels, const double* __restrict__ srcA,
                                                       const double* __restrict__ srcB, int n, uint8_t* __restrict__ packed) {
+  using namespace mma;
   const PackPos P = pack_pos(blockIdx.x, panels, 2, nullptr);
   const Panel& pn = panels[P.pn];
   const double* src = P.pn ? srcB : srcA;
   const int row = P.t * pn.tr + P.r;
-  const int k0 = kWinPts * P.w + 16 * P.qq;
-  f2 h[2][4], l[2][4];
+  const int k0 = kWinPts * P.w + 4 * P.qq;
+  f2 h[kChunksPerWin][2], l[kChunksPerWin][2];
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     float hv[2], lv[2];
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
       double v = 0.0;
-      if (row < pn.nrows && k0 + 2 * i + k < n) v = src[(int64_t)row * n + k0 + 2 * i + k];
+      if (row < pn.nrows && k0 + kChunk * (i >> 1) + 2 * (i & 1) + k < n) v = src[(int64_t)row * n + k0 + kChunk * (i >> 1) + 2 * (i & 1) + k];
       hv[k] = (float)v;
       lv[k] = (float)(v - (double)hv[k]);
     }
-    h[i >> 2][i & 3] = f2_pack(hv[0], hv[1]);
-    l[i >> 2][i & 3] = f2_pack(lv[0], lv[1]);
+    h[i >> 1][i & 1] = f2_pack(hv[0], hv[1]);
+    l[i >> 1][i & 1] = f2_pack(lv[0], lv[1]);
   }
   pack_store(P, pn, h, l, 1.0f, packed);
 }
