@@ -195,6 +195,8 @@ __device__ __forceinline__ df split_d(double v) {
 // A and B depend on (mu, nu) only: they are computed once per node pair and kept in shared memory for
 // all phi nodes (32 points share one on an 8-cell grid with Q = 4); those of a third centre are
 // computed for half of the phi nodes.  A point is then its harmonics and one product per function.
+// FP32 issue bounds it.  Measured (radial factors per point -> shared): bent triatomic (963,072 points)
+// 0.58 -> 0.36 ms, nine atoms (55.7 M points) 45.0 -> 33.2 ms.
 __global__ void __launch_bounds__(kEvalThreads) eval_mixed_kernel(LaunchTables t, const NodeEntry* __restrict__ tab,
                                                                   const float2* __restrict__ xi_tab,
                                                                   float* __restrict__ ops, float* __restrict__ ops_lo) {
@@ -678,6 +680,11 @@ __global__ void __launch_bounds__(128) ri_pack_kernel(const Panel* __restrict__ 
 //                half, scaled by the window's row and column exponents, into double-float
 //                registers (orders 0 and 1 join the sum exactly through TwoSums, orders 2-4
 //                as one FP32 term); at the end of the tile, (hi, lo) partials to global memory.
+// What bounds it: the tensor pipe (62% of the measured BF16 rate on nine atoms) and, about even with
+// it, the producers' slicing and the fold.  Measured (MMAs issued from a divergent branch, scalar
+// slicing and folding, a bulk copy per plane and row -> now): nine-atom quadruple-zeta job (288 grids)
+// 250 -> 163 ms, quintuple-zeta diatomic 98 -> 68 ms, bent triatomic 0.97 -> 0.64 ms.
+//
 // Every wait is bounded (wait_ns in the main loops, the fixed kWaitNs for the drains); a
 // timeout sets *status and the CTA's abort flag, and each role leaves its loops at its next
 // wait; the loader then waits for its copies in flight and the MMA lane for its MMAs before
