@@ -1662,11 +1662,11 @@ size_t psq::status_offset(psq_job* job, unsigned mask) {
 
 namespace {
 psq_status run_plan(psq_job* job, Plan* P, unsigned mask, char* ws, double* d_out[5], cudaStream_t s,
-                    bool timing = true);
+                    bool timing = true, bool overlap = true);
 }
 
 psq_status psq::compute_on(psq_job* job, unsigned mask, void* d_workspace, size_t ws_bytes, double* d_out[5],
-                           void* stream, bool plan_must_exist) {
+                           void* stream, bool plan_must_exist, bool overlap) {
   if (!job) return fail(PSQ_ERR_ARG, "job is NULL");
   if (job->ctx->device < 0) return fail(PSQ_ERR_ARG, "the job's context has no device (planning only)");
   if (mask & ~31u) return fail(PSQ_ERR_ARG, "mask 0x%x has unknown bits", mask);
@@ -1695,14 +1695,14 @@ psq_status psq::compute_on(psq_job* job, unsigned mask, void* d_workspace, size_
     return fail(PSQ_ERR_ARG, "device %d is current, the job's context is on device %d", dev, job->ctx->device);
   // the allocation-free path (plan_must_exist outside a capture) records no timing events:
   // creating them would allocate
-  return run_plan(job, P, mask, (char*)d_workspace, d_out, (cudaStream_t)stream, !plan_must_exist);
+  return run_plan(job, P, mask, (char*)d_workspace, d_out, (cudaStream_t)stream, !plan_must_exist, overlap);
 }
 
 namespace {
 
 // The launch sequence of one psq_compute on plan P (arguments checked by the caller).
 psq_status run_plan(psq_job* job, Plan* P, unsigned mask, char* ws, double* d_out[5], cudaStream_t s,
-                    bool timing) {
+                    bool timing, bool overlap) {
   auto mark = [&](psq_job* j, int kind, cudaStream_t st) { return timing ? ::mark(j, kind, st) : cudaSuccess; };
   CUDA_TRY(mark(job, 0, s));
   CUDA_TRY(cudaMemcpyAsync(ws, P->staging, P->table_bytes, cudaMemcpyHostToDevice, s));
@@ -1752,6 +1752,7 @@ psq_status run_plan(psq_job* job, Plan* P, unsigned mask, char* ws, double* d_ou
   const int* aa = (const int*)(ws + P->o_aa);
   const int* al = (const int*)(ws + P->o_al);
   const unsigned cls[4] = {PSQ_S, PSQ_T, PSQ_V, PSQ_J2};
+  bool after = false;  // another assembly comes before this one, and this one may start beside it
   for (int c = 0; c < 4; ++c) {
     if (!(mask & cls[c])) continue;
     const int n = c == 3 ? job->naux : job->nbf;
@@ -1762,11 +1763,12 @@ psq_status run_plan(psq_job* job, Plan* P, unsigned mask, char* ws, double* d_ou
     CUDA_TRY(launch_assemble((int)cls[c], job->nat, n, 0, at, lo, nullptr, nullptr,
                              (const SrcEntry*)(ws + P->o_src[c]), (const int*)(ws + P->o_ptr[c]), nullptr,
                              closed ? (const DevShell*)(ws + P->o_bsh) : nullptr,
-                             closed ? (const int*)(ws + P->o_fs) : nullptr, res, d_out[c], s));
+                             closed ? (const int*)(ws + P->o_fs) : nullptr, res, d_out[c], after, s));
+    after = after || (overlap && n > 0);
   }
   if (mask & PSQ_J3)
     CUDA_TRY(launch_assemble(16, job->nat, job->nbf, job->naux, fa, fl, aa, al, nullptr, nullptr,
-                             (const J3Src*)(ws + P->o_j3), nullptr, nullptr, res, d_out[4], s));
+                             (const J3Src*)(ws + P->o_j3), nullptr, nullptr, res, d_out[4], after, s));
   CUDA_TRY(mark(job, -1, s));
   return PSQ_OK;
 }

@@ -118,7 +118,7 @@ void launch(psq_server* S, Request* r) {
     o += align256(r->out_bytes[c]);
   }
   r->t_start = now_s();
-  psq_status st = psq::compute_on(r->job, r->mask, base, r->ws_bytes, d_out, s, true);
+  psq_status st = psq::compute_on(r->job, r->mask, base, r->ws_bytes, d_out, s, true, false);
   if (st == PSQ_OK) {
     for (int c = 0; c < 5 && st == PSQ_OK; ++c) {
       if (!((r->mask >> c) & 1)) continue;
