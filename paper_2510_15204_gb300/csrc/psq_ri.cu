@@ -527,7 +527,7 @@ extern "C" psq_status psq_ri_eri_mixed(int n, int64_t m, const double* d_B, int6
     return launched();
   if (launch_reduce_mixed((const DevGrid*)(ws + L.o_grid), (const MmaBlock*)(ws + L.o_blk), 1,
                           (const int64_t*)(ws + L.o_eb), 0, nc * nd, (const short2*)(ws + L.o_rows),
-                          (const double*)(ws + L.o_rowc), (const float2*)(ws + L.o_part), d_out, s) != cudaSuccess)
+                          nullptr, (const float2*)(ws + L.o_part), d_out, s) != cudaSuccess)
     return launched();
   return launched();
 }
