@@ -129,8 +129,9 @@ __device__ __forceinline__ void store_b(Smem& sm, uint32_t off, const double (&v
 }
 
 // The exponent field a window is scaled by, from its largest |high word|: one more where the largest
-// value is within 2^-7 of the next power of two (its leading digit would round up to 128).
-__device__ __forceinline__ int field(int mx) { return (mx + 0x2040) >> 20; }
+// value is within 2^-7 of the next power of two (its leading digit would round up to 128).  A NaN's
+// payload counts for nothing (its sum would leave the range of an int).
+__device__ __forceinline__ int field(int mx) { return (min(mx, 0x7ff00000) + 0x2040) >> 20; }
 
 __device__ __forceinline__ int hi_abs(double v) { return __double2hiint(v) & 0x7fffffff; }
 
