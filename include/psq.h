@@ -64,7 +64,10 @@ typedef struct { int n_mu, n_nu, n_phi, q_mu, q_nu, q_phi, n_sp; } psq_grid_spec
 typedef enum {
   PSQ_FP64 = 0,  /* plain path: FP64 values throughout.  The (P|Q) and (P|ij) sums run on the tensor
                     cores on exact integer digits of the FP64 values (63 bits of each 64-point
-                    window's largest), one FP64 rounding per window; the other sums are FP64 FMAs */
+                    window's largest), one FP64 rounding per window; an element whose two factors
+                    are large at different points of a window sums that window by FP64 FMAs, as
+                    the other classes do throughout.  Within 1e-12 of each element's sum of
+                    absolute terms */
   PSQ_MIXED = 1  /* FP64 node tables, third-centre offsets, row constants and range sums;
                     double-float (FP32 hi + lo, ~48 bits) weights, STO values and aux
                     potentials; contraction on tcgen05 tensor cores: five 8-bit integer slices
@@ -254,8 +257,10 @@ const char* psq_last_error(void);
  * and B = L^-1 (P|ij), (ij|kl) = sum_R B[R][ij] B[R][kl].  FP64 matrices throughout; the large
  * products (the solve's off-diagonal blocks, the (ij|kl) sums) run on the tensor cores on exact
  * integer digits of the FP64 values (62 bits of each 64-row window's largest, one FP64 rounding
- * per window), the rest on the FP64 pipe.  On the device, asynchronous on `stream` (a
- * cudaStream_t; NULL = legacy default stream), on the current device.  Matrices are row-major; the pair index of (P|ij) is ij = i * n_bf + j, so its
+ * per window; FP64 FMAs for an element whose two factors are large in different rows of a window),
+ * the rest on the FP64 pipe: an error of at most (n + 4) 2^-52 of the sum of absolute products.  On
+ * the device, asynchronous on `stream` (a cudaStream_t; NULL = legacy default stream), on the
+ * current device.  Matrices are row-major; the pair index of (P|ij) is ij = i * n_bf + j, so its
  * n_aux x n_bf x n_bf layout is B's n x m layout with m = n_bf^2.  The caller owns every
  * buffer.  Errors: PSQ_ERR_ARG for negative sizes, NULL or non-8-byte-aligned pointers with
  * nonzero sizes, or column ranges outside [0, m); PSQ_ERR_CUDA on a failed launch. */

@@ -11,14 +11,27 @@
 // accumulate per order in FP32: an order's sum over 64 points stays within 64 x 8 x 2^14 = 2^23,
 // so the accumulation is exact.  The order sums join in one 64-bit integer T and the FP64
 // accumulator of an element takes T by one FMA per window: where a chain of FP64 FMAs rounds 64
-// times, this rounds once.  What is dropped (the truncation of small values, orders above 7) stays
-// below about 2^-59 of the largest |a| times the largest |b| per window, against 2^-53 of the
-// running sum per FMA of the chain.
+// times, this rounds once.
 //
-// Rows whose window lies below 2^-958 count as zeros.  Rows that hold an infinity, a NaN or a value of 2^478 and above take the plain FP64 chain for the
-// window (their products with the other operand may leave the range of the integer path).
+// What is dropped, of a product of scales S = 2^(e_a + e_b): the seven products of order 8 and those
+// above, at most 64 x 7 x 2^14 x 2^-78 (1 + 2^-8) = 2^-55.2 S, and the truncation of small values, at
+// most 64 x 2 x 2^-63 = 2^-56 S; typically 2^-61 S.  That is an error relative to the largest values
+// of the window, not to an element's own terms.  So a row's bits in `near` mark the points where it is
+// above 2^-4 of its scale (kNear), and an element whose two rows share such a point has terms of at
+// least 2^-8 S: its error stays within 2^-46.5 of the sum of its absolute terms, about the bound of the
+// chain it stands for (63 roundings, 2^-47).  Where the rows share none (two steep functions that
+// peak at opposite ends of the window), the element's window is summed by that chain instead: none to
+// one element in 10^5 on grids with whole cells per window (bent triatomic, triple
+// zeta), one in 10^3 to 10^2 on coarse grids with cells of 27 or 45 points.
+// Measured (no near bits, no chain -> now): bent triatomic 4.86 -> 5.13 ms, RI of 693 aux functions
+// 8.69 -> 9.11 ms, H2 and RI of 82 unchanged.
 //
-// Layout.  Two CTAs per SM (82 KB of shared memory and 256 of the 512 TMEM columns each), so that
+// Rows with an infinity, a NaN or a value of 2^478 and above take the chain too (their products may
+// leave the range of the integer path).  Rows below 2^-959 (a steep function far out) are lifted by
+// 2^200 first, and sums whose unit lies below 2^-1022 are scaled in two steps: nothing is flushed that
+// FP64 would keep.
+//
+// Layout.  Two CTAs per SM (84 KB of shared memory and 256 of the 512 TMEM columns each), so that
 // one slices or folds while the other's MMAs run.  The digits of 32 points are eight planes of
 // 64-byte rows in the 64-byte swizzle (A: 8 x 8 KB, B: 8 x 2 KB); the B planes are contiguous, so
 // A plane i against B planes 0..7-i is one MMA of N = 32 (8 - i) whose columns land on the order
@@ -37,11 +50,15 @@ constexpr int kWin = 64;                // points per scale window
 constexpr int kDigits = 8;
 constexpr uint32_t kTmemCols = kDigits * kCols;
 constexpr int kBigField = 1500;         // exponent field from which a row takes the FP64 chain
+constexpr int kLift = 200;              // power of two by which a row of tiny values is lifted
+constexpr int kBias = 256;              // keeps the stored field of a lifted row positive
+constexpr int kNear = 2;                // a value of a field at most this below its row's counts as large
 
 struct Smem {
   alignas(1024) uint8_t a[kDigits][kRows * 64];
   alignas(1024) uint8_t b[kDigits][kCols * 64];
-  int ea[2][kRows], eb[2][kCols];  // exponent fields, of even and odd windows
+  int ea[2][kRows], eb[2][kCols];  // exponent fields + kBias, of even and odd windows (0: all zeros)
+  alignas(8) uint8_t na[2][kRows][kWin / 8], nb[2][kCols][kWin / 8];  // bit p: the value at point p is large
   alignas(8) uint64_t done;
   uint32_t tmem;
 };
@@ -88,10 +105,11 @@ __device__ __forceinline__ int b_col() { return 4 * (threadIdx.x >> 5) + ((threa
 __device__ __forceinline__ int b_pt(int c) { return 32 * c + 4 * (threadIdx.x & 7); }
 
 // Biased digits of v (byte k of the result = digit 7 - k plus 128) in a window whose largest
-// exponent field is E (E = 4000: a row of zeros).
-__device__ __forceinline__ uint64_t digits(double v, int E) {
+// exponent field is E (E = 4000: a row of zeros).  near takes a bit at its low end: v is large.
+__device__ __forceinline__ uint64_t digits(double v, int E, uint32_t& near) {
   const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
   const int t = min(E - (int)((hi >> 20) & 0x7ffu), 63);
+  near = __funnelshift_l((uint32_t)(t - 2 - kNear), near, 1);  // (the difference's sign)
   const uint64_t m = ((uint64_t)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
   const uint64_t x = (m << 10) >> t;
   const uint64_t s = (uint64_t)((int64_t)(int32_t)hi >> 63);
@@ -107,67 +125,117 @@ __device__ __forceinline__ uint32_t plane(uint64_t y0, uint64_t y1, int k) {
   return *reinterpret_cast<const uint32_t*>(&d);
 }
 
-// Eight consecutive points of a row into its 16-byte group of every plane (offset off).
-__device__ __forceinline__ void store_a(Smem& sm, uint32_t off, const double (&v)[8], int E) {
+// Eight consecutive points of a row into its 16-byte group of every plane (offset off); their near bits.
+__device__ __forceinline__ uint32_t store_a(Smem& sm, uint32_t off, const double (&v)[8], int E) {
   uint64_t y[8];
+  uint32_t near = 0;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) y[i] = digits(v[i], E);
+  for (int i = 0; i < 8; ++i) y[i] = digits(v[i], E, near);
 #pragma unroll
   for (int k = 0; k < kDigits; ++k)
     *reinterpret_cast<uint4*>(sm.a[k] + off) =
         make_uint4(plane(y[0], y[1], k), plane(y[2], y[3], k), plane(y[4], y[5], k), plane(y[6], y[7], k));
+  return near;
 }
 
 // Four consecutive points of a column into their half group.
-__device__ __forceinline__ void store_b(Smem& sm, uint32_t off, const double (&v)[4], int E) {
+__device__ __forceinline__ uint32_t store_b(Smem& sm, uint32_t off, const double (&v)[4], int E) {
   uint64_t y[4];
+  uint32_t near = 0;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) y[i] = digits(v[i], E);
+  for (int i = 0; i < 4; ++i) y[i] = digits(v[i], E, near);
 #pragma unroll
   for (int k = 0; k < kDigits; ++k)
     *reinterpret_cast<uint2*>(sm.b[k] + off) = make_uint2(plane(y[0], y[1], k), plane(y[2], y[3], k));
+  return near;
 }
 
-// The exponent field a window is scaled by, from its largest |high word|: one more where the largest
-// value is within 2^-7 of the next power of two (its leading digit would round up to 128).  A NaN's
-// payload counts for nothing (its sum would leave the range of an int).
-__device__ __forceinline__ int field(int mx) { return (min(mx, 0x7ff00000) + 0x2040) >> 20; }
+// The size of v as an integer: exponent and the mantissa's first 21 bits (0 below 2^-1043: low_bits).
+__device__ __forceinline__ uint32_t mag(double v) {
+  return __funnelshift_l((uint32_t)__double2loint(v), (uint32_t)__double2hiint(v), 1);
+}
+__device__ __forceinline__ uint32_t low_bits(double v) { return (uint32_t)__double2loint(v); }
+// The exponent field a window is scaled by, from its largest size: one more where the largest value is within
+// 2^-7 of the next power of two (its leading digit would round up to 128).  A NaN's payload counts for
+// nothing (the sum would wrap).
+__device__ __forceinline__ int field(uint32_t mx) { return (int)((min(mx, 0xffe00000u) + 0x4080u) >> 21); }
+constexpr uint32_t kLow = 64u << 21;  // rows below it are lifted
 
-__device__ __forceinline__ int hi_abs(double v) { return __double2hiint(v) & 0x7fffffff; }
+// What a row's or column's window is scaled by: the field its digits are cut with (4000 for zeros: their
+// own field, 0, must be 63 below it), the stored one, and the value of its near bits where they are the
+// same for all points (zeros meet anything; rows out of the digits' range meet nothing).
+struct Scale {
+  int E, stored;
+  uint32_t set, keep;
+  __device__ __forceinline__ Scale(uint32_t mx, int low) {
+    E = field(mx);
+    stored = mx == 0 ? 0 : E + kBias - low;
+    set = mx == 0 ? ~0u : 0u;
+    keep = E >= kBigField ? 0u : ~0u;
+    if (mx == 0) E = 4000;
+  }
+  __device__ __forceinline__ uint32_t bits(uint32_t near) const { return (near | set) & keep; }
+};
 
 // One window: the tile's accumulators (element row 32 (warp % 4) + lane, columns 16 (warp / 4) + j,
 // acc[j]) take sum_p a_r(p) b_c(p).  Only the first `rows` rows and `cols` columns are kept up
 // (8-row groups and 4-column groups past them are left out).  win: the windows done so far by this
 // CTA.  chain(row, col): the plain FP64 sum of the window for a row or column out of the integer
-// path's range.  ok turns false when a wait ran out (the caller ends its loop when the return
+// path's range and for an element whose rows are not large at a common point.  ok turns false when a wait ran out (the caller ends its loop when the return
 // value, the same for all threads, is false, and asks all threads once more at the end).
 template <typename Chain>
-__device__ __forceinline__ bool window(Smem& sm, uint32_t tmem, const double (&va)[4][8], const double (&vb)[2][4],
+__device__ __forceinline__ bool window(Smem& sm, uint32_t tmem, double (&va)[4][8], double (&vb)[2][4],
                                        double (&acc)[16], uint32_t& phase, uint32_t win, int rows, int cols, bool& ok,
                                        Chain chain) {
   constexpr unsigned kFull = 0xffffffffu;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int set = win & 1;
-  int E[2], Eb = 0;
-#pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    int mx = 0;
+  auto over_a = [&](int u, auto part) {  // the largest part of row u's values
+    uint32_t m = 0;
 #pragma unroll
     for (int c = 0; c < 2; ++c)
 #pragma unroll
-      for (int i = 0; i < 8; ++i) mx = max(mx, hi_abs(va[2 * c + u][i]));
-    mx = max(mx, __shfl_xor_sync(kFull, mx, 1));
-    E[u] = field(max(mx, __shfl_xor_sync(kFull, mx, 2)));
-    if ((lane & 3) == 0) sm.ea[set][a_row(u)] = E[u];
-    if (E[u] < 64) E[u] = 4000;  // a zero's own field, 0, must be 63 below that of a row that counts
+      for (int i = 0; i < 8; ++i) m = max(m, part(va[2 * c + u][i]));
+    m = max(m, __shfl_xor_sync(kFull, m, 1));
+    return max(m, __shfl_xor_sync(kFull, m, 2));
+  };
+  auto over_b = [&](auto part) {
+    uint32_t m = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) m = max(m, max(part(vb[0][i]), part(vb[1][i])));
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) m = max(m, __shfl_xor_sync(kFull, m, o));
+    return m;
+  };
+  uint32_t ma[2] = {over_a(0, mag), over_a(1, mag)}, mb = over_b(mag);
+  // zeros, or values below 2^-1043?
+  if (__any_sync(kFull, (ma[0] == 0 && a_row(0) < rows) || (ma[1] == 0 && a_row(1) < rows) || (mb == 0 && b_col() < cols))) {
+    ma[0] = max(ma[0], min(over_a(0, low_bits), 1u));
+    ma[1] = max(ma[1], min(over_a(1, low_bits), 1u));
+    mb = max(mb, min(over_b(low_bits), 1u));
   }
+  const bool la0 = ma[0] - 1 < kLow - 1, la1 = ma[1] - 1 < kLow - 1, lb = mb - 1 < kLow - 1;
+  if (__any_sync(kFull, la0 || la1 || lb)) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i) Eb = max(Eb, max(hi_abs(vb[0][i]), hi_abs(vb[1][i])));
+    for (int c = 0; c < 2; ++c) {
 #pragma unroll
-  for (int o = 1; o < 8; o <<= 1) Eb = max(Eb, __shfl_xor_sync(kFull, Eb, o));
-  Eb = field(Eb);
-  if ((lane & 7) == 0) sm.eb[set][b_col()] = Eb;
-  if (Eb < 64) Eb = 4000;
+      for (int i = 0; i < 8; ++i) {
+        va[2 * c][i] *= la0 ? 0x1p200 : 1.0;
+        va[2 * c + 1][i] *= la1 ? 0x1p200 : 1.0;
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) vb[c][i] *= lb ? 0x1p200 : 1.0;
+    }
+    ma[0] = over_a(0, mag);
+    ma[1] = over_a(1, mag);
+    mb = over_b(mag);
+  }
+  const Scale ea[2] = {Scale(ma[0], la0 ? kLift : 0), Scale(ma[1], la1 ? kLift : 0)}, eb(mb, lb ? kLift : 0);
+  if ((lane & 3) == 0) {
+    sm.ea[set][a_row(0)] = ea[0].stored;
+    sm.ea[set][a_row(1)] = ea[1].stored;
+  }
+  if ((lane & 7) == 0) sm.eb[set][b_col()] = eb.stored;
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
     if (c == 1 && ok) {
@@ -176,8 +244,15 @@ __device__ __forceinline__ bool window(Smem& sm, uint32_t tmem, const double (&v
     }
 #pragma unroll
     for (int u = 0; u < 2; ++u)
-      if (64 * u + 8 * warp < rows) store_a(sm, mma::swz(a_row(u), lane & 3), va[2 * c + u], E[u]);
-    if (4 * warp < cols) store_b(sm, mma::swz(b_col(), (lane & 7) >> 1) + 8u * (lane & 1), vb[c], Eb);
+      if (64 * u + 8 * warp < rows) {
+        const uint32_t near = store_a(sm, mma::swz(a_row(u), lane & 3), va[2 * c + u], ea[u].E);
+        sm.na[set][a_row(u)][4 * c + (lane & 3)] = (uint8_t)ea[u].bits(near);
+      }
+    if (4 * warp < cols) {
+      uint32_t near = eb.bits(store_b(sm, mma::swz(b_col(), (lane & 7) >> 1) + 8u * (lane & 1), vb[c], eb.E)) & 15u;
+      near = (near << 4) | __shfl_down_sync(kFull, near, 1);  // the pair's first points in the high bits, as in na
+      if ((lane & 1) == 0) sm.nb[set][b_col()][4 * c + ((lane & 7) >> 1)] = (uint8_t)near;
+    }
     mma::fence_async_smem();
     mma::fence_before();
     if (!__syncthreads_and(ok)) return false;
@@ -203,16 +278,20 @@ __device__ __forceinline__ bool window(Smem& sm, uint32_t tmem, const double (&v
   if (32 * (warp & 3) < rows) {
     const uint32_t base = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0;
     const int er = sm.ea[set][row];
+    const uint2 near = row < rows ? *reinterpret_cast<const uint2*>(sm.na[set][row]) : make_uint2(~0u, ~0u);
+    uint32_t apart = 0;  // bit j: element j takes the chain
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       if (c0 + 4 * q >= cols) break;
       float o[kDigits][4];
+      __syncwarp();
 #pragma unroll
       for (int k = 0; k < kDigits; ++k) mma::tmem_ld4(base + (uint32_t)(kCols * k + 4 * q), o[k]);
       mma::tmem_wait_ld();
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int ec = sm.eb[set][c0 + 4 * q + j];
+        const uint2 nc = *reinterpret_cast<const uint2*>(sm.nb[set][c0 + 4 * q + j]);
         // orders 0..3 are integers of at most 2^22: their low bits by the magic number 1.5 x 2^23
         int s[6];
 #pragma unroll
@@ -225,13 +304,25 @@ __device__ __forceinline__ bool window(Smem& sm, uint32_t tmem, const double (&v
         const bool small = (uint32_t)((int)(t >> 32) + (1 << 22)) < (1u << 23);
         t = (small ? t << 7 : t) +
             __float2int_rn(fmaf(o[6][j], 0.00390625f, o[7][j] * 1.52587890625e-5f) * (small ? 128.0f : 1.0f));
-        const int f = er + ec - 2044 - 54 + 1023 - (small ? 7 : 0);  // exponent field of t's unit
-        double& r = acc[4 * q + j];
-        if (er >= kBigField || ec >= kBigField)
-          r += chain(row, c0 + 4 * q + j);
+        int f = er + ec - 2 * kBias - 2044 - 54 + 1023 - (small ? 7 : 0);  // exponent field of t's unit
+        double x = __ll2double_rn(t);
+        if (f <= 0) {  // a unit below 2^-1022: in two steps
+          x *= 0x1p-600;
+          f = max(f + 600, 0);
+        }
+        if (((near.x & nc.x) | (near.y & nc.y)) == 0)
+          apart |= 1u << (4 * q + j);
         else
-          r = fma(__ll2double_rn(t), __hiloint2double(f > 0 ? f << 20 : 0, 0), r);
+          acc[4 * q + j] = fma(x, __hiloint2double(f << 20, 0), acc[4 * q + j]);
       }
+    }
+#pragma unroll 1
+    for (; apart; apart &= apart - 1) {
+      const int e = __ffs(apart) - 1;
+      const double s = chain(row, c0 + e);
+#pragma unroll
+      for (int j = 0; j < 16; ++j)
+        if (j == e) acc[j] += s;
     }
   }
   mma::fence_before();  // the next window's MMAs come after its first barrier

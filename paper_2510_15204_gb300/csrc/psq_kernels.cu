@@ -448,12 +448,14 @@ cudaError_t launch_eval_fp64(const LaunchTables& t, double* ops, int /*kinds*/, 
 // partial sums go to their own slot, so the result does not depend on scheduling.
 //
 // GB300's FP64 pipe (two FMAs per clock and SM) bounds every FP64 sum, so the (P|Q) and (P|ij) sums
-// run on the tensor cores in exact digits.  There one factor (V^P) varies slowly over a window and the
-// other (w times an aux function or a pair product, formed before it is cut) is scaled by
-// its own largest value, so an element keeps its precision relative to its own terms.  The overlap,
+// run on the tensor cores in exact digits.  There one factor (V^P) mostly varies slowly over a window and
+// the other (w times an aux function or a pair product, formed before it is cut) is scaled by
+// its own largest value; an element whose factors are large at different points of a window (a window
+// that runs across cells, a steep V^P of high l) takes the window's FP64 chain instead, so that every
+// element keeps the precision of its own terms (psq_fx.cuh).  The overlap,
 // kinetic and V_ne sums multiply two steep functions of different atoms, whose largest values in a
-// window can lie at its opposite ends: on coarse or long grids the digits of both would be spent on
-// terms that never meet.  They stay on the FP64 pipe, with less to do: the nuclear weights of a
+// window can lie at its opposite ends, where an element would take the chain all the same.
+// They stay on the FP64 pipe, with less to do: the nuclear weights of a
 // grid are summed first, and symmetric blocks are summed once.
 //
 // Measured on a bent triatomic (26 basis / 82 aux functions, 963,072 points; all sums on the FP64
