@@ -394,23 +394,38 @@ void row_constants(const psq_job* j, const DevGrid& g, int kind, std::vector<dou
 }
 
 // The evaluation CTAs of grid g: all node pairs of a column and all its phi rows where their tables
-// fit the CTA's shared memory, else fewer pairs, then fewer phi rows; the phi rows in at least `split`
-// parts (as far as there are rows).
+// fit the CTA's shared memory, else fewer pairs, then fewer phi rows, then fewer shells (about 3,070 shells of
+// a pair, or 380 of a third centre at Q_phi = 16, fill the tables of one node pair and phi row); the phi
+// rows in at least `split` parts (as far as there are rows).
 void point_blocks(int gi, const DevGrid& g, int split, std::vector<PointBlock>& out) {
   const bool third = g.C >= 0;
-  const int pair_entries = 2 * ((g.shb_A1 - g.shb_A0) + (g.shb_B1 - g.shb_B0) +
-                                (third ? 0 : (g.sha_1 - g.sha_0) + (g.sha_3 - g.sha_2)));
-  const int node_entries = third ? g.sha_1 - g.sha_0 + 1 : 0;  // per phi node (and its distance from the centre)
+  const int n_basis = (g.shb_A1 - g.shb_A0) + (g.shb_B1 - g.shb_B0), n_aux = (g.sha_1 - g.sha_0) + (g.sha_3 - g.sha_2);
+  const int shells = n_basis + n_aux, n_pair = third ? n_basis : shells;  // the first n_pair have a value per node pair
+  const int node_entries = third ? n_aux + 1 : 0;  // per phi node (and its distance from the centre)
   const int budget = kEvalTabBytes / 8, np = g.q_mu * g.q_nu;
   int npb = np;
-  while (npb > 1 && (pair_entries + g.q_phi * node_entries) * npb > budget) npb = (npb + 1) / 2;
+  while (npb > 1 && (2 * (int64_t)n_pair + g.q_phi * (int64_t)node_entries) * npb > budget) npb = (npb + 1) / 2;
+  // ranges of shells whose tables fit with npb node pairs and one phi row
+  std::vector<int> ends;
+  int64_t used = third ? g.q_phi : 0;
+  for (int s = 0; s < shells; ++s) {
+    const int more = s < n_pair ? 2 : g.q_phi;
+    if ((used + more) * npb > budget) {
+      ends.push_back(s);
+      used = third ? g.q_phi : 0;
+    }
+    used += more;
+  }
+  ends.push_back(shells);
   auto column = [&](int col, int rows) {
     const int half = (rows + 1) / 2;
     int hc = std::min((half + split - 1) / split, std::max(1, kEvalMaxNodes / g.q_phi));
-    if (node_entries) hc = std::max(1, std::min(hc, (budget / npb - pair_entries) / (g.q_phi * node_entries)));
+    if (ends.size() > 1) hc = 1;
+    else if (node_entries) hc = std::max(1, std::min(hc, (budget / npb - 2 * n_pair) / (g.q_phi * node_entries)));
     for (int u = 0; u < half; u += hc)
       for (int q = 0; q < np; q += npb)
-        out.push_back(PointBlock{gi, col, u, std::min(half, u + hc), (short)q, (short)std::min(np, q + npb)});
+        for (size_t k = 0; k < ends.size(); ++k)
+          out.push_back(PointBlock{gi, col, u, std::min(half, u + hc), (short)q, (short)std::min(np, q + npb), k ? ends[k - 1] : 0, ends[k]});
   };
   for (int c = 0; c < g.n_mu * g.n_nu; ++c) column(c, g.n_phi);
   if (g.n_touch > 0)

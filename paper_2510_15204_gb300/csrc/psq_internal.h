@@ -174,11 +174,36 @@ struct J3Src { int64_t off; int s_pair, s_aux, mode, nloc, offY, offW; };
 // its phi rows (columns 0 .. n_mu n_nu - 1: the volume elements; then the (mu, nu) sub-row pairs of
 // the split ones).  The CTA takes the (mu, nu) node pairs [pr0, pr1) of the column (pair = i q_nu + j)
 // and the phi rows [u0, u1) of the first half with their mirror rows: the grid is symmetric under
-// phi -> -phi, and so is the distance from a third centre (which lies at phi = 0).
+// phi -> -phi, and so is the distance from a third centre (which lies at phi = 0).  It evaluates the shells
+// [s0, s1) of the grid's (basis of A, of B, aux of the first centre, of the second): all of them where
+// the tables of one node pair and one phi row fit, else the CTAs of other ranges take the rest.
 struct PointBlock {
   int grid, col, u0, u1;
   short pr0, pr1;
+  int s0, s1;
 };
+// The shells of centre c (A, B, C) that an evaluation CTA takes: basis shells [b0, b1), shell s at entry
+// s + bt of the CTA's tables, and aux shells [a0, a1), entry s + at.
+struct CentreShells {
+  int b0, b1, bt, a0, a1, at;
+};
+inline
+#ifdef __CUDACC__
+    __host__ __device__
+#endif
+    CentreShells centre_shells(const DevGrid& g, const PointBlock& pb, int c) {
+  const int nbA = g.shb_A1 - g.shb_A0, nb = nbA + g.shb_B1 - g.shb_B0, na0 = g.sha_1 - g.sha_0;
+  auto part = [&](int s0, int s1, int at, int& lo, int& hi) {  // shells [s0, s1), the grid's at-th and on
+    lo = s0 + pb.s0 - at > s0 ? s0 + pb.s0 - at : s0;
+    hi = s0 + pb.s1 - at < s1 ? s0 + pb.s1 - at : s1;
+    return at - s0 - pb.s0;  // entry of shell 0
+  };
+  CentreShells r{};
+  if (c < 2) r.bt = c == 0 ? part(g.shb_A0, g.shb_A1, 0, r.b0, r.b1) : part(g.shb_B0, g.shb_B1, nbA, r.b0, r.b1);
+  r.at = c == 1 ? part(g.sha_2, g.sha_3, nb + na0, r.a0, r.a1) : part(g.sha_0, g.sha_1, nb, r.a0, r.a1);
+  if (c == 2) r.at = (pb.s0 > nb ? nb - pb.s0 : 0) - g.sha_0;  // C's own table starts with its first shell here
+  return r;
+}
 // Shared memory of an evaluation CTA: values kept per (node pair, shell and kind) and, for a third
 // centre, per (node pair, phi node, shell).
 constexpr int kEvalThreads = 256, kEvalTabBytes = 48 << 10, kEvalMaxNodes = 256;  // phi nodes of [u0, u1)

@@ -234,10 +234,11 @@ struct EvalNodes {
   double nu[kMaxQ][5];             // sin, cos, sin^2(v/2), cos^2(v/2), weight
   double ph[2 * kEvalMaxNodes][3];  // sin, cos, weight: the rows [u0, u1), then their mirrors
   int meta[4];                     // lmax of A, B, C; functions of the first aux centre
+  CentreShells shells[3];
 };
 constexpr int kEvalFp64Smem = (int)sizeof(EvalNodes) + kEvalTabBytes;
 
-__global__ void __launch_bounds__(kEvalThreads) eval_fp64_kernel(LaunchTables t, double* __restrict__ ops) {
+__global__ void __launch_bounds__(kEvalThreads, 3) eval_fp64_kernel(LaunchTables t, double* __restrict__ ops) {
   extern __shared__ __align__(16) uint8_t raw[];
   EvalNodes& nd = *reinterpret_cast<EvalNodes*>(raw);
   const int tid = threadIdx.x;
@@ -249,7 +250,9 @@ __global__ void __launch_bounds__(kEvalThreads) eval_fp64_kernel(LaunchTables t,
   const bool basis = g.row_F >= 0 || g.row_L >= 0, aux = g.row_G >= 0 || g.row_U >= 0;
   const int n_pair = nbA + nbB + (third ? 0 : na0 + na1);  // shells with a value per node pair
   double* tp = reinterpret_cast<double*>(raw + sizeof(EvalNodes));  // [2 shell + kind][pair]
-  double* tr = tp + 2 * n_pair * np;                                // [phi node][pair]: distance from C
+  const int p0 = min(pb.s0, n_pair), p1 = min(pb.s1, n_pair);       // this CTA's shells: of those,
+  const int q0 = third ? max(pb.s0 - n_pair, 0) : 0, q1 = third ? max(pb.s1 - n_pair, 0) : 0;  // and of C
+  double* tr = tp + 2 * (p1 - p0) * np;                             // [phi node][pair]: distance from C
   double* tc = tr + (third ? nn * np : 0);                          // [shell of C][phi node][pair]
   // the column: its element rows, its points, its phi rows
   const int nreg = g.n_mu * g.n_nu, ns = g.n_sp, q3 = g.q_mu * g.q_nu * g.q_phi;
@@ -329,6 +332,7 @@ __global__ void __launch_bounds__(kEvalThreads) eval_fp64_kernel(LaunchTables t,
     int nf = 0;
     for (int s = g.sha_0; s < g.sha_1; ++s) nf += 2 * t.ashell[s].l + 1;
     nd.meta[3] = nf;
+    for (int c = 0; c < 3; ++c) nd.shells[c] = centre_shells(g, pb, c);
   }
   __syncthreads();
   const double a = g.a;
@@ -340,24 +344,24 @@ __global__ void __launch_bounds__(kEvalThreads) eval_fp64_kernel(LaunchTables t,
       tr[e] = sqrt(x * x + y * y + z * z);
     }
   // radial factors per node pair
-  for (int e = tid; e < n_pair * np; e += kEvalThreads) {
-    const int s = e / np, pq = e - s * np, pr = pb.pr0 + pq, qi = pr / g.q_nu, qj = pr - qi * g.q_nu;
+  for (int e = tid; e < (p1 - p0) * np; e += kEvalThreads) {
+    const int i = e / np, s = p0 + i, pq = e - i * np, pr = pb.pr0 + pq, qi = pr / g.q_nu, qj = pr - qi * g.q_nu;
     const bool isb = s < nbA + nbB, onA = isb ? s < nbA : s < nbA + nbB + na0;
     if (isb ? !basis : !aux) continue;
     const DevShell& q = isb ? t.bshell[s < nbA ? g.shb_A0 + s : g.shb_B0 + s - nbA]
                             : t.ashell[onA ? g.sha_0 + s - nbA - nbB : g.sha_2 + s - nbA - nbB - na0];
     const double r = 2.0 * a * (nd.mu[qi][2] + nd.nu[qj][onA ? 2 : 3]), ex = exp(-q.zeta * r), ir = 1.0 / r;
     const bool ka = isb ? g.row_F >= 0 : g.row_G >= 0, kb = isb ? g.row_L >= 0 : g.row_U >= 0;
-    if (ka) tp[2 * s * np + pq] = radial_value(q, 0, r, ir, ex);
-    if (kb) tp[(2 * s + 1) * np + pq] = radial_value(q, isb ? 1 : 2, r, ir, ex);
+    if (ka) tp[2 * i * np + pq] = radial_value(q, 0, r, ir, ex);
+    if (kb) tp[(2 * i + 1) * np + pq] = radial_value(q, isb ? 1 : 2, r, ir, ex);
   }
   if (third && aux) {
     __syncthreads();
     const int kind = g.row_U >= 0 ? 2 : 0;  // (a refined grid has one aux kind)
-    for (int e = tid; e < na0 * nn * np; e += kEvalThreads) {
-      const int s = e / (nn * np);
-      const DevShell& q = t.ashell[g.sha_0 + s];
-      const double r = tr[e - s * nn * np];
+    for (int e = tid; e < (q1 - q0) * nn * np; e += kEvalThreads) {
+      const int i = e / (nn * np);
+      const DevShell& q = t.ashell[g.sha_0 + q0 + i];
+      const double r = tr[e - i * nn * np];
       tc[e] = radial_value(q, kind, r, 0.0, exp(-q.zeta * r));
     }
   }
@@ -390,20 +394,21 @@ __global__ void __launch_bounds__(kEvalThreads) eval_fp64_kernel(LaunchTables t,
       // the nuclear weights that V_ne elements of this grid are summed with: on a pair grid those of the
       // A x B elements and the square roots of those of the A x A and B x B elements (an atom's own
       // nucleus only on its one-centre grid), on a refined grid the third nucleus's
-      if (g.n_W == 3) {
+      // (written with the first shells)
+      if (g.n_W == 3 && pb.s0 == 0) {
         const double wa = g.zA / rA, wb = g.zB / rB;
         base[(int64_t)(g.row_W + 0) * rs + p] = wa + wb;
         base[(int64_t)(g.row_W + 1) * rs + p] = sqrt(g.own_A ? wa + wb : wb);
         base[(int64_t)(g.row_W + 2) * rs + p] = sqrt(g.own_B ? wa + wb : wa);
-      } else if (g.n_W == 1) {
+      } else if (g.n_W == 1 && pb.s0 == 0) {
         base[(int64_t)g.row_W * rs + p] = g.zC / rC;
       }
     }
     const double x = a * sh * sn * ph[1], y = a * sh * sn * ph[0];
 #pragma unroll 1
     for (int ctr = 0; ctr < 3; ++ctr) {  // A, B, C
-      const int b0 = ctr == 0 ? g.shb_A0 : g.shb_B0, b1 = ctr == 0 ? g.shb_A1 : g.shb_B1;
-      const int a0 = ctr == 1 ? g.sha_2 : g.sha_0, a1 = ctr == 1 ? g.sha_3 : g.sha_1;
+      const CentreShells& own = nd.shells[ctr];
+      const int b0 = own.b0, b1 = own.b1, a0 = own.a0, a1 = own.a1;
       const bool hb = basis && ctr < 2 && b1 > b0, ha = aux && (ctr == 2) == third && a1 > a0;
       if (!hb && !ha) continue;
       const double ir = 1.0 / (ctr == 0 ? rA : (ctr == 1 ? rB : rC));
@@ -412,23 +417,23 @@ __global__ void __launch_bounds__(kEvalThreads) eval_fp64_kernel(LaunchTables t,
       real_ylm(nd.meta[ctr], g.R[0] * dx + g.R[1] * dy + g.R[2] * dz, g.R[3] * dx + g.R[4] * dy + g.R[5] * dz,
                g.R[6] * dx + g.R[7] * dy + g.R[8] * dz, Y);
       if (hb) {
-        const int roff = ctr == 0 ? 0 : g.nFA, e0 = ctr == 0 ? 0 : nbA;
+        const int roff = ctr == 0 ? 0 : g.nFA;
         for (int s = b0; s < b1; ++s) {
           const DevShell& q = t.bshell[s];
-          const double* tv = tp + 2 * (e0 + s - b0) * np + pq;
+          const double* tv = tp + 2 * (s + own.bt) * np + pq;
           if (g.row_F >= 0) store_shell(q, wf * tv[0], Y, base, rs, p, g.row_F + roff);
           if (g.row_L >= 0) store_shell(q, wf * tv[np], Y, base, rs, p, g.row_L + roff);
         }
       }
       if (ha) {
-        const int roff = ctr == 1 ? nd.meta[3] : 0, e0 = nbA + nbB + (ctr == 1 ? na0 : 0);
+        const int roff = ctr == 1 ? nd.meta[3] : 0;
         for (int s = a0; s < a1; ++s) {
           const DevShell& q = t.ashell[s];
           if (ctr == 2) {
-            const double v = tc[((s - a0) * nn + f) * np + pq];
+            const double v = tc[((s + own.at) * nn + f) * np + pq];
             store_shell(q, g.row_U >= 0 ? v : wg * v, Y, base, rs, p, g.row_U >= 0 ? g.row_U : g.row_G);
           } else {
-            const double* tv = tp + 2 * (e0 + s - a0) * np + pq;
+            const double* tv = tp + 2 * (s + own.at) * np + pq;
             if (g.row_G >= 0) store_shell(q, wg * tv[0], Y, base, rs, p, g.row_G + roff);
             if (g.row_U >= 0) store_shell(q, tv[np], Y, base, rs, p, g.row_U + roff);
           }

@@ -203,6 +203,7 @@ __global__ void __launch_bounds__(kEvalThreads) eval_mixed_kernel(LaunchTables t
   extern __shared__ __align__(16) uint8_t raw[];
   __shared__ float2 etab[64];
   __shared__ int meta[5];  // lmax of A, B, C; functions of the first aux centre
+  __shared__ CentreShells shells[3];
   const int tid = threadIdx.x;
   if (tid < 64) etab[tid] = c_exp_tab[tid];
   const PointBlock pb = t.pblocks[blockIdx.x];
@@ -213,7 +214,9 @@ __global__ void __launch_bounds__(kEvalThreads) eval_mixed_kernel(LaunchTables t
   const bool basis = g.row_F >= 0 || g.row_L >= 0, aux = g.row_G >= 0 || g.row_U >= 0;
   const int n_pair = nbA + nbB + (third ? 0 : na0 + na1);  // shells with a value per node pair
   float2* tp = reinterpret_cast<float2*>(raw);             // [2 shell + kind][pair]
-  float2* tr = tp + 2 * n_pair * np;                       // [phi node][pair]: distance from C
+  const int p0 = min(pb.s0, n_pair), p1 = min(pb.s1, n_pair);  // this CTA's shells: of those,
+  const int q0 = third ? max(pb.s0 - n_pair, 0) : 0, q1 = third ? max(pb.s1 - n_pair, 0) : 0;  // and of C
+  float2* tr = tp + 2 * (p1 - p0) * np;                    // [phi node][pair]: distance from C
   float2* tc = tr + (third ? nn * np : 0);                 // [shell of C][phi node][pair]
   // the column's node rows
   const int nreg = g.n_mu * g.n_nu, ns = g.n_sp;
@@ -253,6 +256,7 @@ __global__ void __launch_bounds__(kEvalThreads) eval_mixed_kernel(LaunchTables t
     int nf = 0;
     for (int s = g.sha_0; s < g.sha_1; ++s) nf += 2 * t.ashell[s].l + 1;
     meta[3] = nf;
+    for (int c = 0; c < 3; ++c) shells[c] = centre_shells(g, pb, c);
   }
   // third centre: distances at the phi nodes of the half, FP64 offsets
   if (third) {
@@ -266,8 +270,8 @@ __global__ void __launch_bounds__(kEvalThreads) eval_mixed_kernel(LaunchTables t
   }
   __syncthreads();
   const float2* xi = xi_tab + g.xi_off;  // basis A, basis B, aux c0, aux c1 shells
-  for (int e = tid; e < n_pair * np; e += kEvalThreads) {
-    const int s = e / np, pq = e - s * np, pr = pb.pr0 + pq, qi = pr / g.q_nu, qj = pr - qi * g.q_nu;
+  for (int e = tid; e < (p1 - p0) * np; e += kEvalThreads) {
+    const int i = e / np, s = p0 + i, pq = e - i * np, pr = pb.pr0 + pq, qi = pr / g.q_nu, qj = pr - qi * g.q_nu;
     const bool isb = s < nbA + nbB, onA = isb ? s < nbA : s < nbA + nbB + na0;
     if (isb ? !basis : !aux) continue;
     const DevShell& q = isb ? t.bshell[s < nbA ? g.shb_A0 + s : g.shb_B0 + s - nbA]
@@ -277,19 +281,19 @@ __global__ void __launch_bounds__(kEvalThreads) eval_mixed_kernel(LaunchTables t
     const bool ka = isb ? g.row_F >= 0 : g.row_G >= 0, kb = isb ? g.row_L >= 0 : g.row_U >= 0;
     if (ka) {
       const df r = dfa::radial(0, q.n, q.l, x, ex, ix, c_factd, c_rcpf);
-      tp[2 * s * np + pq] = make_float2(r.h, r.l);
+      tp[2 * i * np + pq] = make_float2(r.h, r.l);
     }
     if (kb) {
       const df r = dfa::radial(isb ? 1 : 2, q.n, q.l, x, ex, ix, c_factd, c_rcpf);
-      tp[(2 * s + 1) * np + pq] = make_float2(r.h, r.l);
+      tp[(2 * i + 1) * np + pq] = make_float2(r.h, r.l);
     }
   }
   if (third && aux) {
     const int kind = g.row_U >= 0 ? 2 : 0;  // (a refined grid has one aux kind)
-    for (int e = tid; e < na0 * nn * np; e += kEvalThreads) {
-      const int s = e / (nn * np);
-      const DevShell& q = t.ashell[g.sha_0 + s];
-      const df x = dfa::mul(ld2(xi[nbA + nbB + s]), ld2(tr[e - s * nn * np]));
+    for (int e = tid; e < (q1 - q0) * nn * np; e += kEvalThreads) {
+      const int i = e / (nn * np);
+      const DevShell& q = t.ashell[g.sha_0 + q0 + i];
+      const df x = dfa::mul(ld2(xi[n_pair + q0 + i]), ld2(tr[e - i * nn * np]));
       const df r = dfa::radial(kind, q.n, q.l, x, dfa::exp_neg(x, c_expc, etab), dfa::rcp(x), c_factd, c_rcpf);
       tc[e] = make_float2(r.h, r.l);
     }
@@ -317,7 +321,7 @@ __global__ void __launch_bounds__(kEvalThreads) eval_mixed_kernel(LaunchTables t
     const df rhoA = dfa::add_same(s2m, s2n), rhoB = dfa::add_same(s2m, c2n);
     df rC = dfa::mk(1.0f);
     if (third) rC = ld2(tr[f * np + pq]);
-    if (g.row_W >= 0) {
+    if (g.row_W >= 0 && pb.s0 == 0) {
       df w = dfa::mk(0.0f);
       if (!dead) {
         const df gw = dfa::mul(dfa::mul(ld2(M.fw), ld2(N.fw)), ld2(F.fw));
@@ -333,8 +337,8 @@ __global__ void __launch_bounds__(kEvalThreads) eval_mixed_kernel(LaunchTables t
     const df xs = dfa::mul(shsn, ld2(F.fc)), ys = dfa::mul(shsn, ld2(F.fs)), s2mc = dfa::mul(s2m, ld2(N.fc));
 #pragma unroll 1
     for (int ctr = 0; ctr < 3; ++ctr) {  // A, B, C
-      const int b0 = ctr == 0 ? g.shb_A0 : g.shb_B0, b1 = ctr == 0 ? g.shb_A1 : g.shb_B1;
-      const int a0 = ctr == 1 ? g.sha_2 : g.sha_0, a1 = ctr == 1 ? g.sha_3 : g.sha_1;
+      const CentreShells& own = shells[ctr];
+      const int b0 = own.b0, b1 = own.b1, a0 = own.a0, a1 = own.a1;
       const bool hb = basis && ctr < 2 && b1 > b0, ha = aux && (ctr == 2) == third && a1 > a0;
       if (!hb && !ha) continue;
       df u3[3];
@@ -347,24 +351,24 @@ __global__ void __launch_bounds__(kEvalThreads) eval_mixed_kernel(LaunchTables t
       }
       dfa::real_ylm(meta[ctr], u3[0], u3[1], u3[2], Y, c_rcpf);
       if (hb) {
-        const int roff = ctr == 0 ? 0 : g.nFA, e0 = ctr == 0 ? 0 : nbA;
+        const int roff = ctr == 0 ? 0 : g.nFA;
 #pragma unroll 1
         for (int s = b0; s < b1; ++s) {
           const DevShell& q = t.bshell[s];
-          const float2* tv = tp + 2 * (e0 + s - b0) * np + pq;
+          const float2* tv = tp + 2 * (s + own.bt) * np + pq;
           if (g.row_F >= 0) store_shell(q, ld2(tv[0]), Y, bh, bl, rs, p, g.row_F + roff);
           if (g.row_L >= 0) store_shell(q, ld2(tv[np]), Y, bh, bl, rs, p, g.row_L + roff);
         }
       }
       if (ha) {
-        const int roff = ctr == 1 ? meta[3] : 0, e0 = nbA + nbB + (ctr == 1 ? na0 : 0);
+        const int roff = ctr == 1 ? meta[3] : 0;
 #pragma unroll 1
         for (int s = a0; s < a1; ++s) {
           const DevShell& q = t.ashell[s];
           if (ctr == 2) {
-            store_shell(q, ld2(tc[((s - a0) * nn + f) * np + pq]), Y, bh, bl, rs, p, g.row_U >= 0 ? g.row_U : g.row_G);
+            store_shell(q, ld2(tc[((s + own.at) * nn + f) * np + pq]), Y, bh, bl, rs, p, g.row_U >= 0 ? g.row_U : g.row_G);
           } else {
-            const float2* tv = tp + 2 * (e0 + s - a0) * np + pq;
+            const float2* tv = tp + 2 * (s + own.at) * np + pq;
             if (g.row_G >= 0) store_shell(q, ld2(tv[0]), Y, bh, bl, rs, p, g.row_G + roff);
             if (g.row_U >= 0) store_shell(q, ld2(tv[np]), Y, bh, bl, rs, p, g.row_U + roff);
           }
