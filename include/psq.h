@@ -192,18 +192,19 @@ psq_status psq_compute_noalloc(psq_job* job, unsigned mask, double* d_out[5], vo
 psq_status psq_check(psq_job* job, unsigned mask, void* d_workspace, void* stream);
 
 /* Failure detection (no paper counterpart): the limit, in nanoseconds, of every bounded wait
- * in the main loops of the tensor-core contraction for this job's later psq_compute calls
- * (default 4e9; 1 <= ns <= 6e10).  A wait that runs out makes the kernel record a status
+ * in the main loops of the tensor-core contractions (of both precisions) for this job's later
+ * psq_compute calls (default 4e9; 1 <= ns <= 6e10).  A wait that runs out makes the kernel record a status
  * (psq_check then returns PSQ_ERR_TIMEOUT), stop its loops, wait (4 s at most) for its own
  * copies and MMAs in flight, release its tensor memory and return: the context stays usable
  * and the next psq_compute starts afresh.  Graphs captured before keep the limit they were
  * captured with.  Errors: PSQ_ERR_ARG for a NULL job or a limit out of range. */
 psq_status psq_job_set_wait_limit(psq_job* job, uint64_t ns);
 
-/* Failure-detection test hook (no paper counterpart): while `on`, every psq_compute of a
- * PSQ_MIXED job raises a flag in its workspace that nothing clears; the contraction's loader
- * waits for it to clear, gives up when the wait limit runs out and the compute ends with
- * PSQ_ERR_TIMEOUT in psq_check, exercising the timeout path without a GPU fault.  Errors:
+/* Failure-detection test hook (no paper counterpart): while `on`, every psq_compute of
+ * the job raises a flag in its workspace that nothing clears; the tensor-core contraction (PSQ_FP64:
+ * of (P|Q) and (P|ij), which then read NaN) waits for it to clear, gives up when the wait limit runs
+ * out and the compute ends with PSQ_ERR_TIMEOUT in psq_check, exercising the timeout path without a
+ * GPU fault.  Errors:
  * PSQ_ERR_ARG for a NULL job. */
 psq_status psq_job_test_stall(psq_job* job, int on);
 
@@ -262,7 +263,9 @@ const char* psq_last_error(void);
  * the device, asynchronous on `stream` (a cudaStream_t; NULL = legacy default stream), on the
  * current device.  Matrices are row-major; the pair index of (P|ij) is ij = i * n_bf + j, so its
  * n_aux x n_bf x n_bf layout is B's n x m layout with m = n_bf^2.  The caller owns every
- * buffer.  Errors: PSQ_ERR_ARG for negative sizes, NULL or non-8-byte-aligned pointers with
+ * buffer.  The tensor-core products wait for their MMAs, 4 s at most: if that ever runs out,
+ * psq_ri_solve leaves NaN in the columns concerned and psq_ri_eri in the elements (they have no
+ * status word).  Errors: PSQ_ERR_ARG for negative sizes, NULL or non-8-byte-aligned pointers with
  * nonzero sizes, or column ranges outside [0, m); PSQ_ERR_CUDA on a failed launch. */
 
 /* Cholesky factor of the symmetric positive definite n x n matrix d_J2 (its lower triangle is

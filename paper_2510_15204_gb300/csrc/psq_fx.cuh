@@ -186,7 +186,7 @@ struct Scale {
 template <typename Chain>
 __device__ __forceinline__ bool window(Smem& sm, uint32_t tmem, double (&va)[4][8], double (&vb)[2][4],
                                        double (&acc)[16], uint32_t& phase, uint32_t win, int rows, int cols, bool& ok,
-                                       Chain chain) {
+                                       Chain chain, uint64_t wait_ns = mma::kWaitNs) {
   constexpr unsigned kFull = 0xffffffffu;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int set = win & 1;
@@ -239,7 +239,7 @@ __device__ __forceinline__ bool window(Smem& sm, uint32_t tmem, double (&va)[4][
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
     if (c == 1 && ok) {
-      ok = mma::mbar_wait(mma::smem_u32(&sm.done), phase & 1);
+      ok = mma::mbar_wait(mma::smem_u32(&sm.done), phase & 1, nullptr, wait_ns);
       phase += ok ? 1u : 0u;
     }
 #pragma unroll
@@ -269,7 +269,7 @@ __device__ __forceinline__ bool window(Smem& sm, uint32_t tmem, double (&va)[4][
       mma::mma_commit(mma::smem_u32(&sm.done));
     }
   }
-  ok = mma::mbar_wait(mma::smem_u32(&sm.done), phase & 1);
+  ok = mma::mbar_wait(mma::smem_u32(&sm.done), phase & 1, nullptr, wait_ns);
   phase += ok ? 1u : 0u;
   if (!__all_sync(kFull, ok)) { ok = false; return true; }
   mma::fence_after();

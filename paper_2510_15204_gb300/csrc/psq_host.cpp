@@ -1757,7 +1757,8 @@ psq_status run_plan(psq_job* job, Plan* P, unsigned mask, char* ws, double* d_ou
     CUDA_TRY(mark(job, 1, s));
     CUDA_TRY(launch_eval_fp64(t, ops, 0, s));
     CUDA_TRY(mark(job, 2, s));
-    CUDA_TRY(launch_contract_fp64(t, ops, part, s));
+    int* status = (int*)(ws + P->o_status);
+    CUDA_TRY(launch_contract_fp64(t, ops, part, status, job->wait_ns, job->test_stall ? status + 1 : nullptr, s));
     CUDA_TRY(mark(job, 3, s));
     CUDA_TRY(launch_reduce(t, part, res, s));
   }

@@ -231,7 +231,9 @@ struct LaunchTables {
 cudaError_t prepare_kernels_fp64();  // per-device kernel attributes (context creation)
 void upload_gl_tables(const double* x, const double* w, const double* klm);  // host constants
 cudaError_t launch_eval_fp64(const LaunchTables& t, double* ops, int kinds, cudaStream_t s);
-cudaError_t launch_contract_fp64(const LaunchTables& t, const double* ops, double* part, cudaStream_t s);
+// status, wait_ns, hold: as launch_contract_ws; every CTA of the tensor-core sums heeds hold (NULL: none raised).
+cudaError_t launch_contract_fp64(const LaunchTables& t, const double* ops, double* part, int* status, uint64_t wait_ns,
+                                 const int* hold, cudaStream_t s);
 cudaError_t launch_reduce(const LaunchTables& t, const double* part, double* res, cudaStream_t s);
 // shells / fn_shell (S and T only, else NULL): the basis shells and each function's shell,
 // for the one-centre elements, which take their closed forms.

@@ -605,7 +605,8 @@ __device__ __forceinline__ void contract_fma(const LaunchTables& t, const GemmIt
 }
 
 __global__ void __launch_bounds__(fx::kThreads, 2) contract_fp64_kernel(LaunchTables t, const double* __restrict__ ops,
-                                                                        double* __restrict__ part) {
+                                                                        double* __restrict__ part, int* __restrict__ status,
+                                                                        uint64_t wait_ns, const int* hold) {
   extern __shared__ __align__(1024) uint8_t raw[];
   const GemmItem it = t.items[blockIdx.x];
   const GemmBlock b = t.gblocks[it.block];
@@ -645,6 +646,15 @@ __global__ void __launch_bounds__(fx::kThreads, 2) contract_fp64_kernel(LaunchTa
   double acc[16] = {};
   uint32_t phase = 0, win = 0;
   bool ok = true, run = true;
+  bool issued = true;  // (no MMA in flight where none was)
+  if (hold) {  // failure-detection test: a raised flag holds the CTA back until the wait limit runs out
+    if (threadIdx.x == 0) {
+      const uint64_t t0 = mma::global_ns();
+      while ((ok = *(volatile const int*)hold == 0) == false && mma::global_ns() - t0 <= wait_ns) {
+      }
+    }
+    issued = run = __syncthreads_and(ok);
+  }
   for (int k = k0; k < k1 && run; k += kFpWin, ++win) {
     double va[4][8], vb[2][4];
     const double* win0 = base + (int64_t)(k >> 7) * g.ws + (k & 127);  // the window's first point (row 0)
@@ -694,18 +704,19 @@ __global__ void __launch_bounds__(fx::kThreads, 2) contract_fp64_kernel(LaunchTa
         for (int p = k; p < min(k1, k + kFpWin); ++p) s = fma(value(qa, p), value(qb, p), s);
       }
       return s;
-    });
+    }, wait_ns);
   }
   if (run) run = __syncthreads_and(ok);
+  if (!run && threadIdx.x == 0) atomicCAS(status, 0, 9);  // a wait that ran out (the first failure's code stays)
   double* out = part + b.part_off + (int64_t)it.chunk * b.m * b.n;
   const int r = 32 * (warp & 3) + lane;
 #pragma unroll
   for (int j = 0; j < 16; ++j) {
     const int c = 16 * (warp >> 2) + j;
-    // a wait that ran out leaves NaN: no result is better than a wrong one
+    // a wait that ran out leaves NaN as well: no result is better than a wrong one
     if (r < rows && c < cols) out[(int64_t)(r0 + r) * b.n + c0 + c] = run ? acc[j] : __longlong_as_double(0x7ff8000000000000ll);
   }
-  fx::close(sm, tmem, run, phase);
+  fx::close(sm, tmem, run || !issued, phase);
 }
 
 cudaError_t prepare_kernels_fp64() {
@@ -716,9 +727,10 @@ cudaError_t prepare_kernels_fp64() {
   return e != cudaSuccess ? e : cudaFuncSetAttribute(contract_fp64_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 80);
 }
 
-cudaError_t launch_contract_fp64(const LaunchTables& t, const double* ops, double* part, cudaStream_t s) {
+cudaError_t launch_contract_fp64(const LaunchTables& t, const double* ops, double* part, int* status, uint64_t wait_ns,
+                                 const int* hold, cudaStream_t s) {
   if (t.n_items == 0) return cudaSuccess;
-  contract_fp64_kernel<<<t.n_items, fx::kThreads, fx::kSmemBytes, s>>>(t, ops, part);
+  contract_fp64_kernel<<<t.n_items, fx::kThreads, fx::kSmemBytes, s>>>(t, ops, part, status, wait_ns, hold);
   return cudaGetLastError();
 }
 
