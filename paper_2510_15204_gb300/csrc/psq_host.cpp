@@ -121,7 +121,7 @@ struct Plan {
   std::vector<PointBlock> pblocks;
   std::vector<GemmBlock> gblocks;
   std::vector<GemmItem> items;
-  std::vector<short2> pairs;
+  std::vector<int2> pairs;
   std::vector<int64_t> elem_begin;
   // assembly sources
   std::vector<SrcEntry> src[4];
@@ -522,7 +522,7 @@ psq_status make_plan(psq_job* j, unsigned mask, Plan& P) {
       return k.A == g.A && k.B == g.B && k.C == -1;
     };
     auto add_rows = [&](int row0, int n, int w) {
-      for (int i = 0; i < n; ++i) P.pairs.push_back(make_short2(row0 + i, w));
+      for (int i = 0; i < n; ++i) P.pairs.push_back(make_int2(row0 + i, w));
     };
     auto add_block = [&](int g, int kind, int a_off, int m, int b_off, int n) {
       GemmBlock b{};
@@ -600,7 +600,7 @@ psq_status make_plan(psq_job* j, unsigned mask, Plan& P) {
               first[c] = list() - a_off;
               const int y0 = Y == g.A ? FA : FB, w0 = Wt == g.A ? FA : FB;
               for (int i = 0; i < j->nb[Y]; ++i)
-                for (int jj = Y == Wt ? i : 0; jj < j->nb[Wt]; ++jj) P.pairs.push_back(make_short2(y0 + i, w0 + jj));
+                for (int jj = Y == Wt ? i : 0; jj < j->nb[Wt]; ++jj) P.pairs.push_back(make_int2(y0 + i, w0 + jj));
             }
             const int m = list() - a_off, b_off = list();
             if (m == 0) continue;
@@ -623,7 +623,7 @@ psq_status make_plan(psq_job* j, unsigned mask, Plan& P) {
         if ((mask & PSQ_J3) && j->na[g.C] > 0) {
           const int a_off = list(), nx = j->na[g.C];
           for (int i = 0; i < nA; ++i)
-            for (int jj = 0; jj < nB; ++jj) P.pairs.push_back(make_short2(FA + i, FB + jj));
+            for (int jj = 0; jj < nB; ++jj) P.pairs.push_back(make_int2(FA + i, FB + jj));
           const int b_off = list();
           add_rows(g.row_U, nx, -1);
           const int64_t off = add_block(gint, kFpDigits, a_off, nA * nB, b_off, nx);
@@ -800,7 +800,7 @@ psq_status make_plan(psq_job* j, unsigned mask, Plan& P) {
           int order[kPairTileRows], place[kPairTileRows];
           for (int k = 0; k < t.nrows; ++k) order[k] = k;
           std::sort(order, order + t.nrows, [&](int x, int y) { return t.rows[x] < t.rows[y]; });
-          short rows[kPairTileRows];
+          int rows[kPairTileRows];
           for (int k = 0; k < t.nrows; ++k) {
             rows[k] = t.rows[order[k]];
             place[order[k]] = k;
@@ -823,9 +823,9 @@ psq_status make_plan(psq_job* j, unsigned mask, Plan& P) {
         const int need = (slot(pr.x) < 0) + (pr.y != pr.x && slot(pr.y) < 0);
         if (t.ncols == kMmaN || t.nrows + need > kPairTileRows) flush();
         int sx = slot(pr.x);
-        if (sx < 0) { sx = t.nrows; t.rows[t.nrows++] = (short)pr.x; }
+        if (sx < 0) { sx = t.nrows; t.rows[t.nrows++] = pr.x; }
         int sy = slot(pr.y);
-        if (sy < 0) { sy = t.nrows; t.rows[t.nrows++] = (short)pr.y; }
+        if (sy < 0) { sy = t.nrows; t.rows[t.nrows++] = pr.y; }
         t.dx[t.ncols] = (unsigned char)sx;
         t.dy[t.ncols] = (unsigned char)sy;
         t.col[t.ncols] = pr.col;
@@ -850,7 +850,7 @@ psq_status make_plan(psq_job* j, unsigned mask, Plan& P) {
         int pu[2] = {-1, -1}, u_off = -1;
         if (j3 || j2) {
           u_off = (int)P.pairs.size();
-          for (int q = 0; q < g.nG; ++q) P.pairs.push_back(make_short2(g.row_U + q, W));
+          for (int q = 0; q < g.nG; ++q) P.pairs.push_back(make_int2(g.row_U + q, W));
           if (split) {
             pu[0] = add_panel((int)gi, u_off, naA, kMmaM);
             pu[1] = add_panel((int)gi, u_off + naA, naB, kMmaM);
@@ -862,7 +862,7 @@ psq_status make_plan(psq_job* j, unsigned mask, Plan& P) {
           // all local pairs i <= j, result columns in packed row-major order
           const int b_off = (int)P.pairs.size();
           for (int i = 0; i < nl; ++i)
-            for (int jj = i; jj < nl; ++jj) P.pairs.push_back(make_short2(g.row_F + i, g.row_F + jj));
+            for (int jj = i; jj < nl; ++jj) P.pairs.push_back(make_int2(g.row_F + i, g.row_F + jj));
           // pair tiles per class (A,A), (A,B), (B,B), in that order, each in 6 x 8 blocks of
           // (i, j): 48 columns from at most 14 distinct rows
           const int nA = g.nFA;
@@ -905,28 +905,28 @@ psq_status make_plan(psq_job* j, unsigned mask, Plan& P) {
           const int a_off = (int)P.pairs.size();
           if (mask & PSQ_T) {
             gb.rowT = 0;
-            for (int i = 0; i < nl; ++i) P.pairs.push_back(make_short2(g.row_L + i, W));
+            for (int i = 0; i < nl; ++i) P.pairs.push_back(make_int2(g.row_L + i, W));
           }
           if (mask & PSQ_S) {
             gb.rowS = (int)P.pairs.size() - a_off;
-            for (int i = 0; i < nl; ++i) P.pairs.push_back(make_short2(g.row_F + i, W));
+            for (int i = 0; i < nl; ++i) P.pairs.push_back(make_int2(g.row_F + i, W));
           }
           if (mask & PSQ_V) {
             gb.rowVA = (int)P.pairs.size() - a_off;
-            for (int i = 0; i < nl; ++i) P.pairs.push_back(make_short2(g.row_F + i, W + 1));
+            for (int i = 0; i < nl; ++i) P.pairs.push_back(make_int2(g.row_F + i, W + 1));
             gb.rowVB = (int)P.pairs.size() - a_off;
-            for (int i = 0; i < nl; ++i) P.pairs.push_back(make_short2(g.row_F + i, W + 2));
+            for (int i = 0; i < nl; ++i) P.pairs.push_back(make_int2(g.row_F + i, W + 2));
           }
           const int na_rows = (int)P.pairs.size() - a_off;
           const int pk = add_panel((int)gi, a_off, na_rows, kMmaM);
           const int b_off = (int)P.pairs.size();
-          for (int i = 0; i < nl; ++i) P.pairs.push_back(make_short2(g.row_F + i, -1));
+          for (int i = 0; i < nl; ++i) P.pairs.push_back(make_int2(g.row_F + i, -1));
           const int pf = add_panel((int)gi, b_off, nl, kMmaN);
           gb.kin = add_mblock((int)gi, na_rows, nl, a_off, b_off, pk, pf, -1, 0);
         }
         if (j2) {
           const int b_off = (int)P.pairs.size();
-          for (int q = 0; q < g.nG; ++q) P.pairs.push_back(make_short2(g.row_G + q, -1));
+          for (int q = 0; q < g.nG; ++q) P.pairs.push_back(make_int2(g.row_G + q, -1));
           const int pg = add_panel((int)gi, b_off, g.nG, kMmaN);
           if (split) {  // rows of A, then rows of B (consecutive results, as one nG x nG block)
             gb.j2 = add_mblock((int)gi, naA, g.nG, u_off, b_off, pu[0], pg, -1, 0);
@@ -940,13 +940,13 @@ psq_status make_plan(psq_job* j, unsigned mask, Plan& P) {
         if (j3 || (mask & PSQ_V)) {
           const int a_off = (int)P.pairs.size();
           if (j3)
-            for (int q = 0; q < g.nG; ++q) P.pairs.push_back(make_short2(g.row_U + q, W));
-          if (mask & PSQ_V) { gb.rowVC = (int)P.pairs.size() - a_off; P.pairs.push_back(make_short2(W + 3, -1)); }
+            for (int q = 0; q < g.nG; ++q) P.pairs.push_back(make_int2(g.row_U + q, W));
+          if (mask & PSQ_V) { gb.rowVC = (int)P.pairs.size() - a_off; P.pairs.push_back(make_int2(W + 3, -1)); }
           const int na_rows = (int)P.pairs.size() - a_off;
           const int pc = add_panel((int)gi, a_off, na_rows, kMmaM);
           const int b_off = (int)P.pairs.size();
           for (int i = 0; i < g.nFA; ++i)
-            for (int jj = 0; jj < g.nFB; ++jj) P.pairs.push_back(make_short2(g.row_F + i, g.row_F + g.nFA + jj));
+            for (int jj = 0; jj < g.nFB; ++jj) P.pairs.push_back(make_int2(g.row_F + i, g.row_F + g.nFA + jj));
           std::vector<PairRef> pl;
           for (int ib = 0; ib < g.nFA; ib += 6)
             for (int jb = 0; jb < g.nFB; jb += 8)
@@ -1302,7 +1302,7 @@ psq_status make_plan(psq_job* j, unsigned mask, Plan& P) {
   P.o_pb = sec(sizeof(PointBlock) * P.pblocks.size());
   P.o_gb = sec(sizeof(GemmBlock) * P.gblocks.size());
   P.o_it = sec(sizeof(GemmItem) * P.items.size());
-  P.o_pairs = sec(sizeof(short2) * P.pairs.size());
+  P.o_pairs = sec(sizeof(int2) * P.pairs.size());
   P.o_eb = sec(sizeof(int64_t) * P.elem_begin.size());
   P.o_fa = sec(sizeof(int) * j->fn_atom.size());
   P.o_fl = sec(sizeof(int) * j->fn_local.size());
@@ -1363,7 +1363,7 @@ psq_status make_plan(psq_job* j, unsigned mask, Plan& P) {
   put(P.o_pb, P.pblocks.data(), sizeof(PointBlock) * P.pblocks.size());
   put(P.o_gb, P.gblocks.data(), sizeof(GemmBlock) * P.gblocks.size());
   put(P.o_it, P.items.data(), sizeof(GemmItem) * P.items.size());
-  put(P.o_pairs, P.pairs.data(), sizeof(short2) * P.pairs.size());
+  put(P.o_pairs, P.pairs.data(), sizeof(int2) * P.pairs.size());
   put(P.o_eb, P.elem_begin.data(), sizeof(int64_t) * P.elem_begin.size());
   put(P.o_fa, j->fn_atom.data(), sizeof(int) * j->fn_atom.size());
   put(P.o_fl, j->fn_local.data(), sizeof(int) * j->fn_local.size());
@@ -1443,7 +1443,7 @@ LaunchTables tables_at(const Plan& P, char* ws) {
   t.n_gblocks = (int)P.gblocks.size();
   t.items = (const GemmItem*)(ws + P.o_it);
   t.n_items = (int)P.items.size();
-  t.pairs = (const short2*)(ws + P.o_pairs);
+  t.pairs = (const int2*)(ws + P.o_pairs);
   t.elem_begin = (const int64_t*)(ws + P.o_eb);
   t.n_elems = P.elem_begin.empty() ? 0 : P.elem_begin.back();
   return t;

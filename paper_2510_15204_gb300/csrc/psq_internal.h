@@ -122,7 +122,7 @@ constexpr int kPackHintJobs = 256;  // packing jobs per entry of a wave's panel 
 constexpr int kPairTileRows = 16;
 struct PairTile {
   int ncols, nrows;
-  short rows[kPairTileRows];
+  int rows[kPairTileRows];
   unsigned char dx[kMmaN], dy[kMmaN];
   int col[kMmaN];
 };
@@ -224,7 +224,7 @@ struct LaunchTables {
   int n_gblocks;
   const GemmItem* items;
   int n_items;
-  const short2* pairs;
+  const int2* pairs;
   const int64_t* elem_begin;  // prefix sums of m*n over blocks (n_gblocks + 1)
   int64_t n_elems;
 };
@@ -255,7 +255,7 @@ cudaError_t prepare_kernels();  // per-device kernel attributes (context creatio
 // hint: per block of kPackHintJobs jobs (numbered from 0 in panels[0]), the index of the panel
 // holding the block's first job (or NULL: bisection).
 cudaError_t launch_pack(const DevGrid* grids, const Panel* panels, int n_panels, const int* hint, int64_t n_jobs,
-                        const short2* rows, const float* ops, const float* ops_lo, uint8_t* packed, cudaStream_t s);
+                        const int2* rows, const float* ops, const float* ops_lo, uint8_t* packed, cudaStream_t s);
 // Packed panels of the RI 4-index product from FP64 rows (panels[0] from srcA, panels[1] from
 // srcB, rows of n values); n_jobs covers both panels' packing jobs.
 cudaError_t launch_ri_pack(const Panel* panels, int64_t n_jobs, const double* srcA, const double* srcB, int n,
@@ -270,7 +270,7 @@ cudaError_t launch_contract_ws(const DevGrid* grids, const MmaBlock* blocks, con
                                uint64_t wait_ns, const int* hold, cudaStream_t s);
 // Reduces the elements [e0, e1) of the blocks (prefix sums elem_begin).
 cudaError_t launch_reduce_mixed(const DevGrid* grids, const MmaBlock* blocks, int n_blocks, const int64_t* elem_begin,
-                                int64_t e0, int64_t e1, const short2* rows, const double* rowc, const float2* part,
+                                int64_t e0, int64_t e1, const int2* rows, const double* rowc, const float2* part,
                                 double* res, cudaStream_t s);
 
 // Host side (psq_host.cpp): psq_compute on a given workspace; with plan_must_exist the call

@@ -560,7 +560,7 @@ __device__ __forceinline__ void contract_fma(const LaunchTables& t, const GemmIt
     const bool rs = tid < kFpFmaRegs;
     const int i = rs ? tid : tid - kFpFmaRegs;
     if (i < (rs ? nr : nl)) {
-      const short2 q = t.pairs[(rs ? roff : loff) + i];
+      const int2 q = t.pairs[(rs ? roff : loff) + i];
       sm.x[tid] = q.x * g.rs;
       sm.y[tid] = q.y >= 0 ? q.y * g.rs : -1;
     }
@@ -630,16 +630,16 @@ __global__ void __launch_bounds__(fx::kThreads, 2) contract_fp64_kernel(LaunchTa
   int64_t ax[2], ay[2], bx, by;
 #pragma unroll
   for (int u = 0; u < 2; ++u) {
-    const short2 q = t.pairs[b.a_off + r0 + min(fx::a_row(u), rows - 1)];
+    const int2 q = t.pairs[b.a_off + r0 + min(fx::a_row(u), rows - 1)];
     ax[u] = q.x * rs;
     ay[u] = q.y >= 0 ? q.y * rs : -1;
   }
   {
-    const short2 q = t.pairs[b.b_off + c0 + min(fx::b_col(), cols - 1)];
+    const int2 q = t.pairs[b.b_off + c0 + min(fx::b_col(), cols - 1)];
     bx = q.x * rs;
     by = q.y >= 0 ? q.y * rs : -1;
   }
-  auto value = [&](short2 q, int p) {
+  auto value = [&](int2 q, int p) {
     const double* at = base + (int64_t)(p >> 7) * g.ws + (p & 127);
     return q.y >= 0 ? at[q.x * rs] * at[q.y * rs] : at[q.x * rs];
   };
@@ -700,7 +700,7 @@ __global__ void __launch_bounds__(fx::kThreads, 2) contract_fp64_kernel(LaunchTa
     run = fx::window(sm, tmem, va, vb, acc, phase, win, rows, cols, ok, [&](int r, int c) {
       double s = 0.0;
       if (r < rows && c < cols) {
-        const short2 qa = t.pairs[b.a_off + r0 + r], qb = t.pairs[b.b_off + c0 + c];
+        const int2 qa = t.pairs[b.a_off + r0 + r], qb = t.pairs[b.b_off + c0 + c];
         for (int p = k; p < min(k1, k + kFpWin); ++p) s = fma(value(qa, p), value(qb, p), s);
       }
       return s;

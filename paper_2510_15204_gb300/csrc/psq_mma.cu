@@ -576,7 +576,7 @@ __device__ __forceinline__ void pack_store(const PackPos& P, const Panel& pn, co
 // half; with four points of each chunk it uses them whole (and 64 registers instead of 70: eight CTAs
 // per SM).  Whole steps before -> after: bent triatomic 1.503 -> 1.421 ms, C3H6 225.2 -> 219.9 ms.
 __global__ void __launch_bounds__(128) pack_kernel(const DevGrid* __restrict__ grids, const Panel* __restrict__ panels,
-                                                   int n_panels, const int* __restrict__ hint, const short2* __restrict__ rows,
+                                                   int n_panels, const int* __restrict__ hint, const int2* __restrict__ rows,
                                                    const float* __restrict__ ops, const float* __restrict__ ops_lo,
                                                    uint8_t* __restrict__ packed) {
   using namespace mma;
@@ -588,7 +588,7 @@ __global__ void __launch_bounds__(128) pack_kernel(const DevGrid* __restrict__ g
   const int64_t blk = g.op_off + (int64_t)P.w * g.ws + 4 * P.qq;  // (kWinPts = 128: one block)
   int64_t src = -1, mul = -1;
   if (row < pn.nrows) {
-    const short2 q = rows[pn.rows_off + row];
+    const int2 q = rows[pn.rows_off + row];
     src = blk + q.x * g.rs;
     if (q.y >= 0) mul = blk + q.y * g.rs;
   }
@@ -1352,7 +1352,7 @@ __global__ void __launch_bounds__(ws::kThreads, 1)
 __global__ void __launch_bounds__(256) reduce_mixed_kernel(const DevGrid* __restrict__ grids,
                                                            const MmaBlock* __restrict__ blocks, int n_blocks,
                                                            const int64_t* __restrict__ elem_begin, int64_t e0,
-                                                           int64_t e1, const short2* __restrict__ rows,
+                                                           int64_t e1, const int2* __restrict__ rows,
                                                            const double* __restrict__ rowc,
                                                            const float2* __restrict__ part, double* __restrict__ res) {
   const int64_t idx = e0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1375,7 +1375,7 @@ __global__ void __launch_bounds__(256) reduce_mixed_kernel(const DevGrid* __rest
   if (rowc) {
     const int r = mn <= 0x7fffffff ? (int)((uint32_t)e / (uint32_t)b.n) : (int)(e / b.n), col = (int)(e - (int64_t)r * b.n);
     const double* rc = rowc + grids[b.grid].rc_off;
-    const short2 qa = rows[b.a_off + r], qb = rows[b.b_off + col];
+    const int2 qa = rows[b.a_off + r], qb = rows[b.b_off + col];
     double ca = rc[qa.x], cb = rc[qb.x];
     if (qa.y >= 0) ca *= rc[qa.y];
     if (qb.y >= 0) cb *= rc[qb.y];
@@ -1431,7 +1431,7 @@ cudaError_t prepare_kernels() {
 }
 
 cudaError_t launch_pack(const DevGrid* grids, const Panel* panels, int n_panels, const int* hint, int64_t n_jobs,
-                        const short2* rows, const float* ops, const float* ops_lo, uint8_t* packed, cudaStream_t s) {
+                        const int2* rows, const float* ops, const float* ops_lo, uint8_t* packed, cudaStream_t s) {
   if (n_jobs == 0) return cudaSuccess;
   pack_kernel<<<(unsigned)n_jobs, 128, 0, s>>>(grids, panels, n_panels, hint, rows, ops, ops_lo, packed);
   return cudaGetLastError();
@@ -1455,7 +1455,7 @@ cudaError_t launch_ri_pack(const Panel* panels, int64_t n_jobs, const double* sr
 }
 
 cudaError_t launch_reduce_mixed(const DevGrid* grids, const MmaBlock* blocks, int n_blocks, const int64_t* elem_begin,
-                                int64_t e0, int64_t e1, const short2* rows, const double* rowc, const float2* part,
+                                int64_t e0, int64_t e1, const int2* rows, const double* rowc, const float2* part,
                                 double* res, cudaStream_t s) {
   if (e1 <= e0) return cudaSuccess;
   reduce_mixed_kernel<<<(unsigned)((e1 - e0 + 255) / 256), 256, 0, s>>>(grids, blocks, n_blocks, elem_begin, e0, e1,

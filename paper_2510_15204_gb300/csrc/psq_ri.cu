@@ -339,7 +339,7 @@ RiMixedLayout ri_mixed_layout(int n, int64_t nc, int64_t nd, int sm_count) {
   L.o_blk = sec(sizeof(MmaBlock));
   L.o_items = sec(sizeof(GemmItem) * (size_t)L.n_items);
   L.o_cb = sec(sizeof(int) * (size_t)(L.n_ctas + 1));
-  L.o_rows = sec(sizeof(short2) * (size_t)(nc + nd));
+  L.o_rows = sec(sizeof(int2) * (size_t)(nc + nd));
   L.o_rowc = sec(sizeof(double));
   L.o_eb = sec(2 * sizeof(int64_t));
   L.o_bt = sec(sizeof(double) * (size_t)(nc + nd) * n);
@@ -387,7 +387,7 @@ __global__ void ri_setup_kernel(RiMixedLayout L, char* __restrict__ ws) {
     const int64_t slot = bcta * q + (bcta < rem ? bcta : rem) + j;
     reinterpret_cast<GemmItem*>(ws + L.o_items)[slot] = GemmItem{0, t / L.tnB, t % L.tnB, chunk};
   }
-  if (i < L.nc + L.nd) reinterpret_cast<short2*>(ws + L.o_rows)[i] = make_short2(0, -1);
+  if (i < L.nc + L.nd) reinterpret_cast<int2*>(ws + L.o_rows)[i] = make_int2(0, -1);
 }
 
 // Bt[r][R] = B[R][col0 + r] for r < count: the pair columns as rows (32 x 32 tiles).
@@ -526,7 +526,7 @@ extern "C" psq_status psq_ri_eri_mixed(int n, int64_t m, const double* d_B, int6
                          nullptr, s) != cudaSuccess)
     return launched();
   if (launch_reduce_mixed((const DevGrid*)(ws + L.o_grid), (const MmaBlock*)(ws + L.o_blk), 1,
-                          (const int64_t*)(ws + L.o_eb), 0, nc * nd, (const short2*)(ws + L.o_rows),
+                          (const int64_t*)(ws + L.o_eb), 0, nc * nd, (const int2*)(ws + L.o_rows),
                           nullptr, (const float2*)(ws + L.o_part), d_out, s) != cudaSuccess)
     return launched();
   return launched();
