@@ -183,7 +183,7 @@ psq_status psq_profile_read(psq_job* job, double ms[8], int counts[8]);
  * (cudaGetSymbolAddress) with that device current; make that first call before any stream
  * capture.  Every call, on every stream, shares the one array and leaves its contents for the
  * next: calls whose work overlaps on the GPU race and give undefined results. */
-#define PSQ_NOALLOC_SCRATCH_BYTES ((size_t)64 << 20)
+#define PSQ_NOALLOC_SCRATCH_BYTES ((size_t)65 << 20)  /* 64 MiB of operands and sums, and the tables */
 psq_status psq_compute_noalloc(psq_job* job, unsigned mask, double* d_out[5], void* stream);
 
 /* Waits for `stream` and reports whether a kernel of the last psq_compute on this workspace
