@@ -455,8 +455,11 @@ extern "C" psq_status psq_ri_solve(int n, int64_t m, const double* d_L, double* 
     return set_error(PSQ_ERR_ARG, "psq_ri_solve: NULL or misaligned matrix");
   if ((m + 63) / 64 > 0x7fffffff) return set_error(PSQ_ERR_ARG, "psq_ri_solve: m too large");
   cudaStream_t s = (cudaStream_t)stream;
-  // few columns: fewer per CTA, so that the serial substitutions spread over the SMs
-  const int64_t per = (m + 2 * 152 - 1) / (2 * 152);
+  int dev = 0, sms = 152;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return launched();
+  // few columns: fewer per CTA, so that the serial substitutions spread over the SMs (two CTAs each)
+  const int64_t per = (m + 2 * sms - 1) / (2 * sms);
   const int cols = per >= 97 ? 128 : (int)((per + 31) / 32 * 32);
   if (!fx_attr((const void*)trsv_kernel)) return launched();
   trsv_kernel<<<(unsigned)((m + cols - 1) / cols), fx::kThreads, fx::kSmemBytes, s>>>(n, m, cols, d_L, d_B);
