@@ -275,8 +275,9 @@ cudaError_t launch_reduce_mixed(const DevGrid* grids, const MmaBlock* blocks, in
 
 // Host side (psq_host.cpp): psq_compute on a given workspace; with plan_must_exist the call
 // plans nothing (no host or device allocation) and fails if mask was never planned.  overlap: the
-// assembly kernels may start beside one another (the server's jobs do without: on several streams
-// the gaps are filled already, and the six-job batch took 10.99 instead of 10.87 ms with it).
+// assembly kernels may start beside one another.  The server's jobs do without: on several streams
+// the gaps are filled already (six-job batch against one fixed build, three runs each: 0.991 to 0.996x
+// with it, 1.003 to 1.008x without; the runs of one side differ by 0.2 to 0.7%).
 psq_status compute_on(psq_job* job, unsigned mask, void* d_workspace, size_t ws_bytes, double* d_out[5],
                       void* stream, bool plan_must_exist, bool overlap = true);
 psq_status set_error(psq_status s, const char* msg);
