@@ -20,18 +20,6 @@ namespace {
 
 constexpr int kB = 32;  // block size of the factor and the solve
 
-// 1/sqrt(d), d > 0: one step of Halley's third-order iteration from the hardware's approximation (about
-// 22 bits).  A pivot's root heads a serial chain, and an FP64 operation takes 64 cycles here, dependent
-// or not: five of them, where sqrt and a division take 675 and 354 cycles.
-__device__ __forceinline__ double rsqrt_fast(double d) {
-  const int hi = __double2hiint(d);
-  if (hi < ((1023 - 1000) << 20) || hi >= ((1023 + 1000) << 20)) return 1.0 / sqrt(d);  // outside [2^-1000, 2^1000)
-  double r;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-  const double h = fma(-d * r, r, 1.0);
-  return fma(fma(0.375, h, 0.5), r * h, r);
-}
-
 // One block column: the kb x kb diagonal block at (k0, k0) and the panel below it, a CTA per 32 rows.
 // Four lanes share a row (lane q its columns 4 i + q): one warp's FP64 instruction occupies its quarter
 // of the SM for 64 cycles, so the work is spread over four warps.  Every CTA factors the diagonal block
@@ -42,7 +30,7 @@ __device__ __forceinline__ double rsqrt_fast(double d) {
 // that is not positive records info = k0 + j + 1 (the first one wins) and continues with 1 so that
 // nothing divides by zero.
 // Measured with the update below: n = 693 from 2.55 ms (three launches per block column, roots and
-// divisions by one thread between barriers) to 1.10, n = 82 from 266 us to 129.
+// divisions by one thread between barriers) to 1.07, n = 82 from 266 us to 126.
 __global__ void __launch_bounds__(128) chol_panel_kernel(int n, int k0, int kb, double* __restrict__ L, int* __restrict__ info) {
   __shared__ double d[kB][kB + 1];  // column-wise: d[j][i] = D[i][j]
   __shared__ double piv[2], inv[kB];  // reciprocal pivots
@@ -68,7 +56,7 @@ __global__ void __launch_bounds__(128) chol_panel_kernel(int n, int k0, int kb, 
         if (blockIdx.x == 0 && tid == 0 && !(p > 0.0)) atomicCAS(info, 0, k0 + j + 1);
         if (!(p > 0.0)) p = 1.0;
       }
-      const double y = rsqrt_fast(p);
+      const double y = rsqrt(p);
       if (q == qq) {
         // the diagonal entry keeps the pivot itself for now (its root: below, all at once)
         a[jj] = row > j ? a[jj] * y : (row == j ? p : 0.0);
