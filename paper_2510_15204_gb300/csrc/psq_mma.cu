@@ -424,8 +424,7 @@ __device__ __forceinline__ float pow2f(int k) {
 
 namespace mma {
 
-// JOIN: the digit after which the lo parts join the remainder.  JOIN = 2 for normalised pairs
-// (|lo| <= 2^-24 |hi|; s3 <= 256); JOIN = 1 for products left unnormalised (|lo| <= 3 2^-24
+// The lo parts join the remainder after digit kJoin = 1: products are left unnormalised (|lo| <= 3 2^-24
 // |hi|: the join adds at most 1.5 to s2, which stays <= 130, and rounds at 2^-17 of s2's unit,
 // 2^-40 of the window's largest value).
 //
@@ -439,6 +438,7 @@ namespace mma {
 constexpr float kRneMagic = 12582912.0f;         // 1.5 x 2^23
 constexpr float kRneMagic256 = 3221225472.0f;    // 256 x 1.5 x 2^23 = 1.5 x 2^31
 constexpr int kDigitScaleExp = 8;                // |stored digit| = 2^8 |s|
+constexpr int kJoin = 1;
 
 // BF16x2 bits of two floats that are exact in BF16 (at most 8 significant bits: their low 16
 // bits are zero), first value in the low half.
@@ -447,17 +447,16 @@ __device__ __forceinline__ uint32_t pack_bf16_exact(float lo, float hi) {
 }
 
 // The window scale of a row whose largest |value| is below 2^e, for the hi words (sc) and
-// for the lo words joining after digit JOIN (sc 256^(JOIN + 1), capped at 2^127: rows below
+// for the lo words joining after digit kJoin (sc 256^(kJoin + 1), capped at 2^127: rows below
 // 2^-96, whose lo parts are below 2^-120, join them at a smaller weight).
-template <int JOIN>
 __device__ __forceinline__ void window_scales(int e, float& sc, float& scj) {
   sc = e == kZeroExp ? 0.0f : pow2f(7 - e);
-  scj = e == kZeroExp ? 0.0f : pow2f(7 - e + 8 * (JOIN + 1));
+  scj = e == kZeroExp ? 0.0f : pow2f(7 - e + 8 * (kJoin + 1));
 }
 
 // The planes of 2 NP consecutive points (NP = 4: a 16-byte group) given as pairs, NP words each; the
 // values are sgn vh + vl (sgn: the sign the hi words' scale sc carries).
-template <int JOIN, int NP>
+template <int NP>
 __device__ __forceinline__ void slice_f2(const f2 (&vh)[NP], const f2 (&vl)[NP], float sc, float scj, uint32_t (&o)[kSlices][NP]) {
   const f2 s0 = f2_both(sc), s256 = f2_both(sc * 256.0f), sj = f2_both(scj);  // |sc 256| at most 2^125
   const f2 magic = f2_both(kRneMagic), magic256 = f2_both(kRneMagic256), m256 = f2_both(-256.0f), p256 = f2_both(256.0f);
@@ -475,7 +474,7 @@ __device__ __forceinline__ void slice_f2(const f2 (&vh)[NP], const f2 (&vl)[NP],
       o[k][q] = pack_bf16_exact(d0, d1);
       if (k + 1 < kSlices) {
         r = k == 0 ? f2_fma(vh[q], s256, d) : f2_fma(r, p256, d);
-        if (k == JOIN) r = f2_add(r, l);
+        if (k == kJoin) r = f2_add(r, l);
       }
     }
   }
@@ -556,7 +555,7 @@ __device__ __forceinline__ void pack_store(const PackPos& P, const Panel& pn, co
   const int rt = min(pn.tr, pn.nrows - P.t * pn.tr);
   if (P.r >= rt) return;
   float sc, scj;
-  window_scales<1>(e, sc, scj);
+  window_scales(e, sc, scj);
   const int plane = rt * kRowB, left = pn.nch - kChunksPerWin * P.w;  // chunks of the window that exist
   uint8_t* dst = packed + pn.pack_off + (int64_t)P.t * pn.nch * (kSlices * pn.tr * kRowB) +
                  (int64_t)kChunksPerWin * P.w * (kSlices * plane) + swz(P.r, P.qq >> 1) + 8 * (P.qq & 1);
@@ -564,7 +563,7 @@ __device__ __forceinline__ void pack_store(const PackPos& P, const Panel& pn, co
   for (int c = 0; c < kChunksPerWin; ++c) {
     if (c >= left) break;
     uint32_t wv[kSlices][2];
-    slice_f2<1, 2>(h[c], l[c], sgn * sc, scj, wv);
+    slice_f2<2>(h[c], l[c], sgn * sc, scj, wv);
 #pragma unroll
     for (int k = 0; k < kSlices; ++k) *reinterpret_cast<uint2*>(dst + (c * kSlices + k) * plane) = make_uint2(wv[k][0], wv[k][1]);
   }
@@ -1147,7 +1146,7 @@ __global__ void __launch_bounds__(ws::kThreads, 1)
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
           if (g == 0) sm.eb[set][col[u]] = e[u];
-          window_scales<1>(e[u], sc[u], scj[u]);
+          window_scales(e[u], sc[u], scj[u]);
         }
 #pragma unroll
         for (int cc = 0; cc < kChunksPerWin; ++cc) {
@@ -1161,7 +1160,7 @@ __global__ void __launch_bounds__(ws::kThreads, 1)
 #pragma unroll
               for (int u = 0; u < 2; ++u) {
                 uint32_t wv[kSlices][2];
-                slice_f2<1, 2>(vh[cc][u], vl[cc][u], -sc[u], scj[u], wv);
+                slice_f2<2>(vh[cc][u], vl[cc][u], -sc[u], scj[u], wv);
 #pragma unroll
                 for (int k = 0; k < kSlices; ++k)
                   *reinterpret_cast<uint2*>(sm.b[sb][k] + swz(col[u], g >> 1) + 8 * (g & 1)) = make_uint2(wv[k][0], wv[k][1]);

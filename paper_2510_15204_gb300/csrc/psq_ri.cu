@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(fx::kThreads, 2) eri_kernel(int n, int64_t m, 
 // place of the points: the pair columns of B become operand rows (transposed into Bt), are
 // packed as in the mixed path (five 8-bit slices per value under a power-of-two scale per
 // row and 128 aux functions), and the tcgen05 contraction and its FP64 range reduction run
-// unchanged on them (one block, A = the c pairs, B = the d pairs, all row constants 1).
+// unchanged on them (one block, A = the c pairs, B = the d pairs, no row constants).
 
 constexpr size_t kAlign = 256;
 size_t up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
@@ -299,7 +299,7 @@ struct RiMixedLayout {
   int64_t nc, nd;
   int n, nch, nwin, tmA, tnB, n_ranges, win_per, n_ctas;
   int64_t n_items, jobsA, jobsB;
-  size_t o_grid, o_pn, o_blk, o_items, o_cb, o_rows, o_rowc, o_eb, o_status, o_bt, o_pack, o_part, total;
+  size_t o_grid, o_pn, o_blk, o_items, o_cb, o_eb, o_status, o_bt, o_pack, o_part, total;
   int64_t packA, expA, packB, expB;  // panel offsets within the packed area
 };
 
@@ -327,8 +327,6 @@ RiMixedLayout ri_mixed_layout(int n, int64_t nc, int64_t nd, int sm_count) {
   L.o_blk = sec(sizeof(MmaBlock));
   L.o_items = sec(sizeof(GemmItem) * (size_t)L.n_items);
   L.o_cb = sec(sizeof(int) * (size_t)(L.n_ctas + 1));
-  L.o_rows = sec(sizeof(int2) * (size_t)(nc + nd));
-  L.o_rowc = sec(sizeof(double));
   L.o_eb = sec(2 * sizeof(int64_t));
   L.o_bt = sec(sizeof(double) * (size_t)(nc + nd) * n);
   size_t pk = 0;
@@ -351,7 +349,6 @@ __global__ void ri_setup_kernel(RiMixedLayout L, char* __restrict__ ws) {
     *reinterpret_cast<int*>(ws + L.o_status) = 0;
     DevGrid* g = reinterpret_cast<DevGrid*>(ws + L.o_grid);
     g->K = L.n;
-    g->rc_off = 0;
     Panel* pn = reinterpret_cast<Panel*>(ws + L.o_pn);
     pn[0].grid = 0; pn[0].rows_off = 0; pn[0].nrows = (int)L.nc; pn[0].tr = kMmaM; pn[0].n_tiles = L.tmA;
     pn[0].nch = L.nch; pn[0].nwin = L.nwin; pn[0].pack_off = L.packA; pn[0].exp_off = L.expA; pn[0].job_begin = 0;
@@ -361,7 +358,6 @@ __global__ void ri_setup_kernel(RiMixedLayout L, char* __restrict__ ws) {
     b->grid = 0; b->m = (int)L.nc; b->n = (int)L.nd; b->a_off = 0; b->b_off = (int)L.nc;
     b->n_ranges = L.n_ranges; b->win_per = L.win_per; b->a_panel = 0; b->b_panel = 1;
     b->ptile_off = 0; b->n_btiles = 0; b->res_off = 0; b->part_off = 0;
-    *reinterpret_cast<double*>(ws + L.o_rowc) = 1.0;
     int64_t* eb = reinterpret_cast<int64_t*>(ws + L.o_eb);
     eb[0] = 0;
     eb[1] = L.nc * L.nd;
@@ -375,7 +371,6 @@ __global__ void ri_setup_kernel(RiMixedLayout L, char* __restrict__ ws) {
     const int64_t slot = bcta * q + (bcta < rem ? bcta : rem) + j;
     reinterpret_cast<GemmItem*>(ws + L.o_items)[slot] = GemmItem{0, t / L.tnB, t % L.tnB, chunk};
   }
-  if (i < L.nc + L.nd) reinterpret_cast<int2*>(ws + L.o_rows)[i] = make_int2(0, -1);
 }
 
 // Bt[r][R] = B[R][col0 + r] for r < count: the pair columns as rows (32 x 32 tiles).
@@ -502,7 +497,7 @@ extern "C" psq_status psq_ri_eri_mixed(int n, int64_t m, const double* d_B, int6
   if (prepare_kernels() != cudaSuccess) return launched();
   char* ws = (char*)d_workspace;
   if (cudaMemsetAsync(ws, 0, L.o_bt, s) != cudaSuccess) return launched();  // tables (zeroed, then set)
-  const int64_t setup_n = std::max<int64_t>(std::max<int64_t>(L.n_items, nc + nd), L.n_ctas + 1);
+  const int64_t setup_n = std::max<int64_t>(L.n_items, L.n_ctas + 1);
   ri_setup_kernel<<<(unsigned)((setup_n + 255) / 256), 256, 0, s>>>(L, ws);
   double* btA = (double*)(ws + L.o_bt);
   double* btB = btA + (size_t)nc * n;
@@ -517,8 +512,7 @@ extern "C" psq_status psq_ri_eri_mixed(int n, int64_t m, const double* d_B, int6
                          nullptr, s) != cudaSuccess)
     return launched();
   if (launch_reduce_mixed((const DevGrid*)(ws + L.o_grid), (const MmaBlock*)(ws + L.o_blk), 1,
-                          (const int64_t*)(ws + L.o_eb), 0, nc * nd, (const int2*)(ws + L.o_rows),
-                          nullptr, (const float2*)(ws + L.o_part), d_out, s) != cudaSuccess)
+                          (const int64_t*)(ws + L.o_eb), 0, nc * nd, nullptr, nullptr, (const float2*)(ws + L.o_part), d_out, s) != cudaSuccess)
     return launched();
   return launched();
 }
