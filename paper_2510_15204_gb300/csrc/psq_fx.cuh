@@ -20,11 +20,14 @@
 // above 2^-4 of its scale (kNear), and an element whose two rows share such a point has terms of at
 // least 2^-8 S: its error stays within 2^-46.5 of the sum of its absolute terms, about the bound of the
 // chain it stands for (63 roundings, 2^-47).  Where the rows share none (two steep functions that
-// peak at opposite ends of the window), the element's window is summed by that chain instead: none to
-// one element in 10^5 on grids with whole cells per window (bent triatomic, triple
-// zeta), one in 10^3 to 10^2 on coarse grids with cells of 27 or 45 points.
-// Measured (no near bits, no chain -> now): bent triatomic 4.86 -> 5.13 ms, RI of 693 aux functions
-// 8.69 -> 9.11 ms, H2 and RI of 82 unchanged.
+// peak at opposite ends of the window) and the running sum is below S as well (above it, what is
+// dropped stays below half a rounding of that sum), the element's window is summed by that chain
+// instead: none to one element in 10^5 on grids with whole cells per window, one in 10^3 to 10^2 on
+// coarse grids with cells of 27 or 45 points.  A column's chains are taken by the whole warp one after
+// the other, two points a lane, or by their own lanes where more than kTogether of the 32 rows ask.
+// Measured (no near bits, no chain -> now): bent triatomic 4.87 -> 5.14 ms, RI of 693 aux functions
+// 8.72 -> 8.66 ms, H2 unchanged; quintuple-zeta N-O on 8 x 6 x 3 cells of 5 x 3 x 3 points, (P|Q) and (P|ij)
+// 4.7 -> 9.6 ms (FP64 FMAs throughout: 28.0).
 //
 // Rows with an infinity, a NaN or a value of 2^478 and above take the chain too (their products may
 // leave the range of the integer path).  Rows below 2^-959 (a steep function far out) are lifted by
@@ -48,10 +51,12 @@ constexpr int kThreads = 256;
 constexpr int kRows = 128, kCols = 32;  // tile of a CTA
 constexpr int kWin = 64;                // points per scale window
 constexpr int kDigits = 8;
+constexpr int kTogether = 8;            // chains of a column's 32 rows that the warp sums one by one, all lanes on each
 constexpr uint32_t kTmemCols = kDigits * kCols;
 constexpr int kBigField = 1500;         // exponent field from which a row takes the FP64 chain
 constexpr int kLift = 200;              // power of two by which a row of tiny values is lifted
 constexpr int kBias = 256;              // keeps the stored field of a lifted row positive
+constexpr int kFar = 8000;              // stored field of a row that always takes the chain
 constexpr int kNear = 2;                // a value of a field at most this below its row's counts as large
 
 struct Smem {
@@ -150,6 +155,7 @@ __device__ __forceinline__ uint32_t store_b(Smem& sm, uint32_t off, const double
   return near;
 }
 
+__device__ __forceinline__ int hi_abs(double v) { return __double2hiint(v) & 0x7fffffff; }
 // The size of v as an integer: exponent and the mantissa's first 21 bits (0 below 2^-1043: low_bits).
 __device__ __forceinline__ uint32_t mag(double v) {
   return __funnelshift_l((uint32_t)__double2loint(v), (uint32_t)__double2hiint(v), 1);
@@ -161,26 +167,21 @@ __device__ __forceinline__ uint32_t low_bits(double v) { return (uint32_t)__doub
 __device__ __forceinline__ int field(uint32_t mx) { return (int)((min(mx, 0xffe00000u) + 0x4080u) >> 21); }
 constexpr uint32_t kLow = 64u << 21;  // rows below it are lifted
 
-// What a row's or column's window is scaled by: the field its digits are cut with (4000 for zeros: their
-// own field, 0, must be 63 below it), the stored one, and the value of its near bits where they are the
-// same for all points (zeros meet anything; rows out of the digits' range meet nothing).
-struct Scale {
-  int E, stored;
-  uint32_t set, keep;
-  __device__ __forceinline__ Scale(uint32_t mx, int low) {
-    E = field(mx);
-    stored = mx == 0 ? 0 : E + kBias - low;
-    set = mx == 0 ? ~0u : 0u;
-    keep = E >= kBigField ? 0u : ~0u;
-    if (mx == 0) E = 4000;
-  }
-  __device__ __forceinline__ uint32_t bits(uint32_t near) const { return (near | set) & keep; }
-};
+// What a row's or column's window is scaled by: the field its digits are cut with (kZeros for zeros: their
+// own field, 0, must be 63 below it) and the stored one.
+constexpr int kZeros = 4000;
+__device__ __forceinline__ int digit_field(uint32_t mx) { return mx == 0 ? kZeros : field(mx); }
+__device__ __forceinline__ int stored_field(uint32_t mx, bool lifted) {
+  const int E = field(mx);
+  return mx == 0 ? 0 : (E >= kBigField ? kFar : E + kBias - (lifted ? kLift : 0));
+}
+// The near bits as the fold wants them: zeros meet anything, rows out of the digits' range nothing.
+__device__ __forceinline__ uint32_t near_bits(uint32_t near, int E) { return E < kBigField ? near : (E == kZeros ? ~0u : 0u); }
 
 // One window: the tile's accumulators (element row 32 (warp % 4) + lane, columns 16 (warp / 4) + j,
 // acc[j]) take sum_p a_r(p) b_c(p).  Only the first `rows` rows and `cols` columns are kept up
 // (8-row groups and 4-column groups past them are left out).  win: the windows done so far by this
-// CTA.  chain(row, col): the plain FP64 sum of the window for a row or column out of the integer
+// CTA.  chain(row, col, p, step): the plain FP64 sum of the window's points p, p + step, ... for a row or column out of the integer
 // path's range and for an element whose rows are not large at a common point.  ok turns false when a wait ran out (the caller ends its loop when the return
 // value, the same for all threads, is false, and asks all threads once more at the end).
 template <typename Chain>
@@ -230,12 +231,12 @@ __device__ __forceinline__ bool window(Smem& sm, uint32_t tmem, double (&va)[4][
     ma[1] = over_a(1, mag);
     mb = over_b(mag);
   }
-  const Scale ea[2] = {Scale(ma[0], la0 ? kLift : 0), Scale(ma[1], la1 ? kLift : 0)}, eb(mb, lb ? kLift : 0);
+  const int ea[2] = {digit_field(ma[0]), digit_field(ma[1])}, eb = digit_field(mb);
   if ((lane & 3) == 0) {
-    sm.ea[set][a_row(0)] = ea[0].stored;
-    sm.ea[set][a_row(1)] = ea[1].stored;
+    sm.ea[set][a_row(0)] = stored_field(ma[0], la0);
+    sm.ea[set][a_row(1)] = stored_field(ma[1], la1);
   }
-  if ((lane & 7) == 0) sm.eb[set][b_col()] = eb.stored;
+  if ((lane & 7) == 0) sm.eb[set][b_col()] = stored_field(mb, lb);
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
     if (c == 1 && ok) {
@@ -245,11 +246,11 @@ __device__ __forceinline__ bool window(Smem& sm, uint32_t tmem, double (&va)[4][
 #pragma unroll
     for (int u = 0; u < 2; ++u)
       if (64 * u + 8 * warp < rows) {
-        const uint32_t near = store_a(sm, mma::swz(a_row(u), lane & 3), va[2 * c + u], ea[u].E);
-        sm.na[set][a_row(u)][4 * c + (lane & 3)] = (uint8_t)ea[u].bits(near);
+        const uint32_t near = store_a(sm, mma::swz(a_row(u), lane & 3), va[2 * c + u], ea[u]);
+        sm.na[set][a_row(u)][4 * c + (lane & 3)] = (uint8_t)near_bits(near, ea[u]);
       }
     if (4 * warp < cols) {
-      uint32_t near = eb.bits(store_b(sm, mma::swz(b_col(), (lane & 7) >> 1) + 8u * (lane & 1), vb[c], eb.E)) & 15u;
+      uint32_t near = near_bits(store_b(sm, mma::swz(b_col(), (lane & 7) >> 1) + 8u * (lane & 1), vb[c], eb), eb) & 15u;
       near = (near << 4) | __shfl_down_sync(kFull, near, 1);  // the pair's first points in the high bits, as in na
       if ((lane & 1) == 0) sm.nb[set][b_col()][4 * c + ((lane & 7) >> 1)] = (uint8_t)near;
     }
@@ -305,24 +306,43 @@ __device__ __forceinline__ bool window(Smem& sm, uint32_t tmem, double (&va)[4][
         t = (small ? t << 7 : t) +
             __float2int_rn(fmaf(o[6][j], 0.00390625f, o[7][j] * 1.52587890625e-5f) * (small ? 128.0f : 1.0f));
         int f = er + ec - 2 * kBias - 2044 - 54 + 1023 - (small ? 7 : 0);  // exponent field of t's unit
-        double x = __ll2double_rn(t);
-        if (f <= 0) {  // a unit below 2^-1022: in two steps
-          x *= 0x1p-600;
+        // t as FP64; where its unit lies below 2^-1022, 2^600 go over from t (by its exponent bits: the FP64
+        // pipe is the scarce one) to the unit
+        const double x = __ll2double_rn(t);
+        int hx = __double2hiint(x);
+        if (f <= 0) {
+          hx -= t == 0 ? 0 : 600 << 20;
           f = max(f + 600, 0);
         }
-        if (((near.x & nc.x) | (near.y & nc.y)) == 0)
+        // no common large point, and the running sum below S
+        if (((near.x & nc.x) | (near.y & nc.y)) == 0 &&
+            (hi_abs(acc[4 * q + j]) >> 20) < er + ec - 2 * kBias - 2044 + 1023)
           apart |= 1u << (4 * q + j);
         else
-          acc[4 * q + j] = fma(x, __hiloint2double(f << 20, 0), acc[4 * q + j]);
+          acc[4 * q + j] = fma(__hiloint2double(hx, __double2loint(x)), __hiloint2double(f << 20, 0), acc[4 * q + j]);
       }
     }
+    // the chains: few of a column's rows at a time by the whole warp, many by their own lanes
+    if (__any_sync(kFull, apart)) {
 #pragma unroll 1
-    for (; apart; apart &= apart - 1) {
-      const int e = __ffs(apart) - 1;
-      const double s = chain(row, c0 + e);
+      for (int j = 0; j < 16; ++j, apart >>= 1) {
+        uint32_t m = __ballot_sync(kFull, apart & 1);
+        double mine = 0.0;
+        if (__popc(m) > kTogether) {
+          if (apart & 1) mine = chain(row, c0 + j, 0, 1);
+        } else {
+          for (; m; m &= m - 1) {
+            const int l = __ffs(m) - 1;
+            double s = chain(32 * (warp & 3) + l, c0 + j, lane, 32);
 #pragma unroll
-      for (int j = 0; j < 16; ++j)
-        if (j == e) acc[j] += s;
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
+            if (l == lane) mine = s;
+          }
+        }
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+          if (k == j && (apart & 1)) acc[k] += mine;
+      }
     }
   }
   mma::fence_before();  // the next window's MMAs come after its first barrier

@@ -604,6 +604,28 @@ __device__ __forceinline__ void contract_fma(const LaunchTables& t, const GemmIt
   }
 }
 
+// The plain sum of points from, from + step, ... below `to` for element (r, c) of an item's tile (outside the
+// kernel's loop, whose registers it would take).
+__device__ __noinline__ double chain_sum(const GemmItem* item, const GemmBlock* blocks, const DevGrid* grids, const int2* pairs,
+                                         const double* ops, int r, int c, int from, int to, int step) {
+  const GemmBlock& b = blocks[item->block];
+  const DevGrid& g = grids[b.grid];
+  const int row = item->tm * kFpDigitRows + r, col = item->tn * kFpDigitCols + c;
+  if (row >= b.m || col >= b.n) return 0.0;
+  const int2 qa = pairs[b.a_off + row], qb = pairs[b.b_off + col];
+  const int64_t rs = g.rs, ws = g.ws;
+  double s = 0.0;
+#pragma unroll 4
+  for (int p = from; p < to; p += step) {
+    const double* at = ops + g.op_off + (int64_t)(p >> 7) * ws + (p & 127);
+    double x = at[qa.x * rs], y = at[qb.x * rs];
+    if (qa.y >= 0) x *= at[qa.y * rs];
+    if (qb.y >= 0) y *= at[qb.y * rs];
+    s = fma(x, y, s);
+  }
+  return s;
+}
+
 __global__ void __launch_bounds__(fx::kThreads, 2) contract_fp64_kernel(LaunchTables t, const double* __restrict__ ops,
                                                                         double* __restrict__ part, int* __restrict__ status,
                                                                         uint64_t wait_ns, const int* hold) {
@@ -620,14 +642,14 @@ __global__ void __launch_bounds__(fx::kThreads, 2) contract_fp64_kernel(LaunchTa
   }
   fx::Smem& sm = fx::smem_at(raw);
   const uint32_t tmem = fx::open(sm);
-  const int64_t rs = g.rs;
+  const int rs = (int)g.rs;  // (128: offsets within a block of points fit 32 bits)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int r0 = it.tm * kFpDigitRows, c0 = it.tn * kFpDigitCols;
   const int rows = min(kFpDigitRows, b.m - r0), cols = min(kFpDigitCols, b.n - c0);
   const int K = (int)g.K;  // below 2^31 - 256 (the planner checks)
   const int k0 = it.chunk * b.win_per * kFpWin, k1 = (int)min((int64_t)K, (int64_t)k0 + (int64_t)b.win_per * kFpWin);
   // this thread's operand rows (element offsets from base; the second one -1: none)
-  int64_t ax[2], ay[2], bx, by;
+  int ax[2], ay[2], bx, by;
 #pragma unroll
   for (int u = 0; u < 2; ++u) {
     const int2 q = t.pairs[b.a_off + r0 + min(fx::a_row(u), rows - 1)];
@@ -639,10 +661,6 @@ __global__ void __launch_bounds__(fx::kThreads, 2) contract_fp64_kernel(LaunchTa
     bx = q.x * rs;
     by = q.y >= 0 ? q.y * rs : -1;
   }
-  auto value = [&](int2 q, int p) {
-    const double* at = base + (int64_t)(p >> 7) * g.ws + (p & 127);
-    return q.y >= 0 ? at[q.x * rs] * at[q.y * rs] : at[q.x * rs];
-  };
   double acc[16] = {};
   uint32_t phase = 0, win = 0;
   bool ok = true, run = true;
@@ -655,7 +673,15 @@ __global__ void __launch_bounds__(fx::kThreads, 2) contract_fp64_kernel(LaunchTa
     }
     issued = run = __syncthreads_and(ok);
   }
-  for (int k = k0; k < k1 && run; k += kFpWin, ++win) {
+  // A window ends where a mu row of cells does as well: its last points lie at one nucleus, the next ones
+  // at the other, and two to ten times as many elements would take the chain (psq_fx.cuh).  Points
+  // [from, to) of an aligned window.
+  const uint32_t row_pts = (uint32_t)(g.n_nu * g.n_phi * g.q_mu * g.q_nu * g.q_phi);
+  uint32_t cut = ((uint32_t)k0 / row_pts + 1) * row_pts;  // (below 2^32)
+  for (int from = k0; from < k1 && run; ++win) {
+    if (cut > g.K_reg) cut = ~0u;
+    const int k = from & -kFpWin, to = (int)min(cut, (uint32_t)min(k + kFpWin, k1));
+    const bool whole = to - from == kFpWin;
     double va[4][8], vb[2][4];
     const double* win0 = base + (int64_t)(k >> 7) * g.ws + (k & 127);  // the window's first point (row 0)
 #pragma unroll
@@ -663,9 +689,8 @@ __global__ void __launch_bounds__(fx::kThreads, 2) contract_fp64_kernel(LaunchTa
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
         double(&v)[8] = va[2 * c + u];
-        const int left = 64 * u + 8 * warp < rows ? k1 - k - fx::a_pt(c) : 0;
         const double* at = win0 + fx::a_pt(c);
-        if (left >= 8) {
+        if (whole && 64 * u + 8 * warp < rows) {
           const double2* x = reinterpret_cast<const double2*>(at + ax[u]);
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
@@ -686,7 +711,8 @@ __global__ void __launch_bounds__(fx::kThreads, 2) contract_fp64_kernel(LaunchTa
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
             v[i] = 0.0;
-            if (i < left) v[i] = at[ax[u] + i] * (ay[u] >= 0 ? at[ay[u] + i] : 1.0);
+            const int p = k + fx::a_pt(c) + i;
+            if (64 * u + 8 * warp < rows && p >= from && p < to) v[i] = at[ax[u] + i] * (ay[u] >= 0 ? at[ay[u] + i] : 1.0);
           }
         }
       }
@@ -694,17 +720,15 @@ __global__ void __launch_bounds__(fx::kThreads, 2) contract_fp64_kernel(LaunchTa
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         vb[c][i] = 0.0;
-        if (fx::b_col() < cols && k + fx::b_pt(c) + i < k1) vb[c][i] = __ldg(at + bx + i) * (by >= 0 ? __ldg(at + by + i) : 1.0);
+        const int p = k + fx::b_pt(c) + i;
+        if (fx::b_col() < cols && (whole || (p >= from && p < to))) vb[c][i] = __ldg(at + bx + i) * (by >= 0 ? __ldg(at + by + i) : 1.0);
       }
     }
-    run = fx::window(sm, tmem, va, vb, acc, phase, win, rows, cols, ok, [&](int r, int c) {
-      double s = 0.0;
-      if (r < rows && c < cols) {
-        const int2 qa = t.pairs[b.a_off + r0 + r], qb = t.pairs[b.b_off + c0 + c];
-        for (int p = k; p < min(k1, k + kFpWin); ++p) s = fma(value(qa, p), value(qb, p), s);
-      }
-      return s;
+    run = fx::window(sm, tmem, va, vb, acc, phase, win, rows, cols, ok, [&](int r, int c, int at, int step) {
+      return chain_sum(t.items + blockIdx.x, t.gblocks, t.grids, t.pairs, ops, r, c, from + at, to, step);
     }, wait_ns);
+    if ((uint32_t)to == cut) cut += row_pts;
+    from = to;
   }
   if (run) run = __syncthreads_and(ok);
   if (!run && threadIdx.x == 0) atomicCAS(status, 0, 9);  // a wait that ran out (the first failure's code stays)
