@@ -30,7 +30,7 @@ constexpr int kB = 32;  // block size of the factor and the solve
 // that is not positive records info = k0 + j + 1 (the first one wins) and continues with 1 so that
 // nothing divides by zero.
 // Measured with the update below: n = 693 from 2.55 ms (three launches per block column, roots and
-// divisions by one thread between barriers) to 1.07, n = 82 from 266 us to 126.
+// divisions by one thread between barriers) to 1.07, n = 82 from 266 us to 123 (past kb nothing is computed: a matrix of one to eight rows 32 -> 23 us).
 __global__ void __launch_bounds__(128) chol_panel_kernel(int n, int k0, int kb, double* __restrict__ L, int* __restrict__ info) {
   __shared__ double d[kB][kB + 1];  // column-wise: d[j][i] = D[i][j]
   __shared__ double piv[2], inv[kB];  // reciprocal pivots
@@ -44,7 +44,8 @@ __global__ void __launch_bounds__(128) chol_panel_kernel(int n, int k0, int kb, 
   }
   // column j = 4 jj + qq: jj unrolled (registers), qq rolled (code that runs once is bound by its fetch)
 #pragma unroll
-  for (int jj = 0; jj < kB / 4; ++jj)
+  for (int jj = 0; jj < kB / 4; ++jj) {
+    if (4 * jj >= kb) break;
 #pragma unroll 1
     for (int qq = 0; qq < 4; ++qq) {
       const int j = 4 * jj + qq;
@@ -69,8 +70,9 @@ __global__ void __launch_bounds__(128) chol_panel_kernel(int n, int k0, int kb, 
       for (int i = jj; i < kB / 4; ++i)
         if (i > jj || q > qq) a[i] = fma(l, d[j][4 * i + q], a[i]);
     }
+  }
   __syncthreads();
-  if (tid < kB) {  // the diagonal: sqrt(p) = p y, corrected by its residual
+  if (tid < kb) {  // the diagonal: sqrt(p) = p y, corrected by its residual
     const double p = d[tid][tid], y = inv[tid], r = p * y;
     const double t = fma(fma(-r, r, p), 0.5 * y, r);
     d[tid][tid] = (__double2hiint(t) & 0x7ff00000) == 0x7ff00000 ? sqrt(p) : t;
