@@ -241,6 +241,78 @@ __global__ void __launch_bounds__(fx::kThreads, 2) trsv_kernel(int n, int64_t m,
   fx::close(sm, tmem, run, phase);
 }
 
+// Few columns (psq_ri_solve has the rule): right-looking, two launches per block, so that the rows below a
+// block spread over the SMs, on the FP64 pipe.
+//
+// Forward substitution on the diagonal block: B[k0 + r][col] for r < kb, one thread per
+// column.
+__global__ void __launch_bounds__(256) trsv_diag_kernel(int n, int64_t m, int k0, int kb,
+                                                        const double* __restrict__ L, double* __restrict__ B) {
+  __shared__ double d[kB][kB + 1];
+  for (int t = threadIdx.x; t < kB * kB; t += blockDim.x) {
+    const int r = t >> 5, c = t & 31;
+    d[r][c] = (r < kb && c <= r) ? L[(int64_t)(k0 + r) * n + k0 + c] : 0.0;
+  }
+  __syncthreads();
+  const int64_t col = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (col >= m) return;
+  double* b = B + (int64_t)k0 * m + col;
+  double x[kB];
+#pragma unroll
+  for (int j = 0; j < kB; ++j) {
+    if (j < kb) {
+      double s = b[(int64_t)j * m];
+#pragma unroll
+      for (int q = 0; q < j; ++q) s -= d[j][q] * x[q];
+      x[j] = s / d[j][j];
+      b[(int64_t)j * m] = x[j];
+    }
+  }
+}
+
+// B[k1 + r][col] -= sum_q L[k1 + r][k0 + q] B[k0 + q][col]: 64 x 64 tiles, 256 threads with
+// 4 x 4 outputs each.
+__global__ void __launch_bounds__(256) trsv_update_kernel(int n, int64_t m, int k0, int kb,
+                                                          const double* __restrict__ L, double* __restrict__ B) {
+  __shared__ double ls[64][kB + 1];
+  __shared__ double bs[kB][64];
+  const int k1 = k0 + kb;
+  const int i0 = k1 + blockIdx.y * 64;
+  const int64_t c0 = (int64_t)blockIdx.x * 64;
+  for (int t = threadIdx.x; t < 64 * kB; t += blockDim.x) {
+    const int r = t / kB, q = t % kB;
+    ls[r][q] = (i0 + r < n && q < kb) ? L[(int64_t)(i0 + r) * n + k0 + q] : 0.0;
+  }
+  for (int t = threadIdx.x; t < kB * 64; t += blockDim.x) {
+    const int q = t / 64, c = t % 64;
+    bs[q][c] = (q < kb && c0 + c < m) ? B[(int64_t)(k0 + q) * m + c0 + c] : 0.0;
+  }
+  __syncthreads();
+  const int tr = threadIdx.x / 16, tc = threadIdx.x % 16;  // rows tr + 16a, columns tc + 16b
+  double acc[4][4] = {};
+  for (int q = 0; q < kb; ++q) {
+    double lv[4], bv[4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) lv[a] = ls[tr + 16 * a][q];
+#pragma unroll
+    for (int b = 0; b < 4; ++b) bv[b] = bs[q][tc + 16 * b];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) acc[a][b] = fma(lv[a], bv[b], acc[a][b]);
+  }
+#pragma unroll
+  for (int a = 0; a < 4; ++a) {
+    const int i = i0 + tr + 16 * a;
+    if (i >= n) continue;
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const int64_t c = c0 + tc + 16 * b;
+      if (c < m) B[(int64_t)i * m + c] -= acc[a][b];
+    }
+  }
+}
+
 // out[c][d] = sum_R B[R][c0 + c] B[R][d0 + d]: a CTA per 128 x 32 output tile, R in windows of 64.
 __global__ void __launch_bounds__(fx::kThreads, 2) eri_kernel(int n, int64_t m, const double* __restrict__ B, int64_t c0,
                                                               int64_t nc, int64_t d0, int64_t nd, double* __restrict__ out) {
@@ -443,6 +515,27 @@ extern "C" psq_status psq_ri_solve(int n, int64_t m, const double* d_L, double* 
   int dev = 0, sms = 152;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return launched();
+  // The tensor-core kernel walks down the blocks within a CTA: where its CTAs are one wave, about 7.6 us for each of
+  // the nb^2 / 4 windows and 38 us for each diagonal block.  Two launches per block on the FP64 pipe: about 70 us and
+  // n^2 m FMAs at 0.59 per ps in all.  Measured, tensor cores against FP64 pipe: n = 2000, 1 and 40 columns 9.9 against
+  // 4.4 ms; n = 3000, 500 columns 20.6 against 10.8 ms; n = 693, 1 column 1.73 against 1.51 ms, 300 columns 1.77
+  // against 1.92 ms; n = 200, 200 columns 0.33 against 0.51 ms.
+  // A single block has no products: 16 rows or fewer (n = 8, 3,000 columns 15 against 12 us), columns of one CTA
+  // (n = 32, 50 columns 44 against 37 us) or more than the tensor-core kernel's first CTAs hold (n = 32, 3,000
+  // columns 43 against 54 us, 51,984 columns 115 against 102 us) take the FP64 one too.
+  const int64_t nb = (n + kB - 1) / kB;
+  const bool fp64 = nb == 1 ? n <= 16 || m <= 256 || m > 160LL * sms
+                            : m <= 2LL * fx::kRows * sms &&
+                                  70.0 * nb + (double)n * n * m / 1.18e6 < 7.6 * (nb * nb / 4) + 38.0 * nb;
+  if (fp64) {
+    for (int k0 = 0; k0 < n; k0 += kB) {
+      const int kb = n - k0 < kB ? n - k0 : kB, rest = n - k0 - kb;
+      trsv_diag_kernel<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(n, m, k0, kb, d_L, d_B);
+      if (rest > 0)
+        trsv_update_kernel<<<dim3((unsigned)((m + 63) / 64), (rest + 63) / 64), 256, 0, s>>>(n, m, k0, kb, d_L, d_B);
+    }
+    return launched();
+  }
   // few columns: fewer per CTA, so that the serial substitutions spread over the SMs (two CTAs each)
   const int64_t per = (m + 2 * sms - 1) / (2 * sms);
   const int cols = per >= 97 ? 128 : (int)((per + 31) / 32 * 32);
