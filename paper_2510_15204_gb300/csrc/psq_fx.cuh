@@ -25,9 +25,10 @@
 // instead: none to one element in 10^5 on grids with whole cells per window, one in 10^3 to 10^2 on
 // coarse grids with cells of 27 or 45 points.  A column's chains are taken by the whole warp one after
 // the other, two points a lane, or by their own lanes where more than kTogether of the 32 rows ask.
-// Measured (no near bits, no chain -> now): bent triatomic 4.87 -> 5.14 ms, RI of 693 aux functions
-// 8.72 -> 8.66 ms, H2 unchanged; quintuple-zeta N-O on 8 x 6 x 3 cells of 5 x 3 x 3 points, (P|Q) and (P|ij)
-// 4.7 -> 9.6 ms (FP64 FMAs throughout: 28.0).
+// Measured (no near bits, no chain -> now): bent triatomic 4.98 -> 5.14 ms, RI of 693 aux functions
+// 8.70 -> 8.53 ms, H2 unchanged, 2-centre Coulomb of 18 functions on 7.6 M points (tiles of few rows, bound by each
+// window's latency) 11.6 -> 13.6 ms; quintuple-zeta N-O on 8 x 6 x 3 cells of 5 x 3 x 3 points, (P|Q) and
+// (P|ij) 4.7 -> 7.9 ms (FP64 FMAs throughout: 28.0).
 //
 // Rows with an infinity, a NaN or a value of 2^478 and above take the chain too (their products may
 // leave the range of the integer path).  Rows below 2^-959 (a steep function far out) are lifted by
@@ -178,6 +179,30 @@ __device__ __forceinline__ int stored_field(uint32_t mx, bool lifted) {
 // The near bits as the fold wants them: zeros meet anything, rows out of the digits' range nothing.
 __device__ __forceinline__ uint32_t near_bits(uint32_t near, int E) { return E < kBigField ? near : (E == kZeros ? ~0u : 0u); }
 
+// The chains of a warp's 32 rows and 16 columns, added to its sums (bit j of apart: this lane's row with column
+// c0 + j): few of a column's rows one by one by all lanes, many by their own.  A function of its own,
+// on a copy of the sums, so that what it needs stays out of the window's registers.
+template <typename Chain>
+__device__ __noinline__ void chains(Chain chain, double* sums, uint32_t apart, int row0, int c0) {
+  constexpr unsigned kFull = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  for (int j = 0; j < 16; ++j, apart >>= 1) {
+    uint32_t m = __ballot_sync(kFull, apart & 1);
+    if (__popc(m) > kTogether) {
+      if (apart & 1) sums[j] += chain(row0 + lane, c0 + j, 0, 1);
+      __syncwarp();
+    } else {
+      for (; m; m &= m - 1) {
+        const int l = __ffs(m) - 1;
+        double s = chain(row0 + l, c0 + j, lane, 32);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
+        if (l == lane) sums[j] += s;
+      }
+    }
+  }
+}
+
 // One window: the tile's accumulators (element row 32 (warp % 4) + lane, columns 16 (warp / 4) + j,
 // acc[j]) take sum_p a_r(p) b_c(p).  Only the first `rows` rows and `cols` columns are kept up
 // (8-row groups and 4-column groups past them are left out).  win: the windows done so far by this
@@ -209,27 +234,28 @@ __device__ __forceinline__ bool window(Smem& sm, uint32_t tmem, double (&va)[4][
     return m;
   };
   uint32_t ma[2] = {over_a(0, mag), over_a(1, mag)}, mb = over_b(mag);
-  // zeros, or values below 2^-1043?
-  if (__any_sync(kFull, (ma[0] == 0 && a_row(0) < rows) || (ma[1] == 0 && a_row(1) < rows) || (mb == 0 && b_col() < cols))) {
-    ma[0] = max(ma[0], min(over_a(0, low_bits), 1u));
-    ma[1] = max(ma[1], min(over_a(1, low_bits), 1u));
-    mb = max(mb, min(over_b(low_bits), 1u));
-  }
-  const bool la0 = ma[0] - 1 < kLow - 1, la1 = ma[1] - 1 < kLow - 1, lb = mb - 1 < kLow - 1;
-  if (__any_sync(kFull, la0 || la1 || lb)) {
+  // small rows: those that are not zero (also below 2^-1043) are lifted
+  bool la0 = false, la1 = false, lb = false;
+  if (__any_sync(kFull, (ma[0] < kLow && a_row(0) < rows) || (ma[1] < kLow && a_row(1) < rows) || (mb < kLow && b_col() < cols))) {
+    const uint32_t wa0 = over_a(0, low_bits), wa1 = over_a(1, low_bits), wb = over_b(low_bits);  // (all lanes shuffle)
+    la0 = ma[0] < kLow && (ma[0] | wa0) != 0;
+    la1 = ma[1] < kLow && (ma[1] | wa1) != 0;
+    lb = mb < kLow && (mb | wb) != 0;
+    if (__any_sync(kFull, la0 || la1 || lb)) {
 #pragma unroll
-    for (int c = 0; c < 2; ++c) {
+      for (int c = 0; c < 2; ++c) {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        va[2 * c][i] *= la0 ? 0x1p200 : 1.0;
-        va[2 * c + 1][i] *= la1 ? 0x1p200 : 1.0;
+        for (int i = 0; i < 8; ++i) {
+          va[2 * c][i] *= la0 ? 0x1p200 : 1.0;
+          va[2 * c + 1][i] *= la1 ? 0x1p200 : 1.0;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) vb[c][i] *= lb ? 0x1p200 : 1.0;
       }
-#pragma unroll
-      for (int i = 0; i < 4; ++i) vb[c][i] *= lb ? 0x1p200 : 1.0;
+      ma[0] = over_a(0, mag);
+      ma[1] = over_a(1, mag);
+      mb = over_b(mag);
     }
-    ma[0] = over_a(0, mag);
-    ma[1] = over_a(1, mag);
-    mb = over_b(mag);
   }
   const int ea[2] = {digit_field(ma[0]), digit_field(ma[1])}, eb = digit_field(mb);
   if ((lane & 3) == 0) {
@@ -322,27 +348,13 @@ __device__ __forceinline__ bool window(Smem& sm, uint32_t tmem, double (&va)[4][
           acc[4 * q + j] = fma(__hiloint2double(hx, __double2loint(x)), __hiloint2double(f << 20, 0), acc[4 * q + j]);
       }
     }
-    // the chains: few of a column's rows at a time by the whole warp, many by their own lanes
     if (__any_sync(kFull, apart)) {
-#pragma unroll 1
-      for (int j = 0; j < 16; ++j, apart >>= 1) {
-        uint32_t m = __ballot_sync(kFull, apart & 1);
-        double mine = 0.0;
-        if (__popc(m) > kTogether) {
-          if (apart & 1) mine = chain(row, c0 + j, 0, 1);
-        } else {
-          for (; m; m &= m - 1) {
-            const int l = __ffs(m) - 1;
-            double s = chain(32 * (warp & 3) + l, c0 + j, lane, 32);
+      double sums[16];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
-            if (l == lane) mine = s;
-          }
-        }
+      for (int j = 0; j < 16; ++j) sums[j] = acc[j];
+      chains(chain, sums, apart, row - lane, c0);
 #pragma unroll
-        for (int k = 0; k < 16; ++k)
-          if (k == j && (apart & 1)) acc[k] += mine;
-      }
+      for (int j = 0; j < 16; ++j) acc[j] = sums[j];
     }
   }
   mma::fence_before();  // the next window's MMAs come after its first barrier

@@ -604,27 +604,33 @@ __device__ __forceinline__ void contract_fma(const LaunchTables& t, const GemmIt
   }
 }
 
-// The plain sum of points from, from + step, ... below `to` for element (r, c) of an item's tile (outside the
-// kernel's loop, whose registers it would take).
-__device__ __noinline__ double chain_sum(const GemmItem* item, const GemmBlock* blocks, const DevGrid* grids, const int2* pairs,
-                                         const double* ops, int r, int c, int from, int to, int step) {
-  const GemmBlock& b = blocks[item->block];
-  const DevGrid& g = grids[b.grid];
-  const int row = item->tm * kFpDigitRows + r, col = item->tn * kFpDigitCols + c;
-  if (row >= b.m || col >= b.n) return 0.0;
-  const int2 qa = pairs[b.a_off + row], qb = pairs[b.b_off + col];
-  const int64_t rs = g.rs, ws = g.ws;
-  double s = 0.0;
+// The plain sum of an item's points [from, to) for element (r, c) of its tile: fx::window's chain.
+struct ItemChain {
+  const GemmItem* item;
+  const GemmBlock* blocks;
+  const DevGrid* grids;
+  const int2* pairs;
+  const double* ops;
+  int from, to;
+  __device__ __forceinline__ double operator()(int r, int c, int p0, int step) const {
+    const GemmBlock& b = blocks[item->block];
+    const DevGrid& g = grids[b.grid];
+    const int row = item->tm * kFpDigitRows + r, col = item->tn * kFpDigitCols + c;
+    if (row >= b.m || col >= b.n) return 0.0;
+    const int2 qa = pairs[b.a_off + row], qb = pairs[b.b_off + col];
+    const int64_t rs = g.rs, ws = g.ws;
+    double s = 0.0;
 #pragma unroll 4
-  for (int p = from; p < to; p += step) {
-    const double* at = ops + g.op_off + (int64_t)(p >> 7) * ws + (p & 127);
-    double x = at[qa.x * rs], y = at[qb.x * rs];
-    if (qa.y >= 0) x *= at[qa.y * rs];
-    if (qb.y >= 0) y *= at[qb.y * rs];
-    s = fma(x, y, s);
+    for (int p = from + p0; p < to; p += step) {
+      const double* at = ops + g.op_off + (int64_t)(p >> 7) * ws + (p & 127);
+      double x = at[qa.x * rs], y = at[qb.x * rs];
+      if (qa.y >= 0) x *= at[qa.y * rs];
+      if (qb.y >= 0) y *= at[qb.y * rs];
+      s = fma(x, y, s);
+    }
+    return s;
   }
-  return s;
-}
+};
 
 __global__ void __launch_bounds__(fx::kThreads, 2) contract_fp64_kernel(LaunchTables t, const double* __restrict__ ops,
                                                                         double* __restrict__ part, int* __restrict__ status,
@@ -724,9 +730,8 @@ __global__ void __launch_bounds__(fx::kThreads, 2) contract_fp64_kernel(LaunchTa
         if (fx::b_col() < cols && (whole || (p >= from && p < to))) vb[c][i] = __ldg(at + bx + i) * (by >= 0 ? __ldg(at + by + i) : 1.0);
       }
     }
-    run = fx::window(sm, tmem, va, vb, acc, phase, win, rows, cols, ok, [&](int r, int c, int at, int step) {
-      return chain_sum(t.items + blockIdx.x, t.gblocks, t.grids, t.pairs, ops, r, c, from + at, to, step);
-    }, wait_ns);
+    run = fx::window(sm, tmem, va, vb, acc, phase, win, rows, cols, ok,
+                     ItemChain{t.items + blockIdx.x, t.gblocks, t.grids, t.pairs, ops, from, to}, wait_ns);
     if ((uint32_t)to == cut) cut += row_pts;
     from = to;
   }

@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(fx::kThreads, 2) trsv_kernel(int n, int64_t m,
 #pragma unroll
         for (int i = 0; i < 4; ++i) vb[c][i] = fx::b_col() < kb && q0 + fx::b_pt(c) + i < k0 ? p[i] : 0.0;
       }
-      run = fx::window(sm, tmem, va, vb, acc, phase, win, live, kb, ok, [&](int r, int c, int at, int step) {
+      run = fx::window(sm, tmem, va, vb, acc, phase, win, live, kb, ok, [=](int r, int c, int at, int step) {
         double s = 0.0;
         if (r < live && c < kb)
           for (int q = q0 + at; q < min(k0, q0 + fx::kWin); q += step) s = fma(B[(int64_t)q * m + c0 + r], L[(int64_t)(k0 + c) * n + q], s);
@@ -340,7 +340,7 @@ __global__ void __launch_bounds__(fx::kThreads, 2) eri_kernel(int n, int64_t m, 
 #pragma unroll
       for (int i = 0; i < 4; ++i) vb[c][i] = fx::b_col() < cols && R0 + fx::b_pt(c) + i < n ? __ldg(p + i * m) : 0.0;
     }
-    run = fx::window(sm, tmem, va, vb, acc, phase, win, rows, cols, ok, [&](int r, int c, int at, int step) {
+    run = fx::window(sm, tmem, va, vb, acc, phase, win, rows, cols, ok, [=](int r, int c, int at, int step) {
       double s = 0.0;
       if (r < rows && c < cols)
         for (int R = R0 + at; R < min(n, R0 + fx::kWin); R += step)
