@@ -227,8 +227,8 @@ __device__ __forceinline__ void store_shell(const DevShell& q, double v, const d
 // those of a third centre for half of the phi nodes (phi -> -phi is a symmetry of the grid).  A point
 // is then its harmonics and one product per function.  Row layout: F/L rows are A's basis functions
 // then B's (fn0 counted within each atom), G/U rows the aux functions of the grid's aux centres.
-// Measured (a thread per point -> now): bent triatomic (963,072 points) 4.4 -> 1.0 ms, H2 (57,600
-// points) 0.21 -> 0.06 ms.
+// Measured (a thread per point -> now): bent triatomic (963,072 points) 4.5 -> 1.1 ms, H2 (57,600
+// points) 0.22 -> 0.06 ms.
 struct EvalNodes {
   double mu[kMaxQ][4];             // sinh, cosh, sinh^2(v/2), weight
   double nu[kMaxQ][5];             // sin, cos, sin^2(v/2), cos^2(v/2), weight
@@ -464,9 +464,9 @@ cudaError_t launch_eval_fp64(const LaunchTables& t, double* ops, int /*kinds*/, 
 // grid are summed first, and symmetric blocks are summed once.
 //
 // Measured on a bent triatomic (26 basis / 82 aux functions, 963,072 points; all sums on the FP64
-// pipe before -> now): 11.85 -> 3.88 ms ((P|ij) alone 2.35, (P|Q) 0.95, the three others 0.91).
-// One-electron matrices alone (90 functions, 4.5 M points): 36.0 -> 30.3 ms, 0.80 TFLOP/s on the FP64
-// pipe, its bound; H2 (57,600 points): 268 -> 150 us (launch and window latency).
+// pipe before -> now): 11.82 -> 4.08 ms ((P|ij) alone 2.45, (P|Q) 0.97, the three others 0.89).
+// One-electron matrices alone (90 functions, 4.5 M points): 36.0 -> 30.7 ms, 0.79 TFLOP/s on the FP64
+// pipe, its bound; H2 (57,600 points): 249 -> 113 us (launch and window latency).
 //
 // The FMA part: the warps of the CTA share the tile and take every eighth group of 8 points each, so
 // that no barrier stands between a warp's loads and its FMAs; a lane holds one column and up to 16

@@ -1,7 +1,7 @@
 // RI 4-index assembly (Section 3, eq 14): (ij|kl) ~ sum_PQ (ij|P) [(PQ)^-1] (Q|kl).  The metric
 // (P|Q) is factored as L L^T (blocked right-looking Cholesky), B = L^-1 (P|ij) by blocked
-// forward substitution, and (ij|kl) = sum_R B[R][ij] B[R][kl], either to FP64 rounding on exact
-// digits (psq_fx.cuh, as the solve's off-diagonal products) or, for large blocks, to 2^-38
+// forward substitution, and (ij|kl) = sum_R B[R][ij] B[R][kl], either on exact digits, each element to
+// the precision of its terms (psq_fx.cuh, as the solve's off-diagonal products) or, for large blocks, to 2^-38
 // through the mixed path's packing and contraction.  The factor and the diagonal blocks stay on
 // the FP64 pipe.  Blocks of 32 rows; every loop bound is a size argument (no waits outside the
 // tensor-core products' bounded ones).
