@@ -23,12 +23,13 @@
 // peak at opposite ends of the window) and the running sum is below S as well (above it, what is
 // dropped stays below half a rounding of that sum), the element's window is summed by that chain
 // instead: none to one element in 10^5 on grids with whole cells per window, one in 10^3 to 10^2 on
-// coarse grids with cells of 27 or 45 points.  A column's chains are taken by the whole warp one after
-// the other, two points a lane, or by their own lanes where more than kTogether of the 32 rows ask.
-// Measured (no near bits, no chain -> now): bent triatomic 4.98 -> 5.14 ms, RI of 693 aux functions
-// 8.70 -> 8.53 ms, H2 unchanged, 2-centre Coulomb of 18 functions on 7.6 M points (tiles of few rows, bound by each
-// window's latency) 11.6 -> 13.6 ms; quintuple-zeta N-O on 8 x 6 x 3 cells of 5 x 3 x 3 points, (P|Q) and
-// (P|ij) 4.7 -> 7.9 ms (FP64 FMAs throughout: 28.0).
+// coarse grids with cells of 27 or 45 points, a quarter of the elements in the RI of a molecule's integrals
+// (whose rows are graded).
+// Measured (no near bits, no chain -> now): bent triatomic 4.95 -> 5.15 ms, RI of 693 aux functions
+// (random) 8.73 -> 8.61 ms, H2 unchanged, 2-centre Coulomb of 18 functions on 7.6 M points (tiles of few rows, bound by
+// each window's latency) 11.6 -> 13.6 ms; quintuple-zeta N-O on 8 x 6 x 3 cells of 5 x 3 x 3 points, (P|Q) and
+// (P|ij) 4.7 -> 8.6 ms (FP64 FMAs throughout: 28.0).  RI of CO's own integrals (178 aux functions, 3,600 pairs): block
+// 0.49 -> 2.3 ms, solve 0.31 -> 0.69 ms (FP64 FMAs: 4.2 and 0.51 ms).
 //
 // Rows with an infinity, a NaN or a value of 2^478 and above take the chain too (their products may
 // leave the range of the integer path).  Rows below 2^-959 (a steep function far out) are lifted by
@@ -52,7 +53,7 @@ constexpr int kThreads = 256;
 constexpr int kRows = 128, kCols = 32;  // tile of a CTA
 constexpr int kWin = 64;                // points per scale window
 constexpr int kDigits = 8;
-constexpr int kTogether = 8;            // chains of a column's 32 rows that the warp sums one by one, all lanes on each
+constexpr int kTogether = 16;           // chains of four columns that the warp sums one by one, all lanes on each
 constexpr uint32_t kTmemCols = kDigits * kCols;
 constexpr int kBigField = 1500;         // exponent field from which a row takes the FP64 chain
 constexpr int kLift = 200;              // power of two by which a row of tiny values is lifted
@@ -180,25 +181,41 @@ __device__ __forceinline__ int stored_field(uint32_t mx, bool lifted) {
 __device__ __forceinline__ uint32_t near_bits(uint32_t near, int E) { return E < kBigField ? near : (E == kZeros ? ~0u : 0u); }
 
 // The chains of a warp's 32 rows and 16 columns, added to its sums (bit j of apart: this lane's row with column
-// c0 + j): few of a column's rows one by one by all lanes, many by their own.  A function of its own,
-// on a copy of the sums, so that what it needs stays out of the window's registers.
+// c0 + j), four columns at a time: few of them one by one by all lanes (two points a lane), more by
+// their own lanes, four columns' operands in flight.  A function of its own, on a copy of the sums, so that
+// what it needs stays out of the window's registers.
 template <typename Chain>
 __device__ __noinline__ void chains(Chain chain, double* sums, uint32_t apart, int row0, int c0) {
   constexpr unsigned kFull = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  for (int j = 0; j < 16; ++j, apart >>= 1) {
-    uint32_t m = __ballot_sync(kFull, apart & 1);
-    if (__popc(m) > kTogether) {
-      if (apart & 1) sums[j] += chain(row0 + lane, c0 + j, 0, 1);
+#pragma unroll 1
+  for (int q = 0; q < 16; q += 4, apart >>= 4) {
+    uint32_t m[4];
+    int count = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      m[j] = __ballot_sync(kFull, apart >> j & 1);
+      count += __popc(m[j]);
+    }
+    if (count > kTogether) {
+      double s[4] = {};
+      if (apart & 15u) chain(row0 + lane, c0 + q, 0, 1, s);
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (apart >> j & 1) sums[q + j] += s[j];
       __syncwarp();
     } else {
-      for (; m; m &= m - 1) {
-        const int l = __ffs(m) - 1;
-        double s = chain(row0 + l, c0 + j, lane, 32);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
-        if (l == lane) sums[j] += s;
-      }
+      for (int j = 0; j < 4; ++j)
+#pragma unroll 1
+        for (; m[j]; m[j] &= m[j] - 1) {
+          const int l = __ffs(m[j]) - 1;
+          double s[1] = {};
+          chain(row0 + l, c0 + q + j, lane, 32, s);
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) s[0] += __shfl_xor_sync(kFull, s[0], o);
+          if (l == lane) sums[q + j] += s[0];
+        }
     }
   }
 }
@@ -206,7 +223,8 @@ __device__ __noinline__ void chains(Chain chain, double* sums, uint32_t apart, i
 // One window: the tile's accumulators (element row 32 (warp % 4) + lane, columns 16 (warp / 4) + j,
 // acc[j]) take sum_p a_r(p) b_c(p).  Only the first `rows` rows and `cols` columns are kept up
 // (8-row groups and 4-column groups past them are left out).  win: the windows done so far by this
-// CTA.  chain(row, col, p, step): the plain FP64 sum of the window's points p, p + step, ... for a row or column out of the integer
+// CTA.  chain(row, col, p, step, s): the plain FP64 sums of the window's points p, p + step, ... for a row and the
+// s's size of columns from col, for rows or columns out of the integer
 // path's range and for an element whose rows are not large at a common point.  ok turns false when a wait ran out (the caller ends its loop when the return
 // value, the same for all threads, is false, and asks all threads once more at the end).
 template <typename Chain>

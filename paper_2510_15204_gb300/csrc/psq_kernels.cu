@@ -604,7 +604,8 @@ __device__ __forceinline__ void contract_fma(const LaunchTables& t, const GemmIt
   }
 }
 
-// The plain sum of an item's points [from, to) for element (r, c) of its tile: fx::window's chain.
+// The plain sums of an item's points [from, to) for element (r, c) of its tile and the next columns:
+// fx::window's chain.
 struct ItemChain {
   const GemmItem* item;
   const GemmBlock* blocks;
@@ -612,23 +613,29 @@ struct ItemChain {
   const int2* pairs;
   const double* ops;
   int from, to;
-  __device__ __forceinline__ double operator()(int r, int c, int p0, int step) const {
+  template <int N>
+  __device__ __forceinline__ void operator()(int r, int c, int p0, int step, double (&s)[N]) const {
     const GemmBlock& b = blocks[item->block];
     const DevGrid& g = grids[b.grid];
     const int row = item->tm * kFpDigitRows + r, col = item->tn * kFpDigitCols + c;
-    if (row >= b.m || col >= b.n) return 0.0;
-    const int2 qa = pairs[b.a_off + row], qb = pairs[b.b_off + col];
+    if (row >= b.m || col >= b.n) return;
+    const int2 qa = pairs[b.a_off + row];
+    int2 qb[N];
+#pragma unroll
+    for (int j = 0; j < N; ++j) qb[j] = pairs[b.b_off + min(col + j, b.n - 1)];
     const int64_t rs = g.rs, ws = g.ws;
-    double s = 0.0;
 #pragma unroll 4
     for (int p = from + p0; p < to; p += step) {
       const double* at = ops + g.op_off + (int64_t)(p >> 7) * ws + (p & 127);
-      double x = at[qa.x * rs], y = at[qb.x * rs];
+      double x = at[qa.x * rs];
       if (qa.y >= 0) x *= at[qa.y * rs];
-      if (qb.y >= 0) y *= at[qb.y * rs];
-      s = fma(x, y, s);
+#pragma unroll
+      for (int j = 0; j < N; ++j) {
+        double y = at[qb[j].x * rs];
+        if (qb[j].y >= 0) y *= at[qb[j].y * rs];
+        s[j] = fma(x, y, s[j]);
+      }
     }
-    return s;
   }
 };
 

@@ -161,6 +161,29 @@ __global__ void finish_factor_kernel(int n, double* __restrict__ L) {
   }
 }
 
+// The plain sums of a window's products for row r and the columns from c (fx::window's chain): factor a of row r
+// and point p at a[p ap + r ar], factor b of column c at b[p bp + c bc].
+struct ProductChain {
+  const double* a;
+  int64_t ap, ar;
+  const double* b;
+  int64_t bp, bc;
+  int rows, cols, points;
+  template <int N>
+  __device__ __forceinline__ void operator()(int r, int c, int p0, int step, double (&s)[N]) const {
+    if (r >= rows || c >= cols) return;
+    int64_t col[N];
+#pragma unroll
+    for (int j = 0; j < N; ++j) col[j] = min(c + j, cols - 1) * bc;
+#pragma unroll 8
+    for (int p = p0; p < points; p += step) {
+      const double x = a[p * ap + r * ar];
+#pragma unroll
+      for (int j = 0; j < N; ++j) s[j] = fma(x, b[p * bp + col[j]], s[j]);
+    }
+  }
+};
+
 // Forward substitution B <- L^-1 B, left-looking, one launch: a CTA owns up to 128 columns and
 // walks down the 32-row blocks.  Block k's rows take sum_{q < 32 k} L[r][q] B[q][col] from the
 // tensor cores (fx::window: the columns are the tile's rows, the block's rows of L its columns),
@@ -196,12 +219,9 @@ __global__ void __launch_bounds__(fx::kThreads, 2) trsv_kernel(int n, int64_t m,
 #pragma unroll
         for (int i = 0; i < 4; ++i) vb[c][i] = fx::b_col() < kb && q0 + fx::b_pt(c) + i < k0 ? p[i] : 0.0;
       }
-      run = fx::window(sm, tmem, va, vb, acc, phase, win, live, kb, ok, [=](int r, int c, int at, int step) {
-        double s = 0.0;
-        if (r < live && c < kb)
-          for (int q = q0 + at; q < min(k0, q0 + fx::kWin); q += step) s = fma(B[(int64_t)q * m + c0 + r], L[(int64_t)(k0 + c) * n + q], s);
-        return s;
-      });
+      run = fx::window(sm, tmem, va, vb, acc, phase, win, live, kb, ok,
+                       ProductChain{B + (int64_t)q0 * m + c0, m, 1, L + (int64_t)k0 * n + q0, 1, n, live, kb,
+                                    min(k0 - q0, fx::kWin)});
     }
     if (k0 > 0 && run) run = __syncthreads_and(ok);  // and no MMA reads the planes any more
     if (!run) break;
@@ -340,13 +360,9 @@ __global__ void __launch_bounds__(fx::kThreads, 2) eri_kernel(int n, int64_t m, 
 #pragma unroll
       for (int i = 0; i < 4; ++i) vb[c][i] = fx::b_col() < cols && R0 + fx::b_pt(c) + i < n ? __ldg(p + i * m) : 0.0;
     }
-    run = fx::window(sm, tmem, va, vb, acc, phase, win, rows, cols, ok, [=](int r, int c, int at, int step) {
-      double s = 0.0;
-      if (r < rows && c < cols)
-        for (int R = R0 + at; R < min(n, R0 + fx::kWin); R += step)
-          s = fma(B[(int64_t)R * m + c0 + tc0 + r], B[(int64_t)R * m + d0 + td0 + c], s);
-      return s;
-    });
+    run = fx::window(sm, tmem, va, vb, acc, phase, win, rows, cols, ok,
+                     ProductChain{B + (int64_t)R0 * m + c0 + tc0, m, 1, B + (int64_t)R0 * m + d0 + td0, m, 1, rows, cols,
+                                  min(n - R0, fx::kWin)});
   }
   if (run) run = __syncthreads_and(ok);
   const int r = 32 * (warp & 3) + lane;
