@@ -7,8 +7,10 @@
 // tensor-core products' bounded ones).
 //
 // Measured (693 aux functions, 51,984 pairs; FP64-pipe kernels before -> exact digits now):
-// (ij|kl) block of 4096 x 4096 18.9 -> 1.81 ms (12.8 useful TFLOP/s, ten times the FP64 pipe's
-// nominal rate; ALU pipe 53% busy slicing, tensor pipe 20%), solve of all pairs 24.0 -> 5.0 ms.
+// (ij|kl) block of 4096 x 4096 18.9 -> 2.1 ms (10.9 useful TFLOP/s, nine times the FP64 pipe's
+// nominal rate; ALU pipe 56% busy slicing, tensor pipe 17%), solve of all pairs 24.0 -> 5.3 ms (FP64
+// pipe 56% with the diagonal blocks, ALU pipe 31%).  Random data; a molecule's own integrals, whose rows are
+// graded, take FP64 chains for a quarter of the elements (psq_fx.cuh).
 #include "psq_internal.h"
 #include "psq_fx.cuh"
 
